@@ -114,13 +114,25 @@ def _weight(g, N, K, std=0.02):
     return (std * torch.randn(N, K, device="cuda", generator=g)).to(torch.bfloat16)
 
 
-def _quantized_weight(W):
-    N, K = W.shape
-    wq = torch.empty(N, K // 2, dtype=torch.uint8, device="cuda")
-    sfw = torch.empty(B.sf_bytes(N, K, B.PQ_SF_TCGEN05), dtype=torch.uint8, device="cuda")
-    ts_w = torch.empty(1, dtype=torch.float32, device="cuda")
-    B.pq_quant_weight(W, None, None, wq, sfw, B.PQ_SF_TCGEN05, ts_w, B.workspace(B.OP_QUANT_WEIGHT, N, K))
-    return wq, sfw, ts_w
+def _hadamard(x, dtype):
+    """x (H_m (x) H_{2^n}) / sqrt(K) of every row, K = m 2^n with m = 1 or 12 (Paley's matrix of order 12)."""
+    M, K = x.shape
+    m = 12 if K % 3 == 0 else 1
+    y = x.to(dtype).view(M, m, K // m)
+    if m == 12:
+        squares = {i * i % 11 for i in range(1, 11)}
+        H = torch.eye(12, dtype=dtype)
+        for i in range(12):
+            for j in range(12):
+                if i != j:
+                    H[i, j] = 1.0 if i == 0 else -1.0 if j == 0 else (1.0 if (i - j) % 11 in squares else -1.0)
+        y = torch.einsum("rab,ac->rcb", y, H.to(x.device))
+    stride = 1
+    while stride < K // m:
+        y = y.reshape(M, -1, 2, stride)
+        y = torch.stack((y[:, :, 0] + y[:, :, 1], y[:, :, 0] - y[:, :, 1]), 2)
+        stride *= 2
+    return y.reshape(M, K) / math.sqrt(K)
 
 
 def _tensor_scale(t):
@@ -131,38 +143,58 @@ def _order(g, K):
     return torch.randperm(K, device="cuda", generator=g).to(torch.int32)
 
 
-def prepare(case, seed):
-    """Inputs, quantized weight and layer object a program holds before the call."""
+def _inputs(case, seed):
     g = torch.Generator(device="cuda")
     g.manual_seed(seed)
     kind, M, K = case["kind"], case["M"], case["K"]
     scale = _channel_scale(g, K, 2.0 if case.get("gelu") else 1.5, not case.get("gelu"))
-    if kind == "fakequant":
-        X = _activations(g, M, K, scale)
-        return dict(kind=kind, X=X, fmt=(B.KIND_INT, case["bits"], case["group"]),
-                    order=_order(g, K) if case["order"] else None, out=torch.empty_like(X))
-    N = case["N"]
+    t = dict(order=None)
     if kind == "calibrate":
-        fmt = pipeline.NVFP4 if case["bits"] == 0 else (B.KIND_INT, case["bits"], case["group"])
-        return dict(kind=kind, batches=[_activations(g, M, K, scale) for _ in range(case["batches"])], W=_weight(g, N, K), fmt=fmt)
-    wq, sfw, ts_w = _quantized_weight(_weight(g, N, K))
+        t["batches"] = [_activations(g, M, K, scale) for _ in range(case["batches"])]
+    else:
+        t["X"] = _activations(g, M, K, scale, case.get("gelu", False))
+    if kind == "fakequant":
+        t["order"] = _order(g, K) if case["order"] else None
+        return t
+    t["W"] = _weight(g, case["N"], K)
     if kind == "linear":
-        X = _activations(g, M, K, scale, case["gelu"])
-        return dict(kind=kind, X=X, layer=pipeline.QuantLinear(wq, sfw, ts_w, _tensor_scale(X), M))
+        t["ts_x"] = _tensor_scale(t["X"])
+    elif kind == "hadamard":
+        t["ts_x"] = _tensor_scale(_hadamard(t["X"], torch.float32))
+        t["order"] = _order(g, K)
+    elif kind == "norm":
+        rms = case["rms"]
+        t["a"] = 1.0 + 0.2 * torch.randn(K, device="cuda", generator=g) if rms else 0.2 * torch.randn(K, device="cuda", generator=g)
+        t["b"] = None if rms else 0.2 * torch.randn(K, device="cuda", generator=g)
+        t["order"] = _order(g, K) if case["order"] else None
+        x = t["X"].float()
+        t["ts_x"] = _tensor_scale(x / (x.square().mean(1, keepdim=True) + EPS).sqrt())  # stands in for the calibrated scale
+    return t
+
+
+def _format(case):
+    return pipeline.NVFP4 if case["bits"] == 0 else (B.KIND_INT, case["bits"], case["group"])
+
+
+def prepare(case, seed):
+    """Inputs, quantized weight and layer object a program holds before the call."""
+    kind, M, K = case["kind"], case["M"], case["K"]
+    t = _inputs(case, seed)
+    if kind == "fakequant":
+        return dict(kind=kind, X=t["X"], fmt=_format(case), order=t["order"], out=torch.empty_like(t["X"]))
+    if kind == "calibrate":
+        return dict(kind=kind, batches=t["batches"], W=t["W"], fmt=_format(case))
+    N = case["N"]
+    wq = torch.empty(N, K // 2, dtype=torch.uint8, device="cuda")
+    sfw = torch.empty(B.sf_bytes(N, K, B.PQ_SF_TCGEN05), dtype=torch.uint8, device="cuda")
+    ts_w = torch.empty(1, dtype=torch.float32, device="cuda")
+    B.pq_quant_weight(t["W"], None, None, wq, sfw, B.PQ_SF_TCGEN05, ts_w, B.workspace(B.OP_QUANT_WEIGHT, N, K))
+    if kind == "linear":
+        return dict(kind=kind, X=t["X"], layer=pipeline.QuantLinear(wq, sfw, ts_w, t["ts_x"], M))
     if kind == "hadamard":
-        X = _activations(g, M, K, scale)
-        basis = torch.empty_like(X)
-        B.pq_hadamard_quant_nvfp4(X, None, None, None, None, B.PQ_SF_LINEAR, basis)
-        return dict(kind=kind, X=X, layer=pipeline.QuantLinearH(wq, sfw, ts_w, _tensor_scale(basis), M, _order(g, K)))
-    H = _activations(g, M, K, scale)
-    rms = case["rms"]
-    a = 1.0 + 0.2 * torch.randn(K, device="cuda", generator=g) if rms else 0.2 * torch.randn(K, device="cuda", generator=g)
-    b = None if rms else 0.2 * torch.randn(K, device="cuda", generator=g)
-    order = _order(g, K) if case["order"] else None
-    x = H.float()
-    x = x / (x.square().mean(1, keepdim=True) + EPS).sqrt()  # its absmax stands in for the calibrated tensor scale
-    return dict(kind=kind, H=H, norm=B.NORM_RMS if rms else B.NORM_ADALN, a=a, b=b, order=order, ts_x=_tensor_scale(x),
-                codes=torch.empty(M, K // 2, dtype=torch.uint8, device="cuda"),
+        return dict(kind=kind, X=t["X"], layer=pipeline.QuantLinearH(wq, sfw, ts_w, t["ts_x"], M, t["order"]))
+    return dict(kind=kind, H=t["X"], norm=B.NORM_RMS if case["rms"] else B.NORM_ADALN, a=t["a"], b=t["b"], order=t["order"],
+                ts_x=t["ts_x"], codes=torch.empty(M, K // 2, dtype=torch.uint8, device="cuda"),
                 sf=torch.empty(B.sf_bytes(M, K, B.PQ_SF_TCGEN05), dtype=torch.uint8, device="cuda"),
                 wq=wq, sfw=sfw, ts_w=ts_w, Y=torch.empty(M, N, dtype=torch.bfloat16, device="cuda"),
                 ws=B.workspace(B.OP_GEMM, M, K, N))
@@ -183,6 +215,95 @@ def run(state):
     c = pipeline.calibrate(state["batches"], state["W"], fmt=state["fmt"])
     return dict(sumsq_a=c.sumsq_a, sumsq_w=c.sumsq_w, amax_a=c.amax_a, ts_x=c.ts_x, ts_w=c.ts_w, perms=c.perms, err_x=c.err_x,
                 err_w=c.err_w, lam=c.lam, E=c.E, select=c.select, wq=c.wq, sfw=c.sfw)
+
+
+# ------------------------------------------------------------------------------------------------- the same in 64 bits
+# The quantizers are defined in fp32 (scale = E4M3 or fp32 quotient, one reciprocal, one product per element), so a code
+# is taken from these operations; everything that is a sum, a product of decoded values or a transform is float64.
+_E2M1 = (0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0)
+
+
+def _decoded(x, ts, fmt):
+    """Quantized-dequantized values of fp32 rows x: (levels, decode scales), both float64, groups along the last dim."""
+    _, bits, group = fmt
+    xg = x.view(x.shape[0], -1, group)
+    amax = xg.abs().amax(-1, keepdim=True)
+    if fmt[0] == B.KIND_INT:
+        Q = float((1 << (bits - 1)) - 1)
+        d = amax / Q
+        z = torch.round(xg * torch.where(d > 0, 1.0 / d, 0.0)).clamp(-Q, Q)
+    else:
+        sf = (amax / (6.0 * ts)).clamp(max=448.0).to(torch.float8_e4m3fn).float()
+        d = sf * ts
+        y = xg * torch.where(d > 0, 1.0 / d, 0.0)
+        grid = torch.tensor(_E2M1, device=x.device)
+        mid = (grid[1:] + grid[:-1]) / 2
+        mag = y.abs().contiguous()
+        # nearest level; a midpoint goes to the code with the even number
+        lower, upper = torch.bucketize(mag, mid), torch.bucketize(mag, mid, right=True)
+        z = torch.where(y < 0, -1.0, 1.0) * grid[torch.where(upper % 2 == 0, upper, lower)]
+    return z.double(), d.double()
+
+
+def _decode(x, ts, fmt):
+    z, d = _decoded(x, ts, fmt)
+    return (z * d).view(x.shape)
+
+
+def _weight_ts(W):
+    return (W.abs().amax().float() / 2688.0).reshape(1)
+
+
+def _tensor_errors(x, ts, fmt, perms):
+    """Sum over the rows of the squared group errors, original order first, then every candidate: float64 [P + 1, K / g]."""
+    err = []
+    for perm in [None] + list(perms):
+        total = 0
+        for rows in x.split(4608):
+            v = (rows if perm is None else rows[:, perm.long()]).float()
+            z, d = _decoded(v, ts, fmt)
+            total = total + (v.double().view(z.shape) - z * d).square().sum((0, 2))
+        err.append(total)
+    return torch.stack(err)
+
+
+def exact(case, seed):
+    """What run returns for these inputs in float64; whole values (codes, scale bytes, orders, decisions) have no such value."""
+    t = _inputs(case, seed)
+    kind, K = case["kind"], case["K"]
+    if kind == "fakequant":
+        x = t["X"] if t["order"] is None else t["X"][:, t["order"].long()]
+        return _decode(x.float(), None, _format(case))
+    W = t["W"]
+    if kind == "calibrate":
+        fmt, J = _format(case), 5
+        x = torch.cat(t["batches"])
+        sa = sum(b.double().square().sum(0) for b in t["batches"])
+        sw = W.double().square().sum(0)
+        amax = x.abs().amax(0).float()
+        ts_x, ts_w = (amax.amax() / 2688.0).reshape(1), _weight_ts(W)
+        a, w = sa / x.shape[0], sw / W.shape[0]
+        perms = torch.stack([torch.argsort(a ** j * w ** (J - j), descending=True, stable=True) for j in range(J + 1)])
+        err_x, err_w = _tensor_errors(x, ts_x, fmt, perms), _tensor_errors(W, ts_w, fmt, perms)
+        lam = torch.stack((1.0 / sa.sum(), 1.0 / sw.sum()))
+        return dict(sumsq_a=sa, sumsq_w=sw, amax_a=amax.double(), ts_x=ts_x.double(), ts_w=ts_w.double(), perms=None, err_x=err_x,
+                    err_w=err_w, lam=lam, E=lam[0] * err_x.sum(1) + lam[1] * err_w.sum(1), select=None, wq=None, sfw=None)
+    x = t["X"]
+    if kind == "hadamard":
+        x = _hadamard(x, torch.float64)
+    elif kind == "norm":
+        x = x.double()
+        if case["rms"]:
+            x = x / (x.square().mean(1, keepdim=True) + EPS).sqrt()
+        else:
+            x = (x - x.mean(1, keepdim=True)) / (x.var(1, unbiased=False, keepdim=True) + EPS).sqrt()
+    if t["order"] is not None:
+        x = x[:, t["order"].long()]
+    if kind == "norm":
+        x = x * t["a"].double() if case["rms"] else x * (1.0 + t["a"].double()) + t["b"].double()
+    wd = _decode(W.float(), _weight_ts(W), pipeline.NVFP4).T
+    y = torch.cat([_decode(rows.float().contiguous(), t["ts_x"], pipeline.NVFP4) @ wd for rows in x.split(4608)])
+    return (y, None, None) if kind == "norm" else y
 
 
 # ------------------------------------------------------------------------------------------------- what a pass cannot do without

@@ -19,8 +19,6 @@
 
 namespace {
 
-constexpr int kErrThreads = 256;
-
 // ---------------------------------------------------------------- original order
 constexpr int kDirectThreads = 128;
 constexpr int kDirectRows = 4;  // rows in flight per thread (2 x 16 bytes each)
@@ -35,37 +33,12 @@ __device__ __forceinline__ void build_scale_table(float2 *table, float ts) {
     }
 }
 
-// Two fp32 lanes in one 64-bit register and the packed IEEE operations on them: one issue slot
-// for two results, each rounded exactly like the scalar instruction.
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
-__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
+using pq::add2;
+using pq::fma2;
+using pq::max_bf16x2;
+using pq::mul2;
+using pq::pack2;
+using pq::unpack2;
 
 // Error of one row's 16 channels held by this lane; TEAM16 = group / 16 adjacent lanes share a group.
 // c6 = 6 * ts (NVFP4 only).  The lane's two 8-channel runs are carried side by side in packed
@@ -190,100 +163,337 @@ group_error_direct(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int6
 }
 
 // ---------------------------------------------------------------- candidate orders
-// One block per (chunk of 16 rows, candidate order).  The chunk goes through shared memory four rows at a
-// time, interleaved per channel (8 bytes per channel: one 64-bit load gathers a channel for four rows, so a
-// random order costs a quarter of the shared-memory wavefronts of a row-by-row gather); the 16-byte pieces of
-// an octet are XOR-swizzled by bits of the octet index, which makes the transposing stores conflict-free.  A
-// thread owns whole 16-channel runs (GPT of them, blockDim apart), keeps their 16 channel positions packed
-// in registers for the whole chunk, and for every row rebuilds the two 16-byte words the original-order
-// kernel loads, so the error of a run is computed by the same routine, in row order.
-constexpr int kMaxGpt = 4;  // 256 threads x 4 runs x 16 channels = 16384 channels
+// A thread group (whole warps, one named barrier) owns a chunk of 16 rows.  It passes them through shared
+// memory four at a time as magnitudes, interleaved per channel, and runs every order of its block over the
+// staged rows before it fetches the next four: the staging is paid once for up to eight orders instead of
+// once per order.  A lane takes a run of 16 positions: its slots come from a table of 16-bit indices the
+// block prepared once per order, one 64-bit load per position brings that channel of four rows, and the
+// error of TWO ROWS is carried side by side in packed fp32 registers (row_pair_sse).  The words the gather
+// returns hold the same channel of two rows, so they are widened as they are; the one-row-at-a-time form
+// had to re-pair them by byte permutes first (half an instruction per element), read the original-order
+// kernel's decode tables (two per element; the hardware E2M1 -> f16 -> fp32 converts take one and a half)
+// and divide once per group and row (the scale tables below take a clamp and two loads).
+// Blocks are persistent, one per SM; the groups of a block only share the slot and scale tables.
+//
+// What bounds it: shared-memory wavefronts (a 64-bit gather through a random order takes about 6 of them
+// where 2 would do: 0.05 per element) and instruction issue, in about equal parts.
+constexpr int kGatherThreads = 768;  // 80 registers per thread; 960 threads at 64 spill
+constexpr int kMaxGroups = 15;                                           // named barriers 1..15
+constexpr int kSfTabMax = 2624;  // bf16 magnitudes from "scale byte 0" to "saturated": 19 binades and the edges
 
-__device__ __forceinline__ int quad_piece(int o, int k) { return 4 * o + (k ^ ((o >> 1) & 3)); }   // 16-byte piece k of octet o
-__device__ __forceinline__ uint32_t quad_channel(uint32_t c) { return c ^ (((c >> 4) & 3u) << 1); }  // 8-byte slot of channel c
+__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("min.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
 
-// one run per thread (up to 4096 channels): held to 64 registers, five 192-thread blocks per SM instead of four
-template <int KIND, int TEAM16, int GPT>
-__global__ void __launch_bounds__(kErrThreads, GPT == 1 ? 4 : 1)
-group_error_gather(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int64_t ld,
-                   const float *__restrict__ ts_ptr, float Qf, const int32_t *__restrict__ perms, int P,
-                   float *__restrict__ part /*[chunks, P, K/g]*/) {
-    extern __shared__ __align__(16) uint16_t quad_s[];  // [K][4 rows]
-    __shared__ float2 scale_table[KIND == 0 ? 256 : 1];
+// What a group's scale is looked up in, per side (activations / weight: they differ in the tensor scale).
+//   NVFP4    {1 / d, -d} for the decode scale d, as a function of the group's absmax, a bf16 magnitude: every magnitude
+//            up to `lo` gives scale byte 0 and every one from `hi` on the saturated byte, the ones between are
+//            tabulated from the definition.
+//   integer  s = amax / Q and 1 / s by the seven mantissa bits of amax, as bit patterns to which the exponent is
+//            added: scaling by a power of two commutes with both roundings while nothing is subnormal, i.e. for
+//            biased exponents kIntExpLo .. kIntExpHi (s >= 2^-125, 1/s >= 2^-124).
+struct ScaleTab {
+    float2 rd[kSfTabMax];
+    uint32_t lo, hi, pad[2];
+};
+constexpr uint32_t kIntExpLo = 9, kIntExpHi = 250;
+
+__device__ __forceinline__ float bf16_pattern(uint32_t a) { return __uint_as_float(a << 16); }
+
+__device__ __forceinline__ void build_scale_tab(ScaleTab &tab, float ts) {
+    const float c6 = __fmul_rn(6.0f, ts), mag = fabsf(c6);
+    // (signed) byte 0 up to |c6| 2^-10, half the smallest subnormal (ties to even); saturated from 448 |c6| on.  A
+    // zero c6 makes every quotient but 0 / 0 infinite; with an infinite or NaN one every decode scale is NaN.
+    uint32_t lo = 0, hi = 0;
+    if (mag == 0.0f) hi = 1;
+    else if (mag < __uint_as_float(0x7F800000u)) {
+        lo = __float_as_uint(__fmul_rz(mag, 0.0009765625f)) >> 16;
+        hi = min(0x7F80u, (__float_as_uint(__fmul_rn(mag, 448.0f)) >> 16) + 2u);
+    }
+    if (threadIdx.x == 0) tab.lo = lo, tab.hi = hi;
+    for (uint32_t i = threadIdx.x; i <= hi - lo && i < kSfTabMax; i += blockDim.x) {
+        const float d = __fmul_rn(pq::e4m3_to_f32(pq::f32_to_e4m3(__fdiv_rn(bf16_pattern(lo + i), c6))), ts);
+        tab.rd[i] = make_float2(d > 0.0f ? __frcp_rn(d) : 0.0f, -d);
+    }
+}
+__device__ __forceinline__ void build_int_tab(uint2 *tab, float Qf) {
+    for (uint32_t m = threadIdx.x; m < 128; m += blockDim.x) {
+        const float s = __fdiv_rn(__uint_as_float(0x3F800000u | (m << 16)), Qf);
+        tab[m] = make_uint2(__float_as_uint(__frcp_rn(s)) + (127u << 23),
+                            __float_as_uint(s) - (127u << 23) + 0x80000000u);  // mod 2^32: -s once the exponent is added
+    }
+}
+
+// E2M1 of the two floats of a pair and back to fp32 (E2M1 -> f16 is exact, f16 -> f32 too).
+__device__ __forceinline__ uint64_t e2m1_pair(uint64_t y2) {
+    float lo, hi;
+    unpack2(y2, lo, hi);
+    uint32_t h2;
+    asm("{\n"
+        ".reg .b8 c;\n"
+        "cvt.rn.satfinite.e2m1x2.f32 c, %2, %1;\n"
+        "cvt.rn.f16x2.e2m1x2 %0, c;\n"
+        "}\n"
+        : "=r"(h2)
+        : "f"(lo), "f"(hi));
+    return pack2(__half2float(__ushort_as_half(static_cast<uint16_t>(h2 & 0xFFFFu))),
+                 __half2float(__ushort_as_half(static_cast<uint16_t>(h2 >> 16))));
+}
+
+// One row of a pair by the definition of the integer formats: for scales in subnormal or non-finite territory.
+struct RunWords {
+    uint32_t u[16];
+};
+template <int TEAM16>
+__device__ __noinline__ float int_row_sse_words(const RunWords words, int row, float amax, float Qf) {
+    float d, rc, run[2];
+    pq::int_scale(amax, Qf, d, rc);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        run[h] = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t w = words.u[8 * h + i];
+            const float x = __uint_as_float(row ? w & 0xFFFF0000u : w << 16);
+            const float z = fminf(__fadd_rn(__fadd_rn(__fmul_rn(x, rc), 12582912.0f), -12582912.0f), Qf);
+            const float delta = __fmaf_rn(-z, d, x);
+            run[h] = __fmaf_rn(delta, delta, run[h]);
+        }
+    }
+    return pq::team_sum<TEAM16>(__fadd_rn(run[0], run[1]));
+}
+template <int TEAM16>
+__device__ __forceinline__ float int_row_sse(const uint32_t (&u)[16], int row, float amax, float Qf) {
+    RunWords words;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) words.u[i] = u[i];
+    return int_row_sse_words<TEAM16>(words, row, amax, Qf);
+}
+
+// Errors of a run of 16 positions in two rows: u[i] = magnitudes of position i in row 0 (low half) and row 1
+// (high half).  Per row the operations and their order are those of row_sse16.
+template <int KIND, int TEAM16>
+__device__ __forceinline__ void row_pair_sse(const uint32_t (&u)[16], const ScaleTab *tab, uint32_t lo2, uint32_t hi2,
+                                             const uint2 *int_tab, float Qf, float &e0, float &e1) {
+    // absmax of both rows at once (a maximum of magnitudes selects one of its inputs)
+    uint32_t mx[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mx[i] = max_bf16x2(u[i], u[i + 8]);
+#pragma unroll
+    for (int s = 4; s; s >>= 1)
+#pragma unroll
+        for (int i = 0; i < s; ++i) mx[i] = max_bf16x2(mx[i], mx[i + s]);
+    uint32_t am = mx[0];
+#pragma unroll
+    for (int m = 1; m < TEAM16; m <<= 1) am = max_bf16x2(am, __shfl_xor_sync(0xFFFFFFFFu, am, m));
+    uint64_t r2, nd2;
+    if (KIND == 0) {
+        const uint32_t cl = min_u16x2(max_u16x2(am, lo2), hi2);
+        const float2 *rd = tab->rd - (lo2 & 0xFFFFu);
+        const float2 d0 = rd[cl & 0xFFFFu], d1 = rd[cl >> 16];
+        r2 = pack2(d0.x, d1.x), nd2 = pack2(d0.y, d1.y);
+    } else {
+        const uint32_t a0 = am & 0xFFFFu, a1 = am >> 16;
+        // an all-zero group may use any finite scale: its levels and residuals are zero
+        const bool odd0 = a0 != 0u && a0 - (kIntExpLo << 7) >= ((kIntExpHi - kIntExpLo + 1u) << 7);
+        const bool odd1 = a1 != 0u && a1 - (kIntExpLo << 7) >= ((kIntExpHi - kIntExpLo + 1u) << 7);
+        if (__any_sync(0xFFFFFFFFu, odd0 || odd1)) {
+            e0 = int_row_sse<TEAM16>(u, 0, bf16_pattern(a0), Qf), e1 = int_row_sse<TEAM16>(u, 1, bf16_pattern(a1), Qf);
+            return;
+        }
+        const uint32_t c0 = max(a0, kIntExpLo << 7), c1 = max(a1, kIntExpLo << 7);
+        const uint2 t0 = int_tab[c0 & 0x7Fu], t1 = int_tab[c1 & 0x7Fu];
+        const uint32_t x0 = (c0 & 0x7F80u) << 16, x1 = (c1 & 0x7F80u) << 16;
+        r2 = pack2(__uint_as_float(t0.x - x0), __uint_as_float(t1.x - x1));
+        nd2 = pack2(__uint_as_float(t0.y + x0), __uint_as_float(t1.y + x1));
+    }
+
+    uint64_t run2[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint64_t acc2 = 0;  // {+0, +0}
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t w = u[8 * h + i];
+            const uint64_t x2 = pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+            const uint64_t y2 = mul2(x2, r2);
+            uint64_t q2;
+            if (KIND == 0) {
+                q2 = e2m1_pair(y2);
+            } else {
+                // rint by adding and subtracting 1.5 * 2^23 (see row_sse16 for the form of the first addition).  No clamp:
+                // |x| / s <= Q (1 + 2^-22) here, which rounds to Q at most.
+                const uint64_t magic = pack2(12582912.0f, 12582912.0f), unmagic = pack2(-12582912.0f, -12582912.0f);
+                q2 = add2(fma2(y2, pack2(1.0f, 1.0f), magic), unmagic);
+            }
+            const uint64_t delta = fma2(q2, nd2, x2);
+            acc2 = fma2(delta, delta, acc2);
+        }
+        run2[h] = acc2;
+    }
+    float s0, s1;
+    unpack2(add2(run2[0], run2[1]), s0, s1);
+    e0 = pq::team_sum<TEAM16>(s0), e1 = pq::team_sum<TEAM16>(s1);
+}
+
+struct GatherParams {
+    const uint16_t *T;
+    int64_t rows, ld;
+    const float *ts;
+    int K, P;                  // P orders
+    const int32_t *perms;      // [P, K]
+    int opb;                   // orders per block (blockIdx.y picks the subset)
+    int groups, group_threads;
+    int64_t chunks;
+    float Qf;
+    float *part;               // [chunks, P, K/g]
+};
+
+constexpr int kTabBytes = (static_cast<int>(sizeof(ScaleTab)) + 15) / 16 * 16;
+
+inline size_t gather_smem_bytes(int64_t K, int opb, int groups) {
+    return static_cast<size_t>(groups) * K * 8 + static_cast<size_t>(opb) * K * 2 +
+           static_cast<size_t>(groups) * opb * (K / 16) * 4 + kTabBytes;
+}
+
+template <int KIND, int TEAM16>
+__global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __grid_constant__ GatherParams p) {
+    // [groups][K][4 rows] bf16 magnitudes | [opb][K] 16-bit slots | scale tables | [groups][opb][runs] fp32 chunk sums
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int K = p.K, octs = K >> 3, runs = K >> 4;
+    const int o0 = blockIdx.y * p.opb, no = min(p.opb, p.P - o0);
+    uint16_t *slot_s = reinterpret_cast<uint16_t *>(smem + static_cast<size_t>(p.groups) * K * 8);
+    unsigned char *tab_s = reinterpret_cast<unsigned char *>(slot_s + static_cast<size_t>(p.opb) * K);
+    ScaleTab *tab = reinterpret_cast<ScaleTab *>(tab_s);
+    uint2 *int_tab = reinterpret_cast<uint2 *>(tab_s);
     pq::dependents_may_launch();
-    const int64_t chunk = blockIdx.x;
-    const int p = blockIdx.y;
-    const int32_t *perm = perms + static_cast<int64_t>(p) * K;
-    const int octs = static_cast<int>(K >> 3), runs = static_cast<int>(K >> 4);
-    const int64_t r0 = chunk * PQ_CHUNK_ROWS;
-    const float ts = (KIND == 0) ? __ldg(ts_ptr) : 1.0f;
-    const float c6 = __fmul_rn(6.0f, ts);
-    if (KIND == 0) build_scale_table(scale_table, ts);  // the first barrier below publishes it
+    pq::wait_for_prior_grid();
 
-    // positions of this thread's channels in the interleaved image, two per register
-    uint32_t ch[GPT][8];
-    float acc[GPT];
-#pragma unroll
-    for (int t = 0; t < GPT; ++t) {
-        acc[t] = 0.0f;
-        const int q = threadIdx.x + t * blockDim.x;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            uint32_t lo = 0, hi = 0;
-            if (q < runs) {
-                lo = quad_channel(static_cast<uint32_t>(perm[q * 16 + 2 * w]));
-                hi = quad_channel(static_cast<uint32_t>(perm[q * 16 + 2 * w + 1]));
-            }
-            ch[t][w] = lo | (hi << 16);
-        }
+    const int32_t *perm = p.perms + static_cast<int64_t>(o0) * K;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < no * K; i += blockDim.x) {
+        const int o = i / K, j = i - o * K;
+        // the two 16-byte halves of a run's slots lie in separate planes: lanes read consecutive 16-byte words
+        slot_s[o * K + ((j >> 3) & 1) * (K >> 1) + (j >> 4) * 8 + (j & 7)] = static_cast<uint16_t>(pq::quad_channel(__ldg(perm + i)));
     }
+    const float ts = KIND == 0 ? __ldg(p.ts) : 1.0f;
+    if (KIND == 0) build_scale_tab(*tab, ts);
+    else build_int_tab(int_tab, p.Qf);
+    __syncthreads();
 
-    uint4 *quad4 = reinterpret_cast<uint4 *>(quad_s);
-    const uint2 *quad2 = reinterpret_cast<const uint2 *>(quad_s);
-#pragma unroll 1
-    for (int quad = 0; quad < PQ_CHUNK_ROWS / 4; ++quad) {
-        const int64_t row = r0 + 4 * quad;
-        __syncthreads();  // the previous four rows have been used
-        for (int o = threadIdx.x; o < octs; o += blockDim.x) {
-            uint4 v[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)  // rows past the end are zeros: their error is +0.0 and adding it changes nothing
-                v[r] = row + r < rows ? __ldg(reinterpret_cast<const uint4 *>(T + (row + r) * ld) + o) : make_uint4(0, 0, 0, 0);
-            const uint32_t *w0 = &v[0].x, *w1 = &v[1].x, *w2 = &v[2].x, *w3 = &v[3].x;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                quad4[quad_piece(o, k)] = make_uint4(__byte_perm(w0[k], w1[k], 0x5410), __byte_perm(w2[k], w3[k], 0x5410),
-                                                     __byte_perm(w0[k], w1[k], 0x7632), __byte_perm(w2[k], w3[k], 0x7632));
-        }
-        __syncthreads();
-#pragma unroll
-        for (int t = 0; t < GPT; ++t) {
-            if (t * static_cast<int>(blockDim.x) >= runs) break;  // uniform over the block
-            uint2 g[16];
-#pragma unroll
-            for (int w = 0; w < 8; ++w) {
-                g[2 * w] = quad2[ch[t][w] & 0xFFFFu];
-                g[2 * w + 1] = quad2[ch[t][w] >> 16];
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                uint32_t pr[8];
-#pragma unroll
-                for (int w = 0; w < 8; ++w) {
-                    const uint32_t a = r < 2 ? g[2 * w].x : g[2 * w].y, b = r < 2 ? g[2 * w + 1].x : g[2 * w + 1].y;
-                    pr[w] = __byte_perm(a, b, (r & 1) ? 0x7632 : 0x5410);
-                }
-                acc[t] = __fadd_rn(acc[t], row_sse16<KIND, TEAM16>(make_uint4(pr[0], pr[1], pr[2], pr[3]),
-                                                                   make_uint4(pr[4], pr[5], pr[6], pr[7]), c6, scale_table, Qf));
-            }
-        }
-    }
+    const int grp = threadIdx.x / p.group_threads, tid = threadIdx.x - grp * p.group_threads;
+    if (grp >= p.groups) return;
+    auto group_sync = [&]() {
+        if (p.group_threads == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(p.group_threads) : "memory");
+    };
+    uint4 *quad4 = reinterpret_cast<uint4 *>(smem + static_cast<size_t>(grp) * K * 8);
+    const uint32_t quad_addr = static_cast<uint32_t>(__cvta_generic_to_shared(quad4));
+    float *acc_s = reinterpret_cast<float *>(tab_s + kTabBytes) + static_cast<size_t>(grp) * p.opb * runs;
+    const uint4 *slot4 = reinterpret_cast<const uint4 *>(slot_s);
+    const uint32_t lo2 = KIND == 0 ? tab->lo * 0x10001u : 0u, hi2 = KIND == 0 ? tab->hi * 0x10001u : 0u;
     const int64_t Kg = runs / TEAM16;
+
+    for (int64_t chunk = static_cast<int64_t>(blockIdx.x) * p.groups + grp; chunk < p.chunks;
+         chunk += static_cast<int64_t>(gridDim.x) * p.groups) {
+        const int64_t r0 = chunk * PQ_CHUNK_ROWS;
+#pragma unroll 1
+        for (int quad = 0; quad < PQ_CHUNK_ROWS / 4; ++quad) {
+            const int64_t row = r0 + 4 * quad;
+            if (row >= p.rows) break;  // no rows left: their error is +0.0
+            group_sync();              // the previous four rows have been used
+            const uint16_t *src = p.T + row * p.ld;
+#pragma unroll 2
+            for (int o = tid; o < octs; o += p.group_threads) {
+                uint4 v[4];
 #pragma unroll
-    for (int t = 0; t < GPT; ++t) {
-        const int q = threadIdx.x + t * blockDim.x;
-        if (q < runs && (q % TEAM16) == 0) part[(chunk * P + p) * Kg + q / TEAM16] = acc[t];
+                for (int r = 0; r < 4; ++r) {  // rows past the end are zeros: their error is +0.0 and adding it changes nothing
+                    v[r] = row + r < p.rows ? __ldg(reinterpret_cast<const uint4 *>(src + r * p.ld) + o) : make_uint4(0, 0, 0, 0);
+                    v[r].x &= 0x7FFF7FFFu, v[r].y &= 0x7FFF7FFFu, v[r].z &= 0x7FFF7FFFu, v[r].w &= 0x7FFF7FFFu;
+                }
+                pq::store_quad_octet(quad4, o, v);
+            }
+            group_sync();
+#pragma unroll 1
+            for (int o = 0; o < no; ++o) {
+#pragma unroll 1
+                for (int q0 = 0; q0 < runs; q0 += p.group_threads) {
+                    const int q = q0 + tid;
+                    const bool live = q < runs;  // runs % TEAM16 == 0: a team is live or dead as a whole
+                    const int at = o * (K >> 3) + (live ? q : 0);
+                    const uint4 i0 = slot4[at], i1 = slot4[at + runs];
+                    const uint32_t iw[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
+                    uint32_t lo[16], hi[16];
+#pragma unroll
+                    for (int w = 0; w < 8; ++w) {
+                        // byte address 8 * slot + base of either half of the word: one dot product each
+                        const uint32_t x = __dp2a_lo(iw[w], 0x0008u, quad_addr), y = __dp2a_lo(iw[w], 0x0800u, quad_addr);
+                        asm("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(lo[2 * w]), "=r"(hi[2 * w]) : "r"(x) : "memory");
+                        asm("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(lo[2 * w + 1]), "=r"(hi[2 * w + 1]) : "r"(y) : "memory");
+                    }
+                    float e0, e1, e2, e3;
+                    row_pair_sse<KIND, TEAM16>(lo, tab, lo2, hi2, int_tab, p.Qf, e0, e1);
+                    row_pair_sse<KIND, TEAM16>(hi, tab, lo2, hi2, int_tab, p.Qf, e2, e3);
+                    if (live) {
+                        float acc = quad ? acc_s[o * runs + q] : 0.0f;
+                        acc = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(acc, e0), e1), e2), e3);
+                        acc_s[o * runs + q] = acc;
+                    }
+                }
+            }
+        }
+        // every thread writes out the sums it kept itself
+        for (int o = 0; o < no; ++o)
+            for (int q = tid; q < runs; q += p.group_threads)
+                if ((q % TEAM16) == 0) p.part[(chunk * p.P + o0 + o) * Kg + q / TEAM16] = acc_s[o * runs + q];
     }
+}
+
+// Orders per block, groups per block and threads per group for `chunks` chunks of K channels under P orders:
+// the configuration with the shortest estimated schedule.  A group of W warps works through
+// ceil(chunks * subsets / (blocks * groups)) chunks; a chunk costs one unit per order and run of each
+// lane, plus about a quarter of a unit of staging per run; an SM is taken to be saturated by 20 warps, fewer
+// are proportionally slower.
+struct GatherConfig {
+    int opb = 0, groups = 0, group_threads = 0;
+};
+inline GatherConfig gather_config(int64_t chunks, int64_t K, int P, int sms) {
+    GatherConfig best;
+    double best_cost = 0.0;
+    const int runs = static_cast<int>(K / 16);
+    for (int per_lane = 1; per_lane <= 4; ++per_lane) {
+        const int threads = static_cast<int>(pq_ceil_div(pq_ceil_div(runs, per_lane), 32)) * 32;
+        if (threads > kGatherThreads) continue;
+        for (int opb = 1; opb <= P; ++opb) {
+            const int64_t subsets = pq_ceil_div(P, opb);
+            for (int groups = 1; groups <= kMaxGroups && groups * threads <= kGatherThreads; ++groups) {
+                if (gather_smem_bytes(K, opb, groups) > 226 * 1024) break;
+                const int64_t blocks = sms / subsets > 0 ? sms / subsets : 1;
+                const int64_t rounds = pq_ceil_div(chunks, blocks * groups);
+                const int warps = groups * threads / 32;
+                const double cost = static_cast<double>(rounds) * threads * groups * per_lane * (opb + 0.25) * (warps < 20 ? 20.0 / warps : 1.0);
+                if (!best.groups || cost < best_cost) {
+                    best_cost = cost;
+                    best.opb = opb, best.groups = groups, best.group_threads = threads;
+                }
+            }
+        }
+        if (threads <= 32) break;
+    }
+    return best;
+}
+
+int sm_count() {
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
 }
 
 template <typename PT, int PER_SLAB>
@@ -303,24 +513,21 @@ pq_status launch(const uint16_t *T, int64_t rows, int64_t K, int64_t ld, const f
         if (pq_launch_status() != PQ_OK) return PQ_ERR_CUDA;
         return fold<double, 1>(ws, slabs, Kg, err, st);
     }
-    const int runs = static_cast<int>(K >> 4);
-    const int threads = runs >= kErrThreads ? kErrThreads : ((runs + 31) / 32) * 32;
-    const int gpt = static_cast<int>(pq_ceil_div(runs, threads));
-    if (gpt > kMaxGpt) return PQ_ERR_SHAPE;
-    const size_t smem = static_cast<size_t>(K) * 8;  // four rows, interleaved per channel
-    dim3 grid(static_cast<unsigned>(chunks), static_cast<unsigned>(P));
-    auto run = [&](auto kern) -> pq_status {
-        if (smem > 40 * 1024)  // the kernel's static shared memory counts towards the 48 KB default limit
-            PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        kern<<<grid, threads, smem, st>>>(T, rows, K, ld, ts, Qf, perms, P, static_cast<float *>(ws));
-        return PQ_OK;
-    };
-    constexpr int TEAM16 = TEAM / 2;
-    const pq_status rl = gpt == 1   ? run(group_error_gather<KIND, TEAM16, 1>)
-                         : gpt == 2 ? run(group_error_gather<KIND, TEAM16, 2>)
-                                    : run(group_error_gather<KIND, TEAM16, 4>);
-    if (rl != PQ_OK) return rl;
-    if (pq_launch_status() != PQ_OK) return PQ_ERR_CUDA;
+    const int sms = sm_count();
+    const GatherConfig cfg = gather_config(chunks, K, P, sms);
+    if (!cfg.groups) return PQ_ERR_SHAPE;
+    GatherParams p;
+    p.T = T, p.rows = rows, p.ld = ld, p.ts = ts, p.K = static_cast<int>(K), p.P = P, p.perms = perms;
+    p.opb = cfg.opb, p.groups = cfg.groups, p.group_threads = cfg.group_threads;
+    p.chunks = chunks, p.Qf = Qf, p.part = static_cast<float *>(ws);
+    const int64_t subsets = pq_ceil_div(P, cfg.opb), share = sms / subsets > 0 ? sms / subsets : 1;
+    const int64_t want = pq_ceil_div(chunks, cfg.groups);
+    const size_t smem = gather_smem_bytes(K, cfg.opb, cfg.groups);
+    auto kern = group_error_gather<KIND, TEAM / 2>;
+    if (smem > 48 * 1024)
+        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(want < share ? want : share), static_cast<unsigned>(subsets)),
+                                    dim3(static_cast<unsigned>(cfg.groups * cfg.group_threads)), smem, st, p));
     return fold<float, kSlabChunks>(ws, chunks, static_cast<int64_t>(P) * Kg, err, st);
 }
 

@@ -255,6 +255,25 @@ pq_status pq_quant_weight(const void *Wt, int64_t N, int64_t K, int64_t ld, cons
                           const int32_t *perm_select, uint8_t *codes, uint8_t *sf, int sf_layout,
                           float *ts_w, void *ws, size_t ws_bytes, void *stream);
 
+/* The offline pass of a layer in one call: pq_calib_stats over every batch and the weight, both tensor
+ * scales, pq_select_perm, pq_group_error of the original order and of the J + 1 candidates over every batch
+ * and the weight, pq_error_weights, pq_accept and pq_quant_weight -- the same results bit for bit, in a few
+ * launches that walk over all tensors at once.  Everything is enqueued on `stream`, nothing is read back.
+ *   X, rows, ld : host arrays of n device pointers (bf16 [rows[i], K], ld[i]) and their sizes; n >= 1.
+ *   Wt          : bf16 [N, K], ldw.   fmt : the format whose error drives the decision.   1 <= J <= 7.
+ *   outputs     : as of the calls named above, overwritten (nothing has to be zeroed): sumsq_a, sumsq_w
+ *                 fp64 [K], amax_a fp32 [K], ts_x, ts_w fp32 scalars, perms int32 [J+1, K], err_x, err_w
+ *                 fp64 [J+2, K/g] (row 0 = original order), lambda fp64 [2], E fp64 [J+2] or NULL,
+ *                 select int32 [2] = {best, accept}, codes / sf of the weight in the chosen order.
+ *   ws          : pq_calibrate_workspace_bytes(n, rows, N, K, fmt, J), 256-byte aligned (0 on bad input). */
+size_t pq_calibrate_workspace_bytes(int n, const int64_t *rows, int64_t N, int64_t K, pq_format fmt, int J);
+pq_status pq_calibrate(int n, const void *const *X, const int64_t *rows, const int64_t *ld, const void *Wt,
+                       int64_t N, int64_t K, int64_t ldw, pq_format fmt, int J, double tau, int sf_layout,
+                       double *sumsq_a, double *sumsq_w, float *amax_a, float *ts_x, float *ts_w,
+                       int32_t *perms, double *err_x, double *err_w, double *lambda, double *E,
+                       int32_t *select, uint8_t *codes, uint8_t *sf, void *ws, size_t ws_bytes,
+                       void *stream);
+
 /* Runtime activation quantizer (dynamic per-group scales, static tensor scale *ts_x from
  * calibration).  Per row and 16-channel group: absmax -> E4M3(absmax / (6 ts)) -> 16 E2M1 codes
  * of x / (scale * ts), round to nearest even, saturating.  Channels arrive already permuted.

@@ -53,6 +53,9 @@ _SIGNATURES = {
     "pq_error_weights": (_int, [_vp, _vp, _i64, _vp, _vp]),
     "pq_accept": (_int, [_vp, _vp, _vp, _int, _i64, C.c_double, _vp, _vp, _vp, _vp]),
     "pq_quant_weight": (_int, [_vp, _i64, _i64, _i64, _vp, _vp, _vp, _vp, _int, _vp, _vp, _sz, _vp]),
+    "pq_calibrate_workspace_bytes": (_sz, [_int, _vp, _i64, _i64, pq_format, _int]),
+    "pq_calibrate": (_int, [_int, _vp, _vp, _vp, _vp, _i64, _i64, _i64, pq_format, _int, C.c_double, _int] + [_vp] * 14
+                     + [_sz, _vp]),
     "pq_quant_act_nvfp4": (_int, [_vp, _i64, _i64, _i64, _vp, _vp, _vp, _int, _vp]),
     "pq_gemm_w4a4": (_int, [_vp, _vp, _vp, _vp, _vp, _vp, _i64, _i64, _i64, _vp, _i64, _vp, _sz, _vp]),
     "pq_linear_w4a4": (_int, [_vp, _i64, _i64, _i64, _vp, _vp, _vp, _vp, _vp, _vp, _i64, _vp, _i64,
@@ -248,6 +251,27 @@ def pq_quant_weight(Wt, perm, perm_select, codes, sf, sf_layout, ts_w, ws):
     _check("pq_quant_weight", lib().pq_quant_weight(_p(Wt), Wt.shape[0], Wt.shape[1], Wt.stride(0), _p(perm),
                                                     _p(perm_select), _p(codes), _p(sf), sf_layout, _p(ts_w),
                                                     w, wb, _stream()))
+
+
+def pq_calibrate(Xs, Wt, fmt, J, tau, sf_layout, sumsq_a, sumsq_w, amax_a, ts_x, ts_w, perms, err_x, err_w, lam, E, select,
+                 codes, sf):
+    """The offline pass over the batches Xs (list of bf16 [T, K]) and the weight Wt; the outputs are overwritten."""
+    n, (N, K) = len(Xs), _bf16(Wt).shape
+    for x in Xs:
+        assert _bf16(x).shape[1] == K and x.is_cuda, "device tensors of the weight's width only"
+    f64, f32, i32 = torch.float64, torch.float32, torch.int32
+    for t, dtype in ((sumsq_a, f64), (sumsq_w, f64), (amax_a, f32), (ts_x, f32), (ts_w, f32), (perms, i32), (err_x, f64),
+                     (err_w, f64), (lam, f64), (E, f64), (select, i32), (codes, torch.uint8), (sf, torch.uint8)):
+        assert t.dtype == dtype and t.is_contiguous()
+    ptrs = (C.c_void_p * n)(*[x.data_ptr() for x in Xs])
+    rows, lds = (C.c_int64 * n)(*[x.shape[0] for x in Xs]), (C.c_int64 * n)(*[x.stride(0) for x in Xs])
+    form = pq_format(*fmt)
+    need = int(lib().pq_calibrate_workspace_bytes(n, rows, N, K, form, J))
+    ws = torch.empty(max(need, 256), dtype=torch.uint8, device=Wt.device)
+    _check("pq_calibrate", lib().pq_calibrate(
+        n, ptrs, rows, lds, _p(Wt), N, K, Wt.stride(0), form, J, float(tau), sf_layout, _p(sumsq_a), _p(sumsq_w), _p(amax_a),
+        _p(ts_x), _p(ts_w), _p(perms), _p(err_x), _p(err_w), _p(lam), _p(E), _p(select), _p(codes), _p(sf), _p(ws), ws.numel(),
+        _stream()))
 
 
 def pq_quant_act_nvfp4(X, ts_x, codes, sf, sf_layout):

@@ -15,6 +15,8 @@
 //     at a time, interleaved per channel, and a thread gathers the 16 channels of its run for four rows
 //     with 64-bit loads, then runs the original-order kernel's error routine on them; the tensor is
 //     fetched from HBM once per chunk and served from L2 to the other orders' blocks.
+#include <type_traits>
+
 #include "pq_common.cuh"
 
 namespace {
@@ -344,78 +346,88 @@ __device__ __forceinline__ void row_pair_sse(const uint32_t (&u)[16], const Scal
 }
 
 struct GatherParams {
-    const uint16_t *T;
-    int64_t rows, ld;
-    const float *ts;
-    int K, P;                  // P orders
-    const int32_t *perms;      // [P, K]
+    PqTensorList list;
+    const float *ts[2];        // tensor scale per side (NVFP4)
+    int K, P, identity;        // P orders; identity != 0: order 0 is the original one and perms holds the others
+    const int32_t *perms;      // [P - identity, K]
     int opb;                   // orders per block (blockIdx.y picks the subset)
     int groups, group_threads;
-    int64_t chunks;
+    int chunks;                // eight per slab; the chunks of a last slab that hold no rows may be left out
     float Qf;
     float *part;               // [chunks, P, K/g]
+    PqErrorWeights weights;    // added up by one more warp of the block(s) in front, behind the gather's back
 };
 
 constexpr int kTabBytes = (static_cast<int>(sizeof(ScaleTab)) + 15) / 16 * 16;
 
-inline size_t gather_smem_bytes(int64_t K, int opb, int groups) {
+inline size_t gather_smem_bytes(int64_t K, int opb, int groups, int sides) {
     return static_cast<size_t>(groups) * K * 8 + static_cast<size_t>(opb) * K * 2 +
-           static_cast<size_t>(groups) * opb * (K / 16) * 4 + kTabBytes;
+           static_cast<size_t>(groups) * opb * (K / 16) * 4 + static_cast<size_t>(sides) * kTabBytes;
 }
 
 template <int KIND, int TEAM16>
-__global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __grid_constant__ GatherParams p) {
+__global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(const __grid_constant__ GatherParams p) {
     // [groups][K][4 rows] bf16 magnitudes | [opb][K] 16-bit slots | scale tables | [groups][opb][runs] fp32 chunk sums
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.K, octs = K >> 3, runs = K >> 4;
     const int o0 = blockIdx.y * p.opb, no = min(p.opb, p.P - o0);
     uint16_t *slot_s = reinterpret_cast<uint16_t *>(smem + static_cast<size_t>(p.groups) * K * 8);
     unsigned char *tab_s = reinterpret_cast<unsigned char *>(slot_s + static_cast<size_t>(p.opb) * K);
-    ScaleTab *tab = reinterpret_cast<ScaleTab *>(tab_s);
     uint2 *int_tab = reinterpret_cast<uint2 *>(tab_s);
     pq::dependents_may_launch();
     pq::wait_for_prior_grid();
 
-    const int32_t *perm = p.perms + static_cast<int64_t>(o0) * K;
-#pragma unroll 4
     for (int i = threadIdx.x; i < no * K; i += blockDim.x) {
-        const int o = i / K, j = i - o * K;
+        const int o = i / K, j = i - o * K, order = o0 + o - p.identity;
+        const uint32_t ch = order < 0 ? static_cast<uint32_t>(j) : static_cast<uint32_t>(__ldg(p.perms + static_cast<int64_t>(order) * K + j));
         // the two 16-byte halves of a run's slots lie in separate planes: lanes read consecutive 16-byte words
-        slot_s[o * K + ((j >> 3) & 1) * (K >> 1) + (j >> 4) * 8 + (j & 7)] = static_cast<uint16_t>(pq::quad_channel(__ldg(perm + i)));
+        slot_s[o * K + ((j >> 3) & 1) * (K >> 1) + (j >> 4) * 8 + (j & 7)] = static_cast<uint16_t>(pq::quad_channel(ch));
     }
-    const float ts = KIND == 0 ? __ldg(p.ts) : 1.0f;
-    if (KIND == 0) build_scale_tab(*tab, ts);
-    else build_int_tab(int_tab, p.Qf);
+    const int sides = p.ts[1] ? 2 : 1;
+    if (KIND == 0) {
+        for (int s = 0; s < sides; ++s) build_scale_tab(reinterpret_cast<ScaleTab *>(tab_s + s * kTabBytes)[0], __ldg(p.ts[s]));
+    } else {
+        build_int_tab(int_tab, p.Qf);
+    }
     __syncthreads();
 
     const int grp = threadIdx.x / p.group_threads, tid = threadIdx.x - grp * p.group_threads;
-    if (grp >= p.groups) return;
+    if (grp >= p.groups) {  // the extra warp
+        for (int s = 0; s < 2; ++s)
+            if (blockIdx.y == 0 && blockIdx.x == min(static_cast<unsigned>(s), gridDim.x - 1)) {
+                const double sum = pq::ordered_sum(s ? p.weights.sumsq_w : p.weights.sumsq_a, K);
+                if ((threadIdx.x & 31) == 0) p.weights.lambda[s] = __ddiv_rn(1.0, sum);
+            }
+        return;
+    }
     auto group_sync = [&]() {
         if (p.group_threads == 32) __syncwarp();
         else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(p.group_threads) : "memory");
     };
     uint4 *quad4 = reinterpret_cast<uint4 *>(smem + static_cast<size_t>(grp) * K * 8);
     const uint32_t quad_addr = static_cast<uint32_t>(__cvta_generic_to_shared(quad4));
-    float *acc_s = reinterpret_cast<float *>(tab_s + kTabBytes) + static_cast<size_t>(grp) * p.opb * runs;
+    float *acc_s = reinterpret_cast<float *>(tab_s + (KIND == 0 ? sides : 1) * kTabBytes) + static_cast<size_t>(grp) * p.opb * runs;
     const uint4 *slot4 = reinterpret_cast<const uint4 *>(slot_s);
-    const uint32_t lo2 = KIND == 0 ? tab->lo * 0x10001u : 0u, hi2 = KIND == 0 ? tab->hi * 0x10001u : 0u;
     const int64_t Kg = runs / TEAM16;
 
-    for (int64_t chunk = static_cast<int64_t>(blockIdx.x) * p.groups + grp; chunk < p.chunks;
-         chunk += static_cast<int64_t>(gridDim.x) * p.groups) {
-        const int64_t r0 = chunk * PQ_CHUNK_ROWS;
+    for (int chunk = blockIdx.x * p.groups + grp; chunk < p.chunks; chunk += gridDim.x * p.groups) {
+        const int slab = chunk / kSlabChunks, t = pq::tensor_of_slab(p.list, slab);
+        const int64_t r0 = static_cast<int64_t>(slab - p.list.slab0[t]) * PQ_SLAB_ROWS + chunk % kSlabChunks * PQ_CHUNK_ROWS;
+        const int64_t ld = p.list.ld[t], left = p.list.rows[t] - r0;
+        const int n = left >= PQ_CHUNK_ROWS ? PQ_CHUNK_ROWS : (left > 0 ? static_cast<int>(left) : 0);
+        const uint16_t *src = p.list.ptr[t] + r0 * ld;
+        const ScaleTab *tab = reinterpret_cast<const ScaleTab *>(tab_s + (KIND == 0 && t >= p.list.n_x ? kTabBytes : 0));
+        const uint32_t lo2 = KIND == 0 ? tab->lo * 0x10001u : 0u, hi2 = KIND == 0 ? tab->hi * 0x10001u : 0u;
 #pragma unroll 1
         for (int quad = 0; quad < PQ_CHUNK_ROWS / 4; ++quad) {
-            const int64_t row = r0 + 4 * quad;
-            if (row >= p.rows) break;  // no rows left: their error is +0.0
+            if (4 * quad >= n) break;  // no rows left: their error is +0.0
             group_sync();              // the previous four rows have been used
-            const uint16_t *src = p.T + row * p.ld;
 #pragma unroll 2
             for (int o = tid; o < octs; o += p.group_threads) {
                 uint4 v[4];
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {  // rows past the end are zeros: their error is +0.0 and adding it changes nothing
-                    v[r] = row + r < p.rows ? __ldg(reinterpret_cast<const uint4 *>(src + r * p.ld) + o) : make_uint4(0, 0, 0, 0);
+                    v[r] = 4 * quad + r < n ? __ldg(reinterpret_cast<const uint4 *>(src + (4 * quad + r) * ld) + o) : make_uint4(0, 0, 0, 0);
                     v[r].x &= 0x7FFF7FFFu, v[r].y &= 0x7FFF7FFFu, v[r].z &= 0x7FFF7FFFu, v[r].w &= 0x7FFF7FFFu;
                 }
                 pq::store_quad_octet(quad4, o, v);
@@ -452,7 +464,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __
         // every thread writes out the sums it kept itself
         for (int o = 0; o < no; ++o)
             for (int q = tid; q < runs; q += p.group_threads)
-                if ((q % TEAM16) == 0) p.part[(chunk * p.P + o0 + o) * Kg + q / TEAM16] = acc_s[o * runs + q];
+                if ((q % TEAM16) == 0) p.part[(static_cast<int64_t>(chunk) * p.P + o0 + o) * Kg + q / TEAM16] = n ? acc_s[o * runs + q] : 0.0f;
     }
 }
 
@@ -464,7 +476,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __
 struct GatherConfig {
     int opb = 0, groups = 0, group_threads = 0;
 };
-inline GatherConfig gather_config(int64_t chunks, int64_t K, int P, int sms) {
+inline GatherConfig gather_config(int64_t chunks, int64_t K, int P, int sides, int sms) {
     GatherConfig best;
     double best_cost = 0.0;
     const int runs = static_cast<int>(K / 16);
@@ -474,7 +486,7 @@ inline GatherConfig gather_config(int64_t chunks, int64_t K, int P, int sms) {
         for (int opb = 1; opb <= P; ++opb) {
             const int64_t subsets = pq_ceil_div(P, opb);
             for (int groups = 1; groups <= kMaxGroups && groups * threads <= kGatherThreads; ++groups) {
-                if (gather_smem_bytes(K, opb, groups) > 226 * 1024) break;
+                if (gather_smem_bytes(K, opb, groups, sides) > 226 * 1024) break;
                 const int64_t blocks = sms / subsets > 0 ? sms / subsets : 1;
                 const int64_t rounds = pq_ceil_div(chunks, blocks * groups);
                 const int warps = groups * threads / 32;
@@ -502,6 +514,26 @@ pq_status fold(const void *part, int64_t count, int64_t n, double *err, cudaStre
     return pq_launch_status();
 }
 
+// list, ts, identity, perms, chunks and weights of p are set by the caller.
+template <int KIND, int TEAM>
+pq_status launch_gather(GatherParams &p, int64_t K, int P, float Qf, float *part, cudaStream_t st) {
+    const int sms = sm_count(), sides = KIND == 0 && p.ts[1] ? 2 : 1;
+    const GatherConfig cfg = gather_config(p.chunks, K, P, sides, sms);
+    if (!cfg.groups) return PQ_ERR_SHAPE;
+    p.K = static_cast<int>(K), p.P = P, p.Qf = Qf, p.part = part;
+    p.opb = cfg.opb, p.groups = cfg.groups, p.group_threads = cfg.group_threads;
+    const int64_t subsets = pq_ceil_div(P, cfg.opb), share = sms / subsets > 0 ? sms / subsets : 1;
+    const int64_t want = pq_ceil_div(p.chunks, cfg.groups);
+    const size_t smem = gather_smem_bytes(K, cfg.opb, cfg.groups, sides);
+    auto kern = group_error_gather<KIND, TEAM / 2>;
+    if (smem > 48 * 1024)
+        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    const unsigned threads = static_cast<unsigned>(cfg.groups * cfg.group_threads + (p.weights.lambda ? 32 : 0));
+    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(want < share ? want : share), static_cast<unsigned>(subsets)),
+                                    dim3(threads), smem, st, p));
+    return pq_launch_status();
+}
+
 template <int KIND, int TEAM>  // TEAM = group / 8
 pq_status launch(const uint16_t *T, int64_t rows, int64_t K, int64_t ld, const float *ts, float Qf,
                  const int32_t *perms, int P, void *ws, double *err, cudaStream_t st) {
@@ -513,23 +545,29 @@ pq_status launch(const uint16_t *T, int64_t rows, int64_t K, int64_t ld, const f
         if (pq_launch_status() != PQ_OK) return PQ_ERR_CUDA;
         return fold<double, 1>(ws, slabs, Kg, err, st);
     }
-    const int sms = sm_count();
-    const GatherConfig cfg = gather_config(chunks, K, P, sms);
-    if (!cfg.groups) return PQ_ERR_SHAPE;
     GatherParams p;
-    p.T = T, p.rows = rows, p.ld = ld, p.ts = ts, p.K = static_cast<int>(K), p.P = P, p.perms = perms;
-    p.opb = cfg.opb, p.groups = cfg.groups, p.group_threads = cfg.group_threads;
-    p.chunks = chunks, p.Qf = Qf, p.part = static_cast<float *>(ws);
-    const int64_t subsets = pq_ceil_div(P, cfg.opb), share = sms / subsets > 0 ? sms / subsets : 1;
-    const int64_t want = pq_ceil_div(chunks, cfg.groups);
-    const size_t smem = gather_smem_bytes(K, cfg.opb, cfg.groups);
-    auto kern = group_error_gather<KIND, TEAM / 2>;
-    if (smem > 48 * 1024)
-        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(want < share ? want : share), static_cast<unsigned>(subsets)),
-                                    dim3(static_cast<unsigned>(cfg.groups * cfg.group_threads)), smem, st, p));
+    p.list.add(T, rows, ld);
+    p.list.n_x = 1;
+    p.ts[0] = ts, p.ts[1] = nullptr, p.identity = 0, p.perms = perms, p.chunks = static_cast<int>(chunks);
+    p.weights = PqErrorWeights{};
+    if (launch_gather<KIND, TEAM>(p, K, P, Qf, static_cast<float *>(ws), st) != PQ_OK) return PQ_ERR_CUDA;
     return fold<float, kSlabChunks>(ws, chunks, static_cast<int64_t>(P) * Kg, err, st);
 }
+
+// f(KIND, TEAM) for a format that has been checked.
+template <typename F>
+pq_status dispatch_format(pq_format fmt, F &&f) {
+    using std::integral_constant;
+    if (fmt.kind == 0) return f(integral_constant<int, 0>{}, integral_constant<int, 2>{});
+    switch (fmt.group) {
+        case 16: return f(integral_constant<int, 1>{}, integral_constant<int, 2>{});
+        case 32: return f(integral_constant<int, 1>{}, integral_constant<int, 4>{});
+        case 64: return f(integral_constant<int, 1>{}, integral_constant<int, 8>{});
+        case 128: return f(integral_constant<int, 1>{}, integral_constant<int, 16>{});
+        default: return f(integral_constant<int, 1>{}, integral_constant<int, 32>{});  // 256: a whole warp per group
+    }
+}
+float level_max(pq_format fmt) { return fmt.kind == 1 ? static_cast<float>((1 << (fmt.bits - 1)) - 1) : 0.0f; }
 
 }  // namespace
 
@@ -555,13 +593,26 @@ extern "C" pq_status pq_group_error(const void *T, int64_t rows, int64_t K, int6
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint16_t *t = static_cast<const uint16_t *>(T);
-    const float Qf = fmt.kind == 1 ? static_cast<float>((1 << (fmt.bits - 1)) - 1) : 0.0f;
-    if (fmt.kind == 0) return launch<0, 2>(t, rows, K, ld, ts, Qf, perms, P, ws, err, st);
-    switch (group) {
-        case 16: return launch<1, 2>(t, rows, K, ld, ts, Qf, perms, P, ws, err, st);
-        case 32: return launch<1, 4>(t, rows, K, ld, ts, Qf, perms, P, ws, err, st);
-        case 64: return launch<1, 8>(t, rows, K, ld, ts, Qf, perms, P, ws, err, st);
-        case 128: return launch<1, 16>(t, rows, K, ld, ts, Qf, perms, P, ws, err, st);
-        default: return launch<1, 32>(t, rows, K, ld, ts, Qf, perms, P, ws, err, st);   // 256: a whole warp per group
-    }
+    return dispatch_format(fmt, [&](auto kind, auto team) {
+        return launch<decltype(kind)::value, decltype(team)::value>(t, rows, K, ld, ts, level_max(fmt), perms, P, ws, err, st);
+    });
+}
+
+pq_status pq_errors_on_list(const PqTensorList &list, int64_t K, pq_format fmt, const float *const (&ts)[2], const int32_t *perms,
+                            int P, const PqSide (&sides)[2], const PqErrorWeights &weights, void *ws, cudaStream_t st) {
+    GatherParams p;
+    p.list = list;
+    p.ts[0] = ts[0], p.ts[1] = ts[1], p.identity = 1, p.perms = perms, p.chunks = list.slabs() * kSlabChunks;
+    p.weights = weights;
+    float *part = static_cast<float *>(ws);
+    const pq_status rc = dispatch_format(fmt, [&](auto kind, auto team) {
+        return launch_gather<decltype(kind)::value, decltype(team)::value>(p, K, P + 1, level_max(fmt), part, st);
+    });
+    if (rc != PQ_OK) return rc;
+    const int64_t n = (P + 1) * (K / (fmt.kind == 0 ? 16 : fmt.group));
+    const int64_t cx = static_cast<int64_t>(list.slabs_x()) * kSlabChunks, cw = p.chunks - cx;
+    const pq::FoldRange rx{part, nullptr, cx, sides[0].total, nullptr, sides[0].from_zero};
+    const pq::FoldRange rw{part + cx * n, nullptr, cw, sides[1].total, nullptr, sides[1].from_zero};
+    PQ_CUDA_OK((pq::launch_fold<float, kSlabChunks, false>(sides[0].total ? rx : rw, sides[0].total ? rw : pq::FoldRange{}, n, st)));
+    return pq_launch_status();
 }

@@ -25,6 +25,10 @@ struct SortParams {
     int J;                 // joint: blockIdx.y = j = 0..J
     int K, deal_groups, group;
     int32_t *perms;        // [orders, K]
+    int orders;
+    // rows of the grid past the orders: *scale_out[s] = tensor scale from the column maxima scale_max[s]
+    const float *scale_max[2];
+    float *scale_out[2];
 };
 
 __device__ __forceinline__ unsigned long long sort_key(const SortParams &p, int j, int i) {
@@ -77,6 +81,12 @@ __global__ void __launch_bounds__(kSortChunk) order_sort_kernel(const __grid_con
     const int chunks = (p.K + kSortChunk - 1) / kSortChunk;
     pq::dependents_may_launch();
     pq::wait_for_prior_grid();
+    if (j >= p.orders) {  // the whole cluster: nobody waits for it at a cluster barrier
+        if (rank) return;
+        const float a = pq::block_max(p.scale_max[j - p.orders], p.K);
+        if (tid == 0) *p.scale_out[j - p.orders] = (a == 0.0f) ? 1.0f : __fdiv_rn(a, 2688.0f);
+        return;
+    }
     int channel[kSortPerCta];
 #pragma unroll
     for (int t = 0; t < kSortPerCta; ++t) {
@@ -145,20 +155,21 @@ __global__ void __launch_bounds__(kSortChunk) order_sort_kernel(const __grid_con
     cluster_barrier();  // the neighbours may still be reading this CTA's keys
 }
 
-SortParams sort_params(KeyKind kind, const double *a, const double *b, const float *f, int64_t rows_a, int64_t rows_b, int J, int64_t K,
+SortParams sort_params(KeyKind kind, int orders, const double *a, const double *b, const float *f, int64_t rows_a, int64_t rows_b, int J, int64_t K,
                        int32_t *perms) {
     SortParams p;
     p.kind = kind, p.a = a, p.b = b, p.f = f;
     p.rows_a = static_cast<double>(rows_a), p.rows_b = static_cast<double>(rows_b), p.J = J;
-    p.K = static_cast<int>(K), p.deal_groups = 0, p.group = 0, p.perms = perms;
+    p.K = static_cast<int>(K), p.deal_groups = 0, p.group = 0, p.perms = perms, p.orders = orders;
+    p.scale_max[0] = p.scale_max[1] = nullptr, p.scale_out[0] = p.scale_out[1] = nullptr;
     return p;
 }
 
-pq_status launch_sort(const SortParams &p, int orders, cudaStream_t st) {
+pq_status launch_sort(const SortParams &p, cudaStream_t st) {
     const int chunks = static_cast<int>(pq_ceil_div(p.K, kSortChunk));
     const int ctas = chunks < kSortMaxCluster ? chunks : kSortMaxCluster;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(ctas), static_cast<unsigned>(orders));
+    cfg.gridDim = dim3(static_cast<unsigned>(ctas), static_cast<unsigned>(p.orders + (p.scale_out[0] ? 2 : 0)));
     cfg.blockDim = dim3(kSortChunk), cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -206,6 +217,14 @@ accept_kernel(const double *__restrict__ ex, const double *__restrict__ ew, cons
 
 }  // namespace
 
+pq_status pq_orders_and_scales(const double *sumsq_a, int64_t rows_a, const double *sumsq_w, int64_t rows_w, int64_t K, int J,
+                               int32_t *perms, const float *amax_a, const float *amax_w, float *ts_x, float *ts_w, cudaStream_t st) {
+    SortParams p = sort_params(kKeyJoint, J + 1, sumsq_a, sumsq_w, nullptr, rows_a, rows_w, J, K, perms);
+    p.scale_max[0] = amax_a, p.scale_max[1] = amax_w;
+    p.scale_out[0] = ts_x, p.scale_out[1] = ts_w;
+    return launch_sort(p, st);
+}
+
 extern "C" pq_status pq_select_perm(const double *sumsq_a, int64_t rows_a, const double *sumsq_w,
                                     int64_t rows_w, int64_t K, int J, int32_t *perms, void *ws,
                                     size_t ws_bytes, void *stream) {
@@ -215,7 +234,7 @@ extern "C" pq_status pq_select_perm(const double *sumsq_a, int64_t rows_a, const
     PQ_REQUIRE(ws && ws_bytes >= need, PQ_ERR_WORKSPACE);
     PQ_REQUIRE(pq_aligned256(ws), PQ_ERR_ALIGN);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return launch_sort(sort_params(kKeyJoint, sumsq_a, sumsq_w, nullptr, rows_a, rows_w, J, K, perms), J + 1, st);
+    return launch_sort(sort_params(kKeyJoint, J + 1, sumsq_a, sumsq_w, nullptr, rows_a, rows_w, J, K, perms), st);
 }
 
 extern "C" pq_status pq_order_by_absmax(const float *amax, int64_t K, int32_t *perm, void *ws, size_t ws_bytes,
@@ -225,7 +244,7 @@ extern "C" pq_status pq_order_by_absmax(const float *amax, int64_t K, int32_t *p
     PQ_REQUIRE(ws && ws_bytes >= pq_workspace_bytes(PQ_OP_SELECT_PERM, 0, K, 0, 1), PQ_ERR_WORKSPACE);
     PQ_REQUIRE(pq_aligned256(ws), PQ_ERR_ALIGN);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return launch_sort(sort_params(kKeyAbsmax, nullptr, nullptr, amax, 1, 1, 0, K, perm), 1, st);
+    return launch_sort(sort_params(kKeyAbsmax, 1, nullptr, nullptr, amax, 1, 1, 0, K, perm), st);
 }
 
 extern "C" pq_status pq_order_by_variance(const double *sum, const double *sumsq, int64_t rows, int64_t K, int32_t *perm,
@@ -235,7 +254,7 @@ extern "C" pq_status pq_order_by_variance(const double *sum, const double *sumsq
     PQ_REQUIRE(ws && ws_bytes >= pq_workspace_bytes(PQ_OP_SELECT_PERM, 0, K, 0, 1), PQ_ERR_WORKSPACE);
     PQ_REQUIRE(pq_aligned256(ws), PQ_ERR_ALIGN);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return launch_sort(sort_params(kKeyVariance, sum, sumsq, nullptr, rows, 1, 0, K, perm), 1, st);
+    return launch_sort(sort_params(kKeyVariance, 1, sum, sumsq, nullptr, rows, 1, 0, K, perm), st);
 }
 
 extern "C" pq_status pq_order_round_robin(const double *sumsq, int64_t K, int group, int32_t *perm, void *ws,
@@ -245,9 +264,9 @@ extern "C" pq_status pq_order_round_robin(const double *sumsq, int64_t K, int gr
     PQ_REQUIRE(ws && ws_bytes >= pq_workspace_bytes(PQ_OP_SELECT_PERM, 0, K, 0, 1), PQ_ERR_WORKSPACE);
     PQ_REQUIRE(pq_aligned256(ws), PQ_ERR_ALIGN);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    SortParams p = sort_params(kKeyPlain, sumsq, nullptr, nullptr, 1, 1, 0, K, perm);
+    SortParams p = sort_params(kKeyPlain, 1, sumsq, nullptr, nullptr, 1, 1, 0, K, perm);
     p.deal_groups = static_cast<int>(K / group), p.group = group;
-    return launch_sort(p, 1, st);
+    return launch_sort(p, st);
 }
 
 extern "C" pq_status pq_accept(const double *err_x, const double *err_w, const double *lambda, int P,

@@ -396,6 +396,15 @@ extern "C" pq_status pq_quant_act_nvfp4_perm(const void *X, int64_t M, int64_t K
                          static_cast<cudaStream_t>(stream));
 }
 
+pq_status pq_quant_weight_scaled(const void *Wt, int64_t N, int64_t K, int64_t ld, const int32_t *perm, const int32_t *perm_select,
+                                 uint8_t *codes, uint8_t *sf, int sf_layout, const float *ts_w, cudaStream_t st) {
+    if (!perm) return pq_quant_act_nvfp4(Wt, N, K, ld, ts_w, codes, sf, sf_layout, st);
+    // rows of up to 6400 channels: four rows per warp share the indices and one gather
+    if (pq_gather_quant_grouped_fits(K) && pq_aligned16(perm))
+        return pq_gather_quant_grouped(Wt, N, K, ld, perm, perm_select, ts_w, codes, sf, sf_layout, st);
+    return launch_gather(static_cast<const uint16_t *>(Wt), N, K, ld, perm, perm_select, ts_w, codes, sf, sf_layout, st);
+}
+
 extern "C" pq_status pq_quant_weight(const void *Wt, int64_t N, int64_t K, int64_t ld,
                                      const int32_t *perm, const int32_t *perm_select, uint8_t *codes,
                                      uint8_t *sf, int sf_layout, float *ts_w, void *ws, size_t ws_bytes,
@@ -422,11 +431,7 @@ extern "C" pq_status pq_quant_weight(const void *Wt, int64_t N, int64_t K, int64
                           dim3(32, kTileRows), 0, st>>>(w, N, K, ld, amax_bits);
     }
     weight_scale_kernel<<<1, 1, 0, st>>>(amax_bits, ts_w);
-    if (!perm) return pq_quant_act_nvfp4(Wt, N, K, ld, ts_w, codes, sf, sf_layout, stream);
-    // rows of up to 6400 channels: four rows per warp share the indices and one gather
-    if (pq_gather_quant_grouped_fits(K) && pq_aligned16(perm))
-        return pq_gather_quant_grouped(Wt, N, K, ld, perm, perm_select, ts_w, codes, sf, sf_layout, stream);
-    return launch_gather(w, N, K, ld, perm, perm_select, ts_w, codes, sf, sf_layout, st);
+    return pq_quant_weight_scaled(Wt, N, K, ld, perm, perm_select, codes, sf, sf_layout, ts_w, st);
 }
 
 extern "C" pq_status pq_fakequant_int(const void *T, int64_t rows, int64_t K, int64_t ld, pq_format fmt,

@@ -30,8 +30,8 @@ __device__ __forceinline__ void stats_row(const uint4 &v, float (&s)[8], float (
 }
 
 __global__ void __launch_bounds__(kStatsThreads)
-calib_stats_slab(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int64_t ld,
-                 double *__restrict__ slab_sum /*[slabs, K]*/, float *__restrict__ slab_max /*[slabs, K]*/) {
+calib_stats_slab(const __grid_constant__ PqTensorList list, int64_t K, double *__restrict__ slab_sum /*[slabs, K]*/,
+                 float *__restrict__ slab_max /*[slabs, K]*/) {
     __shared__ __align__(16) float sum_s[kSlabChunks][kStatsCols];
     __shared__ __align__(16) float max_s[kSlabChunks][kStatsCols];
     pq::dependents_may_launch();
@@ -39,15 +39,16 @@ calib_stats_slab(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int64_
     const int64_t col0 = static_cast<int64_t>(blockIdx.y) * kStatsCols;
     const int64_t col = col0 + lane * 8;
     const int64_t slab = blockIdx.x;
-    const int64_t r0 = slab * PQ_SLAB_ROWS + w * PQ_CHUNK_ROWS;
-    const int64_t left = rows - r0;
+    const int t = pq::tensor_of_slab(list, blockIdx.x);
+    const int64_t ld = list.ld[t], r0 = (slab - list.slab0[t]) * PQ_SLAB_ROWS + w * PQ_CHUNK_ROWS;
+    const int64_t left = list.rows[t] - r0;
     const int n = left >= PQ_CHUNK_ROWS ? PQ_CHUNK_ROWS : (left > 0 ? static_cast<int>(left) : 0);
 
     float s[8], a[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) s[i] = 0.0f, a[i] = 0.0f;
     if (col < K) {
-        const uint16_t *p = T + r0 * ld + col;
+        const uint16_t *p = list.ptr[t] + r0 * ld + col;
         if (n == PQ_CHUNK_ROWS) {
             uint4 v[PQ_CHUNK_ROWS];
 #pragma unroll
@@ -55,7 +56,7 @@ calib_stats_slab(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int64_
 #pragma unroll
             for (int u = 0; u < PQ_CHUNK_ROWS; ++u) stats_row(v[u], s, a);
         } else {
-            for (int t = 0; t < n; ++t) stats_row(__ldcs(reinterpret_cast<const uint4 *>(p + static_cast<int64_t>(t) * ld)), s, a);
+            for (int u = 0; u < n; ++u) stats_row(__ldcs(reinterpret_cast<const uint4 *>(p + static_cast<int64_t>(u) * ld)), s, a);
         }
     }
     float4 *ds = reinterpret_cast<float4 *>(&sum_s[w][lane * 8]);
@@ -193,16 +194,8 @@ output_error_slab(const float *__restrict__ Yref, int64_t ld_ref, const uint16_t
 }
 
 __global__ void tensor_scale_kernel(const float *__restrict__ amax, int64_t K, float *ts) {
-    __shared__ float red[32];
-    float a = 0.0f;
-    for (int64_t i = threadIdx.x; i < K; i += blockDim.x) a = fmaxf(a, amax[i]);
-    for (int m = 16; m; m >>= 1) a = fmaxf(a, __shfl_xor_sync(0xFFFFFFFFu, a, m));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < static_cast<int>(blockDim.x >> 5); ++w) a = fmaxf(a, red[w]);
-        *ts = (a == 0.0f) ? 1.0f : __fdiv_rn(a, 2688.0f);
-    }
+    const float a = pq::block_max(amax, K);
+    if (threadIdx.x == 0) *ts = (a == 0.0f) ? 1.0f : __fdiv_rn(a, 2688.0f);
 }
 
 // lambda[s] = 1 / (sequential fp64 sum of side s in ascending channel order), one warp per side.
@@ -217,6 +210,19 @@ __global__ void __launch_bounds__(64) error_weights_kernel(const double *__restr
 
 }  // namespace
 
+pq_status pq_stats_on_list(const PqTensorList &list, int64_t K, const PqSide (&sides)[2], void *ws, cudaStream_t st) {
+    const int64_t slabs = list.slabs(), slabs_x = list.slabs_x();
+    dim3 grid(static_cast<unsigned>(slabs), static_cast<unsigned>(pq_ceil_div(K, kStatsCols)));
+    double *slab_sum = static_cast<double *>(ws);
+    float *slab_max = reinterpret_cast<float *>(slab_sum + slabs * K);
+    calib_stats_slab<<<grid, kStatsThreads, 0, st>>>(list, K, slab_sum, slab_max);
+    const pq::FoldRange rx{slab_sum, slab_max, slabs_x, sides[0].total, sides[0].vmax, sides[0].from_zero};
+    const pq::FoldRange rw{slab_sum + slabs_x * K, slab_max + slabs_x * K, slabs - slabs_x, sides[1].total, sides[1].vmax,
+                           sides[1].from_zero};
+    PQ_CUDA_OK((pq::launch_fold<double, 1, true>(sides[0].total ? rx : rw, sides[0].total ? rw : pq::FoldRange{}, K, st)));
+    return pq_launch_status();
+}
+
 extern "C" pq_status pq_calib_stats(const void *T, int64_t rows, int64_t K, int64_t ld,
                                     double *sumsq, float *amax, void *ws, size_t ws_bytes,
                                     void *stream) {
@@ -228,13 +234,10 @@ extern "C" pq_status pq_calib_stats(const void *T, int64_t rows, int64_t K, int6
     PQ_REQUIRE(pq_aligned256(ws), PQ_ERR_ALIGN);
     const int64_t slabs = pq_ceil_div(rows, PQ_SLAB_ROWS);
     PQ_REQUIRE(slabs < (1ll << 31) && K <= 65535ll * kStatsCols, PQ_ERR_SHAPE);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    dim3 grid(static_cast<unsigned>(slabs), static_cast<unsigned>(pq_ceil_div(K, kStatsCols)));
-    double *slab_sum = static_cast<double *>(ws);
-    float *slab_max = reinterpret_cast<float *>(slab_sum + slabs * K);
-    calib_stats_slab<<<grid, kStatsThreads, 0, st>>>(static_cast<const uint16_t *>(T), rows, K, ld, slab_sum, slab_max);
-    PQ_CUDA_OK((pq::launch_fold<double, 1, true>(slab_sum, slab_max, slabs, K, sumsq, amax, st)));
-    return pq_launch_status();
+    PqTensorList list;
+    list.add(T, rows, ld);
+    list.n_x = 1;
+    return pq_stats_on_list(list, K, {{sumsq, amax, false}, {nullptr, nullptr, false}}, ws, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" pq_status pq_calib_sum(const void *T, int64_t rows, int64_t K, int64_t ld, double *sum, void *ws,

@@ -46,49 +46,20 @@ class Calibration:
 def calibrate(batches, Wt, fmt=NVFP4, J=5, tau=0.0, sf_layout=B.PQ_SF_TCGEN05) -> Calibration:
     """Offline pass over calibration batches (list of bf16 [T, K] device tensors) and the weight
     Wt (bf16 [N, K] device tensor).  `fmt` is the format whose error drives the acceptance rule."""
-    dev = Wt.device
     N, K = Wt.shape
-    group = 16 if fmt[0] == B.KIND_NVFP4 else fmt[2]
-    Kg = K // group
-    sumsq_a = torch.zeros(K, dtype=torch.float64, device=dev)
-    sumsq_w = torch.zeros(K, dtype=torch.float64, device=dev)
-    amax_a = torch.zeros(K, dtype=torch.float32, device=dev)
-    amax_w = torch.zeros(K, dtype=torch.float32, device=dev)
-    rows_a = 0
-    max_rows = max([b.shape[0] for b in batches] + [N])
-    ws = B.workspace(B.OP_GROUP_ERROR, max_rows, K, 0, J + 1)     # large enough for every step below
-    ws_stats = B.workspace(B.OP_CALIB_STATS, max_rows, K)
-    for x in batches:
-        B.pq_calib_stats(x, sumsq_a, amax_a, ws_stats)
-        rows_a += x.shape[0]
-    B.pq_calib_stats(Wt, sumsq_w, amax_w, ws_stats)
-    ts_x = torch.empty(1, dtype=torch.float32, device=dev)
-    ts_w_err = torch.empty(1, dtype=torch.float32, device=dev)
-    B.pq_tensor_scale(amax_a, ts_x)
-    B.pq_tensor_scale(amax_w, ts_w_err)
+    Kg = K // (16 if fmt[0] == B.KIND_NVFP4 else fmt[2])
 
-    perms = torch.empty(J + 1, K, dtype=torch.int32, device=dev)
-    B.pq_select_perm(sumsq_a, rows_a, sumsq_w, N, J, perms, B.workspace(B.OP_SELECT_PERM, 0, K, 0, J + 1))
+    def out(dtype, *shape):
+        return torch.empty(shape, dtype=dtype, device=Wt.device)
 
-    err_x = torch.zeros(J + 2, Kg, dtype=torch.float64, device=dev)
-    err_w = torch.zeros(J + 2, Kg, dtype=torch.float64, device=dev)
-    for x in batches:
-        B.pq_group_error(x, fmt, ts_x, None, err_x[0:1], ws)
-        B.pq_group_error(x, fmt, ts_x, perms, err_x[1:], ws)
-    B.pq_group_error(Wt, fmt, ts_w_err, None, err_w[0:1], ws)
-    B.pq_group_error(Wt, fmt, ts_w_err, perms, err_w[1:], ws)
-
-    lam = torch.empty(2, dtype=torch.float64, device=dev)
-    B.pq_error_weights(sumsq_a, sumsq_w, lam)
-    select = torch.zeros(2, dtype=torch.int32, device=dev)
-    E = torch.empty(J + 2, dtype=torch.float64, device=dev)
-    B.pq_accept(err_x, err_w, lam, tau, select[0:1], select[1:2], E)
-
-    wq = torch.empty(N, K // 2, dtype=torch.uint8, device=dev)
-    sfw = torch.empty(B.sf_bytes(N, K, sf_layout), dtype=torch.uint8, device=dev)
-    ts_w = torch.empty(1, dtype=torch.float32, device=dev)
-    B.pq_quant_weight(Wt, perms, select, wq, sfw, sf_layout, ts_w, B.workspace(B.OP_QUANT_WEIGHT, N, K))
-    return Calibration(sumsq_a, sumsq_w, amax_a, ts_x, ts_w, perms, err_x, err_w, lam, E, select, wq, sfw, rows_a)
+    f64, f32, i32, u8 = torch.float64, torch.float32, torch.int32, torch.uint8
+    c = Calibration(sumsq_a=out(f64, K), sumsq_w=out(f64, K), amax_a=out(f32, K), ts_x=out(f32, 1), ts_w=out(f32, 1),
+                    perms=out(i32, J + 1, K), err_x=out(f64, J + 2, Kg), err_w=out(f64, J + 2, Kg), lam=out(f64, 2),
+                    E=out(f64, J + 2), select=out(i32, 2), wq=out(u8, N, K // 2), sfw=out(u8, B.sf_bytes(N, K, sf_layout)),
+                    rows_a=sum(x.shape[0] for x in batches))
+    B.pq_calibrate(batches, Wt, fmt, J, tau, sf_layout, c.sumsq_a, c.sumsq_w, c.amax_a, c.ts_x, c.ts_w, c.perms, c.err_x,
+                   c.err_w, c.lam, c.E, c.select, c.wq, c.sfw)
+    return c
 
 
 def calibrate_h(batches, Wt, fmt=NVFP4, J=5, tau=0.0):

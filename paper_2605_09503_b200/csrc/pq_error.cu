@@ -36,8 +36,11 @@ __device__ __forceinline__ void build_scale_table(float2 *table, float ts) {
 }
 
 using pq::add2;
+using pq::bf16_pattern;
 using pq::fma2;
 using pq::max_bf16x2;
+using pq::max_u16x2;
+using pq::min_u16x2;
 using pq::mul2;
 using pq::pack2;
 using pq::unpack2;
@@ -183,32 +186,15 @@ constexpr int kGatherThreads = 768;  // 80 registers per thread; 960 threads at 
 constexpr int kMaxGroups = 15;                                           // named barriers 1..15
 constexpr int kSfTabMax = 2624;  // bf16 magnitudes from "scale byte 0" to "saturated": 19 binades and the edges
 
-__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("min.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-
 // What a group's scale is looked up in, per side (activations / weight: they differ in the tensor scale).
 //   NVFP4    {1 / d, -d} for the decode scale d, as a function of the group's absmax, a bf16 magnitude: every magnitude
 //            up to `lo` gives scale byte 0 and every one from `hi` on the saturated byte, the ones between are
 //            tabulated from the definition.
-//   integer  s = amax / Q and 1 / s by the seven mantissa bits of amax, as bit patterns to which the exponent is
-//            added: scaling by a power of two commutes with both roundings while nothing is subnormal, i.e. for
-//            biased exponents kIntExpLo .. kIntExpHi (s >= 2^-125, 1/s >= 2^-124).
+//   integer  by the mantissa of amax (pq::build_int_tab).
 struct ScaleTab {
     float2 rd[kSfTabMax];
     uint32_t lo, hi, pad[2];
 };
-constexpr uint32_t kIntExpLo = 9, kIntExpHi = 250;
-
-__device__ __forceinline__ float bf16_pattern(uint32_t a) { return __uint_as_float(a << 16); }
-
 __device__ __forceinline__ void build_scale_tab(ScaleTab &tab, float ts) {
     const float c6 = __fmul_rn(6.0f, ts), mag = fabsf(c6);
     // (signed) byte 0 up to |c6| 2^-10, half the smallest subnormal (ties to even); saturated from 448 |c6| on.  A
@@ -225,14 +211,6 @@ __device__ __forceinline__ void build_scale_tab(ScaleTab &tab, float ts) {
         tab.rd[i] = make_float2(d > 0.0f ? __frcp_rn(d) : 0.0f, -d);
     }
 }
-__device__ __forceinline__ void build_int_tab(uint2 *tab, float Qf) {
-    for (uint32_t m = threadIdx.x; m < 128; m += blockDim.x) {
-        const float s = __fdiv_rn(__uint_as_float(0x3F800000u | (m << 16)), Qf);
-        tab[m] = make_uint2(__float_as_uint(__frcp_rn(s)) + (127u << 23),
-                            __float_as_uint(s) - (127u << 23) + 0x80000000u);  // mod 2^32: -s once the exponent is added
-    }
-}
-
 // E2M1 of the two floats of a pair and back to fp32 (E2M1 -> f16 is exact, f16 -> f32 too).
 __device__ __forceinline__ uint64_t e2m1_pair(uint64_t y2) {
     float lo, hi;
@@ -303,18 +281,14 @@ __device__ __forceinline__ void row_pair_sse(const uint32_t (&u)[16], const Scal
         r2 = pack2(d0.x, d1.x), nd2 = pack2(d0.y, d1.y);
     } else {
         const uint32_t a0 = am & 0xFFFFu, a1 = am >> 16;
-        // an all-zero group may use any finite scale: its levels and residuals are zero
-        const bool odd0 = a0 != 0u && a0 - (kIntExpLo << 7) >= ((kIntExpHi - kIntExpLo + 1u) << 7);
-        const bool odd1 = a1 != 0u && a1 - (kIntExpLo << 7) >= ((kIntExpHi - kIntExpLo + 1u) << 7);
-        if (__any_sync(0xFFFFFFFFu, odd0 || odd1)) {
+        if (__any_sync(0xFFFFFFFFu, pq::int_scale_is_odd(a0) || pq::int_scale_is_odd(a1))) {
             e0 = int_row_sse<TEAM16>(u, 0, bf16_pattern(a0), Qf), e1 = int_row_sse<TEAM16>(u, 1, bf16_pattern(a1), Qf);
             return;
         }
-        const uint32_t c0 = max(a0, kIntExpLo << 7), c1 = max(a1, kIntExpLo << 7);
-        const uint2 t0 = int_tab[c0 & 0x7Fu], t1 = int_tab[c1 & 0x7Fu];
-        const uint32_t x0 = (c0 & 0x7F80u) << 16, x1 = (c1 & 0x7F80u) << 16;
-        r2 = pack2(__uint_as_float(t0.x - x0), __uint_as_float(t1.x - x1));
-        nd2 = pack2(__uint_as_float(t0.y + x0), __uint_as_float(t1.y + x1));
+        float r0, r1, nd0, nd1;
+        pq::int_scale_from_tab(int_tab, a0, r0, nd0);
+        pq::int_scale_from_tab(int_tab, a1, r1, nd1);
+        r2 = pack2(r0, r1), nd2 = pack2(nd0, nd1);
     }
 
     uint64_t run2[2];
@@ -387,7 +361,7 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     if (KIND == 0) {
         for (int s = 0; s < sides; ++s) build_scale_tab(reinterpret_cast<ScaleTab *>(tab_s + s * kTabBytes)[0], __ldg(p.ts[s]));
     } else {
-        build_int_tab(int_tab, p.Qf);
+        pq::build_int_tab(int_tab, p.Qf, true);
     }
     __syncthreads();
 

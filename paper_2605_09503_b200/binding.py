@@ -94,6 +94,20 @@ def lib():
     return _lib
 
 
+_native_module = None
+
+
+def native():
+    """The marshalling module of the runtime entry points (csrc/pq_native.cpp).  Fails loudly like lib()."""
+    global _native_module
+    if _native_module is None:
+        lib()
+        from . import _pq_native
+
+        _native_module = _pq_native
+    return _native_module
+
+
 def status_string(code):
     return lib().pq_status_string(code).decode()
 
@@ -109,14 +123,14 @@ def _check(name, code):
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _p(t):
     if t is None:
         return None
     assert t.is_cuda, "device tensors only"
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _bf16(t):
@@ -253,25 +267,14 @@ def pq_quant_weight(Wt, perm, perm_select, codes, sf, sf_layout, ts_w, ws):
                                                     w, wb, _stream()))
 
 
-def pq_calibrate(Xs, Wt, fmt, J, tau, sf_layout, sumsq_a, sumsq_w, amax_a, ts_x, ts_w, perms, err_x, err_w, lam, E, select,
-                 codes, sf):
-    """The offline pass over the batches Xs (list of bf16 [T, K]) and the weight Wt; the outputs are overwritten."""
-    n, (N, K) = len(Xs), _bf16(Wt).shape
-    for x in Xs:
-        assert _bf16(x).shape[1] == K and x.is_cuda, "device tensors of the weight's width only"
-    f64, f32, i32 = torch.float64, torch.float32, torch.int32
-    for t, dtype in ((sumsq_a, f64), (sumsq_w, f64), (amax_a, f32), (ts_x, f32), (ts_w, f32), (perms, i32), (err_x, f64),
-                     (err_w, f64), (lam, f64), (E, f64), (select, i32), (codes, torch.uint8), (sf, torch.uint8)):
-        assert t.dtype == dtype and t.is_contiguous()
-    ptrs = (C.c_void_p * n)(*[x.data_ptr() for x in Xs])
-    rows, lds = (C.c_int64 * n)(*[x.shape[0] for x in Xs]), (C.c_int64 * n)(*[x.stride(0) for x in Xs])
-    form = pq_format(*fmt)
-    need = int(lib().pq_calibrate_workspace_bytes(n, rows, N, K, form, J))
-    ws = torch.empty(max(need, 256), dtype=torch.uint8, device=Wt.device)
-    _check("pq_calibrate", lib().pq_calibrate(
-        n, ptrs, rows, lds, _p(Wt), N, K, Wt.stride(0), form, J, float(tau), sf_layout, _p(sumsq_a), _p(sumsq_w), _p(amax_a),
-        _p(ts_x), _p(ts_w), _p(perms), _p(err_x), _p(err_w), _p(lam), _p(E), _p(select), _p(codes), _p(sf), _p(ws), ws.numel(),
-        _stream()))
+def pq_calibrate(Xs, Wt, fmt, J, tau, sf_layout):
+    """The offline pass over the batches Xs (list of bf16 [T, K]) and the weight Wt -> (sumsq_a, sumsq_w, amax_a, ts_x, ts_w,
+    perms, err_x, err_w, lam, E, select, codes, sf, number of rows), all but the last on the device."""
+    kind, bits, group = fmt
+    r = native().calibrate(Xs, Wt, kind, bits, group, J, tau, sf_layout)
+    if type(r) is int:
+        _check("pq_calibrate", r)
+    return r
 
 
 def pq_quant_act_nvfp4(X, ts_x, codes, sf, sf_layout):
@@ -292,22 +295,20 @@ def pq_quant_act_nvfp4_perm(X, perm, ts_x, codes, sf, sf_layout):
 
 
 def pq_gemm_w4a4(xq, sfx, ts_x, wq, sfw, ts_w, Y, ws):
-    M, K = xq.shape[0], xq.shape[1] * 2
-    N = wq.shape[0]
-    assert Y.dtype == torch.bfloat16 and Y.shape == (M, N) and Y.stride(1) == 1
-    w, wb = _ws(ws)
-    _check("pq_gemm_w4a4", lib().pq_gemm_w4a4(_p(xq), _p(sfx), _p(ts_x), _p(wq), _p(sfw), _p(ts_w), M, N, K,
-                                              _p(Y), Y.stride(0), w, wb, _stream()))
+    _check("pq_gemm_w4a4", native().gemm(xq, sfx, ts_x, wq, sfw, ts_w, Y, ws))
 
 
 def pq_linear_w4a4(X, ts_x, xq, sfx, wq, sfw, ts_w, Y, ws):
-    _bf16(X)
-    M, K = X.shape
-    N = wq.shape[0]
-    assert Y.dtype == torch.bfloat16 and Y.shape == (M, N) and Y.stride(1) == 1
-    w, wb = _ws(ws)
-    _check("pq_linear_w4a4", lib().pq_linear_w4a4(_p(X), M, K, X.stride(0), _p(ts_x), _p(xq), _p(sfx), _p(wq),
-                                                  _p(sfw), _p(ts_w), N, _p(Y), Y.stride(0), w, wb, _stream()))
+    assert Y is not None
+    linear(X, ts_x, xq, sfx, wq, sfw, ts_w, Y, ws)
+
+
+def linear(X, ts_x, xq, sfx, wq, sfw, ts_w, Y, ws):
+    """pq_linear_w4a4 into Y, or into a new bf16 tensor [M, N] when Y is None; returns the output."""
+    r = native().linear(X, ts_x, xq, sfx, wq, sfw, ts_w, Y, ws)
+    if type(r) is int:
+        _check("pq_linear_w4a4", r)
+    return r
 
 
 def pq_linear_w4a4_batched(Xs, ts_x, xqs, sfxs, wq, sfw, ts_w, Ys, ws):
@@ -363,12 +364,8 @@ def pq_linear_w4a4_host(X_host, ts_x, X_dev, xq, sfx, wq, sfw, ts_w, Y_dev, Y_ho
 
 
 def pq_fakequant_int(T, fmt, perm, out):
-    _bf16(T)
-    _bf16(out)
     kind, bits, group = fmt
-    _check("pq_fakequant_int", lib().pq_fakequant_int(_p(T), T.shape[0], T.shape[1], T.stride(0),
-                                                      pq_format(kind, bits, group), _p(perm), _p(out),
-                                                      out.stride(0), _stream()))
+    _check("pq_fakequant_int", native().fakequant(T, kind, bits, group, perm, out))
 
 
 def pq_sf_to_linear(sf_tc, rows, K, sf_linear):
@@ -379,26 +376,13 @@ NORM_RMS, NORM_ADALN = 0, 1
 
 
 def pq_norm_quant_nvfp4(H, kind, a, b, eps, perm, ts_x, codes, sf, sf_layout, y_out=None):
-    _bf16(H)
-    M, K = H.shape
-    assert a.dtype == torch.float32 and a.numel() == K and (b is None or (b.dtype == torch.float32 and b.numel() == K))
-    assert perm is None or (perm.dtype == torch.int32 and perm.numel() == K)
-    assert y_out is None or (y_out.dtype == torch.bfloat16 and y_out.shape == (M, K) and y_out.is_contiguous())
-    _check("pq_norm_quant_nvfp4", lib().pq_norm_quant_nvfp4(_p(H), M, K, H.stride(0), kind, _p(a), _p(b), eps, _p(perm),
-                                                            _p(ts_x), _p(codes), _p(sf), sf_layout, _p(y_out), _stream()))
+    _check("pq_norm_quant_nvfp4", native().norm_quant(H, kind, a, b, eps, perm, ts_x, codes, sf, sf_layout, y_out))
 
 
 def pq_hadamard_quant_nvfp4(X, perm, ts_x, codes, sf, sf_layout, y_out=None):
     """Rows of X through the Hadamard transform, channels read in the order perm, NVFP4 codes and scales of
     the result (codes = sf = None: transform only, into y_out)."""
-    _bf16(X)
-    M, K = X.shape
-    assert perm is None or (perm.dtype == torch.int32 and perm.numel() == K and perm.is_contiguous())
-    assert (codes is None) == (sf is None)
-    assert codes is None or (codes.dtype == torch.uint8 and sf.dtype == torch.uint8 and ts_x.dtype == torch.float32)
-    assert y_out is None or (y_out.dtype == torch.bfloat16 and y_out.shape == (M, K) and y_out.is_contiguous())
-    _check("pq_hadamard_quant_nvfp4", lib().pq_hadamard_quant_nvfp4(_p(X), M, K, X.stride(0), _p(perm), _p(ts_x),
-                                                                    _p(codes), _p(sf), sf_layout, _p(y_out), _stream()))
+    _check("pq_hadamard_quant_nvfp4", native().hadamard_quant(X, perm, ts_x, codes, sf, sf_layout, y_out))
 
 
 def pq_device_status(ws):

@@ -46,20 +46,7 @@ class Calibration:
 def calibrate(batches, Wt, fmt=NVFP4, J=5, tau=0.0, sf_layout=B.PQ_SF_TCGEN05) -> Calibration:
     """Offline pass over calibration batches (list of bf16 [T, K] device tensors) and the weight
     Wt (bf16 [N, K] device tensor).  `fmt` is the format whose error drives the acceptance rule."""
-    N, K = Wt.shape
-    Kg = K // (16 if fmt[0] == B.KIND_NVFP4 else fmt[2])
-
-    def out(dtype, *shape):
-        return torch.empty(shape, dtype=dtype, device=Wt.device)
-
-    f64, f32, i32, u8 = torch.float64, torch.float32, torch.int32, torch.uint8
-    c = Calibration(sumsq_a=out(f64, K), sumsq_w=out(f64, K), amax_a=out(f32, K), ts_x=out(f32, 1), ts_w=out(f32, 1),
-                    perms=out(i32, J + 1, K), err_x=out(f64, J + 2, Kg), err_w=out(f64, J + 2, Kg), lam=out(f64, 2),
-                    E=out(f64, J + 2), select=out(i32, 2), wq=out(u8, N, K // 2), sfw=out(u8, B.sf_bytes(N, K, sf_layout)),
-                    rows_a=sum(x.shape[0] for x in batches))
-    B.pq_calibrate(batches, Wt, fmt, J, tau, sf_layout, c.sumsq_a, c.sumsq_w, c.amax_a, c.ts_x, c.ts_w, c.perms, c.err_x,
-                   c.err_w, c.lam, c.E, c.select, c.wq, c.sfw)
-    return c
+    return Calibration(*B.pq_calibrate(batches, Wt, fmt, J, tau, sf_layout))
 
 
 def calibrate_h(batches, Wt, fmt=NVFP4, J=5, tau=0.0):
@@ -123,12 +110,9 @@ class QuantLinear:
         self._sets = []          # further (xq, sfx) pairs for forward_batches
 
     def __call__(self, X, Y=None):
-        M = X.shape[0]
-        assert M <= self.M_max and X.shape[1] == self.K
-        if Y is None:
-            Y = torch.empty(M, self.N, dtype=torch.bfloat16, device=X.device)
-        B.pq_linear_w4a4(X, self.ts_x, self.xq[:M], self.sfx, self.wq, self.sfw, self.ts_w, Y, self.ws)
-        return Y
+        M, K = X.shape
+        assert M <= self.M_max and K == self.K
+        return B.linear(X, self.ts_x, self.xq, self.sfx, self.wq, self.sfw, self.ts_w, Y, self.ws)  # uses M rows of xq
 
     def forward_batches(self, Xs, Ys, n_sets=4):
         """Independent batches through the layer, the quantizer of the next batches overlapped with
@@ -160,10 +144,11 @@ class QuantLinearH(QuantLinear):
         self.order = None if order is None else order.to(torch.int32).contiguous()
 
     def __call__(self, X, Y=None):
-        M = X.shape[0]
-        assert M <= self.M_max and X.shape[1] == self.K
+        M, K = X.shape
+        assert M <= self.M_max and K == self.K
         if Y is None:
             Y = torch.empty(M, self.N, dtype=torch.bfloat16, device=X.device)
-        B.pq_hadamard_quant_nvfp4(X, self.order, self.ts_x, self.xq[:M], self.sfx, B.PQ_SF_TCGEN05)
-        B.pq_gemm_w4a4(self.xq[:M], self.sfx, self.ts_x, self.wq, self.sfw, self.ts_w, Y, self.ws)
+        xq = self.xq if M == self.M_max else self.xq[:M]
+        B.pq_hadamard_quant_nvfp4(X, self.order, self.ts_x, xq, self.sfx, B.PQ_SF_TCGEN05)
+        B.pq_gemm_w4a4(xq, self.sfx, self.ts_x, self.wq, self.sfw, self.ts_w, Y, self.ws)
         return Y

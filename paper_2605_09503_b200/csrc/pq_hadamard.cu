@@ -354,6 +354,214 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) hadamard_quant_kernel(
     }
 }
 
+// ---- one warp per row (K = 12 * 256), or per two or four rows (12 * 128, 12 * 64)
+// 32 octet positions of twelve segments are exactly one phase-1 item per lane, so a warp can carry its row(s)
+// through all phases by itself: no block barrier, and the phases of the SM's sixteen warps, which load
+// different units (fp32 pipe, shared memory, conversions), run beside each other.  The block version above
+// holds its rows in step, and its second pass has 384 items for 256 threads: 32.6 us at 4608 x 3072 where this
+// takes 23.5, 18.5 / 14.2 at 4608 x 1536, 26.7 / 13.8 at 9216 x 768, 11.3 / 8.8 at 512 x 3072.  The warp's 12 KB image stays conflict-free: octet b of segment a lies
+// at octet b ^ (a & 3) (the strided column accesses of phase 2: four segments per half warp), its 16-byte halves
+// swapped by bit 2 of b (the stores of phase 1).
+constexpr int kRowWarps = 8;            // per block; two blocks per SM at 128 registers
+constexpr int kRowImage = 3072;         // fp32 values per warp
+
+template <int N>
+__device__ __forceinline__ int row_image_index(int channel) {  // of a channel inside its row's image
+    constexpr int SEG = 1 << N;
+    const int a = channel >> N, b = (channel & (SEG - 1)) >> 3, e = channel & 7;
+    return (a << N) + ((b ^ (a & 3)) << 3) + (e ^ (((b >> 2) & 1) << 2));
+}
+
+// 2^LOG values of one column (of WIDTH neighbouring channels: 1 or 2) at the octet stride, in place.
+template <int LOG, typename T>
+__device__ __forceinline__ void column_pass(float *image, int a_base, int s, int e, float scale) {
+    constexpr int NV = 1 << LOG;
+    T *slot[8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b)
+        slot[b] = reinterpret_cast<T *>(image + a_base + ((b ^ s) << 3) + (e ^ ((b >> 2) << 2)));
+    constexpr int kStep = 64 * sizeof(float) / sizeof(T);  // eight octets further
+    T v[NV];
+#pragma unroll
+    for (int b = 0; b < NV; ++b) v[b] = slot[b & 7][(b >> 3) * kStep];
+#pragma unroll
+    for (int l = 0; l < LOG; ++l) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+            if ((j >> l) & 1) continue;
+            const T p = v[j], q = v[j | (1 << l)];
+            if constexpr (sizeof(T) == 8) {
+                v[j] = add2(p, q);
+                v[j | (1 << l)] = sub2(p, q);
+            } else {
+                v[j] = __fadd_rn(p, q);
+                v[j | (1 << l)] = __fsub_rn(p, q);
+            }
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < NV; ++b) {
+        if constexpr (sizeof(T) == 8) slot[b & 7][(b >> 3) * kStep] = mul2(v[b], pack2(scale, scale));
+        else slot[b & 7][(b >> 3) * kStep] = __fmul_rn(v[b], scale);
+    }
+}
+
+// Column a' of the order-12 combination for one half of an octet (two channel pairs) and strides 1, 2.  The first half
+// waits in the image; the second takes stride 4 with it and writes both.  Half an octet at a time keeps the inputs in
+// 48 registers: with the whole octet (96) the compiler spilled 300 bytes per thread at 128 registers.
+template <int AP, int A>
+__device__ __forceinline__ void combine_segments_half(uint64_t (&acc)[2], const uint64_t (&in)[12][2]) {
+    if constexpr (A < 12) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            if constexpr (Paley12<A, AP>::plus) acc[e] = add2(acc[e], in[A][e]);
+            else acc[e] = sub2(acc[e], in[A][e]);
+        }
+        combine_segments_half<AP, A + 1>(acc, in);
+    }
+}
+template <int N, int HALF, int AP>
+__device__ __forceinline__ void row_column_12(const uint64_t (&in)[12][2], float *row_s, int b) {
+    uint64_t v[2] = {in[0][0], in[0][1]};  // the first row of the matrix is all ones
+    combine_segments_half<AP, 1>(v, in);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) v[e] = butterfly_in_pair(v[e]);
+    const uint64_t c0 = add2(v[0], v[1]), c1 = sub2(v[0], v[1]);
+    const int half = (b >> 2) & 1;
+    ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(row_s + (AP << N) + ((b ^ (AP & 3)) << 3));
+    if (HALF == 0) {
+        dst[half] = make_ulonglong2(c0, c1);
+    } else {
+        const ulonglong2 f = dst[half];
+        dst[half] = make_ulonglong2(add2(f.x, c0), add2(f.y, c1));
+        dst[half ^ 1] = make_ulonglong2(sub2(f.x, c0), sub2(f.y, c1));
+    }
+}
+template <int N, int HALF, int... APs>
+__device__ __forceinline__ void row_columns_12(std::integer_sequence<int, APs...>, const uint4 (&raw)[12], float *row_s, int b) {
+    uint64_t in[12][2];
+#pragma unroll
+    for (int a = 0; a < 12; ++a) {
+        const uint32_t w0 = HALF ? raw[a].z : raw[a].x, w1 = HALF ? raw[a].w : raw[a].y;
+        in[a][0] = pack2(__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xFFFF0000u));
+        in[a][1] = pack2(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xFFFF0000u));
+    }
+    (row_column_12<N, HALF, APs>(in, row_s, b), ...);
+}
+
+template <int SF_LAYOUT, int N>
+__global__ void __launch_bounds__(32 * kRowWarps, 2) hadamard_quant_rows_kernel(const HadParams p) {
+    constexpr int SEG = 1 << N, K = 12 * SEG, OCTS = SEG / 8, RPW = 32 / OCTS, LOG = N - 3, GPR = K / 16;
+    extern __shared__ __align__(16) float had_smem[];  // [warps][3072] fp32, then K 16-bit read-out offsets in two planes
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *image = had_smem + warp * kRowImage;
+    uint16_t *offset_s = reinterpret_cast<uint16_t *>(had_smem + kRowWarps * kRowImage);
+    const uint4 *offset4 = reinterpret_cast<const uint4 *>(offset_s);
+    pq::wait_for_prior_grid();
+    pq::dependents_may_launch();
+    // byte offset of the channel each output position reads; positions 0-7 and 8-15 of a group in separate planes,
+    // so that the lanes' 16-byte reads are adjacent
+    for (int j = threadIdx.x; j < K; j += 32 * kRowWarps)
+        offset_s[((j >> 3) & 1) * (K / 2) + (j >> 4) * 8 + (j & 7)] =
+            static_cast<uint16_t>(row_image_index<N>(p.perm ? __ldg(p.perm + j) : j) << 2);
+    const float ts = p.codes ? __ldg(p.ts) : 1.0f;
+    __syncthreads();
+
+    // warps of different blocks first, so that few rows spread over all SMs
+    const int64_t batches = (p.rows_pad + RPW - 1) / RPW, step = static_cast<int64_t>(gridDim.x) * kRowWarps;
+    for (int64_t batch = static_cast<int64_t>(warp) * gridDim.x + blockIdx.x; batch < batches; batch += step) {
+        const int64_t row0 = batch * RPW;
+        if (row0 < p.rows) {
+            // ---- phase 1: lane = (row, octet); rows past the end are zeros
+            const int r = lane / OCTS, b = lane % OCTS;
+            const uint16_t *src = p.X + (row0 + r) * p.ld + b * 8;
+            const bool have = row0 + r < p.rows;
+            uint4 raw[12];
+#pragma unroll
+            for (int a = 0; a < 12; ++a)
+                raw[a] = have ? __ldcs(reinterpret_cast<const uint4 *>(src + a * SEG)) : make_uint4(0, 0, 0, 0);
+            __syncwarp();  // the previous rows have been read out
+            row_columns_12<N, 0>(std::make_integer_sequence<int, 12>{}, raw, image + r * K, b);
+            row_columns_12<N, 1>(std::make_integer_sequence<int, 12>{}, raw, image + r * K, b);
+            // the next rows of this warp, into L2 while the remaining phases run
+            if (row0 + step * RPW + r < p.rows) {
+#pragma unroll
+                for (int a = 0; a < 12; ++a)
+                    if ((b & 7) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + step * RPW * p.ld + a * SEG));
+            }
+            __syncwarp();
+            // ---- phase 2: the remaining strides, column by column; 48 pair columns per row
+            if constexpr (N == 8) {
+                // 48 pair columns for 32 lanes: 32 of them as pairs, the other 16 as 32 single columns
+                column_pass<LOG, uint64_t>(image, (lane >> 2) << N, (lane >> 2) & 3, (lane & 3) * 2, p.scale);
+                const int a = 8 + (lane >> 3);
+                column_pass<LOG, float>(image, a << N, a & 3, lane & 7, p.scale);
+            } else {
+#pragma unroll 1
+                for (int i = lane; i < 48 * RPW; i += 32) {
+                    const int row = i / 48, c = i - row * 48, a = c >> 2;
+                    column_pass<LOG, uint64_t>(image, row * K + (a << N), a & 3, (c & 3) * 2, p.scale);
+                }
+            }
+            __syncwarp();
+        }
+        // ---- phase 3: one output group per lane, 192 groups
+#pragma unroll 1
+        for (int i = lane; i < RPW * GPR; i += 32) {
+            const int r = i / GPR, g = i - r * GPR;
+            const int64_t row = row0 + r;
+            const bool live = row < p.rows;
+            float out[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) out[j] = 0.0f;
+            if (live) {
+                const uint4 i0 = offset4[g], i1 = offset4[GPR + g];
+                const uint32_t iw[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
+                const char *row_b = reinterpret_cast<const char *>(image + r * K);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    out[2 * j] = *reinterpret_cast<const float *>(row_b + (iw[j] & 0xFFFFu));
+                    out[2 * j + 1] = *reinterpret_cast<const float *>(row_b + (iw[j] >> 16));
+                }
+                if (p.y_out) {
+                    uint32_t yw[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
+                                (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
+                    uint4 *ydst = reinterpret_cast<uint4 *>(p.y_out + row * K) + 2 * g;
+                    ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                    ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                }
+            }
+            if (!p.codes) continue;
+            float amax = 0.0f, d, rcp;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(out[j]));
+            uint32_t sf8;
+            pq::nvfp4_scale(amax, ts, sf8, d, rcp);
+            if (live) {
+                const uint64_t rcp2 = pack2(rcp, rcp);
+                float ylo[8], yhi[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    unpack2(mul2(pack2(out[2 * j], out[2 * j + 1]), rcp2), ylo[2 * j], ylo[2 * j + 1]);
+                    unpack2(mul2(pack2(out[8 + 2 * j], out[9 + 2 * j]), rcp2), yhi[2 * j], yhi[2 * j + 1]);
+                }
+                *reinterpret_cast<uint2 *>(p.codes + row * (K / 2) + g * 8) = make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
+            }
+            // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
+            uint32_t word = sf8;
+            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 1) << 8;
+            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2) << 16;
+            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3) << 24;
+            if ((g & 3) || row >= p.rows_pad) continue;
+            if (SF_LAYOUT == PQ_SF_TCGEN05) *reinterpret_cast<uint32_t *>(p.sf + pq::sf_tc_offset(row, g, GPR >> 2)) = word;
+            else if (live) *reinterpret_cast<uint32_t *>(p.sf + row * GPR + g) = word;
+        }
+    }
+}
+
 // K = m * 2^n with m in {1, 12} and 2^n >= 8; returns false otherwise.
 bool factor_width(int64_t K, int &m, int &n) {
     if (K <= 0) return false;
@@ -398,14 +606,28 @@ extern "C" pq_status pq_hadamard_quant_nvfp4(const void *X, int64_t M, int64_t K
     p.sw = p.log[0] ? 3 + p.log[0] : 30;
     p.scale = static_cast<float>(1.0 / sqrt(static_cast<double>(K)));
     p.perm = perm, p.ts = ts_x, p.codes = codes, p.sf = sf, p.y_out = static_cast<uint16_t *>(y_out);
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (m == 12 && n >= 6 && n <= 8) {  // widths whose rows fit a warp's lanes exactly: 768, 1536, 3072
+        const size_t row_smem = static_cast<size_t>(kRowWarps) * kRowImage * sizeof(float) + static_cast<size_t>(K) * sizeof(uint16_t);
+        const int64_t warps = pq_ceil_div(p.rows_pad, 1 << (8 - n));
+        auto launch_rows = [&](auto kern) -> pq_status {
+            PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(row_smem)));
+            PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(std::min<int64_t>(warps, 2 * sms))), dim3(32 * kRowWarps),
+                                            row_smem, static_cast<cudaStream_t>(stream), p));
+            return pq_launch_status();
+        };
+        const bool tc = sf_layout == PQ_SF_TCGEN05;
+        if (n == 8) return tc ? launch_rows(hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 8>) : launch_rows(hadamard_quant_rows_kernel<PQ_SF_LINEAR, 8>);
+        if (n == 7) return tc ? launch_rows(hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 7>) : launch_rows(hadamard_quant_rows_kernel<PQ_SF_LINEAR, 7>);
+        return tc ? launch_rows(hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 6>) : launch_rows(hadamard_quant_rows_kernel<PQ_SF_LINEAR, 6>);
+    }
     const size_t row_bytes = static_cast<size_t>(K) * sizeof(float);
     p.rows_per_block = static_cast<int>(kSmemBudget / row_bytes < kMaxRows ? kSmemBudget / row_bytes : kMaxRows);
     const int kRows = p.rows_per_block;
     const size_t smem = static_cast<size_t>(kRows) * row_bytes + static_cast<size_t>(K) * sizeof(uint16_t);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // persistent grid: as many blocks as fit on the device at once, walking over the batches of rows
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool wide_block = kRows < kMaxRows;  // fewer rows per block: twice the threads on them, one block per SM
     const int per_sm = static_cast<int>(std::min<size_t>(wide_block ? 1 : kBlocksPerSm, (227 * 1024) / (smem + 1024)));
     const int64_t batches = pq_ceil_div(p.rows_pad, kRows);

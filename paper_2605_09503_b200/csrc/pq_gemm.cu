@@ -21,7 +21,7 @@
 //                boxes in swizzled shared memory and write them with TMA stores (full 128-byte
 //                lines) while the next tile's main loop runs.
 //   warps 10..17 scale-factor stagers: read the stage's scale blocks from shared memory and write
-//                them into one of two scale slots in tensor memory with tcgen05.st (one warp per
+//                them into one of the scale slots in tensor memory with tcgen05.st (one warp per
 //                lane quadrant; two sets of four warps take alternate K iterations).
 // 256 divides every FLUX output width (3072, 9216, 12288).  The 512 tensor-memory columns hold one
 // 256-column accumulator plus two scale slots (2 x 48); the epilogue warps pull the accumulator
@@ -66,11 +66,6 @@ constexpr int kSfaBytes = 4 * kSfBlock;    // 4 K-blocks of one 128-row block
 constexpr int kTmemCols = 512;
 constexpr long long kWaitCycles = 4000000000ll;  // default limit of a wait: about two seconds of SM clock
 
-constexpr int BN = 256, BN_CTA = BN / 2;
-constexpr int kStages = 5;
-constexpr int kBBytes = BN_CTA * BK / 2;   // 16384
-constexpr int kSfbBytes = 2 * kSfaBytes;   // the two 128-row blocks of the tile's 256 B rows
-constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38912 = 38 * 1024
 constexpr int kEpiWarps = 8;               // lane quadrant x column half of the accumulator
 constexpr int kBoxCols = 64;               // output staging box: 32 rows x 64 bf16, one TMA store
 constexpr int kEpiBox = 32 * kBoxCols * 2;
@@ -103,16 +98,35 @@ constexpr int kThreads = 32 * (kFirstStager + 4 * kStagerSets);   // producer, M
 // it - kStages (stage_free, which the producer waited for before it refilled the stage) in front of
 // the sf_ready wait, so that wait is sound whatever the slot count; the assertions keep the original
 // condition as well.
-constexpr int kSfSlots = 2;
-constexpr uint32_t kSfSlotCol0 = BN, kSfbColsPerKb = 8, kSfbOfs = 16;
-constexpr uint32_t kSfSlotCols = 4 * (4 + kSfbColsPerKb);   // 48
-static_assert(kSfSlotCol0 + kSfSlots * kSfSlotCols <= 512, "tensor memory columns");
-static_assert(kSfSlots + kStagerSets <= kStages, "a stager set must know that the previous phase of sf_ready has completed");
-static_assert(kSfSlots <= 2 * kStages - 2, "the stagers' parity waits on stage_free must be unambiguous");
-// barriers: stage_full[S] sf_ready[S] stage_free[S] acc_full acc_empty
-constexpr int kNumBars = 3 * kStages + 2;
-constexpr size_t kSmemBytes = kStages * kStageBytes + kEpiBytes + 1024 /*alignment slack*/ + 8 * kNumBars + 64;
-static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
+//
+// Two tile widths.  The wide tile (256 columns) needs the fewest operand bytes per flop and is what every
+// product of more than one round of tiles runs on.  The narrow tile (128 columns) is for products that have at
+// most one such tile per CTA pair: twice as many pairs work on them, half the MMA time per K step, and since a
+// pair never has a next tile, the epilogue stages its boxes in the operand ring, which leaves room for eight stages.
+template <int BN>
+struct Tile {
+    static constexpr int kNCta = BN / 2;
+    static constexpr bool kOneTile = BN == 128;             // a pair computes one tile; the epilogue stages in the ring
+    static constexpr int kStages = BN == 256 ? 5 : 8;
+    static constexpr int kSfSlots = BN == 256 ? 2 : 4;
+    static constexpr int kNB = BN / 128;                  // 128-row scale blocks of B per tile
+    static constexpr int kBBytes = kNCta * BK / 2;
+    static constexpr int kSfbBytes = kNB * kSfaBytes;     // the 128-row blocks of the tile's B rows
+    static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38 or 28 * 1024
+    static constexpr uint32_t kSfSlotCol0 = BN, kSfbColsPerKb = 4 * kNB, kSfbOfs = 16;
+    static constexpr uint32_t kSfSlotCols = 4 * (4 + kSfbColsPerKb);   // 48 or 32
+    static constexpr int kNumBars = 3 * kStages + 2;      // stage_full[S] sf_ready[S] stage_free[S] acc_full acc_empty
+    static constexpr int kRingBytes = kStages * kStageBytes, kEpi = kOneTile ? 0 : kRingBytes;  // where the boxes start
+    static constexpr size_t kSmemBytes = kRingBytes + (kOneTile ? 0 : kEpiBytes) + 1024 /*alignment slack*/ + 8 * kNumBars + 64;
+    // Instruction descriptor: E2M1 x E2M1, UE4M3 scales, both K-major, M = 256 (pair), N = BN, K = 64.
+    static constexpr uint32_t kIdesc = (1u << 7) | (1u << 10) | (static_cast<uint32_t>(BN >> 3) << 17) | (0u << 23) |
+                                       (static_cast<uint32_t>(BM >> 4) << 24);
+    static_assert(kStageBytes % 1024 == 0, "swizzled operand tiles start on 1024-byte boundaries");
+    static_assert(kSfSlotCol0 + kSfSlots * kSfSlotCols <= 512, "tensor memory columns");
+    static_assert(kSfSlots + kStagerSets <= kStages, "a stager set must know that the previous phase of sf_ready has completed");
+    static_assert(kSfSlots <= 2 * kStages - 2, "the stagers' parity waits on stage_free must be unambiguous");
+    static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
+};
 
 struct GemmParams {
     const uint8_t *sfx, *sfw;
@@ -314,11 +328,6 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t smem_addr) {
     return static_cast<uint64_t>((smem_addr & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) |
            (2ull << 61);
 }
-// Instruction descriptor: E2M1 x E2M1, UE4M3 scales, both K-major, M = 256 (pair), N = BN, K = 64.
-constexpr uint32_t kIdesc = (1u << 7) | (1u << 10) | (static_cast<uint32_t>(BN >> 3) << 17) | (0u << 23) |
-                            (static_cast<uint32_t>(BM >> 4) << 24);
-
-
 // Two accumulator values times alpha, each rounded to bf16 (nearest even), packed low | high.
 #ifndef PQ_GEMM_EPI_PACKED
 #define PQ_GEMM_EPI_PACKED 1
@@ -352,17 +361,22 @@ __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo_bits, uint32_t hi_bits
 // The 1024 registers left there take one warp of a 32-register kernel, so 128-thread blocks of
 // other kernels can still run on the SM beside the GEMM.
 constexpr int kMaxRegs = 96;
+template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kMaxRegs)
 gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                  const __grid_constant__ CUtensorMap map_y, const GemmParams p) {
-    constexpr int kNB = BN / 128;  // 128-row scale blocks of B per tile
+    using T = Tile<BN>;
+    constexpr int kStages = T::kStages, kSfSlots = T::kSfSlots, kNB = T::kNB, BN_CTA = T::kNCta;
+    constexpr int kBBytes = T::kBBytes, kStageBytes = T::kStageBytes, kNumBars = T::kNumBars;
+    constexpr uint32_t kSfbOfs = T::kSfbOfs, kSfbColsPerKb = T::kSfbColsPerKb;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // identical in both CTAs of the pair
     uint8_t *base_ptr = smem_raw + (base - raw);
-    const uint32_t epi = base + kStages * kStageBytes;
-    const uint32_t bars = epi + kEpiBytes;
-    uint8_t *bars_ptr = base_ptr + kStages * kStageBytes + kEpiBytes;
+    constexpr int kBarOfs = T::kRingBytes + (T::kOneTile ? 0 : kEpiBytes);
+    const uint32_t epi = base + T::kEpi;
+    const uint32_t bars = base + kBarOfs;
+    uint8_t *bars_ptr = base_ptr + kBarOfs;
     // stage_full: operand bytes of both CTAs have landed (1 arrival + transaction bytes) and the
     // stage's scales are in tensor memory in both CTAs (8 stager-warp arrivals); leader's copy only
     auto stage_full_bar = [&](int s) { return bars + 8u * s; };
@@ -373,7 +387,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars_ptr + 8 * kNumBars);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_ptr + 8 * kNumBars + 8);
     const WaitCtx wctx{abort_flag, p.status, p.wait_cycles};
-    auto sf_slot_col = [](uint32_t t) { return kSfSlotCol0 + t * kSfSlotCols; };
+    auto sf_slot_col = [](uint32_t t) { return T::kSfSlotCol0 + t * T::kSfSlotCols; };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();  // 0 = pair leader
@@ -488,7 +502,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         for (int kk = 0; kk < 4; ++kk) {
                             if (kk < kb_valid) {
                                 const uint32_t accumulate = acc | static_cast<uint32_t>(kk);
-                                tc_mma_pair(d_tmem, da + 2 * kk, db + 2 * kk, kIdesc, sfa_t + 4 * kk,
+                                tc_mma_pair(d_tmem, da + 2 * kk, db + 2 * kk, T::kIdesc, sfa_t + 4 * kk,
                                             sfb_t + kSfbColsPerKb * kk, accumulate);
                             }
                         }
@@ -563,14 +577,14 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         }
     } else {
         // ------------------------------------------------------------ epilogue
-        // Eight warps: lane quadrant q x column half h.  A warp reads its 32 rows x 128 columns out of
-        // tensor memory, scales and rounds them to bf16 and keeps them packed in 64 registers; the
+        // Eight warps: lane quadrant q x column half h.  A warp reads its 32 rows x BN / 2 columns out of
+        // tensor memory, scales and rounds them to bf16 and keeps them packed in BN / 4 registers; the
         // accumulator goes back to the MMA issuer after those loads (a few hundred cycles), and the
-        // two 64-column boxes leave through one staging box and TMA stores behind the next tile's
+        // 64-column boxes leave through one staging box and TMA stores behind the next tile's
         // main loop.
-        constexpr int kBoxes = 128 / kBoxCols, kChunks = kBoxCols / 8;  // boxes per warp, 16-byte chunks per box row
+        constexpr int kCols = BN / 2, kBoxes = kCols / kBoxCols, kChunks = kBoxCols / 8;  // boxes per warp, 16-byte chunks per box row
         const int q = warp & 3;                // tensor-memory lane quadrant this warp may read
-        const int h = (warp - 2) >> 2;         // 128-column part
+        const int h = (warp - 2) >> 2;         // column half
         const float alpha = __fmul_rn(__ldg(p.ts_x), __ldg(p.ts_w));
         const uint32_t buf = epi + static_cast<uint32_t>(warp - 2) * kEpiBox;
         // 128-byte swizzle of the staging box (what the store's tensor map expects): chunk ^ (row & 7)
@@ -578,23 +592,23 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         uint32_t tcount = 0;
         for (int tile = pair; tile < total_tiles; tile += num_pairs, ++tcount) {
             const int m_blk = tile % p.m_tiles, n_blk = tile / p.m_tiles;
-            const int m0 = m_blk * BM + static_cast<int>(rank) * BM_CTA + q * 32, n0 = n_blk * BN + h * 128;
+            const int m0 = m_blk * BM + static_cast<int>(rank) * BM_CTA + q * 32, n0 = n_blk * BN + h * kCols;
             const bool got = mbar_wait(acc_full_bar, tcount & 1u, wctx);
             if (!__all_sync(0xFFFFFFFFu, got)) break;
             tc_fence_after();
-            const uint32_t acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + h * 128;
-            uint32_t pk[64];  // pk[8 c + i] = columns 16 c + 2 i, 16 c + 2 i + 1 of this lane's row
+            const uint32_t acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + h * kCols;
+            uint32_t pk[kCols / 2];  // pk[8 c + i] = columns 16 c + 2 i, 16 c + 2 i + 1 of this lane's row
             // two loads in flight: chunk c + 1 is on its way while chunk c is scaled and packed
             uint32_t va[16], vb[16];
             tc_ld16(acc, va);
 #pragma unroll
-            for (int c = 0; c < 8; c += 2) {
+            for (int c = 0; c < kCols / 16; c += 2) {
                 tc_wait_ld(va);
                 tc_ld16(acc + (c + 1) * 16, vb);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) pk[8 * c + i] = pack_bf16(va[2 * i], va[2 * i + 1], alpha);
                 tc_wait_ld(vb);
-                if (c + 2 < 8) tc_ld16(acc + (c + 2) * 16, va);
+                if (c + 2 < kCols / 16) tc_ld16(acc + (c + 2) * 16, va);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) pk[8 * (c + 1) + i] = pack_bf16(vb[2 * i], vb[2 * i + 1], alpha);
             }
@@ -715,13 +729,15 @@ bool make_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t row_bytes
 
 // Number of CTA pairs that can be resident at once on the current device (a cluster must fit inside
 // one GPC), after opting the kernel in to its dynamic shared memory there.  Both are per device.
+template <int BN>
 int resident_pairs() {
+    constexpr size_t kSmemBytes = Tile<BN>::kSmemBytes;
     static PqPerDevice cache;
     const int dev = pq_device_slot();
     if (dev < 0) return 0;
     std::lock_guard<std::mutex> guard(cache.lock);
     if (cache.value[dev]) return cache.value[dev];
-    if (cudaFuncSetAttribute(gemm_w4a4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(gemm_w4a4_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kSmemBytes)) != cudaSuccess) {
         (void)cudaGetLastError();
         return 0;
@@ -738,12 +754,66 @@ int resident_pairs() {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_w4a4_kernel, &cfg) != cudaSuccess || n <= 0) {
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_w4a4_kernel<BN>, &cfg) != cudaSuccess || n <= 0) {
         (void)cudaGetLastError();
         return 0;
     }
     cache.value[dev] = n;
     return n;
+}
+
+struct GemmArgs {
+    const uint8_t *xq, *sfx, *wq, *sfw;
+    const float *ts_x, *ts_w;
+    int64_t M, N, K, ldy;
+    void *Y, *ws;
+    cudaStream_t st;
+};
+
+template <int BN>
+pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
+    CUtensorMap map_a, map_b, map_y;
+    if (!make_map(&map_a, g.xq, g.M, g.K / 2, g.K / 2, BM_CTA, 1) || !make_map(&map_b, g.wq, g.N, g.K / 2, g.K / 2, Tile<BN>::kNCta, 1) ||
+        !make_map(&map_y, g.Y, g.M, g.N * 2, g.ldy * 2, 32, 2))
+        return PQ_ERR_CUDA;
+    GemmParams p;
+    p.sfx = g.sfx, p.sfw = g.sfw, p.ts_x = g.ts_x, p.ts_w = g.ts_w;
+    p.M = static_cast<int>(g.M), p.N = static_cast<int>(g.N), p.K = static_cast<int>(g.K);
+    p.m_tiles = static_cast<int>(pq_ceil_div(g.M, BM));
+    p.n_tiles = static_cast<int>(pq_ceil_div(g.N, BN));
+    p.k_tiles = static_cast<int>(pq_ceil_div(g.K, BK));
+    p.kb_total = static_cast<int>(g.K / 64);
+    p.kb4 = p.kb_total;
+    p.m_rowblocks = static_cast<int>(pq_ceil_div(g.M, 128));
+    p.n_rowblocks = static_cast<int>(pq_ceil_div(g.N, 128));
+    p.wait_cycles = kWaitCycles;
+    p.status = static_cast<int *>(g.ws);
+    const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
+    PQ_REQUIRE(!Tile<BN>::kOneTile || tiles <= pairs_max, PQ_ERR_SHAPE);
+    const int pairs = static_cast<int>(tiles < pairs_max ? tiles : pairs_max);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * pairs, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = Tile<BN>::kSmemBytes;
+    cfg.stream = g.st;
+    // Programmatic dependent launch: the kernel may start (barrier set-up, tensor-memory allocation,
+    // tensor-map prefetch) while the kernel in front of it in the stream drains (the quantizer, or
+    // the previous GEMM of a chain of layers); it waits for that kernel to complete with
+    // griddepcontrol.wait before touching global memory, so stream order is what the caller sees.
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    PQ_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel<BN>, map_a, map_b, map_y, p));
+    return PQ_OK;
+}
+
+// One round of narrow tiles covers the product.  Measured on both sides of the line (narrow against wide, us):
+// 128 x 3072 x 3072 6.9 / 8.4, 512 x 3072 x 3072 7.4 / 8.6, 512 x 3072 x 12288 18.1 / 21.0; beyond one round the wide tile wins:
+// 512 x 9216 x 3072 12.2 / 11.0, 1024 x 3072 x 3072 11.2 / 9.7, 4608 x 9216 x 3072 72.8 / 57.5.
+bool narrow_tiles(int64_t M, int64_t N, int pairs) {
+    return pq_ceil_div(M, BM) * pq_ceil_div(N, 128) <= pairs;
 }
 
 pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, const uint8_t *wq, const uint8_t *sfw,
@@ -759,44 +829,10 @@ pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, 
     PQ_REQUIRE(pq_aligned256(ws), PQ_ERR_ALIGN);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-    CUtensorMap map_a, map_b, map_y;
-    if (!make_map(&map_a, xq, M, K / 2, K / 2, BM_CTA, 1) || !make_map(&map_b, wq, N, K / 2, K / 2, BN_CTA, 1) ||
-        !make_map(&map_y, Y, M, N * 2, ldy * 2, 32, 2))
-        return PQ_ERR_CUDA;
-
-    const int pairs_max = resident_pairs();
-    if (pairs_max <= 0) return PQ_ERR_CUDA;
-
-    GemmParams p;
-    p.sfx = sfx, p.sfw = sfw, p.ts_x = ts_x, p.ts_w = ts_w;
-    p.M = static_cast<int>(M), p.N = static_cast<int>(N), p.K = static_cast<int>(K);
-    p.m_tiles = static_cast<int>(pq_ceil_div(M, BM));
-    p.n_tiles = static_cast<int>(pq_ceil_div(N, BN));
-    p.k_tiles = static_cast<int>(pq_ceil_div(K, BK));
-    p.kb_total = static_cast<int>(K / 64);
-    p.kb4 = p.kb_total;
-    p.m_rowblocks = static_cast<int>(pq_ceil_div(M, 128));
-    p.n_rowblocks = static_cast<int>(pq_ceil_div(N, 128));
-    p.wait_cycles = kWaitCycles;
-    p.status = static_cast<int *>(ws);
-    const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
-    const int pairs = static_cast<int>(tiles < pairs_max ? tiles : pairs_max);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pairs, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = st;
-    // Programmatic dependent launch: the kernel may start (barrier set-up, tensor-memory allocation,
-    // tensor-map prefetch) while the kernel in front of it in the stream drains (the quantizer, or
-    // the previous GEMM of a chain of layers); it waits for that kernel to complete with
-    // griddepcontrol.wait before touching global memory, so stream order is what the caller sees.
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    PQ_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel, map_a, map_b, map_y, p));
-    return PQ_OK;
+    const int pairs_max = resident_pairs<256>(), pairs_narrow = resident_pairs<128>();
+    if (pairs_max <= 0 || pairs_narrow <= 0) return PQ_ERR_CUDA;
+    const GemmArgs g{xq, sfx, wq, sfw, ts_x, ts_w, M, N, K, ldy, Y, ws, st};
+    return narrow_tiles(M, N, pairs_narrow) ? launch_tiles<128>(g, pairs_narrow) : launch_tiles<256>(g, pairs_max);
 }
 }  // namespace
 

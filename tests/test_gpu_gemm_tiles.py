@@ -1,0 +1,22 @@
+"""Both tile widths of the GEMM at the line between them (one round of narrow tiles over 74 CTA pairs) and where the
+narrow one's operand ring wraps: exact cases, bit for bit against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import pq_oracle as O
+from test_gpu_gemm import bf16_round, gemm, pack
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,N,K", [(300, 4736, 128), (300, 4744, 128),            # 74 narrow tiles; 76: the wide one
+                                   (256, 128, 64), (1, 8, 2048), (257, 136, 2112),  # 1, 8 and 9 K steps, ragged edges
+                                   (130, 264, 4352)])                             # the ring wraps twice
+def test_exact_at_the_line(M, N, K):
+    rng = np.random.default_rng(M + N + K)
+    pick = np.array([0, 2, 4, 10, 12], np.uint8)
+    xn, wn = pick[rng.integers(0, 5, (M, K))], pick[rng.integers(0, 5, (N, K))]
+    pow2 = np.array([0x30, 0x38, 0x40, 0x48], np.uint8)             # 0.5, 1, 2, 4
+    sfx, sfw = pow2[rng.integers(0, 4, (M, K // 16))], pow2[rng.integers(0, 4, (N, K // 16))]
+    Y = gemm(pack(xn), sfx, 0.5, pack(wn), sfw, 4.0, ldy=N + 8)
+    assert np.array_equal(Y, bf16_round(O.gemm_ref(pack(xn), sfx, 0.5, pack(wn), sfw, 4.0)))

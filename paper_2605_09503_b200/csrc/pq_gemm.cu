@@ -24,7 +24,7 @@
 //                them into one of the scale slots in tensor memory with tcgen05.st (one warp per
 //                lane quadrant; two sets of four warps take alternate K iterations).
 // 256 divides every FLUX output width (3072, 9216, 12288).  The 512 tensor-memory columns hold one
-// 256-column accumulator plus two scale slots (2 x 48); the epilogue warps pull the accumulator
+// 256-column accumulator plus three scale slots (3 x 48); the epilogue warps pull the accumulator
 // into registers as packed bf16 within a few hundred cycles and store it from there.
 //
 // Measurements on B200 behind these choices:
@@ -99,6 +99,10 @@ constexpr int kThreads = 32 * (kFirstStager + 4 * kStagerSets);   // producer, M
 // the sf_ready wait, so that wait is sound whatever the slot count; the assertions keep the original
 // condition as well.
 //
+// Three slots for the wide tile are what the condition allows with five stages: 57.5 -> 56.8 us (4608 x 3072 x 9216)
+// and 66.3 -> 64.1 us (4608 x 12288 x 3072) against two.  A third set of stagers (80 registers per thread) made both
+// slower, 59.5 and 67.3 us.
+//
 // Two tile widths.  The wide tile (256 columns) needs the fewest operand bytes per flop and is what every
 // product of more than one round of tiles runs on.  The narrow tile (128 columns) is for products that have at
 // most one such tile per CTA pair: twice as many pairs work on them, half the MMA time per K step, and since a
@@ -108,7 +112,7 @@ struct Tile {
     static constexpr int kNCta = BN / 2;
     static constexpr bool kOneTile = BN == 128;             // a pair computes one tile; the epilogue stages in the ring
     static constexpr int kStages = BN == 256 ? 5 : 8;
-    static constexpr int kSfSlots = BN == 256 ? 2 : 4;
+    static constexpr int kSfSlots = BN == 256 ? 3 : 4;
     static constexpr int kNB = BN / 128;                  // 128-row scale blocks of B per tile
     static constexpr int kBBytes = kNCta * BK / 2;
     static constexpr int kSfbBytes = kNB * kSfaBytes;     // the 128-row blocks of the tile's B rows
@@ -810,8 +814,8 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
 }
 
 // One round of narrow tiles covers the product.  Measured on both sides of the line (narrow against wide, us):
-// 128 x 3072 x 3072 6.9 / 8.4, 512 x 3072 x 3072 7.4 / 8.6, 512 x 3072 x 12288 18.1 / 21.0; beyond one round the wide tile wins:
-// 512 x 9216 x 3072 12.2 / 11.0, 1024 x 3072 x 3072 11.2 / 9.7, 4608 x 9216 x 3072 72.8 / 57.5.
+// 128 x 3072 x 3072 6.9 / 8.1, 512 x 3072 x 3072 7.4 / 8.3, 512 x 3072 x 12288 18.0 / 20.5; beyond one round the wide tile wins:
+// 512 x 9216 x 3072 12.2 / 10.9, 1024 x 3072 x 3072 11.2 / 9.4, 4608 x 9216 x 3072 72.8 / 56.9.
 bool narrow_tiles(int64_t M, int64_t N, int pairs) {
     return pq_ceil_div(M, BM) * pq_ceil_div(N, 128) <= pairs;
 }

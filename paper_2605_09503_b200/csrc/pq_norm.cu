@@ -2,7 +2,7 @@
 // the channel reordering absorbed into it, and the NVFP4 quantizer of the runtime path (Eq. 8)
 // attached, so the normalized activations never make a bf16 round trip through HBM.
 //
-// A warp owns whole token rows.  A row is read once with coalesced 16-byte loads (lane l owns the
+// A row is read once with coalesced 16-byte loads (lane l owns the
 // octets l, l + 32, ...: the summation order of the row statistics is this walk followed by a
 // butterfly over the lanes, and does not depend on the permutation) and kept in shared memory as
 // bf16; then the lanes walk the OUTPUT order, gather their channels from shared memory through the
@@ -12,11 +12,13 @@
 // one 32-bit store).  The normalized values exist only in registers, in fp32.  Optionally the
 // reordered bf16 tensor of the unfused kernel is written too.
 //
-// Three kernels: rows of up to 6400 channels go four per warp (below, second kernel); wider rows one
-// per warp, eight positions per lane (first kernel); and without a permutation (channels already in
-// output order) rows of up to 4096 channels never leave the registers (third kernel).  KIND 0 is RMSNorm,
-// 1 adaptive LayerNorm; the four-row kernel also exists as KIND 2, no normalization at all: the gather
+// Four kernels: four rows per warp (second) or four rows per block (third) for rows of up to 16384 channels;
+// wider rows one per warp, eight positions per lane (first); and without a permutation (channels already in
+// output order) rows of up to 4096 channels never leave the registers (fourth).  KIND 0 is RMSNorm,
+// 1 adaptive LayerNorm; the four-rows-per-block kernel also exists as KIND 2, no normalization at all: the gather
 // quantizers of the offline path (a candidate order applied to activations or to the weight) run through it.
+#include <algorithm>
+
 #include "pq_common.cuh"
 
 namespace {
@@ -26,6 +28,7 @@ constexpr int kMaxRowsPerBlock = 8;
 #define PQ_NORM_POS 8
 #endif
 constexpr size_t kSmemBudget = 200 * 1024;
+constexpr int kQuadRegs = 80;  // four 192-thread blocks per SM at 3072 channels; 96 registers (three): 20.0 / 24.1 us
 
 __device__ __forceinline__ float lane_butterfly(float p) {
 #pragma unroll
@@ -238,12 +241,9 @@ template <int KIND, int SF_LAYOUT>
 __global__ void __launch_bounds__(32 * kGroupWarps * kSplit, 2)
 norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
                         const float *__restrict__ a, const float *__restrict__ b, float eps,
-                        const int32_t *__restrict__ perm, const int32_t *__restrict__ perm_select,
+                        const int32_t *__restrict__ perm,
                         const float *__restrict__ ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
                         uint16_t *__restrict__ y_out) {
-    // perm_select given: perm is a table of candidate orders [., K] and {best, accept} on the device name the
-    // row best - 1, or the original order (the offline weight quantizer, whose decision never visits the host)
-    if (perm_select) perm = perm_select[1] ? perm + static_cast<int64_t>(perm_select[0] - 1) * K : nullptr;
     extern __shared__ __align__(16) uint16_t row_s[];  // [row groups][K][R rows] bf16 bit patterns
     __shared__ float stat_s[kGroupWarps][2 * kGroupRows];
     constexpr int R = kGroupRows;
@@ -302,20 +302,14 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
                 for (int r = 0; r < R; ++r) {
                     float x[8];
                     pq::unpack8(v[u][r], x);
-                    if (KIND != 2) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) p[r] = KIND == 0 ? __fmaf_rn(x[e], x[e], p[r]) : __fadd_rn(p[r], x[e]);
-                    }
+                    for (int e = 0; e < 8; ++e) p[r] = KIND == 0 ? __fmaf_rn(x[e], x[e], p[r]) : __fadd_rn(p[r], x[e]);
                 }
             }
         }
-        if (KIND != 2) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) p[r] = lane_butterfly(p[r]);
-        }
-        if (KIND == 2) {
-            // no normalization: the values themselves are quantized
-        } else if (KIND == 0) {
+        for (int r = 0; r < R; ++r) p[r] = lane_butterfly(p[r]);
+        if (KIND == 0) {
 #pragma unroll
             for (int r = 0; r < R; ++r)
                 if (r < nlive) inv[r] = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(p[r], static_cast<float>(K)), eps)));
@@ -378,10 +372,8 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
                 if (perm) idx = __ldg(reinterpret_cast<const int4 *>(perm) + (POS / 4) * q + h);
                 g[4 * h + 0] = channel_rows<R>(xs, idx.x), g[4 * h + 1] = channel_rows<R>(xs, idx.y);
                 g[4 * h + 2] = channel_rows<R>(xs, idx.z), g[4 * h + 3] = channel_rows<R>(xs, idx.w);
-                if (KIND != 2) {
-                    const float4 a4 = __ldg(reinterpret_cast<const float4 *>(a) + (POS / 4) * q + h);
-                    w[4 * h + 0] = a4.x, w[4 * h + 1] = a4.y, w[4 * h + 2] = a4.z, w[4 * h + 3] = a4.w;
-                }
+                const float4 a4 = __ldg(reinterpret_cast<const float4 *>(a) + (POS / 4) * q + h);
+                w[4 * h + 0] = a4.x, w[4 * h + 1] = a4.y, w[4 * h + 2] = a4.z, w[4 * h + 3] = a4.w;
                 if (KIND == 1) {
                     const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b) + (POS / 4) * q + h);
                     sh[4 * h + 0] = b4.x, sh[4 * h + 1] = b4.y, sh[4 * h + 2] = b4.z, sh[4 * h + 3] = b4.w;
@@ -401,9 +393,8 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
 #pragma unroll
             for (int j = 0; j < POS; ++j) {
                 const float v = row_value(g[j], r);
-                out[j] = KIND == 2   ? v
-                         : KIND == 0 ? __fmul_rn(__fmul_rn(v, inv[r]), w[j])
-                                     : __fmaf_rn(__fmul_rn(__fsub_rn(v, mu[r]), inv[r]), w[j], sh[j]);
+                out[j] = KIND == 0 ? __fmul_rn(__fmul_rn(v, inv[r]), w[j])
+                                   : __fmaf_rn(__fmul_rn(__fsub_rn(v, mu[r]), inv[r]), w[j], sh[j]);
                 amax = fmaxf(amax, fabsf(out[j]));
             }
             if (!(live && have)) amax = 0.0f;  // nothing of such a row or group is stored but a zero scale byte
@@ -448,6 +439,213 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
             }
         }
     }
+}
+
+// ---- four rows per block ------------------------------------------------------------------------
+// The same computation in smaller pieces: four rows to a block of up to sixteen warps, for fewer rows than the kernel
+// above needs to fill the chip, for rows too wide for two of its blocks per SM, and for the gather without a norm.  The rows arrive by
+// asynchronous 16-byte copies, all in flight at once and through no register; a warp takes the statistics of one row
+// from shared memory; then the image is transposed in place (through registers) to four rows interleaved per
+// channel, so that one 64-bit load gathers a channel for all four and indices and parameters are fetched once for
+// them.  In the walk a lane takes a whole group of 16 output positions: the scale is derived once per group and row
+// and nothing but the scale bytes crosses lanes; neighbouring positions go through packed fp32 arithmetic.  The
+// order of every floating-point operation is that of the one-row kernel.
+// What bounds it: instruction issue at 20-24 warps per SM (ncu: issue slots 58 % busy, stalls on shared memory,
+// fixed latencies and barriers).  Several small blocks share an SM and drift apart, so that some wait for memory while
+// others compute.  RMSNorm / adaptive LayerNorm, us, against the kernel above: 512 x 3072 4.5 / 6.0 against 10.6 / 13.4,
+// 4608 x 6144 35.0 / 46.2 against 42.9 / 53.7; 2304 x 12288 35.9 / 45.8 against 69.5 / 81.5 one row per warp; but
+// 4608 x 3072 17.8 / 22.3 against 17.4 / 21.9 and 4608 x 1088 11.2 / 13.9 against 10.3 / 12.3.  Without a norm: 4608 x 3072
+// 12.7 against 14.4, 18432 x 3072 37.7 against 49.4.
+template <int KIND, int SF_LAYOUT, int ITER>  // ITER = groups per lane
+__global__ void __maxnreg__(kQuadRegs)
+norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
+                       const float *__restrict__ a, const float *__restrict__ b, float eps,
+                       const int32_t *__restrict__ perm, const int32_t *__restrict__ perm_select,
+                       const float *__restrict__ ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
+                       uint16_t *__restrict__ y_out) {
+    extern __shared__ __align__(16) uint4 quad_s[];  // [4 rows][K] bf16, then [K][4 rows]
+    __shared__ float stat_s[8];                      // inv, mu of the four rows
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x, T = blockDim.x;
+    const int64_t row0 = static_cast<int64_t>(blockIdx.x) * 4;
+    const int nlive = static_cast<int>(min(static_cast<int64_t>(4), max(static_cast<int64_t>(0), rows - row0)));
+    const int octs = K >> 3, gpr = K >> 4;
+    pq::wait_for_prior_grid();
+    pq::dependents_may_launch();
+    // perm_select given: perm is a table of candidate orders [., K] and {best, accept} on the device name the
+    // row best - 1, or the original order (the offline weight quantizer, whose decision never visits the host)
+    if (perm_select) perm = perm_select[1] ? perm + static_cast<int64_t>(perm_select[0] - 1) * K : nullptr;
+    const float ts = __ldg(ts_ptr);
+    const uint16_t *src = H + row0 * ld;
+
+    if (KIND == 2) {  // no statistics: straight into the interleaved image
+        for (int o = tid; o < octs; o += T) {
+            uint4 v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                v[r] = r < nlive ? __ldcs(reinterpret_cast<const uint4 *>(src + r * ld) + o) : make_uint4(0, 0, 0, 0);
+            pq::store_quad_octet(quad_s, o, v);
+        }
+    } else {
+        const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(quad_s));
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            for (int o = tid; o < octs; o += T) {
+                if (r < nlive)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + 16u * (r * octs + o)), "l"(src + r * ld + o * 8)
+                                 : "memory");
+                else quad_s[r * octs + o] = make_uint4(0, 0, 0, 0);
+            }
+        }
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (warp < 4) {
+            float inv = 0.0f, mu = 0.0f;
+            if (warp < nlive) {
+                const uint4 *row4 = quad_s + warp * octs;
+                float p = 0.0f;
+#pragma unroll 4
+                for (int o = lane; o < octs; o += 32) {
+                    float x[8];
+                    pq::unpack8(row4[o], x);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) p = KIND == 0 ? __fmaf_rn(x[e], x[e], p) : __fadd_rn(p, x[e]);
+                }
+                p = lane_butterfly(p);
+                if (KIND == 1) {
+                    mu = __fdiv_rn(p, static_cast<float>(K));
+                    p = 0.0f;
+#pragma unroll 4
+                    for (int o = lane; o < octs; o += 32) {
+                        float x[8];
+                        pq::unpack8(row4[o], x);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float d = __fsub_rn(x[e], mu);
+                            p = __fmaf_rn(d, d, p);
+                        }
+                    }
+                    p = lane_butterfly(p);
+                }
+                inv = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(p, static_cast<float>(K)), eps)));
+            }
+            if (lane == 0) stat_s[warp] = inv, stat_s[4 + warp] = mu;
+        }
+        uint4 v[2 * ITER][4];  // this thread's octets of the four rows (octs <= 2 * ITER * T)
+#pragma unroll
+        for (int i = 0; i < 2 * ITER; ++i) {
+            const int o = tid + i * T;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) v[i][r] = o < octs ? quad_s[r * octs + o] : make_uint4(0, 0, 0, 0);
+        }
+        __syncthreads();  // every row has been read, by the statistics too
+#pragma unroll
+        for (int i = 0; i < 2 * ITER; ++i)
+            if (tid + i * T < octs) pq::store_quad_octet(quad_s, tid + i * T, v[i]);
+    }
+    __syncthreads();
+
+    // ---- output order: one group (16 consecutive positions) per lane, for the four rows
+    const uint2 *quad2 = reinterpret_cast<const uint2 *>(quad_s);
+#pragma unroll 1
+    for (int it = 0; it < ITER; ++it) {
+        const int q = tid + it * T;
+        const bool have = q < gpr;
+        const int64_t sf_ofs = SF_LAYOUT == PQ_SF_TCGEN05 ? pq::sf_tc_offset(row0, q, gpr >> 2) : row0 * gpr + q;
+        uint8_t *const out_codes = codes + row0 * (K >> 1) + q * 8;
+        uint2 g[16];
+        uint64_t w2[8], sh2[8];  // parameters of neighbouring positions, packed
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const int j0 = have ? 16 * q + 4 * h : 0;
+            int4 idx = make_int4(j0, j0 + 1, j0 + 2, j0 + 3);
+            if (perm) idx = __ldg(reinterpret_cast<const int4 *>(perm + j0));
+            g[4 * h + 0] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.x))];
+            g[4 * h + 1] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.y))];
+            g[4 * h + 2] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.z))];
+            g[4 * h + 3] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.w))];
+            if (KIND != 2) {
+                float4 a4 = __ldg(reinterpret_cast<const float4 *>(a + j0));
+                if (KIND == 1) {
+                    a4 = make_float4(__fadd_rn(1.0f, a4.x), __fadd_rn(1.0f, a4.y), __fadd_rn(1.0f, a4.z), __fadd_rn(1.0f, a4.w));
+                    const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b + j0));
+                    sh2[2 * h] = pq::pack2(b4.x, b4.y), sh2[2 * h + 1] = pq::pack2(b4.z, b4.w);
+                }
+                w2[2 * h] = pq::pack2(a4.x, a4.y), w2[2 * h + 1] = pq::pack2(a4.z, a4.w);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int64_t row = row0 + r;
+            const bool live = r < nlive && have;
+            uint64_t y2[8];
+            float amax = 0.0f;
+            const uint64_t inv2 = KIND == 2 ? 0 : pq::pack2(stat_s[r], stat_s[r]);
+            const uint64_t nmu2 = KIND == 1 ? pq::pack2(-stat_s[4 + r], -stat_s[4 + r]) : 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t c0 = r < 2 ? g[2 * j].x : g[2 * j].y, c1 = r < 2 ? g[2 * j + 1].x : g[2 * j + 1].y;
+                uint64_t v = (r & 1) ? pq::pack2(__uint_as_float(c0 & 0xFFFF0000u), __uint_as_float(c1 & 0xFFFF0000u))
+                                     : pq::pack2(__uint_as_float(c0 << 16), __uint_as_float(c1 << 16));
+                if (KIND == 0) v = pq::mul2(pq::mul2(v, inv2), w2[j]);
+                if (KIND == 1) v = pq::fma2(pq::mul2(pq::add2(v, nmu2), inv2), w2[j], sh2[j]);
+                y2[j] = v;
+                float lo, hi;
+                pq::unpack2(v, lo, hi);
+                amax = fmaxf(fmaxf(amax, fabsf(lo)), fabsf(hi));
+            }
+            if (!live) amax = 0.0f;  // nothing of such a row or group is stored but a zero scale byte
+            uint32_t sf8;
+            float d, rcp;
+            pq::nvfp4_scale(amax, ts, sf8, d, rcp);
+            if (live) {
+                if (y_out) {
+                    uint32_t yw[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        float lo, hi;
+                        pq::unpack2(y2[j], lo, hi);
+                        yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
+                                (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(hi))) << 16);
+                    }
+                    uint4 *ydst = reinterpret_cast<uint4 *>(y_out + row * K) + 2 * q;
+                    ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                    ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                }
+                const uint64_t rcp2 = pq::pack2(rcp, rcp);
+                float y[16];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) pq::unpack2(pq::mul2(y2[j], rcp2), y[2 * j], y[2 * j + 1]);
+                const float ylo[8] = {y[0], y[1], y[2], y[3], y[4], y[5], y[6], y[7]};
+                const float yhi[8] = {y[8], y[9], y[10], y[11], y[12], y[13], y[14], y[15]};
+                *reinterpret_cast<uint2 *>(out_codes + r * (K >> 1)) = make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
+            }
+            // one scale byte per lane; the lanes of a warp write runs of four adjacent bytes (padding rows write zeros).
+            // row0 is a multiple of four: the rows' bytes lie 16 apart in the tensor-core layout
+            if (have && (SF_LAYOUT == PQ_SF_TCGEN05 ? row < rows_pad : live))
+                sf[SF_LAYOUT == PQ_SF_TCGEN05 ? sf_ofs + 16 * r : sf_ofs + r * gpr] = static_cast<uint8_t>(sf8);
+        }
+    }
+}
+
+// Rows the four-rows-per-block kernel takes: up to two groups per lane of at most 512 threads, 128 KB of image.
+constexpr int64_t kQuadMaxK = 16384;
+
+template <int KIND, int SF_LAYOUT>
+pq_status launch_quad(const uint16_t *H, int64_t rows, int64_t rows_pad, int K, int64_t ld, const float *a, const float *b, float eps,
+                      const int32_t *perm, const int32_t *perm_select, const float *ts, uint8_t *codes, uint8_t *sf, uint16_t *y_out,
+                      cudaStream_t st) {
+    const int gpr = K >> 4, iter = gpr > 512 ? 2 : 1;
+    // one or two groups per lane; four warps at least, one per row for the statistics
+    const int threads = std::max(128, static_cast<int>(pq_ceil_div(pq_ceil_div(gpr, iter), 32)) * 32);
+    const size_t smem = static_cast<size_t>(K) * 8;
+    const int64_t blocks = pq_ceil_div(rows_pad, 4);
+    PQ_REQUIRE(blocks < (1ll << 31), PQ_ERR_SHAPE);
+    auto kern = iter == 1 ? norm_quant_quad_kernel<KIND, SF_LAYOUT, 1> : norm_quant_quad_kernel<KIND, SF_LAYOUT, 2>;
+    if (smem > 47 * 1024)  // the kernel's static shared memory counts towards the 48 KB default limit
+        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks)), dim3(static_cast<unsigned>(threads)), smem, st, H, rows, rows_pad,
+                                    K, ld, a, b, eps, perm, perm_select, ts, codes, sf, y_out));
+    return pq_launch_status();
 }
 
 // ---- channels already in output order --------------------------------------------------------------
@@ -577,18 +775,22 @@ pq_status launch(const uint16_t *H, int64_t M, int64_t rows_pad, int K, int64_t 
         else norm_quant_ordered_kernel<KIND, SF_LAYOUT, 16><<<grid, kDirectThreads, 0, st>>>(H, M, rows_pad, K, ld, a, b, eps, ts, codes, sf, y_out);
         return pq_launch_status();
     }
-    // up to 6400 channels: four rows per warp, four warps per block (two blocks per SM at 3072 channels)
+    // several rows per warp while two blocks of sixteen rows fit on an SM and there is one for every SM at least;
+    // otherwise four rows per block (measurements at that kernel)
     const size_t group_smem = static_cast<size_t>(kGroupWarps) * kGroupRows * K * 2;
-    if (group_smem <= kSmemBudget) {
+    const int64_t group_blocks = pq_ceil_div(rows_pad, kGroupWarps * kGroupRows);
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (2 * (group_smem + 2048) <= 227 * 1024 && group_blocks >= sms) {
         if (group_smem > 40 * 1024)  // the kernel's static shared memory counts towards the 48 KB default limit
             PQ_CUDA_OK(cudaFuncSetAttribute(norm_quant_grouped_kernel<KIND, SF_LAYOUT>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(group_smem)));
-        const int64_t blocks = pq_ceil_div(rows_pad, kGroupWarps * kGroupRows);
-        PQ_REQUIRE(blocks < (1ll << 31), PQ_ERR_SHAPE);
-        norm_quant_grouped_kernel<KIND, SF_LAYOUT><<<static_cast<unsigned>(blocks), kGroupWarps * kSplit * 32, group_smem, st>>>(
-            H, M, rows_pad, K, ld, a, b, eps, perm, nullptr, ts, codes, sf, y_out);
+        PQ_REQUIRE(group_blocks < (1ll << 31), PQ_ERR_SHAPE);
+        norm_quant_grouped_kernel<KIND, SF_LAYOUT><<<static_cast<unsigned>(group_blocks), kGroupWarps * kSplit * 32, group_smem, st>>>(
+            H, M, rows_pad, K, ld, a, b, eps, perm, ts, codes, sf, y_out);
         return pq_launch_status();
     }
+    if (K <= kQuadMaxK) return launch_quad<KIND, SF_LAYOUT>(H, M, rows_pad, K, ld, a, b, eps, perm, nullptr, ts, codes, sf, y_out, st);
     // wider rows: one warp per row, the row as bf16 in shared memory: 8 rows per block up to 12800 channels
     int warps = static_cast<int>(kSmemBudget / (static_cast<size_t>(K) * 2));
     if (warps > kMaxRowsPerBlock) warps = kMaxRowsPerBlock;
@@ -604,36 +806,19 @@ pq_status launch(const uint16_t *H, int64_t M, int64_t rows_pad, int K, int64_t 
     return pq_launch_status();
 }
 
-template <int SF_LAYOUT>
-pq_status launch_gather_only(const uint16_t *X, int64_t M, int64_t rows_pad, int K, int64_t ld, const int32_t *perm,
-                             const int32_t *perm_select, const float *ts, uint8_t *codes, uint8_t *sf, cudaStream_t st) {
-    const size_t group_smem = static_cast<size_t>(kGroupWarps) * kGroupRows * K * 2;
-    if (group_smem > 40 * 1024)
-        PQ_CUDA_OK(cudaFuncSetAttribute(norm_quant_grouped_kernel<2, SF_LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        static_cast<int>(group_smem)));
-    const int64_t blocks = pq_ceil_div(rows_pad, kGroupWarps * kGroupRows);
-    PQ_REQUIRE(blocks < (1ll << 31), PQ_ERR_SHAPE);
-    norm_quant_grouped_kernel<2, SF_LAYOUT><<<static_cast<unsigned>(blocks), kGroupWarps * kSplit * 32, group_smem, st>>>(
-        X, M, rows_pad, K, ld, nullptr, nullptr, 0.0f, perm, perm_select, ts, codes, sf, nullptr);
-    return pq_launch_status();
-}
-
 }  // namespace
 
-// The gather quantizer of pq_quant_act_nvfp4_perm and pq_quant_weight for rows the four-rows-per-warp kernel can
-// hold: that kernel with the normalization left out (the gathered values themselves are quantized).
-bool pq_gather_quant_grouped_fits(int64_t K) {
-    return K > 0 && static_cast<size_t>(kGroupWarps) * kGroupRows * static_cast<size_t>(K) * 2 <= kSmemBudget;
-}
-pq_status pq_gather_quant_grouped(const void *X, int64_t M, int64_t K, int64_t ld, const int32_t *perm,
-                                  const int32_t *perm_select, const float *ts_x, uint8_t *codes, uint8_t *sf,
-                                  int sf_layout, void *stream) {
+// The gather quantizer of pq_quant_act_nvfp4_perm and pq_quant_weight: the four-rows-per-block kernel with the
+// normalization left out (the gathered values themselves are quantized).
+pq_status pq_gather_quant(const void *X, int64_t M, int64_t K, int64_t ld, const int32_t *perm, const int32_t *perm_select,
+                          const float *ts_x, uint8_t *codes, uint8_t *sf, int sf_layout, void *stream) {
     const int64_t rows_pad = sf_layout == PQ_SF_TCGEN05 ? pq_ceil_div(M, 128) * 128 : M;
     const uint16_t *x = static_cast<const uint16_t *>(X);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const int k = static_cast<int>(K);
     return sf_layout == PQ_SF_TCGEN05
-               ? launch_gather_only<PQ_SF_TCGEN05>(x, M, rows_pad, static_cast<int>(K), ld, perm, perm_select, ts_x, codes, sf, st)
-               : launch_gather_only<PQ_SF_LINEAR>(x, M, rows_pad, static_cast<int>(K), ld, perm, perm_select, ts_x, codes, sf, st);
+               ? launch_quad<2, PQ_SF_TCGEN05>(x, M, rows_pad, k, ld, nullptr, nullptr, 0.0f, perm, perm_select, ts_x, codes, sf, nullptr, st)
+               : launch_quad<2, PQ_SF_LINEAR>(x, M, rows_pad, k, ld, nullptr, nullptr, 0.0f, perm, perm_select, ts_x, codes, sf, nullptr, st);
 }
 
 extern "C" pq_status pq_norm_quant_nvfp4(const void *H, int64_t M, int64_t K, int64_t ld, int kind, const float *a,

@@ -9,8 +9,8 @@
 //
 // The permuted variants (weights, fake-quant with a gather) stage each row in shared memory
 // with coalesced 16-byte loads and gather from there, so global memory is still read once.  For
-// NVFP4 and rows of up to 6400 channels the gather runs in the fused producer's kernel (pq_norm.cu,
-// four rows per warp sharing indices and gathers) with its normalization compiled out.
+// NVFP4 the gather runs in the fused producer's kernel (pq_norm.cu, four rows per block sharing indices
+// and gathers) with its normalization compiled out.
 #include "pq_common.cuh"
 
 namespace {
@@ -466,11 +466,9 @@ extern "C" pq_status pq_quant_act_nvfp4_perm(const void *X, int64_t M, int64_t K
     PQ_REQUIRE(M > 0 && K > 0 && K % 16 == 0 && K <= 16384 && ld >= K, PQ_ERR_SHAPE);
     PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || K % 64 == 0, PQ_ERR_SHAPE);
     PQ_REQUIRE(pq_aligned16(X) && ld % 8 == 0 && pq_aligned16(codes) && pq_aligned16(sf), PQ_ERR_ALIGN);
-    // rows of up to 6400 channels: four rows per warp share the indices and one gather (the fused producer's
-    // kernel without its normalization); wider rows, or an index vector it cannot load 16 bytes at a time: one
-    // block per row
-    if (pq_gather_quant_grouped_fits(K) && pq_aligned16(perm))
-        return pq_gather_quant_grouped(X, M, K, ld, perm, nullptr, ts_x, codes, sf, sf_layout, stream);
+    // four rows share the indices and one gather (the fused producer's kernel without its normalization); an index
+    // vector it cannot load 16 bytes at a time: one block per row
+    if (pq_aligned16(perm)) return pq_gather_quant(X, M, K, ld, perm, nullptr, ts_x, codes, sf, sf_layout, stream);
     return launch_gather(static_cast<const uint16_t *>(X), M, K, ld, perm, nullptr, ts_x, codes, sf, sf_layout,
                          static_cast<cudaStream_t>(stream));
 }
@@ -478,9 +476,8 @@ extern "C" pq_status pq_quant_act_nvfp4_perm(const void *X, int64_t M, int64_t K
 pq_status pq_quant_weight_scaled(const void *Wt, int64_t N, int64_t K, int64_t ld, const int32_t *perm, const int32_t *perm_select,
                                  uint8_t *codes, uint8_t *sf, int sf_layout, const float *ts_w, cudaStream_t st) {
     if (!perm) return pq_quant_act_nvfp4(Wt, N, K, ld, ts_w, codes, sf, sf_layout, st);
-    // rows of up to 6400 channels: four rows per warp share the indices and one gather
-    if (pq_gather_quant_grouped_fits(K) && pq_aligned16(perm))
-        return pq_gather_quant_grouped(Wt, N, K, ld, perm, perm_select, ts_w, codes, sf, sf_layout, st);
+    // four rows share the indices and one gather
+    if (pq_aligned16(perm)) return pq_gather_quant(Wt, N, K, ld, perm, perm_select, ts_w, codes, sf, sf_layout, st);
     return launch_gather(static_cast<const uint16_t *>(Wt), N, K, ld, perm, perm_select, ts_w, codes, sf, sf_layout, st);
 }
 

@@ -310,14 +310,18 @@ fakequant_int_gather_kernel(const uint16_t *__restrict__ T, int64_t rows, int K,
     const int live_rows = static_cast<int>(min(static_cast<int64_t>(4), rows - row0));
     const bool aligned = (reinterpret_cast<uintptr_t>(perm) & 15u) == 0;
     T += row0 * ld;
-    for (int o = threadIdx.x; o < octs; o += blockDim.x) {
-        uint4 v[4];
+    auto load_octet = [&](int o, uint4 (&v)[4]) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-            v[r] = r < live_rows ? __ldg(reinterpret_cast<const uint4 *>(T + r * ld) + o) : make_uint4(0, 0, 0, 0);
+            v[r] = o < octs && r < live_rows ? __ldg(reinterpret_cast<const uint4 *>(T + r * ld) + o) : make_uint4(0, 0, 0, 0);
+    };
+    uint4 v[4];
+    load_octet(threadIdx.x, v);
+    pq::build_int_tab(tab, Qf, false);  // while the first rows are on their way
+    for (int o = threadIdx.x; o < octs; o += blockDim.x) {
         pq::store_quad_octet(quad_s, o, v);
+        load_octet(o + blockDim.x, v);
     }
-    pq::build_int_tab(tab, Qf, false);
     __syncthreads();
     const uint2 *quad2 = reinterpret_cast<const uint2 *>(quad_s);
     out += row0 * ldo;

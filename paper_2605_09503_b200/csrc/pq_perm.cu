@@ -1,13 +1,13 @@
 // Sort candidates of the joint second-moment criterion (Eq. 9, Prop. 3.2) and the
 // selection / acceptance rule (Eq. 10).
 //
-// Sorting: a thread-block cluster per order.  The channels are cut into chunks of 1024 keys; a CTA sorts
+// Sorting: a thread-block cluster per order.  The channels are cut into chunks of 512 keys; a CTA sorts
 // its chunks (bitonic, one key per thread: strides below a warp by shuffles, the others through shared
-// memory), then every key finds its rank by binary search in the other chunks, read from the neighbours'
-// shared memory.  The position of a channel is the number of channels that precede it under the total order
+// memory), fetches the neighbours' sorted chunks out of their shared memory, and every key finds its rank by
+// binary search in them.  The position of a channel is the number of channels that precede it under the total order
 // (key descending, channel ascending), so the result is unique, hence identical to any comparison sort.
-// Counting ranks against all K keys instead is K^2 comparisons: 37 us for six orders of 3072 channels on
-// B200 and sixteen times that at 12288, where this takes one launch of a few microseconds.
+// Counting ranks against all K keys instead is K^2 comparisons: 38.9 us for six orders of 3072 channels and
+// 517 us at 12288 on B200, where this takes 8.7 us at 3072.
 // Keys are 64-bit patterns that order like the doubles they stand for: a non-negative double orders
 // like its own bits; a signed one after flipping all bits of a negative value and the sign bit of
 // the others.
@@ -54,8 +54,24 @@ __device__ __forceinline__ unsigned long long sort_key(const SortParams &p, int 
     return static_cast<unsigned long long>(__double_as_longlong(fabs(p.a[i])));
 }
 
-constexpr int kSortChunk = 1024, kSortMaxChunks = 16, kSortMaxCluster = 8;
+constexpr int kSortChunk = 512, kSortMaxChunks = 32, kSortMaxCluster = 8;
 constexpr int kSortPerCta = kSortMaxChunks / kSortMaxCluster;  // chunks a CTA may hold
+
+// (okey, oidx) precedes (key, idx): larger key, or equal key and lower index.  The borrow of a 96-bit subtraction.
+__device__ __forceinline__ bool precedes(unsigned long long okey, uint32_t oidx, unsigned long long key, uint32_t idx) {
+    uint32_t borrow;
+    asm("{\n"
+        ".reg .u32 t;\n"
+        "sub.cc.u32 t, %1, %2;\n"
+        "subc.cc.u32 t, %3, %4;\n"
+        "subc.cc.u32 t, %5, %6;\n"
+        "subc.u32 %0, 0, 0;\n"
+        "}\n"
+        : "=r"(borrow)
+        : "r"(oidx), "r"(idx), "r"(static_cast<uint32_t>(key)), "r"(static_cast<uint32_t>(okey)),
+          "r"(static_cast<uint32_t>(key >> 32)), "r"(static_cast<uint32_t>(okey >> 32)));
+    return borrow != 0;
+}
 
 // Key of the neighbour: shared memory of CTA `rank` of the cluster.
 __device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
@@ -73,10 +89,13 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 // gridDim.x = cluster size; CTA r holds the chunks r, r + cluster size, ...
+// The searches go four chunks at a time in a loop: with all of them unrolled (up to 31) the kernel took 32 us at 512
+// channels, where it has nothing to search, against 4.4 us (instruction fetches).
 __global__ void __launch_bounds__(kSortChunk) order_sort_kernel(const __grid_constant__ SortParams p) {
+    extern __shared__ unsigned long long all_s[];  // [chunks][512] sorted keys of the whole cluster
     __shared__ unsigned long long sorted[kSortPerCta][kSortChunk];
     __shared__ unsigned long long key_x[2][kSortChunk];
-    __shared__ uint16_t idx_x[2][kSortChunk];
+    __shared__ uint16_t idx_x[2][kSortChunk], channel_s[kSortPerCta][kSortChunk];
     const int j = blockIdx.y, rank = blockIdx.x, ctas = gridDim.x, tid = threadIdx.x;
     const int chunks = (p.K + kSortChunk - 1) / kSortChunk;
     pq::dependents_may_launch();
@@ -87,19 +106,21 @@ __global__ void __launch_bounds__(kSortChunk) order_sort_kernel(const __grid_con
         if (tid == 0) *p.scale_out[j - p.orders] = (a == 0.0f) ? 1.0f : __fdiv_rn(a, 2688.0f);
         return;
     }
-    int channel[kSortPerCta];
-#pragma unroll
+#pragma unroll 1
     for (int t = 0; t < kSortPerCta; ++t) {
         const int chunk = rank + t * ctas;
         if (chunk >= chunks) break;  // uniform over the CTA
         const int base = chunk * kSortChunk;
         // a slot past the end holds key 0 at an index above every channel: it precedes nothing
         unsigned long long key = base + tid < p.K ? sort_key(p, j, base + tid) : 0ull;
-        int idx = tid, buf = 0;
+        uint32_t idx = tid;
+        int buf = 0;
+#pragma unroll
         for (int k = 2; k <= kSortChunk; k <<= 1) {
+#pragma unroll
             for (int d = k >> 1; d; d >>= 1) {
                 unsigned long long okey;
-                int oidx;
+                uint32_t oidx;
                 if (d >= 32) {
                     key_x[buf][tid] = key, idx_x[buf][tid] = static_cast<uint16_t>(idx);
                     __syncthreads();  // one barrier per exchange: the other buffer is written next
@@ -108,49 +129,56 @@ __global__ void __launch_bounds__(kSortChunk) order_sort_kernel(const __grid_con
                 } else {
                     okey = __shfl_xor_sync(0xFFFFFFFFu, key, d), oidx = __shfl_xor_sync(0xFFFFFFFFu, idx, d);
                 }
-                const bool other_first = okey > key || (okey == key && oidx < idx);
                 const bool want_first = ((tid & d) == 0) == ((tid & k) == 0);
-                if (want_first == other_first) key = okey, idx = oidx;
+                if (want_first == precedes(okey, oidx, key, idx)) key = okey, idx = oidx;
             }
         }
         sorted[t][tid] = key;
-        channel[t] = base + idx;
+        channel_s[t][tid] = static_cast<uint16_t>(base + idx);
         __syncthreads();  // the exchange buffers may be written again
     }
     cluster_barrier();
-#pragma unroll
+#pragma unroll 4
+    for (int c = 0; c < chunks; ++c)
+        all_s[c * kSortChunk + tid] = cluster_load(cluster_addr(&sorted[c / ctas][tid], static_cast<uint32_t>(c % ctas)));
+    __syncthreads();
+#pragma unroll 1
     for (int t = 0; t < kSortPerCta; ++t) {
         const int chunk = rank + t * ctas;
         if (chunk >= chunks) break;
         const unsigned long long mine = sorted[t][tid];
-        int pos[kSortMaxChunks];
-        uint32_t addr[kSortMaxChunks];
-#pragma unroll
-        for (int c = 0; c < kSortMaxChunks; ++c) {
-            pos[c] = 0;
-            addr[c] = c < chunks ? cluster_addr(&sorted[c / ctas][0], static_cast<uint32_t>(c % ctas)) : 0u;
-        }
-        // keys of an earlier chunk precede mine when they are not smaller, of a later one when larger.  The chunks'
-        // searches are independent, so their (remote) loads overlap.
-        for (int s = kSortChunk / 2; s; s >>= 1) {
-#pragma unroll
-            for (int c = 0; c < kSortMaxChunks; ++c) {
-                if (c >= chunks || c == chunk) continue;
-                const unsigned long long other = cluster_load(addr[c] + 8u * (pos[c] + s - 1));
-                if (c < chunk ? other >= mine : other > mine) pos[c] += s;
-            }
-        }
+        // keys of an earlier chunk precede mine when they are not smaller, of a later one when larger
         int place = tid;
+#pragma unroll 1
+        for (int c0 = 0; c0 < chunks; c0 += 4) {
+            int pos[4];
+            const unsigned long long *keys[4];
+            bool earlier[4];
 #pragma unroll
-        for (int c = 0; c < kSortMaxChunks; ++c) {
-            if (c >= chunks || c == chunk) continue;
-            const unsigned long long other = cluster_load(addr[c] + 8u * pos[c]);
-            place += pos[c] + ((c < chunk ? other >= mine : other > mine) ? 1 : 0);
+            for (int u = 0; u < 4; ++u) {
+                const int c = min(c0 + u, chunks - 1);
+                pos[u] = 0, keys[u] = all_s + c * kSortChunk, earlier[u] = c < chunk;
+            }
+#pragma unroll
+            for (int s = kSortChunk / 2; s; s >>= 1) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const unsigned long long other = keys[u][pos[u] + s - 1];
+                    if (other > mine || (earlier[u] && other == mine)) pos[u] += s;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned long long other = keys[u][pos[u]];
+                if (other > mine || (earlier[u] && other == mine)) ++pos[u];
+                if (c0 + u < chunks && c0 + u != chunk) place += pos[u];
+            }
         }
         // deal_groups == 0: the channel of rank r is read at position r; otherwise the sorted channels are dealt
         // to deal_groups groups in turn: rank r goes to group r % deal_groups, slot r / deal_groups
         const int at = p.deal_groups ? (place % p.deal_groups) * p.group + place / p.deal_groups : place;
-        if (channel[t] < p.K) p.perms[static_cast<int64_t>(j) * p.K + at] = channel[t];
+        const int ch = channel_s[t][tid];
+        if (ch < p.K) p.perms[static_cast<int64_t>(j) * p.K + at] = ch;
     }
     cluster_barrier();  // the neighbours may still be reading this CTA's keys
 }
@@ -171,6 +199,9 @@ pq_status launch_sort(const SortParams &p, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(ctas), static_cast<unsigned>(p.orders + (p.scale_out[0] ? 2 : 0)));
     cfg.blockDim = dim3(kSortChunk), cfg.stream = st;
+    cfg.dynamicSmemBytes = static_cast<size_t>(chunks) * kSortChunk * sizeof(unsigned long long);
+    if (cfg.dynamicSmemBytes > 16 * 1024)  // the kernel's static shared memory counts towards the 48 KB default limit
+        PQ_CUDA_OK(cudaFuncSetAttribute(order_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(cfg.dynamicSmemBytes)));
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = static_cast<unsigned>(ctas), attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;

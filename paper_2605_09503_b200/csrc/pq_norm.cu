@@ -36,6 +36,29 @@ __device__ __forceinline__ float lane_butterfly(float p) {
     return p;
 }
 
+// The statistics over the eight values of an octet in order: plain sum (adaptive LayerNorm) or sum of squares (RMSNorm) ...
+template <int KIND>
+__device__ __forceinline__ float add_octet(float p, const uint4 &v) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        p = KIND == 0 ? pq::add_bf16_square<0>(p, w[i]) : pq::add_bf16<0>(p, w[i]);
+        p = KIND == 0 ? pq::add_bf16_square<1>(p, w[i]) : pq::add_bf16<1>(p, w[i]);
+    }
+    return p;
+}
+// ... and the centred second moment.
+__device__ __forceinline__ float add_centred_octet(float q, const uint4 &v, float mu) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float d0 = pq::bf16_minus<0>(w[i], mu), d1 = pq::bf16_minus<1>(w[i], mu);
+        q = __fmaf_rn(d0, d0, q);
+        q = __fmaf_rn(d1, d1, q);
+    }
+    return q;
+}
+
 template <int KIND, int SF_LAYOUT>
 __global__ void __launch_bounds__(32 * kMaxRowsPerBlock)
 norm_quant_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
@@ -69,10 +92,7 @@ norm_quant_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad
                 const int o = o0 + 32 * u;
                 if (o >= octs) break;
                 reinterpret_cast<uint4 *>(xs)[o] = v[u];
-                float x[8];
-                pq::unpack8(v[u], x);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) p = KIND == 0 ? __fmaf_rn(x[e], x[e], p) : __fadd_rn(p, x[e]);
+                p = add_octet<KIND>(p, v[u]);
             }
         }
         p = lane_butterfly(p);
@@ -81,15 +101,7 @@ norm_quant_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad
         } else {
             mu = __fdiv_rn(p, static_cast<float>(K));
             float q = 0.0f;
-            for (int o = lane; o < octs; o += 32) {  // the lane re-reads what it wrote
-                float x[8];
-                pq::unpack8(reinterpret_cast<const uint4 *>(xs)[o], x);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const float d = __fsub_rn(x[e], mu);
-                    q = __fmaf_rn(d, d, q);
-                }
-            }
+            for (int o = lane; o < octs; o += 32) q = add_centred_octet(q, reinterpret_cast<const uint4 *>(xs)[o], mu);  // what it wrote
             q = lane_butterfly(q);
             inv = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(q, static_cast<float>(K)), eps)));
         }
@@ -237,6 +249,11 @@ __device__ __forceinline__ float row_value(const uint2 &g, int r) {
     return __uint_as_float((r & 1) ? (w & 0xFFFF0000u) : (w << 16));
 }
 
+__device__ __forceinline__ float row_minus(const uint2 &g, int r, float c) {
+    const uint32_t w = r < 2 ? g.x : g.y;
+    return (r & 1) ? pq::bf16_minus<1>(w, c) : pq::bf16_minus<0>(w, c);
+}
+
 template <int KIND, int SF_LAYOUT>
 __global__ void __launch_bounds__(32 * kGroupWarps * kSplit, 2)
 norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
@@ -256,6 +273,8 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
     uint16_t *xs = row_s + static_cast<size_t>(grp_in_block) * K * R;
     uint4 *xs4 = reinterpret_cast<uint4 *>(xs);
     const int octs = K >> 3, gpr = K >> 4;
+    pq::wait_for_prior_grid();
+    pq::dependents_may_launch();
     const float ts = __ldg(ts_ptr);
     float inv[R], mu[R];
 #pragma unroll
@@ -299,12 +318,7 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
                                        __byte_perm(w0[2 * k + 1], w1[2 * k + 1], 0x7632));
                 }
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    float x[8];
-                    pq::unpack8(v[u][r], x);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) p[r] = KIND == 0 ? __fmaf_rn(x[e], x[e], p[r]) : __fadd_rn(p[r], x[e]);
-                }
+                for (int r = 0; r < R; ++r) p[r] = add_octet<KIND>(p[r], v[u][r]);
             }
         }
 #pragma unroll
@@ -327,7 +341,7 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
                         const uint2 ch = R == 4 ? make_uint2(cw[2 * i], cw[2 * i + 1]) : make_uint2(cw[i], 0u);
 #pragma unroll
                         for (int r = 0; r < R; ++r) {
-                            const float d0 = __fsub_rn(row_value(ch, r), mu[r]);
+                            const float d0 = row_minus(ch, r, mu[r]);
                             q[r] = __fmaf_rn(d0, d0, q[r]);
                         }
                     }
@@ -392,9 +406,8 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
             float amax = 0.0f;
 #pragma unroll
             for (int j = 0; j < POS; ++j) {
-                const float v = row_value(g[j], r);
-                out[j] = KIND == 0 ? __fmul_rn(__fmul_rn(v, inv[r]), w[j])
-                                   : __fmaf_rn(__fmul_rn(__fsub_rn(v, mu[r]), inv[r]), w[j], sh[j]);
+                out[j] = KIND == 0 ? __fmul_rn(__fmul_rn(row_value(g[j], r), inv[r]), w[j])
+                                   : __fmaf_rn(__fmul_rn(row_minus(g[j], r, mu[r]), inv[r]), w[j], sh[j]);
                 amax = fmaxf(amax, fabsf(out[j]));
             }
             if (!(live && have)) amax = 0.0f;  // nothing of such a row or group is stored but a zero scale byte
@@ -504,26 +517,13 @@ norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t row
                 const uint4 *row4 = quad_s + warp * octs;
                 float p = 0.0f;
 #pragma unroll 4
-                for (int o = lane; o < octs; o += 32) {
-                    float x[8];
-                    pq::unpack8(row4[o], x);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) p = KIND == 0 ? __fmaf_rn(x[e], x[e], p) : __fadd_rn(p, x[e]);
-                }
+                for (int o = lane; o < octs; o += 32) p = add_octet<KIND>(p, row4[o]);
                 p = lane_butterfly(p);
                 if (KIND == 1) {
                     mu = __fdiv_rn(p, static_cast<float>(K));
                     p = 0.0f;
 #pragma unroll 4
-                    for (int o = lane; o < octs; o += 32) {
-                        float x[8];
-                        pq::unpack8(row4[o], x);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float d = __fsub_rn(x[e], mu);
-                            p = __fmaf_rn(d, d, p);
-                        }
-                    }
+                    for (int o = lane; o < octs; o += 32) p = add_centred_octet(p, row4[o], mu);
                     p = lane_butterfly(p);
                 }
                 inv = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(p, static_cast<float>(K)), eps)));
@@ -580,14 +580,16 @@ norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t row
             uint64_t y2[8];
             float amax = 0.0f;
             const uint64_t inv2 = KIND == 2 ? 0 : pq::pack2(stat_s[r], stat_s[r]);
-            const uint64_t nmu2 = KIND == 1 ? pq::pack2(-stat_s[4 + r], -stat_s[4 + r]) : 0;
+            const float mu = stat_s[4 + r];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const uint32_t c0 = r < 2 ? g[2 * j].x : g[2 * j].y, c1 = r < 2 ? g[2 * j + 1].x : g[2 * j + 1].y;
-                uint64_t v = (r & 1) ? pq::pack2(__uint_as_float(c0 & 0xFFFF0000u), __uint_as_float(c1 & 0xFFFF0000u))
+                uint64_t v = KIND == 1 ? ((r & 1) ? pq::pack2(pq::bf16_minus<1>(c0, mu), pq::bf16_minus<1>(c1, mu))
+                                                  : pq::pack2(pq::bf16_minus<0>(c0, mu), pq::bf16_minus<0>(c1, mu)))
+                             : (r & 1) ? pq::pack2(__uint_as_float(c0 & 0xFFFF0000u), __uint_as_float(c1 & 0xFFFF0000u))
                                      : pq::pack2(__uint_as_float(c0 << 16), __uint_as_float(c1 << 16));
                 if (KIND == 0) v = pq::mul2(pq::mul2(v, inv2), w2[j]);
-                if (KIND == 1) v = pq::fma2(pq::mul2(pq::add2(v, nmu2), inv2), w2[j], sh2[j]);
+                if (KIND == 1) v = pq::fma2(pq::mul2(v, inv2), w2[j], sh2[j]);
                 y2[j] = v;
                 float lo, hi;
                 pq::unpack2(v, lo, hi);
@@ -655,6 +657,8 @@ pq_status launch_quad(const uint16_t *H, int64_t rows, int64_t rows_pad, int K, 
 // ... (the walk the statistics are defined on), the two octets of a 16-channel group sit in neighbouring
 // lanes (one shuffle for the group's absmax), every lane converts its own eight values and stores four bytes of
 // codes (128 contiguous bytes per warp instruction).  No shared memory, nothing but streaming.
+// (The statistics widen their values here: a lane has one chain of additions, and with the mixed-precision forms, whose
+// result is ready later, 18432 x 3072 went from 47 / 61 to 63 / 74 us.)
 constexpr int kDirectMaxOcts = 16;  // octets per lane: rows of up to 4096 channels
 constexpr int kDirectThreads = 128;
 
@@ -786,8 +790,9 @@ pq_status launch(const uint16_t *H, int64_t M, int64_t rows_pad, int K, int64_t 
             PQ_CUDA_OK(cudaFuncSetAttribute(norm_quant_grouped_kernel<KIND, SF_LAYOUT>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(group_smem)));
         PQ_REQUIRE(group_blocks < (1ll << 31), PQ_ERR_SHAPE);
-        norm_quant_grouped_kernel<KIND, SF_LAYOUT><<<static_cast<unsigned>(group_blocks), kGroupWarps * kSplit * 32, group_smem, st>>>(
-            H, M, rows_pad, K, ld, a, b, eps, perm, ts, codes, sf, y_out);
+        PQ_CUDA_OK(pq::launch_dependent(norm_quant_grouped_kernel<KIND, SF_LAYOUT>, dim3(static_cast<unsigned>(group_blocks)),
+                                        dim3(kGroupWarps * kSplit * 32), group_smem, st, H, M, rows_pad, K, ld, a, b, eps, perm, ts,
+                                        codes, sf, y_out));
         return pq_launch_status();
     }
     if (K <= kQuadMaxK) return launch_quad<KIND, SF_LAYOUT>(H, M, rows_pad, K, ld, a, b, eps, perm, nullptr, ts, codes, sf, y_out, st);

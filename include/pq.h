@@ -155,8 +155,8 @@ pq_status pq_tensor_scale(const float *amax, int64_t K, float *ts, void *stream)
  * keys keep ascending channel order.  j = J is the activation-only sort of Prop. 3.2, j = 0 the
  * weight-only sort.
  *   K <= 16384, 1 <= J <= 16.  perms : int32 [J+1, K] out.
- *   ws : pq_workspace_bytes(PQ_OP_SELECT_PERM, 0, K, 0, J + 1) bytes, 256-byte aligned (the sort keys of
- *        every candidate); a NULL or short workspace returns PQ_ERR_WORKSPACE. */
+ *   ws : pq_workspace_bytes(PQ_OP_SELECT_PERM, 0, K, 0, J + 1) bytes, 256-byte aligned (part of the
+ *        interface; the sort itself works in shared memory); a NULL or short one returns PQ_ERR_WORKSPACE. */
 pq_status pq_select_perm(const double *sumsq_a, int64_t rows_a, const double *sumsq_w,
                          int64_t rows_w, int64_t K, int J, int32_t *perms, void *ws,
                          size_t ws_bytes, void *stream);

@@ -99,7 +99,7 @@ pq_status unlocked(F &&call) {
 // linear(X, ts_x, xq, sfx, wq, sfw, ts_w, Y or None, ws) -> Y or status
 PyObject *linear(PyObject *, PyObject *const *a, Py_ssize_t given) {
     return guarded(given, 9, [&]() -> PyObject * {
-        const at::Tensor &X = matrix(a[0]), &W = tensor(a[4]), &scratch = tensor(a[8]);
+        const at::Tensor &X = matrix(a[0]), &W = tensor(a[4]);
         require(W.dim() >= 1, "wq is [N, K / 2]");
         const int64_t M = X.size(0), K = X.size(1), N = W.size(0), ld = X.stride(0);
         const bool make = a[7] == Py_None;
@@ -109,9 +109,9 @@ PyObject *linear(PyObject *, PyObject *const *a, Py_ssize_t given) {
         const float *ts_x = ptr_as<float>(a[1]), *ts_w = ptr_as<float>(a[6]);
         uint8_t *xq = ptr_as<uint8_t>(a[2]), *sfx = ptr_as<uint8_t>(a[3]), *sfw = ptr_as<uint8_t>(a[5]);
         const uint8_t *wq = static_cast<const uint8_t *>(ptr(W));
-        void *y = ptr(Y), *ws = ptr(scratch), *st = stream();
+        void *y = ptr(Y), *ws = ptr_as<void>(a[8]), *st = stream();
         const int64_t ldy = Y.stride(0);
-        const size_t ws_bytes = static_cast<size_t>(scratch.numel());
+        const size_t ws_bytes = ws ? static_cast<size_t>(tensor(a[8]).numel()) : 0;
         const pq_status s = unlocked([&] { return pq_linear_w4a4(x, M, K, ld, ts_x, xq, sfx, wq, sfw, ts_w, N, y, ldy, ws, ws_bytes, st); });
         if (s != PQ_OK) return status(s);
         if (make) return THPVariable_Wrap(std::move(Y));
@@ -123,15 +123,15 @@ PyObject *linear(PyObject *, PyObject *const *a, Py_ssize_t given) {
 // gemm(xq, sfx, ts_x, wq, sfw, ts_w, Y, ws) -> status
 PyObject *gemm(PyObject *, PyObject *const *a, Py_ssize_t given) {
     return guarded(given, 8, [&]() -> PyObject * {
-        const at::Tensor &X = tensor(a[0]), &W = tensor(a[3]), &Y = tensor(a[6]), &scratch = tensor(a[7]);
+        const at::Tensor &X = tensor(a[0]), &W = tensor(a[3]), &Y = tensor(a[6]);
         require(X.dim() == 2 && W.dim() >= 1, "codes are [rows, K / 2]");
         const int64_t M = X.size(0), K = X.size(1) * 2, N = W.size(0), ldy = Y.dim() == 2 ? Y.stride(0) : 0;
         output(Y, M, N);
         const uint8_t *xq = static_cast<const uint8_t *>(ptr(X)), *wq = static_cast<const uint8_t *>(ptr(W));
         const uint8_t *sfx = ptr_as<uint8_t>(a[1]), *sfw = ptr_as<uint8_t>(a[4]);
         const float *ts_x = ptr_as<float>(a[2]), *ts_w = ptr_as<float>(a[5]);
-        void *y = ptr(Y), *ws = ptr(scratch), *st = stream();
-        const size_t ws_bytes = static_cast<size_t>(scratch.numel());
+        void *y = ptr(Y), *ws = ptr_as<void>(a[7]), *st = stream();
+        const size_t ws_bytes = ws ? static_cast<size_t>(tensor(a[7]).numel()) : 0;
         return status(unlocked([&] { return pq_gemm_w4a4(xq, sfx, ts_x, wq, sfw, ts_w, M, N, K, y, ldy, ws, ws_bytes, st); }));
     });
 }

@@ -110,8 +110,8 @@ class QuantLinear:
         self._sets = []          # further (xq, sfx) pairs for forward_batches
 
     def __call__(self, X, Y=None):
-        M, K = X.shape
-        assert M <= self.M_max and K == self.K
+        M = X.shape[0]
+        assert M <= self.M_max and X.shape[1] == self.K
         return B.linear(X, self.ts_x, self.xq, self.sfx, self.wq, self.sfw, self.ts_w, Y, self.ws)  # uses M rows of xq
 
     def forward_batches(self, Xs, Ys, n_sets=4):
@@ -144,8 +144,8 @@ class QuantLinearH(QuantLinear):
         self.order = None if order is None else order.to(torch.int32).contiguous()
 
     def __call__(self, X, Y=None):
-        M, K = X.shape
-        assert M <= self.M_max and K == self.K
+        M = X.shape[0]
+        assert M <= self.M_max and X.shape[1] == self.K
         if Y is None:
             Y = torch.empty(M, self.N, dtype=torch.bfloat16, device=X.device)
         xq = self.xq if M == self.M_max else self.xq[:M]

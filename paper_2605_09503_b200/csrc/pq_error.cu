@@ -183,6 +183,7 @@ group_error_direct(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int6
 // What bounds it: shared-memory wavefronts (a 64-bit gather through a random order takes about 6 of them
 // where 2 would do: 0.05 per element) and instruction issue, in about equal parts.
 constexpr int kGatherThreads = 768;  // 80 registers per thread; 960 threads at 64 spill
+constexpr int kMaxOrders = 9;      // eight candidates and the original order
 constexpr int kMaxGroups = 15;                                           // named barriers 1..15
 constexpr int kSfTabMax = 2624;  // bf16 magnitudes from "scale byte 0" to "saturated": 19 binades and the edges
 
@@ -206,6 +207,7 @@ __device__ __forceinline__ void build_scale_tab(ScaleTab &tab, float ts) {
         hi = min(0x7F80u, (__float_as_uint(__fmul_rn(mag, 448.0f)) >> 16) + 2u);
     }
     if (threadIdx.x == 0) tab.lo = lo, tab.hi = hi;
+#pragma unroll 4
     for (uint32_t i = threadIdx.x; i <= hi - lo && i < kSfTabMax; i += blockDim.x) {
         const float d = __fmul_rn(pq::e4m3_to_f32(pq::f32_to_e4m3(__fdiv_rn(bf16_pattern(lo + i), c6))), ts);
         tab.rd[i] = make_float2(d > 0.0f ? __frcp_rn(d) : 0.0f, -d);
@@ -326,6 +328,7 @@ struct GatherParams {
     const int32_t *perms;      // [P - identity, K]
     int opb;                   // orders per block (blockIdx.y picks the subset)
     int groups, group_threads;
+    uint32_t base[2], rem[2];  // pairs / shares and its remainder: subsets of opb orders, the last subset
     int chunks;                // eight per slab; the chunks of a last slab that hold no rows may be left out
     float Qf;
     float *part;               // [chunks, P, K/g]
@@ -348,20 +351,27 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     uint16_t *slot_s = reinterpret_cast<uint16_t *>(smem + static_cast<size_t>(p.groups) * K * 8);
     unsigned char *tab_s = reinterpret_cast<unsigned char *>(slot_s + static_cast<size_t>(p.opb) * K);
     uint2 *int_tab = reinterpret_cast<uint2 *>(tab_s);
+    if (KIND == 1) pq::build_int_tab(int_tab, p.Qf, true);  // needs nothing of the kernel in front
     pq::dependents_may_launch();
     pq::wait_for_prior_grid();
 
-    for (int i = threadIdx.x; i < no * K; i += blockDim.x) {
-        const int o = i / K, j = i - o * K, order = o0 + o - p.identity;
-        const uint32_t ch = order < 0 ? static_cast<uint32_t>(j) : static_cast<uint32_t>(__ldg(p.perms + static_cast<int64_t>(order) * K + j));
+    for (int j = threadIdx.x; j < K; j += blockDim.x) {
+        // the channel of every order at position j, all loads in flight (one after the other they cost 10 us a launch)
+        uint32_t ch[kMaxOrders];
+#pragma unroll
+        for (int o = 0; o < kMaxOrders; ++o) {
+            const int order = o0 + o - p.identity;
+            ch[o] = o < no && order >= 0 ? static_cast<uint32_t>(__ldg(p.perms + static_cast<int64_t>(order) * K + j)) : static_cast<uint32_t>(j);
+        }
         // the two 16-byte halves of a run's slots lie in separate planes: lanes read consecutive 16-byte words
-        slot_s[o * K + ((j >> 3) & 1) * (K >> 1) + (j >> 4) * 8 + (j & 7)] = static_cast<uint16_t>(pq::quad_channel(ch));
+        uint16_t *slot = slot_s + ((j >> 3) & 1) * (K >> 1) + (j >> 4) * 8 + (j & 7);
+#pragma unroll
+        for (int o = 0; o < kMaxOrders; ++o)
+            if (o < no) slot[o * K] = static_cast<uint16_t>(pq::quad_channel(ch[o]));
     }
     const int sides = p.ts[1] ? 2 : 1;
     if (KIND == 0) {
         for (int s = 0; s < sides; ++s) build_scale_tab(reinterpret_cast<ScaleTab *>(tab_s + s * kTabBytes)[0], __ldg(p.ts[s]));
-    } else {
-        pq::build_int_tab(int_tab, p.Qf, true);
     }
     __syncthreads();
 
@@ -384,8 +394,16 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     const uint4 *slot4 = reinterpret_cast<const uint4 *>(slot_s);
     const int64_t Kg = runs / TEAM16;
 
-    for (int chunk = blockIdx.x * p.groups + grp; chunk < p.chunks; chunk += gridDim.x * p.groups) {
-        const int slab = chunk / kSlabChunks, t = pq::tensor_of_slab(p.list, slab);
+    // The (chunk, order) pairs of this block row, chunk by chunk, in equal shares: a group that has work for a few
+    // chunks only would otherwise wait for the one that has a whole chunk more.
+    const uint32_t share = blockIdx.x * p.groups + grp, base = p.base[o0 + no == p.P], rem = p.rem[o0 + no == p.P];
+    const uint32_t first = share * base + min(share, rem);
+    int pairs = static_cast<int>(base + (share < rem));
+    uint32_t chunk = first / static_cast<uint32_t>(no);
+    int ob = static_cast<int>(first - chunk * no);
+    for (int oe; pairs > 0; pairs -= oe - ob, ob = 0, ++chunk) {
+        oe = min(no, ob + pairs);
+        const int slab = static_cast<int>(chunk / kSlabChunks), t = pq::tensor_of_slab(p.list, slab);
         const int64_t r0 = static_cast<int64_t>(slab - p.list.slab0[t]) * PQ_SLAB_ROWS + chunk % kSlabChunks * PQ_CHUNK_ROWS;
         const int64_t ld = p.list.ld[t], left = p.list.rows[t] - r0;
         const int n = left >= PQ_CHUNK_ROWS ? PQ_CHUNK_ROWS : (left > 0 ? static_cast<int>(left) : 0);
@@ -408,7 +426,7 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
             }
             group_sync();
 #pragma unroll 1
-            for (int o = 0; o < no; ++o) {
+            for (int o = ob; o < oe; ++o) {
 #pragma unroll 1
                 for (int q0 = 0; q0 < runs; q0 += p.group_threads) {
                     const int q = q0 + tid;
@@ -436,17 +454,17 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
             }
         }
         // every thread writes out the sums it kept itself
-        for (int o = 0; o < no; ++o)
+        for (int o = ob; o < oe; ++o)
             for (int q = tid; q < runs; q += p.group_threads)
                 if ((q % TEAM16) == 0) p.part[(static_cast<int64_t>(chunk) * p.P + o0 + o) * Kg + q / TEAM16] = n ? acc_s[o * runs + q] : 0.0f;
     }
 }
 
 // Orders per block, groups per block and threads per group for `chunks` chunks of K channels under P orders:
-// the configuration with the shortest estimated schedule.  A group of W warps works through
-// ceil(chunks * subsets / (blocks * groups)) chunks; a chunk costs one unit per order and run of each
-// lane, plus about a quarter of a unit of staging per run; an SM is taken to be saturated by 20 warps, fewer
-// are proportionally slower.
+// the configuration with the shortest estimated schedule.  A group works through its share of the (chunk, order)
+// pairs; a pair costs one unit per run of each lane, a chunk a quarter of a unit of staging per run (and a share
+// touches one chunk more than it holds whole); an SM is taken to be saturated by 20 warps, fewer are
+// proportionally slower.
 struct GatherConfig {
     int opb = 0, groups = 0, group_threads = 0;
 };
@@ -462,9 +480,9 @@ inline GatherConfig gather_config(int64_t chunks, int64_t K, int P, int sides, i
             for (int groups = 1; groups <= kMaxGroups && groups * threads <= kGatherThreads; ++groups) {
                 if (gather_smem_bytes(K, opb, groups, sides) > 226 * 1024) break;
                 const int64_t blocks = sms / subsets > 0 ? sms / subsets : 1;
-                const int64_t rounds = pq_ceil_div(chunks, blocks * groups);
+                const double pairs = static_cast<double>(pq_ceil_div(chunks * opb, blocks * groups));
                 const int warps = groups * threads / 32;
-                const double cost = static_cast<double>(rounds) * threads * groups * per_lane * (opb + 0.25) * (warps < 20 ? 20.0 / warps : 1.0);
+                const double cost = (pairs + 0.25 * (pairs / opb + 1.0)) * threads * groups * per_lane * (warps < 20 ? 20.0 / warps : 1.0);
                 if (!best.groups || cost < best_cost) {
                     best_cost = cost;
                     best.opb = opb, best.groups = groups, best.group_threads = threads;
@@ -497,13 +515,19 @@ pq_status launch_gather(GatherParams &p, int64_t K, int P, float Qf, float *part
     p.K = static_cast<int>(K), p.P = P, p.Qf = Qf, p.part = part;
     p.opb = cfg.opb, p.groups = cfg.groups, p.group_threads = cfg.group_threads;
     const int64_t subsets = pq_ceil_div(P, cfg.opb), share = sms / subsets > 0 ? sms / subsets : 1;
-    const int64_t want = pq_ceil_div(p.chunks, cfg.groups);
+    const int64_t want = pq_ceil_div(static_cast<int64_t>(p.chunks) * cfg.opb, cfg.groups);
+    const int64_t blocks = want < share ? want : share;
+    for (int last = 0; last < 2; ++last) {
+        const int64_t orders = last ? P - (subsets - 1) * cfg.opb : cfg.opb;
+        const int64_t pairs = p.chunks * orders, shares = blocks * cfg.groups;
+        p.base[last] = static_cast<uint32_t>(pairs / shares), p.rem[last] = static_cast<uint32_t>(pairs % shares);
+    }
     const size_t smem = gather_smem_bytes(K, cfg.opb, cfg.groups, sides);
     auto kern = group_error_gather<KIND, TEAM / 2>;
     if (smem > 48 * 1024)
         PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
     const unsigned threads = static_cast<unsigned>(cfg.groups * cfg.group_threads + (p.weights.lambda ? 32 : 0));
-    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(want < share ? want : share), static_cast<unsigned>(subsets)),
+    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(subsets)),
                                     dim3(threads), smem, st, p));
     return pq_launch_status();
 }

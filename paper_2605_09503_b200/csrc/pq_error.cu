@@ -173,13 +173,16 @@ group_error_direct(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int6
 // staged rows before it fetches the next four: the staging is paid once for up to eight orders instead of
 // once per order.  A lane takes a run of 16 positions: its slots come from a table of 16-bit indices the
 // block prepared once per order, one 64-bit load per position brings that channel of four rows, and the
-// error of TWO ROWS is carried side by side in packed fp32 registers (row_pair_sse).  The words the gather
-// returns hold the same channel of two rows, so they are widened as they are; the one-row-at-a-time form
+// error of TWO ROWS is carried side by side (row_pair_sse): the words the gather returns hold the same channel of
+// two rows, so they are widened as they are; the one-row-at-a-time form
 // had to re-pair them by byte permutes first (half an instruction per element), read the original-order
 // kernel's decode tables (two per element; the hardware E2M1 -> f16 -> fp32 converts take one and a half)
 // and divide once per group and row (the scale tables below take a clamp and two loads).
 // Blocks are persistent, one per SM; the groups of a block only share the slot and scale tables.
 //
+// NVFP4 is scalar arithmetic: packed f32x2 instructions save issue slots but run on one of the two FMA pipes only, and
+// with the f16 converts there too it was 59 % busy (9216 x 3072, six orders: 79 us scalar, 84 packed).  The integer
+// formats, without converts, are packed (4608 x 3072, INT4 g64: 53.4 us, 54.1 scalar).
 // What bounds it: shared-memory wavefronts (a 64-bit gather through a random order takes about 6 of them
 // where 2 would do: 0.05 per element) and instruction issue, in about equal parts.
 constexpr int kGatherThreads = 768;  // 80 registers per thread; 960 threads at 64 spill
@@ -213,10 +216,8 @@ __device__ __forceinline__ void build_scale_tab(ScaleTab &tab, float ts) {
         tab.rd[i] = make_float2(d > 0.0f ? __frcp_rn(d) : 0.0f, -d);
     }
 }
-// E2M1 of the two floats of a pair and back to fp32 (E2M1 -> f16 is exact, f16 -> f32 too).
-__device__ __forceinline__ uint64_t e2m1_pair(uint64_t y2) {
-    float lo, hi;
-    unpack2(y2, lo, hi);
+// E2M1 of two floats and back to fp32 (E2M1 -> f16 is exact, f16 -> f32 too).
+__device__ __forceinline__ void e2m1_pair(float &y0, float &y1) {
     uint32_t h2;
     asm("{\n"
         ".reg .b8 c;\n"
@@ -224,9 +225,9 @@ __device__ __forceinline__ uint64_t e2m1_pair(uint64_t y2) {
         "cvt.rn.f16x2.e2m1x2 %0, c;\n"
         "}\n"
         : "=r"(h2)
-        : "f"(lo), "f"(hi));
-    return pack2(__half2float(__ushort_as_half(static_cast<uint16_t>(h2 & 0xFFFFu))),
-                 __half2float(__ushort_as_half(static_cast<uint16_t>(h2 >> 16))));
+        : "f"(y0), "f"(y1));
+    y0 = __half2float(__ushort_as_half(static_cast<uint16_t>(h2 & 0xFFFFu)));
+    y1 = __half2float(__ushort_as_half(static_cast<uint16_t>(h2 >> 16)));
 }
 
 // One row of a pair by the definition of the integer formats: for scales in subnormal or non-finite territory.
@@ -275,50 +276,55 @@ __device__ __forceinline__ void row_pair_sse(const uint32_t (&u)[16], const Scal
     uint32_t am = mx[0];
 #pragma unroll
     for (int m = 1; m < TEAM16; m <<= 1) am = max_bf16x2(am, __shfl_xor_sync(0xFFFFFFFFu, am, m));
-    uint64_t r2, nd2;
+    float r0, r1, nd0, nd1;  // reciprocal and negated decode scale of either row
     if (KIND == 0) {
         const uint32_t cl = min_u16x2(max_u16x2(am, lo2), hi2);
         const float2 *rd = tab->rd - (lo2 & 0xFFFFu);
         const float2 d0 = rd[cl & 0xFFFFu], d1 = rd[cl >> 16];
-        r2 = pack2(d0.x, d1.x), nd2 = pack2(d0.y, d1.y);
+        r0 = d0.x, r1 = d1.x, nd0 = d0.y, nd1 = d1.y;
     } else {
         const uint32_t a0 = am & 0xFFFFu, a1 = am >> 16;
         if (__any_sync(0xFFFFFFFFu, pq::int_scale_is_odd(a0) || pq::int_scale_is_odd(a1))) {
             e0 = int_row_sse<TEAM16>(u, 0, bf16_pattern(a0), Qf), e1 = int_row_sse<TEAM16>(u, 1, bf16_pattern(a1), Qf);
             return;
         }
-        float r0, r1, nd0, nd1;
         pq::int_scale_from_tab(int_tab, a0, r0, nd0);
         pq::int_scale_from_tab(int_tab, a1, r1, nd1);
-        r2 = pack2(r0, r1), nd2 = pack2(nd0, nd1);
     }
 
-    uint64_t run2[2];
+    float run0[2], run1[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        uint64_t acc2 = 0;  // {+0, +0}
+        if (KIND == 0) {
+            float acc0 = 0.0f, acc1 = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint32_t w = u[8 * h + i];
-            const uint64_t x2 = pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
-            const uint64_t y2 = mul2(x2, r2);
-            uint64_t q2;
-            if (KIND == 0) {
-                q2 = e2m1_pair(y2);
-            } else {
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t w = u[8 * h + i];
+                const float x0 = __uint_as_float(w << 16), x1 = __uint_as_float(w & 0xFFFF0000u);
+                float q0 = __fmul_rn(x0, r0), q1 = __fmul_rn(x1, r1);
+                e2m1_pair(q0, q1);
+                const float d0 = __fmaf_rn(q0, nd0, x0), d1 = __fmaf_rn(q1, nd1, x1);
+                acc0 = __fmaf_rn(d0, d0, acc0), acc1 = __fmaf_rn(d1, d1, acc1);
+            }
+            run0[h] = acc0, run1[h] = acc1;
+        } else {
+            const uint64_t r2 = pack2(r0, r1), nd2 = pack2(nd0, nd1), one2 = pack2(1.0f, 1.0f);
+            const uint64_t magic = pack2(12582912.0f, 12582912.0f), unmagic = pack2(-12582912.0f, -12582912.0f);
+            uint64_t acc2 = 0;  // {+0, +0}
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t w = u[8 * h + i];
+                const uint64_t x2 = pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
                 // rint by adding and subtracting 1.5 * 2^23 (see row_sse16 for the form of the first addition).  No clamp:
                 // |x| / s <= Q (1 + 2^-22) here, which rounds to Q at most.
-                const uint64_t magic = pack2(12582912.0f, 12582912.0f), unmagic = pack2(-12582912.0f, -12582912.0f);
-                q2 = add2(fma2(y2, pack2(1.0f, 1.0f), magic), unmagic);
+                const uint64_t q2 = add2(fma2(mul2(x2, r2), one2, magic), unmagic);
+                const uint64_t d2 = fma2(q2, nd2, x2);
+                acc2 = fma2(d2, d2, acc2);
             }
-            const uint64_t delta = fma2(q2, nd2, x2);
-            acc2 = fma2(delta, delta, acc2);
+            unpack2(acc2, run0[h], run1[h]);
         }
-        run2[h] = acc2;
     }
-    float s0, s1;
-    unpack2(add2(run2[0], run2[1]), s0, s1);
-    e0 = pq::team_sum<TEAM16>(s0), e1 = pq::team_sum<TEAM16>(s1);
+    e0 = pq::team_sum<TEAM16>(__fadd_rn(run0[0], run0[1])), e1 = pq::team_sum<TEAM16>(__fadd_rn(run1[0], run1[1]));
 }
 
 struct GatherParams {

@@ -28,6 +28,7 @@
 // the first pass's window and bit 2 with bit 5.  The first spreads the strided accesses of phase 2 over
 // all banks, the second lets the eight lanes of a 16-byte store wavefront of phase 1 hit distinct banks.
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 
 #include "pq_common.cuh"
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) hadamard_quant_kernel(
     // offset: the same for every row, so it is worked out once per block (K <= 16384: 16 bits)
     for (int j = threadIdx.x; j < p.K; j += THREADS)
         offset_s[j] = static_cast<uint16_t>(swz(p.perm ? __ldg(p.perm + j) : j, p.sw) << 2);
-    const float ts = p.codes ? __ldg(p.ts) : 1.0f;
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldg(p.ts) : 1.0f);
 
     for (int64_t batch = blockIdx.x; batch < batches; batch += gridDim.x) {
         const int64_t row0 = batch * kRows;
@@ -264,93 +265,97 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) hadamard_quant_kernel(
         // the read-out offsets are fetched once for both rows and the two quantizer chains interleave
         const int rows_here = static_cast<int>(min(static_cast<int64_t>(kRows), p.rows_pad - row0));
         const int row_pairs = (rows_here + 1) >> 1;
-        for (int c = warp; c < row_pairs * chunks; c += THREADS / 32) {
-            const int rp = c / chunks, g = (c - rp * chunks) * 32 + lane;
-            const bool have = g < gpr;
-            uint32_t iw[8];
-            if (have) {
-                const uint4 i0 = reinterpret_cast<const uint4 *>(offset_s)[2 * g], i1 = reinterpret_cast<const uint4 *>(offset_s)[2 * g + 1];
-                iw[0] = i0.x, iw[1] = i0.y, iw[2] = i0.z, iw[3] = i0.w, iw[4] = i1.x, iw[5] = i1.y, iw[6] = i1.z, iw[7] = i1.w;
-            } else {
+        auto read_out = [&](auto fast) {
+            for (int c = warp; c < row_pairs * chunks; c += THREADS / 32) {
+                const int rp = c / chunks, g = (c - rp * chunks) * 32 + lane;
+                const bool have = g < gpr;
+                uint32_t iw[8];
+                if (have) {
+                    const uint4 i0 = reinterpret_cast<const uint4 *>(offset_s)[2 * g], i1 = reinterpret_cast<const uint4 *>(offset_s)[2 * g + 1];
+                    iw[0] = i0.x, iw[1] = i0.y, iw[2] = i0.z, iw[3] = i0.w, iw[4] = i1.x, iw[5] = i1.y, iw[6] = i1.z, iw[7] = i1.w;
+                } else {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) iw[j] = 0;
-            }
-            float out[2][16];
-            bool live[2], present[2];
-            int64_t row[2];
+                    for (int j = 0; j < 8; ++j) iw[j] = 0;
+                }
+                float out[2][16];
+                bool live[2], present[2];
+                int64_t row[2];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = 2 * rp + h;
-                row[h] = row0 + r;
-                present[h] = r < rows_here;
-                // the second row of the last pair does not exist when the block holds an odd number of rows (three
-                // at 16384 channels): that index is the first row of the NEXT batch and lies past this image
-                live[h] = present[h] && row[h] < p.rows;
-                const char *row_b = reinterpret_cast<const char *>(had_smem + static_cast<size_t>(r) * p.K);
+                for (int h = 0; h < 2; ++h) {
+                    const int r = 2 * rp + h;
+                    row[h] = row0 + r;
+                    present[h] = r < rows_here;
+                    // the second row of the last pair does not exist when the block holds an odd number of rows (three
+                    // at 16384 channels): that index is the first row of the NEXT batch and lies past this image
+                    live[h] = present[h] && row[h] < p.rows;
+                    const char *row_b = reinterpret_cast<const char *>(had_smem + static_cast<size_t>(r) * p.K);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) out[h][j] = 0.0f;
-                if (live[h] && have) {
+                    for (int j = 0; j < 16; ++j) out[h][j] = 0.0f;
+                    if (live[h] && have) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        out[h][2 * j] = *reinterpret_cast<const float *>(row_b + (iw[j] & 0xFFFFu));
-                        out[h][2 * j + 1] = *reinterpret_cast<const float *>(row_b + (iw[j] >> 16));
+                        for (int j = 0; j < 8; ++j) {
+                            out[h][2 * j] = *reinterpret_cast<const float *>(row_b + (iw[j] & 0xFFFFu));
+                            out[h][2 * j + 1] = *reinterpret_cast<const float *>(row_b + (iw[j] >> 16));
+                        }
+                        if (!p.log[0]) {  // no pass of phase 2 carried the scaling
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) out[h][j] = __fmul_rn(out[h][j], p.scale);
+                        }
+                        if (p.y_out) {
+                            uint32_t yw[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j)
+                                yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[h][2 * j])) |
+                                        (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[h][2 * j + 1]))) << 16);
+                            uint4 *ydst = reinterpret_cast<uint4 *>(p.y_out + row[h] * p.K) + 2 * g;
+                            ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                            ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                        }
                     }
-                    if (!p.log[0]) {  // no pass of phase 2 carried the scaling
+                }
+                if (!p.codes) continue;
+                uint32_t sf8[2];
+                float rcp[2];
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) out[h][j] = __fmul_rn(out[h][j], p.scale);
+                for (int h = 0; h < 2; ++h) {
+                    float amax = 0.0f;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(out[h][j]));
+                    pq::nvfp4_scale<decltype(fast)::value>(amax, scaler, sf8[h], rcp[h]);
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (live[h] && have) {
+                        const uint64_t rcp2 = pack2(rcp[h], rcp[h]);
+                        float ylo[8], yhi[8];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            unpack2(mul2(pack2(out[h][2 * j], out[h][2 * j + 1]), rcp2), ylo[2 * j], ylo[2 * j + 1]);
+                            unpack2(mul2(pack2(out[h][8 + 2 * j], out[h][9 + 2 * j]), rcp2), yhi[2 * j], yhi[2 * j + 1]);
+                        }
+                        *reinterpret_cast<uint2 *>(p.codes + row[h] * (p.K >> 1) + g * 8) =
+                            make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
                     }
-                    if (p.y_out) {
-                        uint32_t yw[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[h][2 * j])) |
-                                    (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[h][2 * j + 1]))) << 16);
-                        uint4 *ydst = reinterpret_cast<uint4 *>(p.y_out + row[h] * p.K) + 2 * g;
-                        ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
-                        ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                    // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
+                    uint32_t word = sf8[h];
+                    word |= __shfl_down_sync(0xFFFFFFFFu, sf8[h], 1) << 8;
+                    word |= __shfl_down_sync(0xFFFFFFFFu, sf8[h], 2) << 16;
+                    word |= __shfl_down_sync(0xFFFFFFFFu, sf8[h], 3) << 24;
+                    if (!have || !present[h]) continue;
+                    if (SF_LAYOUT == PQ_SF_TCGEN05) {
+                        if ((g & 3) == 0) *reinterpret_cast<uint32_t *>(p.sf + pq::sf_tc_offset(row[h], g, gpr >> 2)) = word;
+                    } else if (live[h]) {
+                        if ((gpr & 3) == 0) {
+                            if ((g & 3) == 0) *reinterpret_cast<uint32_t *>(p.sf + row[h] * gpr + g) = word;
+                        } else {
+                            p.sf[row[h] * gpr + g] = static_cast<uint8_t>(sf8[h]);
+                        }
                     }
                 }
             }
-            if (!p.codes) continue;
-            uint32_t sf8[2];
-            float rcp[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float amax = 0.0f, d;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(out[h][j]));
-                pq::nvfp4_scale(amax, ts, sf8[h], d, rcp[h]);
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (live[h] && have) {
-                    const uint64_t rcp2 = pack2(rcp[h], rcp[h]);
-                    float ylo[8], yhi[8];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        unpack2(mul2(pack2(out[h][2 * j], out[h][2 * j + 1]), rcp2), ylo[2 * j], ylo[2 * j + 1]);
-                        unpack2(mul2(pack2(out[h][8 + 2 * j], out[h][9 + 2 * j]), rcp2), yhi[2 * j], yhi[2 * j + 1]);
-                    }
-                    *reinterpret_cast<uint2 *>(p.codes + row[h] * (p.K >> 1) + g * 8) =
-                        make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
-                }
-                // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
-                uint32_t word = sf8[h];
-                word |= __shfl_down_sync(0xFFFFFFFFu, sf8[h], 1) << 8;
-                word |= __shfl_down_sync(0xFFFFFFFFu, sf8[h], 2) << 16;
-                word |= __shfl_down_sync(0xFFFFFFFFu, sf8[h], 3) << 24;
-                if (!have || !present[h]) continue;
-                if (SF_LAYOUT == PQ_SF_TCGEN05) {
-                    if ((g & 3) == 0) *reinterpret_cast<uint32_t *>(p.sf + pq::sf_tc_offset(row[h], g, gpr >> 2)) = word;
-                } else if (live[h]) {
-                    if ((gpr & 3) == 0) {
-                        if ((g & 3) == 0) *reinterpret_cast<uint32_t *>(p.sf + row[h] * gpr + g) = word;
-                    } else {
-                        p.sf[row[h] * gpr + g] = static_cast<uint8_t>(sf8[h]);
-                    }
-                }
-            }
-        }
+        };
+        if (scaler.fast) read_out(std::true_type{});
+        else read_out(std::false_type{});
     }
 }
 
@@ -464,7 +469,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) hadamard_quant_rows_kernel(
     for (int j = threadIdx.x; j < K; j += 32 * kRowWarps)
         offset_s[((j >> 3) & 1) * (K / 2) + (j >> 4) * 8 + (j & 7)] =
             static_cast<uint16_t>(row_image_index<N>(p.perm ? __ldg(p.perm + j) : j) << 2);
-    const float ts = p.codes ? __ldg(p.ts) : 1.0f;
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldg(p.ts) : 1.0f);
     __syncthreads();
 
     // warps of different blocks first, so that few rows spread over all SMs
@@ -506,59 +511,63 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) hadamard_quant_rows_kernel(
             __syncwarp();
         }
         // ---- phase 3: one output group per lane, 192 groups
+        auto read_out = [&](auto fast) {
 #pragma unroll 1
-        for (int i = lane; i < RPW * GPR; i += 32) {
-            const int r = i / GPR, g = i - r * GPR;
-            const int64_t row = row0 + r;
-            const bool live = row < p.rows;
-            float out[16];
+            for (int i = lane; i < RPW * GPR; i += 32) {
+                const int r = i / GPR, g = i - r * GPR;
+                const int64_t row = row0 + r;
+                const bool live = row < p.rows;
+                float out[16];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) out[j] = 0.0f;
-            if (live) {
-                const uint4 i0 = offset4[g], i1 = offset4[GPR + g];
-                const uint32_t iw[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
-                const char *row_b = reinterpret_cast<const char *>(image + r * K);
+                for (int j = 0; j < 16; ++j) out[j] = 0.0f;
+                if (live) {
+                    const uint4 i0 = offset4[g], i1 = offset4[GPR + g];
+                    const uint32_t iw[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
+                    const char *row_b = reinterpret_cast<const char *>(image + r * K);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    out[2 * j] = *reinterpret_cast<const float *>(row_b + (iw[j] & 0xFFFFu));
-                    out[2 * j + 1] = *reinterpret_cast<const float *>(row_b + (iw[j] >> 16));
+                    for (int j = 0; j < 8; ++j) {
+                        out[2 * j] = *reinterpret_cast<const float *>(row_b + (iw[j] & 0xFFFFu));
+                        out[2 * j + 1] = *reinterpret_cast<const float *>(row_b + (iw[j] >> 16));
+                    }
+                    if (p.y_out) {
+                        uint32_t yw[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
+                                    (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
+                        uint4 *ydst = reinterpret_cast<uint4 *>(p.y_out + row * K) + 2 * g;
+                        ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                        ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                    }
                 }
-                if (p.y_out) {
-                    uint32_t yw[8];
+                if (!p.codes) continue;
+                float amax = 0.0f, rcp;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
-                                (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
-                    uint4 *ydst = reinterpret_cast<uint4 *>(p.y_out + row * K) + 2 * g;
-                    ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
-                    ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(out[j]));
+                uint32_t sf8;
+                pq::nvfp4_scale<decltype(fast)::value>(amax, scaler, sf8, rcp);
+                if (live) {
+                    const uint64_t rcp2 = pack2(rcp, rcp);
+                    float ylo[8], yhi[8];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        unpack2(mul2(pack2(out[2 * j], out[2 * j + 1]), rcp2), ylo[2 * j], ylo[2 * j + 1]);
+                        unpack2(mul2(pack2(out[8 + 2 * j], out[9 + 2 * j]), rcp2), yhi[2 * j], yhi[2 * j + 1]);
+                    }
+                    *reinterpret_cast<uint2 *>(p.codes + row * (K / 2) + g * 8) = make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
                 }
+                // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
+                uint32_t word = sf8;
+                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 1) << 8;
+                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2) << 16;
+                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3) << 24;
+                if ((g & 3) || row >= p.rows_pad) continue;
+                if (SF_LAYOUT == PQ_SF_TCGEN05) *reinterpret_cast<uint32_t *>(p.sf + pq::sf_tc_offset(row, g, GPR >> 2)) = word;
+                else if (live) *reinterpret_cast<uint32_t *>(p.sf + row * GPR + g) = word;
             }
-            if (!p.codes) continue;
-            float amax = 0.0f, d, rcp;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(out[j]));
-            uint32_t sf8;
-            pq::nvfp4_scale(amax, ts, sf8, d, rcp);
-            if (live) {
-                const uint64_t rcp2 = pack2(rcp, rcp);
-                float ylo[8], yhi[8];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    unpack2(mul2(pack2(out[2 * j], out[2 * j + 1]), rcp2), ylo[2 * j], ylo[2 * j + 1]);
-                    unpack2(mul2(pack2(out[8 + 2 * j], out[9 + 2 * j]), rcp2), yhi[2 * j], yhi[2 * j + 1]);
-                }
-                *reinterpret_cast<uint2 *>(p.codes + row * (K / 2) + g * 8) = make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
-            }
-            // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
-            uint32_t word = sf8;
-            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 1) << 8;
-            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2) << 16;
-            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3) << 24;
-            if ((g & 3) || row >= p.rows_pad) continue;
-            if (SF_LAYOUT == PQ_SF_TCGEN05) *reinterpret_cast<uint32_t *>(p.sf + pq::sf_tc_offset(row, g, GPR >> 2)) = word;
-            else if (live) *reinterpret_cast<uint32_t *>(p.sf + row * GPR + g) = word;
-        }
+        };
+        if (scaler.fast) read_out(std::true_type{});
+        else read_out(std::false_type{});
     }
 }
 

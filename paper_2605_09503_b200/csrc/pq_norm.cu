@@ -18,6 +18,7 @@
 // 1 adaptive LayerNorm; the four-rows-per-block kernel also exists as KIND 2, no normalization at all: the gather
 // quantizers of the offline path (a candidate order applied to activations or to the weight) run through it.
 #include <algorithm>
+#include <type_traits>
 
 #include "pq_common.cuh"
 
@@ -72,7 +73,7 @@ norm_quant_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad
     const bool live = row < rows;
     uint16_t *xs = row_s + static_cast<size_t>(warp) * K;
     const int octs = K >> 3, gpr = K >> 4;
-    const float ts = __ldg(ts_ptr);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
     float inv = 0.0f, mu = 0.0f;
 
     if (live) {
@@ -113,98 +114,102 @@ norm_quant_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad
     // normalize, quantize; the lanes of a group share its absmax by shuffles and each derive the scale.
     constexpr int POS = PQ_NORM_POS, LPG = 16 / POS;  // lanes per group
     const int slots = K / POS;
-    for (int q0 = 0; q0 < slots; q0 += 32) {
-        const int q = q0 + lane;           // positions POS q .. POS q + POS - 1, group q / LPG
-        const bool have = q < slots;
-        float out[POS];
+    auto walk = [&](auto fast) {
+        for (int q0 = 0; q0 < slots; q0 += 32) {
+            const int q = q0 + lane;           // positions POS q .. POS q + POS - 1, group q / LPG
+            const bool have = q < slots;
+            float out[POS];
 #pragma unroll
-        for (int j = 0; j < POS; ++j) out[j] = 0.0f;
-        if (live && have) {
-            float v[POS], w[POS];
-#pragma unroll
-            for (int h = 0; h < POS / 4; ++h) {
-                if (perm) {
-                    const int4 idx = __ldg(reinterpret_cast<const int4 *>(perm) + q * (POS / 4) + h);
-                    v[4 * h + 0] = pq::bf16_bits_to_f32(xs[idx.x]), v[4 * h + 1] = pq::bf16_bits_to_f32(xs[idx.y]);
-                    v[4 * h + 2] = pq::bf16_bits_to_f32(xs[idx.z]), v[4 * h + 3] = pq::bf16_bits_to_f32(xs[idx.w]);
-                } else {
-                    const uint2 u = reinterpret_cast<const uint2 *>(xs)[q * (POS / 4) + h];
-                    v[4 * h + 0] = __uint_as_float(u.x << 16), v[4 * h + 1] = __uint_as_float(u.x & 0xFFFF0000u);
-                    v[4 * h + 2] = __uint_as_float(u.y << 16), v[4 * h + 3] = __uint_as_float(u.y & 0xFFFF0000u);
-                }
-                const float4 a4 = __ldg(reinterpret_cast<const float4 *>(a) + q * (POS / 4) + h);
-                w[4 * h + 0] = a4.x, w[4 * h + 1] = a4.y, w[4 * h + 2] = a4.z, w[4 * h + 3] = a4.w;
-            }
-            if (KIND == 0) {
-#pragma unroll
-                for (int j = 0; j < POS; ++j) out[j] = __fmul_rn(__fmul_rn(v[j], inv), w[j]);
-            } else {
-                float sh[POS];
+            for (int j = 0; j < POS; ++j) out[j] = 0.0f;
+            if (live && have) {
+                float v[POS], w[POS];
 #pragma unroll
                 for (int h = 0; h < POS / 4; ++h) {
-                    const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b) + q * (POS / 4) + h);
-                    sh[4 * h + 0] = b4.x, sh[4 * h + 1] = b4.y, sh[4 * h + 2] = b4.z, sh[4 * h + 3] = b4.w;
+                    if (perm) {
+                        const int4 idx = __ldg(reinterpret_cast<const int4 *>(perm) + q * (POS / 4) + h);
+                        v[4 * h + 0] = pq::bf16_bits_to_f32(xs[idx.x]), v[4 * h + 1] = pq::bf16_bits_to_f32(xs[idx.y]);
+                        v[4 * h + 2] = pq::bf16_bits_to_f32(xs[idx.z]), v[4 * h + 3] = pq::bf16_bits_to_f32(xs[idx.w]);
+                    } else {
+                        const uint2 u = reinterpret_cast<const uint2 *>(xs)[q * (POS / 4) + h];
+                        v[4 * h + 0] = __uint_as_float(u.x << 16), v[4 * h + 1] = __uint_as_float(u.x & 0xFFFF0000u);
+                        v[4 * h + 2] = __uint_as_float(u.y << 16), v[4 * h + 3] = __uint_as_float(u.y & 0xFFFF0000u);
+                    }
+                    const float4 a4 = __ldg(reinterpret_cast<const float4 *>(a) + q * (POS / 4) + h);
+                    w[4 * h + 0] = a4.x, w[4 * h + 1] = a4.y, w[4 * h + 2] = a4.z, w[4 * h + 3] = a4.w;
                 }
+                if (KIND == 0) {
 #pragma unroll
-                for (int j = 0; j < POS; ++j)
-                    out[j] = __fmaf_rn(__fmul_rn(__fsub_rn(v[j], mu), inv), __fadd_rn(1.0f, w[j]), sh[j]);
+                    for (int j = 0; j < POS; ++j) out[j] = __fmul_rn(__fmul_rn(v[j], inv), w[j]);
+                } else {
+                    float sh[POS];
+#pragma unroll
+                    for (int h = 0; h < POS / 4; ++h) {
+                        const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b) + q * (POS / 4) + h);
+                        sh[4 * h + 0] = b4.x, sh[4 * h + 1] = b4.y, sh[4 * h + 2] = b4.z, sh[4 * h + 3] = b4.w;
+                    }
+#pragma unroll
+                    for (int j = 0; j < POS; ++j)
+                        out[j] = __fmaf_rn(__fmul_rn(__fsub_rn(v[j], mu), inv), __fadd_rn(1.0f, w[j]), sh[j]);
+                }
+            }
+            float amax = 0.0f;
+#pragma unroll
+            for (int j = 0; j < POS; ++j) amax = fmaxf(amax, fabsf(out[j]));
+#pragma unroll
+            for (int m = 1; m < LPG; m <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, m));
+            uint32_t sf8;
+            float r;
+            pq::nvfp4_scale<decltype(fast)::value>(amax, scaler, sf8, r);
+            uint32_t cw = 0;
+#pragma unroll
+            for (int h = 0; h < POS / 4; ++h) {
+                uint16_t c16;
+                asm("{\n"
+                    ".reg .b8 lo, hi;\n"
+                    "cvt.rn.satfinite.e2m1x2.f32 lo, %2, %1;\n"
+                    "cvt.rn.satfinite.e2m1x2.f32 hi, %4, %3;\n"
+                    "mov.b16 %0, {lo, hi};\n"
+                    "}\n"
+                    : "=h"(c16)
+                    : "f"(__fmul_rn(out[4 * h], r)), "f"(__fmul_rn(out[4 * h + 1], r)), "f"(__fmul_rn(out[4 * h + 2], r)),
+                      "f"(__fmul_rn(out[4 * h + 3], r)));
+                cw |= static_cast<uint32_t>(c16) << (16 * h);
+            }
+            if (live && have) {
+                uint8_t *cdst = codes + row * (K >> 1) + q * (POS / 2);
+                if (POS == 4) *reinterpret_cast<uint16_t *>(cdst) = static_cast<uint16_t>(cw);
+                else *reinterpret_cast<uint32_t *>(cdst) = cw;
+                if (y_out) {
+                    uint32_t yw[POS / 2];
+#pragma unroll
+                    for (int j = 0; j < POS / 2; ++j)
+                        yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
+                                (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
+                    if (POS == 4) reinterpret_cast<uint2 *>(y_out + row * K)[q] = make_uint2(yw[0], yw[1]);
+                    else reinterpret_cast<uint4 *>(y_out + row * K)[q] = make_uint4(yw[0], yw[1], yw[POS / 2 - 2], yw[POS / 2 - 1]);
+                }
+            }
+            // scale bytes: the first lane of each group holds its byte; four neighbouring groups sit LPG
+            // lanes apart (padding rows write zeros)
+            uint32_t word = sf8;
+            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, LPG) << 8;
+            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2 * LPG) << 16;
+            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3 * LPG) << 24;
+            if (!have || (q % LPG) != 0) continue;
+            const int g = q / LPG;
+            if (SF_LAYOUT == PQ_SF_TCGEN05) {
+                if ((g & 3) == 0) *reinterpret_cast<uint32_t *>(sf + pq::sf_tc_offset(row, g, gpr >> 2)) = word;
+            } else if (live) {
+                if ((gpr & 3) == 0) {
+                    if ((g & 3) == 0) *reinterpret_cast<uint32_t *>(sf + row * gpr + g) = word;
+                } else {
+                    sf[row * gpr + g] = static_cast<uint8_t>(sf8);
+                }
             }
         }
-        float amax = 0.0f;
-#pragma unroll
-        for (int j = 0; j < POS; ++j) amax = fmaxf(amax, fabsf(out[j]));
-#pragma unroll
-        for (int m = 1; m < LPG; m <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, m));
-        uint32_t sf8;
-        float d, r;
-        pq::nvfp4_scale(amax, ts, sf8, d, r);
-        uint32_t cw = 0;
-#pragma unroll
-        for (int h = 0; h < POS / 4; ++h) {
-            uint16_t c16;
-            asm("{\n"
-                ".reg .b8 lo, hi;\n"
-                "cvt.rn.satfinite.e2m1x2.f32 lo, %2, %1;\n"
-                "cvt.rn.satfinite.e2m1x2.f32 hi, %4, %3;\n"
-                "mov.b16 %0, {lo, hi};\n"
-                "}\n"
-                : "=h"(c16)
-                : "f"(__fmul_rn(out[4 * h], r)), "f"(__fmul_rn(out[4 * h + 1], r)), "f"(__fmul_rn(out[4 * h + 2], r)),
-                  "f"(__fmul_rn(out[4 * h + 3], r)));
-            cw |= static_cast<uint32_t>(c16) << (16 * h);
-        }
-        if (live && have) {
-            uint8_t *cdst = codes + row * (K >> 1) + q * (POS / 2);
-            if (POS == 4) *reinterpret_cast<uint16_t *>(cdst) = static_cast<uint16_t>(cw);
-            else *reinterpret_cast<uint32_t *>(cdst) = cw;
-            if (y_out) {
-                uint32_t yw[POS / 2];
-#pragma unroll
-                for (int j = 0; j < POS / 2; ++j)
-                    yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
-                            (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
-                if (POS == 4) reinterpret_cast<uint2 *>(y_out + row * K)[q] = make_uint2(yw[0], yw[1]);
-                else reinterpret_cast<uint4 *>(y_out + row * K)[q] = make_uint4(yw[0], yw[1], yw[POS / 2 - 2], yw[POS / 2 - 1]);
-            }
-        }
-        // scale bytes: the first lane of each group holds its byte; four neighbouring groups sit LPG
-        // lanes apart (padding rows write zeros)
-        uint32_t word = sf8;
-        word |= __shfl_down_sync(0xFFFFFFFFu, sf8, LPG) << 8;
-        word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2 * LPG) << 16;
-        word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3 * LPG) << 24;
-        if (!have || (q % LPG) != 0) continue;
-        const int g = q / LPG;
-        if (SF_LAYOUT == PQ_SF_TCGEN05) {
-            if ((g & 3) == 0) *reinterpret_cast<uint32_t *>(sf + pq::sf_tc_offset(row, g, gpr >> 2)) = word;
-        } else if (live) {
-            if ((gpr & 3) == 0) {
-                if ((g & 3) == 0) *reinterpret_cast<uint32_t *>(sf + row * gpr + g) = word;
-            } else {
-                sf[row * gpr + g] = static_cast<uint8_t>(sf8);
-            }
-        }
-    }
+    };
+    if (scaler.fast) walk(std::true_type{});
+    else walk(std::false_type{});
 }
 
 // ---- several rows per warp ----------------------------------------------------------------------
@@ -275,7 +280,7 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
     const int octs = K >> 3, gpr = K >> 4;
     pq::wait_for_prior_grid();
     pq::dependents_may_launch();
-    const float ts = __ldg(ts_ptr);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
     float inv[R], mu[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) inv[r] = 0.0f, mu[r] = 0.0f;
@@ -371,87 +376,91 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
     // the indices and parameters are fetched once, the scale is derived once per group and row
     constexpr int POS = 16;
     const bool any_live = nlive > 0;
-    for (int q0 = 32 * part; q0 < gpr; q0 += 32 * kSplit) {
-        const int q = q0 + lane;  // group
-        const bool have = q < gpr;
-        uint2 g[POS];
-        float w[POS], sh[POS];
+    auto walk = [&](auto fast) {
+        for (int q0 = 32 * part; q0 < gpr; q0 += 32 * kSplit) {
+            const int q = q0 + lane;  // group
+            const bool have = q < gpr;
+            uint2 g[POS];
+            float w[POS], sh[POS];
 #pragma unroll
-        for (int j = 0; j < POS; ++j) g[j] = make_uint2(0, 0), w[j] = 0.0f, sh[j] = 0.0f;
-        if (have && any_live) {
+            for (int j = 0; j < POS; ++j) g[j] = make_uint2(0, 0), w[j] = 0.0f, sh[j] = 0.0f;
+            if (have && any_live) {
 #pragma unroll
-            for (int h = 0; h < POS / 4; ++h) {
-                const int j0 = POS * q + 4 * h;
-                int4 idx = make_int4(j0, j0 + 1, j0 + 2, j0 + 3);
-                if (perm) idx = __ldg(reinterpret_cast<const int4 *>(perm) + (POS / 4) * q + h);
-                g[4 * h + 0] = channel_rows<R>(xs, idx.x), g[4 * h + 1] = channel_rows<R>(xs, idx.y);
-                g[4 * h + 2] = channel_rows<R>(xs, idx.z), g[4 * h + 3] = channel_rows<R>(xs, idx.w);
-                const float4 a4 = __ldg(reinterpret_cast<const float4 *>(a) + (POS / 4) * q + h);
-                w[4 * h + 0] = a4.x, w[4 * h + 1] = a4.y, w[4 * h + 2] = a4.z, w[4 * h + 3] = a4.w;
+                for (int h = 0; h < POS / 4; ++h) {
+                    const int j0 = POS * q + 4 * h;
+                    int4 idx = make_int4(j0, j0 + 1, j0 + 2, j0 + 3);
+                    if (perm) idx = __ldg(reinterpret_cast<const int4 *>(perm) + (POS / 4) * q + h);
+                    g[4 * h + 0] = channel_rows<R>(xs, idx.x), g[4 * h + 1] = channel_rows<R>(xs, idx.y);
+                    g[4 * h + 2] = channel_rows<R>(xs, idx.z), g[4 * h + 3] = channel_rows<R>(xs, idx.w);
+                    const float4 a4 = __ldg(reinterpret_cast<const float4 *>(a) + (POS / 4) * q + h);
+                    w[4 * h + 0] = a4.x, w[4 * h + 1] = a4.y, w[4 * h + 2] = a4.z, w[4 * h + 3] = a4.w;
+                    if (KIND == 1) {
+                        const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b) + (POS / 4) * q + h);
+                        sh[4 * h + 0] = b4.x, sh[4 * h + 1] = b4.y, sh[4 * h + 2] = b4.z, sh[4 * h + 3] = b4.w;
+                    }
+                }
                 if (KIND == 1) {
-                    const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b) + (POS / 4) * q + h);
-                    sh[4 * h + 0] = b4.x, sh[4 * h + 1] = b4.y, sh[4 * h + 2] = b4.z, sh[4 * h + 3] = b4.w;
+#pragma unroll
+                    for (int j = 0; j < POS; ++j) w[j] = __fadd_rn(1.0f, w[j]);
                 }
             }
-            if (KIND == 1) {
 #pragma unroll
-                for (int j = 0; j < POS; ++j) w[j] = __fadd_rn(1.0f, w[j]);
-            }
-        }
+            for (int r = 0; r < R; ++r) {
+                const int64_t row = row0 + r;
+                const bool live = r < nlive;  // rows past the end carry inv = mu = 0 and zeros in shared memory
+                float out[POS];
+                float amax = 0.0f;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int64_t row = row0 + r;
-            const bool live = r < nlive;  // rows past the end carry inv = mu = 0 and zeros in shared memory
-            float out[POS];
-            float amax = 0.0f;
-#pragma unroll
-            for (int j = 0; j < POS; ++j) {
-                out[j] = KIND == 0 ? __fmul_rn(__fmul_rn(row_value(g[j], r), inv[r]), w[j])
-                                   : __fmaf_rn(__fmul_rn(row_minus(g[j], r, mu[r]), inv[r]), w[j], sh[j]);
-                amax = fmaxf(amax, fabsf(out[j]));
-            }
-            if (!(live && have)) amax = 0.0f;  // nothing of such a row or group is stored but a zero scale byte
-            uint32_t sf8;
-            float d, rcp;
-            pq::nvfp4_scale(amax, ts, sf8, d, rcp);
-            if (live && have) {
-                float y[8];
-                uint2 cw;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) y[j] = __fmul_rn(out[j], rcp);
-                cw.x = pq::f32x8_to_e2m1(y);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) y[j] = __fmul_rn(out[8 + j], rcp);
-                cw.y = pq::f32x8_to_e2m1(y);
-                *reinterpret_cast<uint2 *>(codes + row * (K >> 1) + q * 8) = cw;
-                if (y_out) {
-                    uint32_t yw[POS / 2];
-#pragma unroll
-                    for (int j = 0; j < POS / 2; ++j)
-                        yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
-                                (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
-                    uint4 *ydst = reinterpret_cast<uint4 *>(y_out + row * K) + 2 * q;
-                    ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
-                    ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                for (int j = 0; j < POS; ++j) {
+                    out[j] = KIND == 0 ? __fmul_rn(__fmul_rn(row_value(g[j], r), inv[r]), w[j])
+                                       : __fmaf_rn(__fmul_rn(row_minus(g[j], r, mu[r]), inv[r]), w[j], sh[j]);
+                    amax = fmaxf(amax, fabsf(out[j]));
                 }
-            }
-            // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
-            uint32_t word = sf8;
-            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 1) << 8;
-            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2) << 16;
-            word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3) << 24;
-            if (!have || row >= rows_pad) continue;
-            if (SF_LAYOUT == PQ_SF_TCGEN05) {
-                if ((q & 3) == 0) *reinterpret_cast<uint32_t *>(sf + pq::sf_tc_offset(row, q, gpr >> 2)) = word;
-            } else if (live) {
-                if ((gpr & 3) == 0) {
-                    if ((q & 3) == 0) *reinterpret_cast<uint32_t *>(sf + row * gpr + q) = word;
-                } else {
-                    sf[row * gpr + q] = static_cast<uint8_t>(sf8);
+                if (!(live && have)) amax = 0.0f;  // nothing of such a row or group is stored but a zero scale byte
+                uint32_t sf8;
+                float rcp;
+                pq::nvfp4_scale<decltype(fast)::value>(amax, scaler, sf8, rcp);
+                if (live && have) {
+                    float y[8];
+                    uint2 cw;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) y[j] = __fmul_rn(out[j], rcp);
+                    cw.x = pq::f32x8_to_e2m1(y);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) y[j] = __fmul_rn(out[8 + j], rcp);
+                    cw.y = pq::f32x8_to_e2m1(y);
+                    *reinterpret_cast<uint2 *>(codes + row * (K >> 1) + q * 8) = cw;
+                    if (y_out) {
+                        uint32_t yw[POS / 2];
+#pragma unroll
+                        for (int j = 0; j < POS / 2; ++j)
+                            yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
+                                    (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
+                        uint4 *ydst = reinterpret_cast<uint4 *>(y_out + row * K) + 2 * q;
+                        ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                        ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                    }
+                }
+                // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
+                uint32_t word = sf8;
+                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 1) << 8;
+                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2) << 16;
+                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3) << 24;
+                if (!have || row >= rows_pad) continue;
+                if (SF_LAYOUT == PQ_SF_TCGEN05) {
+                    if ((q & 3) == 0) *reinterpret_cast<uint32_t *>(sf + pq::sf_tc_offset(row, q, gpr >> 2)) = word;
+                } else if (live) {
+                    if ((gpr & 3) == 0) {
+                        if ((q & 3) == 0) *reinterpret_cast<uint32_t *>(sf + row * gpr + q) = word;
+                    } else {
+                        sf[row * gpr + q] = static_cast<uint8_t>(sf8);
+                    }
                 }
             }
         }
-    }
+    };
+    if (scaler.fast) walk(std::true_type{});
+    else walk(std::false_type{});
 }
 
 // ---- four rows per block ------------------------------------------------------------------------
@@ -487,7 +496,7 @@ norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t row
     // perm_select given: perm is a table of candidate orders [., K] and {best, accept} on the device name the
     // row best - 1, or the original order (the offline weight quantizer, whose decision never visits the host)
     if (perm_select) perm = perm_select[1] ? perm + static_cast<int64_t>(perm_select[0] - 1) * K : nullptr;
-    const float ts = __ldg(ts_ptr);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
     const uint16_t *src = H + row0 * ld;
 
     if (KIND == 2) {  // no statistics: straight into the interleaved image
@@ -546,87 +555,91 @@ norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t row
 
     // ---- output order: one group (16 consecutive positions) per lane, for the four rows
     const uint2 *quad2 = reinterpret_cast<const uint2 *>(quad_s);
+    auto walk = [&](auto fast) {
 #pragma unroll 1
-    for (int it = 0; it < ITER; ++it) {
-        const int q = tid + it * T;
-        const bool have = q < gpr;
-        const int64_t sf_ofs = SF_LAYOUT == PQ_SF_TCGEN05 ? pq::sf_tc_offset(row0, q, gpr >> 2) : row0 * gpr + q;
-        uint8_t *const out_codes = codes + row0 * (K >> 1) + q * 8;
-        uint2 g[16];
-        uint64_t w2[8], sh2[8];  // parameters of neighbouring positions, packed
+        for (int it = 0; it < ITER; ++it) {
+            const int q = tid + it * T;
+            const bool have = q < gpr;
+            const int64_t sf_ofs = SF_LAYOUT == PQ_SF_TCGEN05 ? pq::sf_tc_offset(row0, q, gpr >> 2) : row0 * gpr + q;
+            uint8_t *const out_codes = codes + row0 * (K >> 1) + q * 8;
+            uint2 g[16];
+            uint64_t w2[8], sh2[8];  // parameters of neighbouring positions, packed
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int j0 = have ? 16 * q + 4 * h : 0;
-            int4 idx = make_int4(j0, j0 + 1, j0 + 2, j0 + 3);
-            if (perm) idx = __ldg(reinterpret_cast<const int4 *>(perm + j0));
-            g[4 * h + 0] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.x))];
-            g[4 * h + 1] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.y))];
-            g[4 * h + 2] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.z))];
-            g[4 * h + 3] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.w))];
-            if (KIND != 2) {
-                float4 a4 = __ldg(reinterpret_cast<const float4 *>(a + j0));
-                if (KIND == 1) {
-                    a4 = make_float4(__fadd_rn(1.0f, a4.x), __fadd_rn(1.0f, a4.y), __fadd_rn(1.0f, a4.z), __fadd_rn(1.0f, a4.w));
-                    const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b + j0));
-                    sh2[2 * h] = pq::pack2(b4.x, b4.y), sh2[2 * h + 1] = pq::pack2(b4.z, b4.w);
-                }
-                w2[2 * h] = pq::pack2(a4.x, a4.y), w2[2 * h + 1] = pq::pack2(a4.z, a4.w);
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int64_t row = row0 + r;
-            const bool live = r < nlive && have;
-            uint64_t y2[8];
-            float amax = 0.0f;
-            const uint64_t inv2 = KIND == 2 ? 0 : pq::pack2(stat_s[r], stat_s[r]);
-            const float mu = stat_s[4 + r];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const uint32_t c0 = r < 2 ? g[2 * j].x : g[2 * j].y, c1 = r < 2 ? g[2 * j + 1].x : g[2 * j + 1].y;
-                uint64_t v = KIND == 1 ? ((r & 1) ? pq::pack2(pq::bf16_minus<1>(c0, mu), pq::bf16_minus<1>(c1, mu))
-                                                  : pq::pack2(pq::bf16_minus<0>(c0, mu), pq::bf16_minus<0>(c1, mu)))
-                             : (r & 1) ? pq::pack2(__uint_as_float(c0 & 0xFFFF0000u), __uint_as_float(c1 & 0xFFFF0000u))
-                                     : pq::pack2(__uint_as_float(c0 << 16), __uint_as_float(c1 << 16));
-                if (KIND == 0) v = pq::mul2(pq::mul2(v, inv2), w2[j]);
-                if (KIND == 1) v = pq::fma2(pq::mul2(v, inv2), w2[j], sh2[j]);
-                y2[j] = v;
-                float lo, hi;
-                pq::unpack2(v, lo, hi);
-                amax = fmaxf(fmaxf(amax, fabsf(lo)), fabsf(hi));
-            }
-            if (!live) amax = 0.0f;  // nothing of such a row or group is stored but a zero scale byte
-            uint32_t sf8;
-            float d, rcp;
-            pq::nvfp4_scale(amax, ts, sf8, d, rcp);
-            if (live) {
-                if (y_out) {
-                    uint32_t yw[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        float lo, hi;
-                        pq::unpack2(y2[j], lo, hi);
-                        yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
-                                (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(hi))) << 16);
+            for (int h = 0; h < 4; ++h) {
+                const int j0 = have ? 16 * q + 4 * h : 0;
+                int4 idx = make_int4(j0, j0 + 1, j0 + 2, j0 + 3);
+                if (perm) idx = __ldg(reinterpret_cast<const int4 *>(perm + j0));
+                g[4 * h + 0] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.x))];
+                g[4 * h + 1] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.y))];
+                g[4 * h + 2] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.z))];
+                g[4 * h + 3] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.w))];
+                if (KIND != 2) {
+                    float4 a4 = __ldg(reinterpret_cast<const float4 *>(a + j0));
+                    if (KIND == 1) {
+                        a4 = make_float4(__fadd_rn(1.0f, a4.x), __fadd_rn(1.0f, a4.y), __fadd_rn(1.0f, a4.z), __fadd_rn(1.0f, a4.w));
+                        const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b + j0));
+                        sh2[2 * h] = pq::pack2(b4.x, b4.y), sh2[2 * h + 1] = pq::pack2(b4.z, b4.w);
                     }
-                    uint4 *ydst = reinterpret_cast<uint4 *>(y_out + row * K) + 2 * q;
-                    ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
-                    ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                    w2[2 * h] = pq::pack2(a4.x, a4.y), w2[2 * h + 1] = pq::pack2(a4.z, a4.w);
                 }
-                const uint64_t rcp2 = pq::pack2(rcp, rcp);
-                float y[16];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) pq::unpack2(pq::mul2(y2[j], rcp2), y[2 * j], y[2 * j + 1]);
-                const float ylo[8] = {y[0], y[1], y[2], y[3], y[4], y[5], y[6], y[7]};
-                const float yhi[8] = {y[8], y[9], y[10], y[11], y[12], y[13], y[14], y[15]};
-                *reinterpret_cast<uint2 *>(out_codes + r * (K >> 1)) = make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
             }
-            // one scale byte per lane; the lanes of a warp write runs of four adjacent bytes (padding rows write zeros).
-            // row0 is a multiple of four: the rows' bytes lie 16 apart in the tensor-core layout
-            if (have && (SF_LAYOUT == PQ_SF_TCGEN05 ? row < rows_pad : live))
-                sf[SF_LAYOUT == PQ_SF_TCGEN05 ? sf_ofs + 16 * r : sf_ofs + r * gpr] = static_cast<uint8_t>(sf8);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int64_t row = row0 + r;
+                const bool live = r < nlive && have;
+                uint64_t y2[8];
+                float amax = 0.0f;
+                const uint64_t inv2 = KIND == 2 ? 0 : pq::pack2(stat_s[r], stat_s[r]);
+                const float mu = stat_s[4 + r];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const uint32_t c0 = r < 2 ? g[2 * j].x : g[2 * j].y, c1 = r < 2 ? g[2 * j + 1].x : g[2 * j + 1].y;
+                    uint64_t v = KIND == 1 ? ((r & 1) ? pq::pack2(pq::bf16_minus<1>(c0, mu), pq::bf16_minus<1>(c1, mu))
+                                                      : pq::pack2(pq::bf16_minus<0>(c0, mu), pq::bf16_minus<0>(c1, mu)))
+                                 : (r & 1) ? pq::pack2(__uint_as_float(c0 & 0xFFFF0000u), __uint_as_float(c1 & 0xFFFF0000u))
+                                         : pq::pack2(__uint_as_float(c0 << 16), __uint_as_float(c1 << 16));
+                    if (KIND == 0) v = pq::mul2(pq::mul2(v, inv2), w2[j]);
+                    if (KIND == 1) v = pq::fma2(pq::mul2(v, inv2), w2[j], sh2[j]);
+                    y2[j] = v;
+                    float lo, hi;
+                    pq::unpack2(v, lo, hi);
+                    amax = fmaxf(fmaxf(amax, fabsf(lo)), fabsf(hi));
+                }
+                if (!live) amax = 0.0f;  // nothing of such a row or group is stored but a zero scale byte
+                uint32_t sf8;
+                float rcp;
+                pq::nvfp4_scale<decltype(fast)::value>(amax, scaler, sf8, rcp);
+                if (live) {
+                    if (y_out) {
+                        uint32_t yw[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            float lo, hi;
+                            pq::unpack2(y2[j], lo, hi);
+                            yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
+                                    (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(hi))) << 16);
+                        }
+                        uint4 *ydst = reinterpret_cast<uint4 *>(y_out + row * K) + 2 * q;
+                        ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                        ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+                    }
+                    const uint64_t rcp2 = pq::pack2(rcp, rcp);
+                    float y[16];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) pq::unpack2(pq::mul2(y2[j], rcp2), y[2 * j], y[2 * j + 1]);
+                    const float ylo[8] = {y[0], y[1], y[2], y[3], y[4], y[5], y[6], y[7]};
+                    const float yhi[8] = {y[8], y[9], y[10], y[11], y[12], y[13], y[14], y[15]};
+                    *reinterpret_cast<uint2 *>(out_codes + r * (K >> 1)) = make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
+                }
+                // one scale byte per lane; the lanes of a warp write runs of four adjacent bytes (padding rows write zeros).
+                // row0 is a multiple of four: the rows' bytes lie 16 apart in the tensor-core layout
+                if (have && (SF_LAYOUT == PQ_SF_TCGEN05 ? row < rows_pad : live))
+                    sf[SF_LAYOUT == PQ_SF_TCGEN05 ? sf_ofs + 16 * r : sf_ofs + r * gpr] = static_cast<uint8_t>(sf8);
+            }
         }
-    }
+    };
+    if (scaler.fast) walk(std::true_type{});
+    else walk(std::false_type{});
 }
 
 // Rows the four-rows-per-block kernel takes: up to two groups per lane of at most 512 threads, 128 KB of image.
@@ -673,7 +686,7 @@ norm_quant_ordered_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
     if (row >= rows_pad) return;  // whole warps only
     const bool live = row < rows;
     const int octs = K >> 3, gpr = K >> 4;
-    const float ts = __ldg(ts_ptr);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
     uint4 raw[NOCT];
 #pragma unroll
     for (int u = 0; u < NOCT; ++u) {
@@ -715,52 +728,56 @@ norm_quant_ordered_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
     }
     if (!live) inv = 0.0f, mu = 0.0f;
     // normalize, quantize, store: octet o = lane + 32 u, group o / 2 (its other octet is in lane ^ 1)
+    auto walk = [&](auto fast) {
 #pragma unroll
-    for (int u = 0; u < NOCT; ++u) {
-        const int o = lane + 32 * u;
-        if (32 * u >= octs) break;  // uniform over the warp
-        const bool have = o < octs;
-        float out[8];
+        for (int u = 0; u < NOCT; ++u) {
+            const int o = lane + 32 * u;
+            if (32 * u >= octs) break;  // uniform over the warp
+            const bool have = o < octs;
+            float out[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) out[e] = 0.0f;
-        if (live && have) {
-            float x[8];
-            pq::unpack8(raw[u], x);
-            const float4 a0 = __ldg(reinterpret_cast<const float4 *>(a) + 2 * o), a1 = __ldg(reinterpret_cast<const float4 *>(a) + 2 * o + 1);
-            const float w[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            if (KIND == 0) {
+            for (int e = 0; e < 8; ++e) out[e] = 0.0f;
+            if (live && have) {
+                float x[8];
+                pq::unpack8(raw[u], x);
+                const float4 a0 = __ldg(reinterpret_cast<const float4 *>(a) + 2 * o), a1 = __ldg(reinterpret_cast<const float4 *>(a) + 2 * o + 1);
+                const float w[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+                if (KIND == 0) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) out[e] = __fmul_rn(__fmul_rn(x[e], inv), w[e]);
-            } else {
-                const float4 b0 = __ldg(reinterpret_cast<const float4 *>(b) + 2 * o), b1 = __ldg(reinterpret_cast<const float4 *>(b) + 2 * o + 1);
-                const float sh[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                    for (int e = 0; e < 8; ++e) out[e] = __fmul_rn(__fmul_rn(x[e], inv), w[e]);
+                } else {
+                    const float4 b0 = __ldg(reinterpret_cast<const float4 *>(b) + 2 * o), b1 = __ldg(reinterpret_cast<const float4 *>(b) + 2 * o + 1);
+                    const float sh[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    out[e] = __fmaf_rn(__fmul_rn(__fsub_rn(x[e], mu), inv), __fadd_rn(1.0f, w[e]), sh[e]);
+                    for (int e = 0; e < 8; ++e)
+                        out[e] = __fmaf_rn(__fmul_rn(__fsub_rn(x[e], mu), inv), __fadd_rn(1.0f, w[e]), sh[e]);
+                }
             }
-        }
-        float amax = pq::absmax8(out);
-        amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, 1));
-        uint32_t sf8;
-        float d, rcp;
-        pq::nvfp4_scale(amax, ts, sf8, d, rcp);
-        if (live && have) {
-            *reinterpret_cast<uint32_t *>(codes + row * (K >> 1) + o * 4) = pq::nvfp4_codes(out, rcp);
-            if (y_out) {
-                uint32_t yw[4];
+            float amax = pq::absmax8(out);
+            amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, 1));
+            uint32_t sf8;
+            float rcp;
+            pq::nvfp4_scale<decltype(fast)::value>(amax, scaler, sf8, rcp);
+            if (live && have) {
+                *reinterpret_cast<uint32_t *>(codes + row * (K >> 1) + o * 4) = pq::nvfp4_codes(out, rcp);
+                if (y_out) {
+                    uint32_t yw[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
-                            (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
-                reinterpret_cast<uint4 *>(y_out + row * K)[o] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                    for (int j = 0; j < 4; ++j)
+                        yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
+                                (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
+                    reinterpret_cast<uint4 *>(y_out + row * K)[o] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                }
             }
+            // the scale byte of a group: written by the lane that holds its first octet (padding rows write zeros)
+            if (!have || (o & 1)) continue;
+            const int g = o >> 1;
+            if (SF_LAYOUT == PQ_SF_TCGEN05) sf[pq::sf_tc_offset(row, g, gpr >> 2)] = static_cast<uint8_t>(sf8);
+            else if (live) sf[row * gpr + g] = static_cast<uint8_t>(sf8);
         }
-        // the scale byte of a group: written by the lane that holds its first octet (padding rows write zeros)
-        if (!have || (o & 1)) continue;
-        const int g = o >> 1;
-        if (SF_LAYOUT == PQ_SF_TCGEN05) sf[pq::sf_tc_offset(row, g, gpr >> 2)] = static_cast<uint8_t>(sf8);
-        else if (live) sf[row * gpr + g] = static_cast<uint8_t>(sf8);
-    }
+    };
+    if (scaler.fast) walk(std::true_type{});
+    else walk(std::false_type{});
 }
 
 template <int KIND, int SF_LAYOUT>

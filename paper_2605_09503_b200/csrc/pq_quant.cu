@@ -11,6 +11,8 @@
 // with coalesced 16-byte loads and gather from there, so global memory is still read once.  For
 // NVFP4 the gather runs in the fused producer's kernel (pq_norm.cu, four rows per block sharing indices
 // and gathers) with its normalization compiled out.
+#include <type_traits>
+
 #include "pq_common.cuh"
 
 namespace {
@@ -71,8 +73,6 @@ quant_nvfp4_kernel(const uint16_t *__restrict__ X, int64_t rows, int64_t rows_pa
     // it waits for this grid to complete before reading the results.
     pq::wait_for_prior_grid();
     pq::dependents_may_launch();
-    const float ts = __ldg(ts_ptr);
-
     uint4 lo[kActRows], hi[kActRows];
 #pragma unroll
     for (int i = 0; i < kActRows; ++i) {
@@ -80,28 +80,33 @@ quant_nvfp4_kernel(const uint16_t *__restrict__ X, int64_t rows, int64_t rows_pa
         lo[i] = make_uint4(0, 0, 0, 0), hi[i] = lo[i];
         if (row < rows && g < gpr) load_group<WIDE>(X + row * ld + static_cast<int64_t>(g) * 16, lo[i], hi[i]);
     }
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
+    auto quantize = [&](auto fast) {
 #pragma unroll
-    for (int i = 0; i < kActRows; ++i) {
-        const int64_t row = row0 + i * kActTileRows;
-        const bool in_range = row < rows_pad && g < gpr, live = row < rows && g < gpr;
-        // group absmax on the bf16 pairs (a maximum of magnitudes selects one of its inputs: exact)
-        const uint32_t m = 0x7FFF7FFFu;
-        const uint32_t mx = pq::max_bf16x2(pq::max_bf16x2(pq::max_bf16x2(lo[i].x & m, lo[i].y & m), pq::max_bf16x2(lo[i].z & m, lo[i].w & m)),
-                                           pq::max_bf16x2(pq::max_bf16x2(hi[i].x & m, hi[i].y & m), pq::max_bf16x2(hi[i].z & m, hi[i].w & m)));
-        const float amax = fmaxf(__uint_as_float(mx << 16), __uint_as_float(mx & 0xFFFF0000u));
-        uint32_t sf8;
-        float d, r;
-        pq::nvfp4_scale(amax, ts, sf8, d, r);
-        const uint32_t c0 = pq::nvfp4_codes_packed(lo[i], r), c1 = pq::nvfp4_codes_packed(hi[i], r);
-        // an ordinary store: the GEMM reads the codes next, they should stay in L2 (a streaming store measured
-        // 0.2 us more on quantize + GEMM)
-        if (live) *reinterpret_cast<uint2 *>(codes + row * (K >> 1) + static_cast<int64_t>(g) * 8) = make_uint2(c0, c1);
-        // one scale byte per thread: the lanes of a warp write runs of four adjacent bytes (adjacent in both
-        // layouts) in one instruction; padding rows of the tensor-core layout get zeros
-        if (!in_range) continue;
-        if (SF_LAYOUT == PQ_SF_TCGEN05) sf[pq::sf_tc_offset(row, g, gpr >> 2)] = static_cast<uint8_t>(sf8);
-        else if (live) sf[row * gpr + g] = static_cast<uint8_t>(sf8);
-    }
+        for (int i = 0; i < kActRows; ++i) {
+            const int64_t row = row0 + i * kActTileRows;
+            const bool in_range = row < rows_pad && g < gpr, live = row < rows && g < gpr;
+            // group absmax on the bf16 pairs (a maximum of magnitudes selects one of its inputs: exact)
+            const uint32_t m = 0x7FFF7FFFu;
+            const uint32_t mx = pq::max_bf16x2(pq::max_bf16x2(pq::max_bf16x2(lo[i].x & m, lo[i].y & m), pq::max_bf16x2(lo[i].z & m, lo[i].w & m)),
+                                               pq::max_bf16x2(pq::max_bf16x2(hi[i].x & m, hi[i].y & m), pq::max_bf16x2(hi[i].z & m, hi[i].w & m)));
+            const float amax = fmaxf(__uint_as_float(mx << 16), __uint_as_float(mx & 0xFFFF0000u));
+            uint32_t sf8;
+            float r;
+            pq::nvfp4_scale<decltype(fast)::value>(amax, scaler, sf8, r);
+            const uint32_t c0 = pq::nvfp4_codes_packed(lo[i], r), c1 = pq::nvfp4_codes_packed(hi[i], r);
+            // an ordinary store: the GEMM reads the codes next, they should stay in L2 (a streaming store measured
+            // 0.2 us more on quantize + GEMM)
+            if (live) *reinterpret_cast<uint2 *>(codes + row * (K >> 1) + static_cast<int64_t>(g) * 8) = make_uint2(c0, c1);
+            // one scale byte per thread: the lanes of a warp write runs of four adjacent bytes (adjacent in both
+            // layouts) in one instruction; padding rows of the tensor-core layout get zeros
+            if (!in_range) continue;
+            if (SF_LAYOUT == PQ_SF_TCGEN05) sf[pq::sf_tc_offset(row, g, gpr >> 2)] = static_cast<uint8_t>(sf8);
+            else if (live) sf[row * gpr + g] = static_cast<uint8_t>(sf8);
+        }
+    };
+    if (scaler.fast) quantize(std::true_type{});
+    else quantize(std::false_type{});
 }
 
 // ---------------------------------------------------------------- weights

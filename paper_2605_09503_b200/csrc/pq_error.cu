@@ -11,10 +11,10 @@
 //     eight rows at a time and walks them in order; a block covers the eight chunks of a slab.  The pass streams the tensor once from HBM;
 //     its cost per element is arithmetic (about ten instructions), so it sits between the HBM and
 //     the ALU roof.
-//   candidate orders: one block per (chunk, order); the chunk's rows are staged in shared memory four
-//     at a time, interleaved per channel, and a thread gathers the 16 channels of its run for four rows
-//     with 64-bit loads, then runs the original-order kernel's error routine on them; the tensor is
-//     fetched from HBM once per chunk and served from L2 to the other orders' blocks.
+//   candidate orders: persistent blocks of thread groups; a group stages a chunk's rows in shared memory four at a time,
+//     interleaved per channel, for all orders of its share of the (chunk, order) pairs, and a lane gathers the 16 channels
+//     of its run for four rows with 64-bit loads, two rows side by side in packed registers; the tensor is fetched from HBM
+//     about once.
 #include <type_traits>
 
 #include "pq_common.cuh"
@@ -334,7 +334,9 @@ struct GatherParams {
     const int32_t *perms;      // [P - identity, K]
     int opb;                   // orders per block (blockIdx.y picks the subset)
     int groups, group_threads;
-    uint32_t base[2], rem[2];  // pairs / shares and its remainder: subsets of opb orders, the last subset
+    uint32_t base[2], rem[2];  // pairs of the first `split` chunks / shares and its remainder: subsets of opb orders, the last
+    uint32_t split;
+    int full;                  // whole chunks per share behind them
     int chunks;                // eight per slab; the chunks of a last slab that hold no rows may be left out
     float Qf;
     float *part;               // [chunks, P, K/g]
@@ -400,14 +402,22 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     const uint4 *slot4 = reinterpret_cast<const uint4 *>(slot_s);
     const int64_t Kg = runs / TEAM16;
 
-    // The (chunk, order) pairs of this block row, chunk by chunk, in equal shares: a group that has work for a few
-    // chunks only would otherwise wait for the one that has a whole chunk more.
-    const uint32_t share = blockIdx.x * p.groups + grp, base = p.base[o0 + no == p.P], rem = p.rem[o0 + no == p.P];
+    // An equal part of the (chunk, order) pairs of the first p.split chunks, then p.full whole chunks.  Without the first
+    // part a group that has work for a few chunks only would wait for the one that has a whole chunk more; without the
+    // second a group would stage one more chunk of which it uses some orders (eight batches of 4608 x 3072 and a
+    // 9216 x 3072 weight: 535 us a calibration all in pairs, 518 like this).
+    const uint32_t shares = gridDim.x * p.groups, share = blockIdx.x * p.groups + grp;
+    const uint32_t base = p.base[o0 + no == p.P], rem = p.rem[o0 + no == p.P];
     const uint32_t first = share * base + min(share, rem);
-    int pairs = static_cast<int>(base + (share < rem));
-    uint32_t chunk = first / static_cast<uint32_t>(no);
+    int pairs = static_cast<int>(base + (share < rem)), full = p.full * no;
+    uint32_t chunk = first / static_cast<uint32_t>(no), step = 1;
     int ob = static_cast<int>(first - chunk * no);
-    for (int oe; pairs > 0; pairs -= oe - ob, ob = 0, ++chunk) {
+    for (int oe;; pairs -= oe - ob, ob = 0, chunk += step) {
+        if (pairs == 0) {
+            if (full == 0) break;
+            pairs = full, full = 0, ob = 0;
+            chunk = p.split + share, step = shares;
+        }
         oe = min(no, ob + pairs);
         const int slab = static_cast<int>(chunk / kSlabChunks), t = pq::tensor_of_slab(p.list, slab);
         const int64_t r0 = static_cast<int64_t>(slab - p.list.slab0[t]) * PQ_SLAB_ROWS + chunk % kSlabChunks * PQ_CHUNK_ROWS;
@@ -523,9 +533,11 @@ pq_status launch_gather(GatherParams &p, int64_t K, int P, float Qf, float *part
     const int64_t subsets = pq_ceil_div(P, cfg.opb), share = sms / subsets > 0 ? sms / subsets : 1;
     const int64_t want = pq_ceil_div(static_cast<int64_t>(p.chunks) * cfg.opb, cfg.groups);
     const int64_t blocks = want < share ? want : share;
+    const int64_t shares = blocks * cfg.groups;
+    p.full = static_cast<int>(p.chunks / shares), p.split = static_cast<uint32_t>(p.chunks % shares);
     for (int last = 0; last < 2; ++last) {
         const int64_t orders = last ? P - (subsets - 1) * cfg.opb : cfg.opb;
-        const int64_t pairs = p.chunks * orders, shares = blocks * cfg.groups;
+        const int64_t pairs = p.split * orders;
         p.base[last] = static_cast<uint32_t>(pairs / shares), p.rem[last] = static_cast<uint32_t>(pairs % shares);
     }
     const size_t smem = gather_smem_bytes(K, cfg.opb, cfg.groups, sides);

@@ -11,6 +11,9 @@
 // then one multiplication by fl(1 / sqrt(K)).  Within one stride the butterflies are independent, so how
 // they are spread over threads does not change a bit of the result.
 //
+// Four kernels.  Widths of 768, 1024, 1536, 2048, 3072, 4096, 6144 and 12288 have rows that divide evenly over the lanes of
+// one, two or four warps, which then carry a row through all phases by themselves (second half of this file).
+// Every other width goes through the kernel described here.
 // Work distribution.  A thread block keeps up to 8 rows as K fp32 values each in shared memory and walks
 // over batches of rows (persistent grid):
 //   phase 1  a thread takes one octet position of one row: m 16-byte loads (the same octet of every
@@ -371,14 +374,42 @@ constexpr int kRowWarps = 8;            // per block; two blocks per SM at 128 r
 constexpr int kRowImage = 3072;         // fp32 values per warp
 
 template <int N>
+__device__ __forceinline__ int row_octet(int a, int b) {  // where octet b of segment a lies inside its row's image
+    return (a << N) + ((b ^ ((N > 8 ? b >> 3 : a) & 3)) << 3);
+}
+template <int N>
 __device__ __forceinline__ int row_image_index(int channel) {  // of a channel inside its row's image
-    constexpr int SEG = 1 << N;
-    const int a = channel >> N, b = (channel & (SEG - 1)) >> 3, e = channel & 7;
-    return (a << N) + ((b ^ (a & 3)) << 3) + (e ^ (((b >> 2) & 1) << 2));
+    const int a = channel >> N, b = (channel & ((1 << N) - 1)) >> 3, e = channel & 7;
+    return row_octet<N>(a, b) + (e ^ (((b >> 2) & 1) << 2));
 }
 
-// 2^LOG values of one column (of WIDTH neighbouring channels: 1 or 2) at the octet stride, in place.
-template <int LOG, typename T>
+// The butterflies of NV values (of one channel, or of two neighbouring channels) in ascending stride.
+template <int NV, typename T>
+__device__ __forceinline__ void column_butterflies(T (&v)[NV]) {
+#pragma unroll
+    for (int l = 1; l < NV; l <<= 1) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+            if (j & l) continue;
+            const T p = v[j], q = v[j | l];
+            if constexpr (sizeof(T) == 8) {
+                v[j] = add2(p, q);
+                v[j | l] = sub2(p, q);
+            } else {
+                v[j] = __fadd_rn(p, q);
+                v[j | l] = __fsub_rn(p, q);
+            }
+        }
+    }
+}
+template <typename T>
+__device__ __forceinline__ T column_scaled(T v, float scale) {
+    if constexpr (sizeof(T) == 8) return mul2(v, pack2(scale, scale));
+    else return __fmul_rn(v, scale);
+}
+
+// 2^LOG values of one column (of one channel, or of two neighbouring channels) at the octet stride, in place; LAST: and the scaling.
+template <int LOG, typename T, bool LAST = true>
 __device__ __forceinline__ void column_pass(float *image, int a_base, int s, int e, float scale) {
     constexpr int NV = 1 << LOG;
     T *slot[8];
@@ -389,26 +420,9 @@ __device__ __forceinline__ void column_pass(float *image, int a_base, int s, int
     T v[NV];
 #pragma unroll
     for (int b = 0; b < NV; ++b) v[b] = slot[b & 7][(b >> 3) * kStep];
+    column_butterflies(v);
 #pragma unroll
-    for (int l = 0; l < LOG; ++l) {
-#pragma unroll
-        for (int j = 0; j < NV; ++j) {
-            if ((j >> l) & 1) continue;
-            const T p = v[j], q = v[j | (1 << l)];
-            if constexpr (sizeof(T) == 8) {
-                v[j] = add2(p, q);
-                v[j | (1 << l)] = sub2(p, q);
-            } else {
-                v[j] = __fadd_rn(p, q);
-                v[j | (1 << l)] = __fsub_rn(p, q);
-            }
-        }
-    }
-#pragma unroll
-    for (int b = 0; b < NV; ++b) {
-        if constexpr (sizeof(T) == 8) slot[b & 7][(b >> 3) * kStep] = mul2(v[b], pack2(scale, scale));
-        else slot[b & 7][(b >> 3) * kStep] = __fmul_rn(v[b], scale);
-    }
+    for (int b = 0; b < NV; ++b) slot[b & 7][(b >> 3) * kStep] = LAST ? column_scaled(v[b], scale) : v[b];
 }
 
 // Column a' of the order-12 combination for one half of an octet (two channel pairs) and strides 1, 2.  The first half
@@ -433,7 +447,8 @@ __device__ __forceinline__ void row_column_12(const uint64_t (&in)[12][2], float
     for (int e = 0; e < 2; ++e) v[e] = butterfly_in_pair(v[e]);
     const uint64_t c0 = add2(v[0], v[1]), c1 = sub2(v[0], v[1]);
     const int half = (b >> 2) & 1;
-    ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(row_s + (AP << N) + ((b ^ (AP & 3)) << 3));
+    // row_octet<N>(AP, b) written out: through the call the warp-per-row kernel spilled more (23.8 against 23.1 us)
+    ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(row_s + (AP << N) + ((b ^ (N > 8 ? (b >> 3) & 3 : AP & 3)) << 3));
     if (HALF == 0) {
         dst[half] = make_ulonglong2(c0, c1);
     } else {
@@ -454,9 +469,85 @@ __device__ __forceinline__ void row_columns_12(std::integer_sequence<int, APs...
     (row_column_12<N, HALF, APs>(in, row_s, b), ...);
 }
 
+// The strides above a window of eight octets (segments of more than 256 channels): 2^LOG values, eight octets apart.
+template <int LOG>
+__device__ __forceinline__ void high_column_pass(float *segment, int k, int e, float scale) {
+    constexpr int NV = 1 << LOG;
+    uint64_t *slot[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        slot[j] = reinterpret_cast<uint64_t *>(segment + ((k ^ j) << 3) + (e ^ ((k >> 2) << 2)));
+    uint64_t v[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] = slot[j & 3][j * 32];
+    column_butterflies(v);
+#pragma unroll
+    for (int j = 0; j < NV; ++j) slot[j & 3][j * 32] = column_scaled(v[j], scale);
+}
+
+// Phase 3 of a team of NT threads that holds ROWS transformed rows: one output group per lane.
+template <int SF_LAYOUT, int K, int ROWS, int NT, bool FAST>
+__device__ __forceinline__ void rows_read_out(const HadParams &p, const pq::Nvfp4Scaler &scaler, const float *image,
+                                              const uint4 *offset4, int64_t row0, int tid) {
+    constexpr int GPR = K / 16;
+#pragma unroll 1
+    for (int i = tid; i < ROWS * GPR; i += NT) {
+        const int r = i / GPR, g = i - r * GPR;
+        const int64_t row = row0 + r;
+        const bool live = row < p.rows;
+        float out[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) out[j] = 0.0f;
+        if (live) {
+            const uint4 i0 = offset4[g], i1 = offset4[GPR + g];
+            const uint32_t iw[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
+            const char *row_b = reinterpret_cast<const char *>(image + r * K);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                out[2 * j] = *reinterpret_cast<const float *>(row_b + (iw[j] & 0xFFFFu));
+                out[2 * j + 1] = *reinterpret_cast<const float *>(row_b + (iw[j] >> 16));
+            }
+            if (p.y_out) {
+                uint32_t yw[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
+                            (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
+                uint4 *ydst = reinterpret_cast<uint4 *>(p.y_out + row * K) + 2 * g;
+                ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
+                ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
+            }
+        }
+        if (!p.codes) continue;
+        float amax = 0.0f, rcp;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(out[j]));
+        uint32_t sf8;
+        pq::nvfp4_scale<FAST>(amax, scaler, sf8, rcp);
+        if (live) {
+            const uint64_t rcp2 = pack2(rcp, rcp);
+            float ylo[8], yhi[8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                unpack2(mul2(pack2(out[2 * j], out[2 * j + 1]), rcp2), ylo[2 * j], ylo[2 * j + 1]);
+                unpack2(mul2(pack2(out[8 + 2 * j], out[9 + 2 * j]), rcp2), yhi[2 * j], yhi[2 * j + 1]);
+            }
+            *reinterpret_cast<uint2 *>(p.codes + row * (K / 2) + g * 8) = make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
+        }
+        // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
+        uint32_t word = sf8;
+        word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 1) << 8;
+        word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2) << 16;
+        word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3) << 24;
+        if ((g & 3) || row >= p.rows_pad) continue;
+        if (SF_LAYOUT == PQ_SF_TCGEN05) *reinterpret_cast<uint32_t *>(p.sf + pq::sf_tc_offset(row, g, GPR >> 2)) = word;
+        else if (live) *reinterpret_cast<uint32_t *>(p.sf + row * GPR + g) = word;
+    }
+}
+
 template <int SF_LAYOUT, int N>
 __global__ void __launch_bounds__(32 * kRowWarps, 2) hadamard_quant_rows_kernel(const HadParams p) {
-    constexpr int SEG = 1 << N, K = 12 * SEG, OCTS = SEG / 8, RPW = 32 / OCTS, LOG = N - 3, GPR = K / 16;
+    constexpr int SEG = 1 << N, K = 12 * SEG, OCTS = SEG / 8, RPW = 32 / OCTS, LOG = N - 3;
     extern __shared__ __align__(16) float had_smem[];  // [warps][3072] fp32, then K 16-bit read-out offsets in two planes
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float *image = had_smem + warp * kRowImage;
@@ -510,64 +601,150 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) hadamard_quant_rows_kernel(
             }
             __syncwarp();
         }
-        // ---- phase 3: one output group per lane, 192 groups
+        // through a lambda: with the two calls written directly the 768- and 1536-channel kernels spilled
         auto read_out = [&](auto fast) {
-#pragma unroll 1
-            for (int i = lane; i < RPW * GPR; i += 32) {
-                const int r = i / GPR, g = i - r * GPR;
-                const int64_t row = row0 + r;
-                const bool live = row < p.rows;
-                float out[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) out[j] = 0.0f;
-                if (live) {
-                    const uint4 i0 = offset4[g], i1 = offset4[GPR + g];
-                    const uint32_t iw[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
-                    const char *row_b = reinterpret_cast<const char *>(image + r * K);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        out[2 * j] = *reinterpret_cast<const float *>(row_b + (iw[j] & 0xFFFFu));
-                        out[2 * j + 1] = *reinterpret_cast<const float *>(row_b + (iw[j] >> 16));
-                    }
-                    if (p.y_out) {
-                        uint32_t yw[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            yw[j] = __bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j])) |
-                                    (static_cast<uint32_t>(__bfloat16_as_ushort(__float2bfloat16_rn(out[2 * j + 1]))) << 16);
-                        uint4 *ydst = reinterpret_cast<uint4 *>(p.y_out + row * K) + 2 * g;
-                        ydst[0] = make_uint4(yw[0], yw[1], yw[2], yw[3]);
-                        ydst[1] = make_uint4(yw[4], yw[5], yw[6], yw[7]);
-                    }
-                }
-                if (!p.codes) continue;
-                float amax = 0.0f, rcp;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) amax = fmaxf(amax, fabsf(out[j]));
-                uint32_t sf8;
-                pq::nvfp4_scale<decltype(fast)::value>(amax, scaler, sf8, rcp);
-                if (live) {
-                    const uint64_t rcp2 = pack2(rcp, rcp);
-                    float ylo[8], yhi[8];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        unpack2(mul2(pack2(out[2 * j], out[2 * j + 1]), rcp2), ylo[2 * j], ylo[2 * j + 1]);
-                        unpack2(mul2(pack2(out[8 + 2 * j], out[9 + 2 * j]), rcp2), yhi[2 * j], yhi[2 * j + 1]);
-                    }
-                    *reinterpret_cast<uint2 *>(p.codes + row * (K / 2) + g * 8) = make_uint2(pq::f32x8_to_e2m1(ylo), pq::f32x8_to_e2m1(yhi));
-                }
-                // scale bytes: four neighbouring groups sit in neighbouring lanes (padding rows write zeros)
-                uint32_t word = sf8;
-                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 1) << 8;
-                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 2) << 16;
-                word |= __shfl_down_sync(0xFFFFFFFFu, sf8, 3) << 24;
-                if ((g & 3) || row >= p.rows_pad) continue;
-                if (SF_LAYOUT == PQ_SF_TCGEN05) *reinterpret_cast<uint32_t *>(p.sf + pq::sf_tc_offset(row, g, GPR >> 2)) = word;
-                else if (live) *reinterpret_cast<uint32_t *>(p.sf + row * GPR + g) = word;
-            }
+            rows_read_out<SF_LAYOUT, K, RPW, 32, decltype(fast)::value>(p, scaler, image, offset4, row0, lane);
         };
         if (scaler.fast) read_out(std::true_type{});
         else read_out(std::false_type{});
+    }
+}
+
+// ---- two or four warps per row (K = 12 * 512, 12 * 1024)
+// A team's lanes take one phase-1 item each, as above, and meet at a barrier of their own, so the teams of an SM stay
+// out of step with each other.  4608 x 6144 49.2 us (99.8 with the block kernel, whose rows move in step), 4608 x 12288
+// 92.6 (161.6), 300 x 6144 9.9 (25.6), 200 x 12288 10.6 (21.6); instruction issue and shared memory bound it, as above.  The strides above 4 take two passes: 8 octets side by side, then the rest.  The image
+// XORs an octet's two low bits with the two bits above the first window, which keeps the column accesses of both
+// passes (four neighbouring windows, four neighbouring octets per half warp) and the stores of phase 1 conflict-free.
+// One block of sixteen warps per SM: eight or four images of 24 or 48 KB.
+template <int SF_LAYOUT, int N>
+__global__ void __launch_bounds__(512, 1) hadamard_quant_team_kernel(const HadParams p) {
+    constexpr int SEG = 1 << N, K = 12 * SEG, NT = SEG / 8, TEAMS = 512 / NT, WINDOWS = SEG / 64;
+    extern __shared__ __align__(16) float had_smem[];  // [teams][K] fp32, then K 16-bit read-out offsets in two planes
+    const int team = threadIdx.x / NT, tid = threadIdx.x % NT;
+    float *image = had_smem + team * K;
+    uint16_t *offset_s = reinterpret_cast<uint16_t *>(had_smem + TEAMS * K);
+    const uint4 *offset4 = reinterpret_cast<const uint4 *>(offset_s);
+    pq::wait_for_prior_grid();
+    pq::dependents_may_launch();
+    for (int j = threadIdx.x; j < K; j += 512)
+        offset_s[((j >> 3) & 1) * (K / 2) + (j >> 4) * 8 + (j & 7)] =
+            static_cast<uint16_t>(row_image_index<N>(p.perm ? __ldg(p.perm + j) : j) << 2);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldg(p.ts) : 1.0f);
+    __syncthreads();
+    auto team_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(NT) : "memory"); };
+
+    const int64_t step = static_cast<int64_t>(gridDim.x) * TEAMS;
+    for (int64_t row = static_cast<int64_t>(team) * gridDim.x + blockIdx.x; row < p.rows_pad; row += step) {
+        if (row < p.rows) {
+            const uint16_t *src = p.X + row * p.ld + tid * 8;
+            uint4 raw[12];
+#pragma unroll
+            for (int a = 0; a < 12; ++a) raw[a] = __ldcs(reinterpret_cast<const uint4 *>(src + a * SEG));
+            team_sync();  // the previous row has been read out
+            row_columns_12<N, 0>(std::make_integer_sequence<int, 12>{}, raw, image, tid);
+            row_columns_12<N, 1>(std::make_integer_sequence<int, 12>{}, raw, image, tid);
+            if (row + step < p.rows && (tid & 7) == 0) {  // this team's next row, into L2
+#pragma unroll
+                for (int a = 0; a < 12; ++a) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + step * p.ld + a * SEG));
+            }
+            team_sync();
+#pragma unroll 2
+            for (int i = tid; i < 48 * WINDOWS; i += NT) {
+                const int w = (i >> 2) % WINDOWS, a = (i >> 2) / WINDOWS;
+                column_pass<3, uint64_t, false>(image, (a << N) + (w << 6), w & 3, (i & 3) * 2, 0.0f);
+            }
+            team_sync();
+#pragma unroll 1
+            for (int i = tid; i < 12 * 32; i += NT)
+                high_column_pass<N - 6>(image + ((i >> 5) << N), (i >> 2) & 7, (i & 3) * 2, p.scale);
+            team_sync();
+        }
+        if (scaler.fast) rows_read_out<SF_LAYOUT, K, 1, NT, true>(p, scaler, image, offset4, row, tid);
+        else rows_read_out<SF_LAYOUT, K, 1, NT, false>(p, scaler, image, offset4, row, tid);
+    }
+}
+
+// ---- one warp per row (K = 2048, 4096) or per two rows (1024), without the order-12 factor
+// A lane holds blocks of 2^P1 neighbouring channels (strides 1 ... 2^(P1-1) in registers), then columns of 2^P2 values,
+// one per block: a single pass over shared memory, packed where a lane's columns come in pairs.  16-byte chunk q of
+// block u lies at chunk q ^ (u & 7): the stores of phase 1 (eight blocks per wavefront) and the column accesses (one
+// block per instruction) are conflict-free.  Against the block kernel: 4608 x 1024 8.1 us (16.4), 9000 x 2048 29.8 (55.1),
+// 4608 x 4096 33.0 (81.4), 300 x 1024 4.3 (5.8), 300 x 4096 7.7 (16.5).
+template <int P1>
+__device__ __forceinline__ int pow2_image_index(int channel) {
+    const int u = channel >> P1, c = channel & ((1 << P1) - 1);
+    return (u << P1) + (((c >> 2) ^ (u & 7)) << 2) + (c & 3);
+}
+template <int P1, int P2, typename T>
+__device__ __forceinline__ void pow2_column(float *row_s, int c, float scale) {
+    constexpr int NV = 1 << P2, kStep = (8 << P1) * sizeof(float) / sizeof(T);
+    T *slot[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) slot[j] = reinterpret_cast<T *>(row_s + (j << P1) + (((c >> 2) ^ j) << 2) + (c & 3));
+    T v[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] = slot[j & 7][(j >> 3) * kStep];
+    column_butterflies(v);
+#pragma unroll
+    for (int j = 0; j < NV; ++j) slot[j & 7][(j >> 3) * kStep] = column_scaled(v[j], scale);
+}
+
+// RPW rows per warp; WARPS per block: two blocks' images fit an SM
+template <int SF_LAYOUT, int P1, int P2, int RPW, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 2) hadamard_quant_pow2_kernel(const HadParams p) {
+    constexpr int K = 1 << (P1 + P2), BL = 1 << P1, NB = 1 << P2;
+    extern __shared__ __align__(16) float had_smem[];  // [warps][RPW][K] fp32, then K 16-bit read-out offsets in two planes
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *image = had_smem + warp * (RPW * K);
+    uint16_t *offset_s = reinterpret_cast<uint16_t *>(had_smem + WARPS * RPW * K);
+    const uint4 *offset4 = reinterpret_cast<const uint4 *>(offset_s);
+    pq::wait_for_prior_grid();
+    pq::dependents_may_launch();
+    for (int j = threadIdx.x; j < K; j += 32 * WARPS)
+        offset_s[((j >> 3) & 1) * (K / 2) + (j >> 4) * 8 + (j & 7)] =
+            static_cast<uint16_t>(pow2_image_index<P1>(p.perm ? __ldg(p.perm + j) : j) << 2);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldg(p.ts) : 1.0f);
+    __syncthreads();
+
+    const int64_t batches = (p.rows_pad + RPW - 1) / RPW, step = static_cast<int64_t>(gridDim.x) * WARPS;
+    for (int64_t batch = static_cast<int64_t>(warp) * gridDim.x + blockIdx.x; batch < batches; batch += step) {
+        const int64_t row0 = batch * RPW;
+        if (row0 < p.rows) {
+            __syncwarp();  // the previous rows have been read out
+#pragma unroll 1
+            for (int i = lane; i < RPW * NB; i += 32) {
+                const int r = i / NB, u = i % NB;
+                const uint4 *src = reinterpret_cast<const uint4 *>(p.X + (row0 + r) * p.ld + u * BL);
+                const bool have = row0 + r < p.rows;  // rows past the end are zeros
+                uint4 raw[BL / 8];
+#pragma unroll
+                for (int q = 0; q < BL / 8; ++q) raw[q] = have ? __ldg(src + q) : make_uint4(0, 0, 0, 0);
+                uint64_t v[BL / 2];
+#pragma unroll
+                for (int q = 0; q < BL / 8; ++q) {
+                    uint64_t w[4];
+                    unpack_pairs(raw[q], w);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) v[4 * q + e] = butterfly_in_pair(w[e]);
+                }
+                column_butterflies(v);
+                ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(image + r * K + u * BL);
+#pragma unroll
+                for (int q = 0; q < BL / 4; ++q) dst[q ^ (u & 7)] = make_ulonglong2(v[2 * q], v[2 * q + 1]);
+            }
+            __syncwarp();
+            if constexpr (P2 == 5) {
+                const int r = RPW == 2 ? lane >> 4 : 0, c = RPW == 2 ? lane & 15 : lane;
+                pow2_column<P1, P2, uint64_t>(image + r * K, 2 * c, p.scale);
+            } else {
+#pragma unroll 1
+                for (int c = lane; c < BL; c += 32) pow2_column<P1, P2, float>(image, c, p.scale);
+            }
+            __syncwarp();
+        }
+        if (scaler.fast) rows_read_out<SF_LAYOUT, K, RPW, 32, true>(p, scaler, image, offset4, row0, lane);
+        else rows_read_out<SF_LAYOUT, K, RPW, 32, false>(p, scaler, image, offset4, row0, lane);
     }
 }
 
@@ -617,19 +794,34 @@ extern "C" pq_status pq_hadamard_quant_nvfp4(const void *X, int64_t M, int64_t K
     p.perm = perm, p.ts = ts_x, p.codes = codes, p.sf = sf, p.y_out = static_cast<uint16_t *>(y_out);
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // warps or teams of warps with rows of their own: `images` values per block, `units` units of work of all rows,
+    // `per_sm` blocks of `threads` per SM
+    auto launch_rows = [&](auto kern, int64_t images, int64_t units, int per_sm, int threads) -> pq_status {
+        const size_t smem = static_cast<size_t>(images) * sizeof(float) + static_cast<size_t>(K) * sizeof(uint16_t);
+        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(std::min<int64_t>(units, per_sm * sms))), dim3(threads), smem,
+                                        static_cast<cudaStream_t>(stream), p));
+        return pq_launch_status();
+    };
+    const bool tc = sf_layout == PQ_SF_TCGEN05;
     if (m == 12 && n >= 6 && n <= 8) {  // widths whose rows fit a warp's lanes exactly: 768, 1536, 3072
-        const size_t row_smem = static_cast<size_t>(kRowWarps) * kRowImage * sizeof(float) + static_cast<size_t>(K) * sizeof(uint16_t);
-        const int64_t warps = pq_ceil_div(p.rows_pad, 1 << (8 - n));
-        auto launch_rows = [&](auto kern) -> pq_status {
-            PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(row_smem)));
-            PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(std::min<int64_t>(warps, 2 * sms))), dim3(32 * kRowWarps),
-                                            row_smem, static_cast<cudaStream_t>(stream), p));
-            return pq_launch_status();
+        auto go = [&](auto kern) { return launch_rows(kern, kRowWarps * kRowImage, pq_ceil_div(p.rows_pad, 1 << (8 - n)), 2, 32 * kRowWarps); };
+        if (n == 8) return go(tc ? hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 8> : hadamard_quant_rows_kernel<PQ_SF_LINEAR, 8>);
+        if (n == 7) return go(tc ? hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 7> : hadamard_quant_rows_kernel<PQ_SF_LINEAR, 7>);
+        return go(tc ? hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 6> : hadamard_quant_rows_kernel<PQ_SF_LINEAR, 6>);
+    }
+    if (m == 12 && (n == 9 || n == 10)) {  // two and four times as wide: 6144, 12288
+        auto go = [&](auto kern) { return launch_rows(kern, 16 * kRowImage, p.rows_pad, 1, 512); };
+        if (n == 9) return go(tc ? hadamard_quant_team_kernel<PQ_SF_TCGEN05, 9> : hadamard_quant_team_kernel<PQ_SF_LINEAR, 9>);
+        return go(tc ? hadamard_quant_team_kernel<PQ_SF_TCGEN05, 10> : hadamard_quant_team_kernel<PQ_SF_LINEAR, 10>);
+    }
+    if (m == 1 && n >= 10 && n <= 12) {  // 1024, 2048, 4096
+        auto go = [&](auto kern, int rows, int warps) {
+            return launch_rows(kern, warps * rows * K, pq_ceil_div(p.rows_pad, rows), 2, 32 * warps);
         };
-        const bool tc = sf_layout == PQ_SF_TCGEN05;
-        if (n == 8) return tc ? launch_rows(hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 8>) : launch_rows(hadamard_quant_rows_kernel<PQ_SF_LINEAR, 8>);
-        if (n == 7) return tc ? launch_rows(hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 7>) : launch_rows(hadamard_quant_rows_kernel<PQ_SF_LINEAR, 7>);
-        return tc ? launch_rows(hadamard_quant_rows_kernel<PQ_SF_TCGEN05, 6>) : launch_rows(hadamard_quant_rows_kernel<PQ_SF_LINEAR, 6>);
+        if (n == 10) return go(tc ? hadamard_quant_pow2_kernel<PQ_SF_TCGEN05, 5, 5, 2, 8> : hadamard_quant_pow2_kernel<PQ_SF_LINEAR, 5, 5, 2, 8>, 2, 8);
+        if (n == 11) return go(tc ? hadamard_quant_pow2_kernel<PQ_SF_TCGEN05, 6, 5, 1, 8> : hadamard_quant_pow2_kernel<PQ_SF_LINEAR, 6, 5, 1, 8>, 1, 8);
+        return go(tc ? hadamard_quant_pow2_kernel<PQ_SF_TCGEN05, 6, 6, 1, 6> : hadamard_quant_pow2_kernel<PQ_SF_LINEAR, 6, 6, 1, 6>, 1, 6);
     }
     const size_t row_bytes = static_cast<size_t>(K) * sizeof(float);
     p.rows_per_block = static_cast<int>(kSmemBudget / row_bytes < kMaxRows ? kSmemBudget / row_bytes : kMaxRows);

@@ -1,4 +1,4 @@
-"""The warp-per-row Hadamard kernel over more rows than the grid has warps, with a last, partly filled group of rows."""
+"""The Hadamard kernels with a warp or a team of warps per row over more rows than the grid has warps, with a last, partly filled group of rows."""
 import numpy as np
 import pytest
 import torch
@@ -11,7 +11,9 @@ from test_gpu_gemm import to_tc
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,K", [(2400, 3072), (4737, 1536), (9475, 768), (1, 3072), (3, 768)])
+@pytest.mark.parametrize("M,K", [(2400, 3072), (4737, 1536), (9475, 768), (1, 3072), (3, 768),
+                                 (1187, 6144), (2, 6144), (597, 12288), (1, 12288),
+                                 (4739, 1024), (1, 1024), (2371, 2048), (1779, 4096)])
 def test_rows_kernel_bit_exact(M, K):
     g = torch.Generator().manual_seed(M)
     x = (torch.randn(M, K, generator=g) * torch.exp(torch.randn(K, generator=g))).to(torch.bfloat16)

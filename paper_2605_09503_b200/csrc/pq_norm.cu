@@ -682,6 +682,8 @@ norm_quant_ordered_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
                           const float *__restrict__ ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
                           uint16_t *__restrict__ y_out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pq::wait_for_prior_grid();
+    pq::dependents_may_launch();
     const int64_t row = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + warp;
     if (row >= rows_pad) return;  // whole warps only
     const bool live = row < rows;
@@ -784,24 +786,30 @@ template <int KIND, int SF_LAYOUT>
 pq_status launch(const uint16_t *H, int64_t M, int64_t rows_pad, int K, int64_t ld, const float *a, const float *b,
                  float eps, const int32_t *perm, const float *ts, uint8_t *codes, uint8_t *sf, uint16_t *y_out,
                  cudaStream_t st) {
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // no reordering to apply and a row fits a warp's registers: the streaming kernel
     if (!perm && K <= 256 * kDirectMaxOcts) {
         const int64_t blocks = pq_ceil_div(rows_pad, kDirectThreads / 32);
         PQ_REQUIRE(blocks < (1ll << 31), PQ_ERR_SHAPE);
         const unsigned grid = static_cast<unsigned>(blocks);
         const int noct = static_cast<int>(pq_ceil_div(K, 256));
-        if (noct <= 4) norm_quant_ordered_kernel<KIND, SF_LAYOUT, 4><<<grid, kDirectThreads, 0, st>>>(H, M, rows_pad, K, ld, a, b, eps, ts, codes, sf, y_out);
-        else if (noct <= 8) norm_quant_ordered_kernel<KIND, SF_LAYOUT, 8><<<grid, kDirectThreads, 0, st>>>(H, M, rows_pad, K, ld, a, b, eps, ts, codes, sf, y_out);
-        else if (noct <= 12) norm_quant_ordered_kernel<KIND, SF_LAYOUT, 12><<<grid, kDirectThreads, 0, st>>>(H, M, rows_pad, K, ld, a, b, eps, ts, codes, sf, y_out);
-        else norm_quant_ordered_kernel<KIND, SF_LAYOUT, 16><<<grid, kDirectThreads, 0, st>>>(H, M, rows_pad, K, ld, a, b, eps, ts, codes, sf, y_out);
+        auto kern = noct <= 4    ? norm_quant_ordered_kernel<KIND, SF_LAYOUT, 4>
+                    : noct <= 8  ? norm_quant_ordered_kernel<KIND, SF_LAYOUT, 8>
+                    : noct <= 12 ? norm_quant_ordered_kernel<KIND, SF_LAYOUT, 12>
+                                 : norm_quant_ordered_kernel<KIND, SF_LAYOUT, 16>;
+        // Few rows: the GEMM's launch overlaps this kernel (norm and GEMM, us, plain / dependent: 512 x 3072 x 3072 17.5 / 16.1,
+        // 300 x 2048 x 512 14.4 / 11.9, 2304 x 3072 x 3072 26.7 / 25.4).  Many: its waiting blocks take room on the SMs from
+        // this kernel's (4608 x 3072 x 9216 76.3 / 76.8, 3400 x 3072 without a GEMM 13.0 / 13.5).
+        if (blocks <= 4 * sms)
+            PQ_CUDA_OK(pq::launch_dependent(kern, dim3(grid), dim3(kDirectThreads), 0, st, H, M, rows_pad, K, ld, a, b, eps, ts, codes, sf, y_out));
+        else kern<<<grid, kDirectThreads, 0, st>>>(H, M, rows_pad, K, ld, a, b, eps, ts, codes, sf, y_out);
         return pq_launch_status();
     }
     // several rows per warp while two blocks of sixteen rows fit on an SM and there is one for every SM at least;
     // otherwise four rows per block (measurements at that kernel)
     const size_t group_smem = static_cast<size_t>(kGroupWarps) * kGroupRows * K * 2;
     const int64_t group_blocks = pq_ceil_div(rows_pad, kGroupWarps * kGroupRows);
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (2 * (group_smem + 2048) <= 227 * 1024 && group_blocks >= sms) {
         if (group_smem > 40 * 1024)  // the kernel's static shared memory counts towards the 48 KB default limit
             PQ_CUDA_OK(cudaFuncSetAttribute(norm_quant_grouped_kernel<KIND, SF_LAYOUT>,

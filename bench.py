@@ -563,7 +563,7 @@ def run_ours(args):
         ws_qw = B.workspace(B.OP_QUANT_WEIGHT, N, K)
         stage("quant_weight", graph_loop(torch, lambda i: B.pq_quant_weight(Wt, cal.perms, cal.select, wq2, sfw2, 1, tsw2,
                                                                             ws_qw), max(5, it // 4)),
-              2 * N * K * 2 + N * K // 2 + N * K // 16, note="two reads of W (absmax, then gather + quantize, four rows per warp)")
+              2 * N * K * 2 + N * K // 2 + N * K // 16, note="two reads of W (absmax, then gather + quantize, four rows per block)")
 
         # output-side calibration error: fp32 reference and bf16 layer output of one batch (6 B per element)
         yrefs = [torch.randn(M, N, device=dev) for _ in range(2)]
@@ -575,7 +575,7 @@ def run_ours(args):
         stage("quant_act_nvfp4_candidate_order",
               graph_loop(torch, lambda i: B.pq_quant_act_nvfp4_perm(xs[i % XROT], order, cal.ts_x, xq_rot[i % XROT],
                                                                     sfx_rot[i % XROT], B.PQ_SF_TCGEN05), it),
-              quant_bytes, note="calibration-time gather quantizer: four rows per warp share indices and gathers")
+              quant_bytes, note="calibration-time gather quantizer: four rows per block share indices and gathers")
         del yrefs, yqs
 
     # ---- end to end: host tensors in, host tensor out, through the C ABI

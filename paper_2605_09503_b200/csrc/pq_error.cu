@@ -343,6 +343,7 @@ struct GatherParams {
     PqErrorWeights weights;    // added up by one more warp of the block(s) in front, behind the gather's back
 };
 
+constexpr size_t kGatherSmemMax = 226 * 1024;
 constexpr int kTabBytes = (static_cast<int>(sizeof(ScaleTab)) + 15) / 16 * 16;
 
 inline size_t gather_smem_bytes(int64_t K, int opb, int groups, int sides) {
@@ -494,7 +495,7 @@ inline GatherConfig gather_config(int64_t chunks, int64_t K, int P, int sides, i
         for (int opb = 1; opb <= P; ++opb) {
             const int64_t subsets = pq_ceil_div(P, opb);
             for (int groups = 1; groups <= kMaxGroups && groups * threads <= kGatherThreads; ++groups) {
-                if (gather_smem_bytes(K, opb, groups, sides) > 226 * 1024) break;
+                if (gather_smem_bytes(K, opb, groups, sides) > kGatherSmemMax) break;
                 const int64_t blocks = sms / subsets > 0 ? sms / subsets : 1;
                 const double pairs = static_cast<double>(pq_ceil_div(chunks * opb, blocks * groups));
                 const int warps = groups * threads / 32;
@@ -542,8 +543,7 @@ pq_status launch_gather(GatherParams &p, int64_t K, int P, float Qf, float *part
     }
     const size_t smem = gather_smem_bytes(K, cfg.opb, cfg.groups, sides);
     auto kern = group_error_gather<KIND, TEAM / 2>;
-    if (smem > 48 * 1024)
-        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    PQ_CUDA_OK(pq::allow_smem(kern, smem, kGatherSmemMax));
     const unsigned threads = static_cast<unsigned>(cfg.groups * cfg.group_threads + (p.weights.lambda ? 32 : 0));
     PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(subsets)),
                                     dim3(threads), smem, st, p));

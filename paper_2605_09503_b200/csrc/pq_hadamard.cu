@@ -48,6 +48,7 @@ constexpr int kThreads = 32 * kMaxRows;
 #endif
 constexpr int kBlocksPerSm = PQ_HAD_BLOCKS;
 constexpr size_t kSmemBudget = 192 * 1024;
+constexpr int64_t kMaxK = 16384;
 
 // ---- Paley's Hadamard matrix of order 12 (compile-time)
 constexpr int quadratic_character_11(int r) {
@@ -771,7 +772,7 @@ extern "C" pq_status pq_hadamard_quant_nvfp4(const void *X, int64_t M, int64_t K
     PQ_REQUIRE(!codes || ts_x, PQ_ERR_NULL);
     PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || sf_layout == PQ_SF_TCGEN05, PQ_ERR_FORMAT);
     int m = 0, n = 0;
-    PQ_REQUIRE(M > 0 && K >= 16 && K % 16 == 0 && K <= 16384 && ld >= K && factor_width(K, m, n), PQ_ERR_SHAPE);
+    PQ_REQUIRE(M > 0 && K >= 16 && K % 16 == 0 && K <= kMaxK && ld >= K && factor_width(K, m, n), PQ_ERR_SHAPE);
     PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || !codes || K % 64 == 0, PQ_ERR_SHAPE);
     PQ_REQUIRE(pq_aligned16(X) && ld % 8 == 0 && (!codes || (pq_aligned16(codes) && pq_aligned16(sf))) &&
                    (!perm || pq_aligned16(perm)) && (!y_out || pq_aligned16(y_out)),
@@ -798,7 +799,7 @@ extern "C" pq_status pq_hadamard_quant_nvfp4(const void *X, int64_t M, int64_t K
     // `per_sm` blocks of `threads` per SM
     auto launch_rows = [&](auto kern, int64_t images, int64_t units, int per_sm, int threads) -> pq_status {
         const size_t smem = static_cast<size_t>(images) * sizeof(float) + static_cast<size_t>(K) * sizeof(uint16_t);
-        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        PQ_CUDA_OK(pq::allow_smem(kern, smem, smem));  // a kernel serves one width
         PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(std::min<int64_t>(units, per_sm * sms))), dim3(threads), smem,
                                         static_cast<cudaStream_t>(stream), p));
         return pq_launch_status();
@@ -834,8 +835,7 @@ extern "C" pq_status pq_hadamard_quant_nvfp4(const void *X, int64_t M, int64_t K
     const int64_t batches = pq_ceil_div(p.rows_pad, kRows);
     const int64_t blocks = std::min<int64_t>(batches, static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1));
     auto launch = [&](auto kern) -> pq_status {
-        if (smem > 48 * 1024)
-            PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        PQ_CUDA_OK(pq::allow_smem(kern, smem, kSmemBudget + kMaxK * sizeof(uint16_t)));
         PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks)), dim3(wide_block ? 2 * kThreads : kThreads),
                                         smem, st, p));
         return pq_launch_status();

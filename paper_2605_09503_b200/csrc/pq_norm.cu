@@ -233,6 +233,7 @@ norm_quant_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad
 // the statistics, then all of them share the walk over the output order
 constexpr int kGroupRows = PQ_NORM_ROWS, kGroupWarps = PQ_NORM_WARPS, kSplit = PQ_NORM_SPLIT;
 static_assert(kGroupRows == 2 || kGroupRows == 4, "rows per warp");
+constexpr size_t kGroupSmemMax = 227 * 1024 / 2 - 2048;  // two blocks per SM
 
 // 16-byte chunk k of octet o (R = 4: two channels per chunk, four chunks; R = 2: four channels, two chunks)
 template <int R>
@@ -656,8 +657,7 @@ pq_status launch_quad(const uint16_t *H, int64_t rows, int64_t rows_pad, int K, 
     const int64_t blocks = pq_ceil_div(rows_pad, 4);
     PQ_REQUIRE(blocks < (1ll << 31), PQ_ERR_SHAPE);
     auto kern = iter == 1 ? norm_quant_quad_kernel<KIND, SF_LAYOUT, 1> : norm_quant_quad_kernel<KIND, SF_LAYOUT, 2>;
-    if (smem > 47 * 1024)  // the kernel's static shared memory counts towards the 48 KB default limit
-        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    PQ_CUDA_OK(pq::allow_smem(kern, smem, kQuadMaxK * 8, 1024));
     PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks)), dim3(static_cast<unsigned>(threads)), smem, st, H, rows, rows_pad,
                                     K, ld, a, b, eps, perm, perm_select, ts, codes, sf, y_out));
     return pq_launch_status();
@@ -810,10 +810,8 @@ pq_status launch(const uint16_t *H, int64_t M, int64_t rows_pad, int K, int64_t 
     // otherwise four rows per block (measurements at that kernel)
     const size_t group_smem = static_cast<size_t>(kGroupWarps) * kGroupRows * K * 2;
     const int64_t group_blocks = pq_ceil_div(rows_pad, kGroupWarps * kGroupRows);
-    if (2 * (group_smem + 2048) <= 227 * 1024 && group_blocks >= sms) {
-        if (group_smem > 40 * 1024)  // the kernel's static shared memory counts towards the 48 KB default limit
-            PQ_CUDA_OK(cudaFuncSetAttribute(norm_quant_grouped_kernel<KIND, SF_LAYOUT>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(group_smem)));
+    if (group_smem <= kGroupSmemMax && group_blocks >= sms) {
+        PQ_CUDA_OK(pq::allow_smem(norm_quant_grouped_kernel<KIND, SF_LAYOUT>, group_smem, kGroupSmemMax, 1024));
         PQ_REQUIRE(group_blocks < (1ll << 31), PQ_ERR_SHAPE);
         PQ_CUDA_OK(pq::launch_dependent(norm_quant_grouped_kernel<KIND, SF_LAYOUT>, dim3(static_cast<unsigned>(group_blocks)),
                                         dim3(kGroupWarps * kSplit * 32), group_smem, st, H, M, rows_pad, K, ld, a, b, eps, perm, ts,
@@ -826,9 +824,7 @@ pq_status launch(const uint16_t *H, int64_t M, int64_t rows_pad, int K, int64_t 
     if (warps > kMaxRowsPerBlock) warps = kMaxRowsPerBlock;
     if (warps < 1) return PQ_ERR_SHAPE;
     const size_t smem = static_cast<size_t>(warps) * K * 2;
-    if (smem > 48 * 1024)
-        PQ_CUDA_OK(cudaFuncSetAttribute(norm_quant_kernel<KIND, SF_LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        static_cast<int>(smem)));
+    PQ_CUDA_OK(pq::allow_smem(norm_quant_kernel<KIND, SF_LAYOUT>, smem, kSmemBudget));
     const int64_t blocks = pq_ceil_div(rows_pad, warps);
     PQ_REQUIRE(blocks < (1ll << 31), PQ_ERR_SHAPE);
     norm_quant_kernel<KIND, SF_LAYOUT><<<static_cast<unsigned>(blocks), warps * 32, smem, st>>>(

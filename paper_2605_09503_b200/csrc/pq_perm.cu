@@ -200,8 +200,7 @@ pq_status launch_sort(const SortParams &p, cudaStream_t st) {
     cfg.gridDim = dim3(static_cast<unsigned>(ctas), static_cast<unsigned>(p.orders + (p.scale_out[0] ? 2 : 0)));
     cfg.blockDim = dim3(kSortChunk), cfg.stream = st;
     cfg.dynamicSmemBytes = static_cast<size_t>(chunks) * kSortChunk * sizeof(unsigned long long);
-    if (cfg.dynamicSmemBytes > 16 * 1024)  // the kernel's static shared memory counts towards the 48 KB default limit
-        PQ_CUDA_OK(cudaFuncSetAttribute(order_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(cfg.dynamicSmemBytes)));
+    PQ_CUDA_OK(pq::allow_smem(order_sort_kernel, cfg.dynamicSmemBytes, kSortMaxChunks * kSortChunk * sizeof(unsigned long long), 32 * 1024));
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = static_cast<unsigned>(ctas), attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;

@@ -23,6 +23,7 @@ constexpr int kTileRows = 8;                    // blocks of the streaming kerne
 // sub-partition at 32 registers, which is what fits on an SM beside a GEMM CTA (batched linear path).
 constexpr int kActThreads = 32 * kTileRows;
 constexpr unsigned kGridYMax = 65535;
+constexpr int64_t kOrderMaxK = 16384;           // channels an order may have
 
 // Row block of a (x = column chunk, y/z = row block) grid; y alone is limited to 65535 blocks.
 __device__ __forceinline__ int64_t row_block_index() {
@@ -374,13 +375,6 @@ int grid_for(int64_t work_items, int threads, int per_sm) {
     return static_cast<int>(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
-template <typename Kern>
-pq_status allow_smem(Kern kern, size_t bytes) {
-    if (bytes > 48 * 1024)
-        PQ_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)));
-    return PQ_OK;
-}
-
 }  // namespace
 
 extern "C" size_t pq_sf_bytes(int64_t rows, int64_t K, int sf_layout) {
@@ -450,16 +444,14 @@ extern "C" pq_status pq_quant_act_nvfp4(const void *X, int64_t M, int64_t K, int
 static pq_status launch_gather(const uint16_t *w, int64_t N, int64_t K, int64_t ld, const int32_t *perm,
                                const int32_t *perm_select, const float *ts, uint8_t *codes, uint8_t *sf,
                                int sf_layout, cudaStream_t st) {
-    const size_t smem = static_cast<size_t>(K) * 2;
+    const size_t smem = static_cast<size_t>(K) * 2;  // 32 KB at most
     const int grid = static_cast<int>(N < 148 * 8 ? N : 148 * 8);
     if (sf_layout == PQ_SF_TCGEN05) {
         const int64_t rows_pad = pq_ceil_div(N, 128) * 128;
         if (rows_pad > N) sf_zero_pad_kernel<<<64, 256, 0, st>>>(sf, N, rows_pad, K);
-        if (allow_smem(quant_nvfp4_gather_kernel<PQ_SF_TCGEN05>, smem) != PQ_OK) return PQ_ERR_CUDA;
         quant_nvfp4_gather_kernel<PQ_SF_TCGEN05><<<grid, kQuantThreads, smem, st>>>(
             w, N, K, ld, perm, perm_select, ts, codes, sf);
     } else {
-        if (allow_smem(quant_nvfp4_gather_kernel<PQ_SF_LINEAR>, smem) != PQ_OK) return PQ_ERR_CUDA;
         quant_nvfp4_gather_kernel<PQ_SF_LINEAR><<<grid, kQuantThreads, smem, st>>>(
             w, N, K, ld, perm, perm_select, ts, codes, sf);
     }
@@ -472,7 +464,7 @@ extern "C" pq_status pq_quant_act_nvfp4_perm(const void *X, int64_t M, int64_t K
     if (!perm) return pq_quant_act_nvfp4(X, M, K, ld, ts_x, codes, sf, sf_layout, stream);
     PQ_REQUIRE(X && ts_x && codes && sf, PQ_ERR_NULL);
     PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || sf_layout == PQ_SF_TCGEN05, PQ_ERR_FORMAT);
-    PQ_REQUIRE(M > 0 && K > 0 && K % 16 == 0 && K <= 16384 && ld >= K, PQ_ERR_SHAPE);
+    PQ_REQUIRE(M > 0 && K > 0 && K % 16 == 0 && K <= kOrderMaxK && ld >= K, PQ_ERR_SHAPE);
     PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || K % 64 == 0, PQ_ERR_SHAPE);
     PQ_REQUIRE(pq_aligned16(X) && ld % 8 == 0 && pq_aligned16(codes) && pq_aligned16(sf), PQ_ERR_ALIGN);
     // four rows share the indices and one gather (the fused producer's kernel without its normalization); an index
@@ -497,7 +489,7 @@ extern "C" pq_status pq_quant_weight(const void *Wt, int64_t N, int64_t K, int64
     PQ_REQUIRE(Wt && codes && sf && ts_w, PQ_ERR_NULL);
     PQ_REQUIRE(perm || !perm_select, PQ_ERR_NULL);
     PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || sf_layout == PQ_SF_TCGEN05, PQ_ERR_FORMAT);
-    PQ_REQUIRE(N > 0 && K > 0 && K % 16 == 0 && K <= 16384 && ld >= K, PQ_ERR_SHAPE);
+    PQ_REQUIRE(N > 0 && K > 0 && K % 16 == 0 && K <= kOrderMaxK && ld >= K, PQ_ERR_SHAPE);
     PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || K % 64 == 0, PQ_ERR_SHAPE);
     PQ_REQUIRE(pq_aligned16(Wt) && ld % 8 == 0 && pq_aligned16(codes) && pq_aligned16(sf), PQ_ERR_ALIGN);
     PQ_REQUIRE(ws && ws_bytes >= pq_workspace_bytes(PQ_OP_QUANT_WEIGHT, N, K, 0, 0), PQ_ERR_WORKSPACE);
@@ -525,7 +517,7 @@ extern "C" pq_status pq_fakequant_int(const void *T, int64_t rows, int64_t K, in
     PQ_REQUIRE(fmt.kind == 1 && fmt.bits >= 2 && fmt.bits <= 8, PQ_ERR_FORMAT);
     PQ_REQUIRE(fmt.group == 16 || fmt.group == 32 || fmt.group == 64 || fmt.group == 128 || fmt.group == 256, PQ_ERR_FORMAT);
     PQ_REQUIRE(rows > 0 && K > 0 && K % fmt.group == 0 && ld >= K && ldo >= K, PQ_ERR_SHAPE);
-    PQ_REQUIRE(!perm || K <= 16384, PQ_ERR_SHAPE);
+    PQ_REQUIRE(!perm || K <= kOrderMaxK, PQ_ERR_SHAPE);
     PQ_REQUIRE(pq_aligned16(T) && pq_aligned16(out) && ld % 8 == 0 && ldo % 8 == 0, PQ_ERR_ALIGN);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint16_t *t = static_cast<const uint16_t *>(T);
@@ -541,7 +533,7 @@ extern "C" pq_status pq_fakequant_int(const void *T, int64_t rows, int64_t K, in
     const dim3 grid = tile_grid(pq_ceil_div(K / 8, 32), pq_ceil_div(rows, kTileRows));
 #define PQ_FQ_CASE(TEAM)                                                                              \
     if (perm) {                                                                                       \
-        if (allow_smem(fakequant_int_gather_kernel<TEAM>, smem + 1024) != PQ_OK) return PQ_ERR_CUDA;  \
+        PQ_CUDA_OK(pq::allow_smem(fakequant_int_gather_kernel<TEAM>, smem, kOrderMaxK * 8, 1024));    \
         fakequant_int_gather_kernel<TEAM><<<static_cast<unsigned>(grid_g), threads_g, smem, st>>>(    \
             t, rows, static_cast<int>(K), ld, perm, Qf, o, ldo);                                      \
     } else {                                                                                          \

@@ -12,6 +12,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpq.so")
 NATIVE = os.path.join(HERE, "_pq_native.so")      # marshalling of the runtime calls (torch headers, no device code)
+# What the native module asks the loader for.  libpq.so is also the name of PostgreSQL's client library; under a name of its
+# own the library is found among the loaded ones (binding.lib() loads it by path first) and nothing is searched.
+SONAME = "libpq_permuquant_b200.so"
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", "--fmad=false", "-cudart", "static"]
 
@@ -38,8 +41,8 @@ def build_native(force: bool = False) -> str:
         root = os.path.dirname(torch.__file__)
         subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wall", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
                         f"-I{root}/include", f"-I{root}/include/torch/csrc/api/include", f"-I{sysconfig.get_paths()['include']}",
-                        "-I/usr/local/cuda/include", src, "-o", NATIVE, f"-L{HERE}", "-l:libpq.so", "-Wl,-rpath,$ORIGIN",
-                        f"-L{root}/lib", "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"], check=True)
+                        "-I/usr/local/cuda/include", src, "-o", NATIVE, f"-L{HERE}", "-l:libpq.so", f"-L{root}/lib",
+                        "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"], check=True)
     return NATIVE
 
 
@@ -53,7 +56,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 cmd.insert(1, "-Xptxas=-v")
             subprocess.run(cmd, check=True)
             objs.append(obj)
-        subprocess.run(["nvcc", "-Wno-deprecated-gpu-targets", "-shared", "-cudart", "static", "-o", LIB, *objs, "-ldl", "-lpthread", "-lrt"], check=True)
+        subprocess.run(["nvcc", "-Wno-deprecated-gpu-targets", "-shared", "-cudart", "static", "-Xlinker", f"-soname={SONAME}", "-o", LIB, *objs, "-ldl",
+                        "-lpthread", "-lrt"], check=True)
     build_native(force)
     return LIB
 

@@ -6,9 +6,12 @@ the entry point of the same name in libpq.so.  There is no fallback: if the libr
 missing or the call fails, an exception is raised.
 """
 import ctypes as C
+import importlib.util
 import os
 
 import torch
+
+from .build import native_path
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libpq.so")
@@ -102,9 +105,13 @@ def native():
     global _native_module
     if _native_module is None:
         lib()
-        from . import _pq_native
-
-        _native_module = _pq_native
+        path = native_path()
+        if not os.path.exists(path):
+            raise ImportError(f"{path} not found: run `python -m paper_2605_09503_b200.build`")
+        spec = importlib.util.spec_from_file_location(__package__ + "._pq_native", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native_module = module
     return _native_module
 
 

@@ -6,6 +6,7 @@
 // status code of the entry point; linear() and calibrate() return their outputs on success.
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <memory>
@@ -81,8 +82,8 @@ PyObject *guarded(Py_ssize_t given, Py_ssize_t n, F &&f) {
         return f();
     } catch (const Failed &) {
         return nullptr;
-    } catch (const std::exception &e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {  // torch's own errors keep their Python types (an allocation that fails is torch.OutOfMemoryError)
+        torch::translate_exception_to_python(std::current_exception());
         return nullptr;
     }
 }

@@ -200,12 +200,13 @@ PyObject *calibrate(PyObject *, PyObject *const *a, Py_ssize_t given) {
         std::vector<const void *> xs;
         std::vector<int64_t> rows, lds;
         int64_t total = 0;
-        PyObject *list = PySequence_Fast(a[0], "batches are a list of tensors");
-        if (!list) throw Failed{};
-        const std::unique_ptr<PyObject, void (*)(PyObject *)> hold(list, [](PyObject *o) { Py_DECREF(o); });
-        const Py_ssize_t n = PySequence_Fast_GET_SIZE(list);
+        // a tuple of its own holds the batches: another thread may empty the caller's list while the lock is released below
+        PyObject *held = PySequence_Tuple(a[0]);
+        if (!held) throw Failed{};
+        const std::unique_ptr<PyObject, void (*)(PyObject *)> hold(held, [](PyObject *o) { Py_DECREF(o); });
+        const Py_ssize_t n = PyTuple_GET_SIZE(held);
         for (Py_ssize_t i = 0; i < n; ++i) {
-            const at::Tensor &X = matrix(PySequence_Fast_GET_ITEM(list, i));
+            const at::Tensor &X = matrix(PyTuple_GET_ITEM(held, i));
             require(X.size(1) == K, "batches have the weight's width");
             xs.push_back(ptr(X)), rows.push_back(X.size(0)), lds.push_back(X.stride(0));
             total += X.size(0);

@@ -18,15 +18,20 @@ size_t partial_bytes(int64_t slabs, int64_t K, int group, int P) {
     const size_t a = pq_stats_list_bytes(slabs, K), b = pq_errors_list_bytes(slabs, K, group, P);
     return round256(a > b ? a : b);
 }
-bool known_format(pq_format fmt) {
-    if (fmt.kind == 0) return true;
-    return fmt.kind == 1 && fmt.bits >= 2 && fmt.bits <= 8 &&
-           (fmt.group == 16 || fmt.group == 32 || fmt.group == 64 || fmt.group == 128 || fmt.group == 256);
+// What can be told from the sizes alone; the caller's outputs and the workspace are sized by these.
+pq_status sizes_status(int n, int64_t N, int64_t K, pq_format fmt, int J) {
+    PQ_REQUIRE(fmt.kind == 0 || (fmt.kind == 1 && fmt.bits >= 2 && fmt.bits <= 8 &&
+                                 (fmt.group == 16 || fmt.group == 32 || fmt.group == 64 || fmt.group == 128 || fmt.group == 256)),
+               PQ_ERR_FORMAT);
+    const int group = fmt.kind == 0 ? 16 : fmt.group;
+    PQ_REQUIRE(n >= 1 && N > 0 && K > 0 && K % group == 0 && K % 16 == 0 && K <= 16384, PQ_ERR_SHAPE);
+    PQ_REQUIRE(J >= 1 && J <= 7, PQ_ERR_SHAPE);
+    return PQ_OK;
 }
 }  // namespace
 
 extern "C" size_t pq_calibrate_workspace_bytes(int n, const int64_t *rows, int64_t N, int64_t K, pq_format fmt, int J) {
-    if (n < 1 || !rows || N <= 0 || K <= 0 || J < 1 || !known_format(fmt)) return 0;
+    if (!rows || sizes_status(n, N, K, fmt, J) != PQ_OK) return 0;
     const int group = fmt.kind == 0 ? 16 : fmt.group;
     size_t most = 0;
     for (int i = 0; i < n;) {
@@ -45,14 +50,14 @@ extern "C" pq_status pq_calibrate(int n, const void *const *X, const int64_t *ro
                                   double *sumsq_w, float *amax_a, float *ts_x, float *ts_w, int32_t *perms, double *err_x,
                                   double *err_w, double *lambda, double *E, int32_t *select, uint8_t *codes, uint8_t *sf,
                                   void *ws, size_t ws_bytes, void *stream) {
+    const pq_status sizes = sizes_status(n, N, K, fmt, J);
+    PQ_REQUIRE(sizes == PQ_OK, sizes);
+    PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || sf_layout == PQ_SF_TCGEN05, PQ_ERR_FORMAT);
     PQ_REQUIRE(X && rows && ld && Wt && sumsq_a && sumsq_w && amax_a && ts_x && ts_w && perms && err_x && err_w && lambda &&
                    select && codes && sf,
                PQ_ERR_NULL);
-    PQ_REQUIRE(known_format(fmt) && (sf_layout == PQ_SF_LINEAR || sf_layout == PQ_SF_TCGEN05), PQ_ERR_FORMAT);
     const int group = fmt.kind == 0 ? 16 : fmt.group;
-    PQ_REQUIRE(n >= 1 && N > 0 && K > 0 && K % group == 0 && K % 16 == 0 && K <= 16384 && ldw >= K, PQ_ERR_SHAPE);
-    PQ_REQUIRE(sf_layout == PQ_SF_LINEAR || K % 64 == 0, PQ_ERR_SHAPE);
-    PQ_REQUIRE(J >= 1 && J <= 7, PQ_ERR_SHAPE);
+    PQ_REQUIRE(ldw >= K && (sf_layout == PQ_SF_LINEAR || K % 64 == 0), PQ_ERR_SHAPE);
     PQ_REQUIRE(pq_aligned16(Wt) && ldw % 8 == 0 && pq_aligned16(codes) && pq_aligned16(sf), PQ_ERR_ALIGN);
     int64_t rows_a = 0, slabs = pq_ceil_div(N, PQ_SLAB_ROWS);
     for (int i = 0; i < n; ++i) {

@@ -195,8 +195,6 @@ PyObject *calibrate(PyObject *, PyObject *const *a, Py_ssize_t given) {
         const pq_format fmt = {static_cast<int>(integer(a[2])), static_cast<int>(integer(a[3])), static_cast<int>(integer(a[4]))};
         const int J = static_cast<int>(integer(a[5])), layout = static_cast<int>(integer(a[7]));
         const double tau = number(a[6]);
-        const int64_t group = fmt.kind == 0 ? 16 : fmt.group;
-        require(group > 0 && J >= 0, "group and J are positive");
         std::vector<const void *> xs;
         std::vector<int64_t> rows, lds;
         int64_t total = 0;
@@ -212,25 +210,29 @@ PyObject *calibrate(PyObject *, PyObject *const *a, Py_ssize_t given) {
             total += X.size(0);
         }
         const void *w = ptr(W);
-        const auto like = W.options();
-        const auto f64 = like.dtype(at::kDouble), f32 = like.dtype(at::kFloat), i32 = like.dtype(at::kInt), u8 = like.dtype(at::kByte);
-        const int64_t Kg = K / group;
-        at::Tensor out[13] = {at::empty({K}, f64), at::empty({K}, f64), at::empty({K}, f32), at::empty({1}, f32), at::empty({1}, f32),
-                              at::empty({J + 1, K}, i32), at::empty({J + 2, Kg}, f64), at::empty({J + 2, Kg}, f64), at::empty({2}, f64),
-                              at::empty({J + 2}, f64), at::empty({2}, i32), at::empty({N, K / 2}, u8),
-                              at::empty({static_cast<int64_t>(pq_sf_bytes(N, K, layout))}, u8)};
-        const size_t need = pq_calibrate_workspace_bytes(static_cast<int>(n), rows.data(), N, K, fmt, J);
-        at::Tensor scratch = at::empty({static_cast<int64_t>(need > 256 ? need : 256)}, u8);
-        void *o[13], *ws = ptr(scratch), *st = stream();
-        for (int i = 0; i < 13; ++i) o[i] = out[i].data_ptr();
-        const size_t ws_bytes = static_cast<size_t>(scratch.numel());
-        const pq_status s = unlocked([&] {
+        void *o[13], *st = stream();
+        auto call = [&](void *ws, size_t ws_bytes) {
             return pq_calibrate(static_cast<int>(n), xs.data(), rows.data(), lds.data(), w, N, K, ldw, fmt, J, tau, layout,
                                 static_cast<double *>(o[0]), static_cast<double *>(o[1]), static_cast<float *>(o[2]), static_cast<float *>(o[3]),
                                 static_cast<float *>(o[4]), static_cast<int32_t *>(o[5]), static_cast<double *>(o[6]),
                                 static_cast<double *>(o[7]), static_cast<double *>(o[8]), static_cast<double *>(o[9]),
                                 static_cast<int32_t *>(o[10]), static_cast<uint8_t *>(o[11]), static_cast<uint8_t *>(o[12]), ws, ws_bytes, st);
-        });
+        };
+        const size_t need = pq_calibrate_workspace_bytes(static_cast<int>(n), rows.data(), N, K, fmt, J), sf_size = pq_sf_bytes(N, K, layout);
+        if (!need || !sf_size) {  // nothing is allocated for sizes the call refuses (and without a workspace it launches nothing)
+            for (void *&p : o) p = nullptr;
+            return status(call(nullptr, 0));
+        }
+        const auto like = W.options();
+        const auto f64 = like.dtype(at::kDouble), f32 = like.dtype(at::kFloat), i32 = like.dtype(at::kInt), u8 = like.dtype(at::kByte);
+        const int64_t Kg = K / (fmt.kind == 0 ? 16 : fmt.group);
+        at::Tensor out[13] = {at::empty({K}, f64), at::empty({K}, f64), at::empty({K}, f32), at::empty({1}, f32), at::empty({1}, f32),
+                              at::empty({J + 1, K}, i32), at::empty({J + 2, Kg}, f64), at::empty({J + 2, Kg}, f64), at::empty({2}, f64),
+                              at::empty({J + 2}, f64), at::empty({2}, i32), at::empty({N, K / 2}, u8), at::empty({static_cast<int64_t>(sf_size)}, u8)};
+        at::Tensor scratch = at::empty({static_cast<int64_t>(need)}, u8);
+        void *ws = ptr(scratch);
+        for (int i = 0; i < 13; ++i) o[i] = out[i].data_ptr();
+        const pq_status s = unlocked([&] { return call(ws, need); });
         if (s != PQ_OK) return status(s);
         PyObject *t = PyTuple_New(14);
         if (!t) return nullptr;

@@ -265,7 +265,9 @@ pq_status pq_quant_weight(const void *Wt, int64_t N, int64_t K, int64_t ld, cons
  *                 fp64 [K], amax_a fp32 [K], ts_x, ts_w fp32 scalars, perms int32 [J+1, K], err_x, err_w
  *                 fp64 [J+2, K/g] (row 0 = original order), lambda fp64 [2], E fp64 [J+2] or NULL,
  *                 select int32 [2] = {best, accept}, codes / sf of the weight in the chosen order.
- *   ws          : pq_calibrate_workspace_bytes(n, rows, N, K, fmt, J), 256-byte aligned (0 on bad input). */
+ *   ws          : pq_calibrate_workspace_bytes(n, rows, N, K, fmt, J), 256-byte aligned (0 on bad input): partial sums,
+ *                 (J + 2) K/g * 32 bytes or K * 12 per 128 rows, whichever is more.  The tensors are taken in rounds
+ *                 of 64 MiB of them, so that is the most for any number of batches, or what the largest tensor takes. */
 size_t pq_calibrate_workspace_bytes(int n, const int64_t *rows, int64_t N, int64_t K, pq_format fmt, int J);
 pq_status pq_calibrate(int n, const void *const *X, const int64_t *rows, const int64_t *ld, const void *Wt,
                        int64_t N, int64_t K, int64_t ldw, pq_format fmt, int J, double tau, int sf_layout,

@@ -11,13 +11,35 @@
 namespace {
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
-// Batches [i, end) of one round: as many as a list holds; the weight closes the last list.
-int round_end(int i, int n) { return n - i < kPqListMax ? n : i + kPqListMax; }
+// The batches of a round and whether the weight closes it: as many tensors as a list holds and as the partial sums have room
+// for, one at least.  Without the second limit the sums of up to 64 tensors lie side by side, 400 MB for 64 batches of
+// 4608 x 12288; 64 MiB hold the sums of 600 million elements in NVFP4, whose pass takes milliseconds.
+constexpr size_t kPartialBytes = 64u << 20;
+struct Round {
+    int end;
+    bool with_weight;
+    int64_t slabs;
+};
+Round next_round(int i, int n, const int64_t *rows, int64_t N, int64_t most) {
+    Round r{i, false, 0};
+    int count = 0;
+    for (; r.end < n && count < kPqListMax; ++r.end, ++count) {
+        const int64_t slabs = rows[r.end] > 0 ? pq_ceil_div(rows[r.end], PQ_SLAB_ROWS) : 0;
+        if (count && r.slabs + slabs > most) break;
+        r.slabs += slabs;
+    }
+    const int64_t slabs = pq_ceil_div(N, PQ_SLAB_ROWS);
+    r.with_weight = r.end == n && count < kPqListMax && (!count || r.slabs + slabs <= most);
+    if (r.with_weight) r.slabs += slabs;
+    return r;
+}
 
 size_t partial_bytes(int64_t slabs, int64_t K, int group, int P) {
     const size_t a = pq_stats_list_bytes(slabs, K), b = pq_errors_list_bytes(slabs, K, group, P);
     return round256(a > b ? a : b);
 }
+int64_t slabs_per_round(int64_t K, int group, int P) { return static_cast<int64_t>(kPartialBytes / partial_bytes(1, K, group, P)); }
+
 // What can be told from the sizes alone; the caller's outputs and the workspace are sized by these.
 pq_status sizes_status(int n, int64_t N, int64_t K, pq_format fmt, int J) {
     PQ_REQUIRE(fmt.kind == 0 || (fmt.kind == 1 && fmt.bits >= 2 && fmt.bits <= 8 &&
@@ -33,13 +55,11 @@ pq_status sizes_status(int n, int64_t N, int64_t K, pq_format fmt, int J) {
 extern "C" size_t pq_calibrate_workspace_bytes(int n, const int64_t *rows, int64_t N, int64_t K, pq_format fmt, int J) {
     if (!rows || sizes_status(n, N, K, fmt, J) != PQ_OK) return 0;
     const int group = fmt.kind == 0 ? 16 : fmt.group;
+    const int64_t limit = slabs_per_round(K, group, J + 1);
     size_t most = 0;
-    for (int i = 0; i < n;) {
-        // the weight may ride with the last batches or, where they fill a list, come alone: room for either
-        const int end = round_end(i, n);
-        int64_t slabs = pq_ceil_div(N, PQ_SLAB_ROWS);
-        for (; i < end; ++i) slabs += rows[i] > 0 ? pq_ceil_div(rows[i], PQ_SLAB_ROWS) : 0;
-        const size_t b = partial_bytes(slabs, K, group, J + 1);
+    for (Round r{0, false, 0}; !r.with_weight;) {
+        r = next_round(r.end, n, rows, N, limit);
+        const size_t b = partial_bytes(r.slabs, K, group, J + 1);
         if (b > most) most = b;
     }
     return most + round256(static_cast<size_t>(K) * sizeof(float));
@@ -73,15 +93,18 @@ extern "C" pq_status pq_calibrate(int n, const void *const *X, const int64_t *ro
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float *amax_w = reinterpret_cast<float *>(static_cast<unsigned char *>(ws) + need - round256(static_cast<size_t>(K) * sizeof(float)));
 
+    const int64_t limit = slabs_per_round(K, group, J + 1);
     // f(list, first round, the weight is in the list) for every round of tensors
     auto each_round = [&](auto &&f) -> pq_status {
-        for (int i = 0, w = 0; !w;) {
+        for (Round r{0, false, 0}; !r.with_weight;) {
             PqTensorList list;
+            int i = r.end;
             const bool first = i == 0;
-            for (const int end = round_end(i, n); i < end; ++i) list.add(X[i], rows[i], ld[i]);
+            r = next_round(i, n, rows, N, limit);
+            for (; i < r.end; ++i) list.add(X[i], rows[i], ld[i]);
             list.n_x = list.n;
-            if (i == n && list.n < kPqListMax) list.add(Wt, N, ldw), w = 1;
-            const pq_status rc = f(list, first, w != 0);
+            if (r.with_weight) list.add(Wt, N, ldw);
+            const pq_status rc = f(list, first, r.with_weight);
             if (rc != PQ_OK) return rc;
         }
         return PQ_OK;

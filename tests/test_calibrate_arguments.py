@@ -44,6 +44,17 @@ def test_workspace_size_of_bad_sizes_is_zero():
     assert [size(n=0), size(N=0), size(K=0), size(kind=2), size(J=0), size(J=8), size(J=10 ** 9)] == [0] * 7
 
 
+@pytest.mark.parametrize("rows,N,K,group,J", [([4608] * 64, 9216, 12288, 16, 7), ([4608] * 64, 3072, 3072, 16, 5), ([18432] * 200, 12288, 3072, 64, 5),
+                                              ([200000, 5], 64, 3072, 16, 5), ([5, 200000], 64, 16384, 256, 1)])
+def test_workspace_does_not_grow_with_the_number_of_batches(rows, N, K, group, J):
+    """64 MiB of partial sums are enough for any number of batches, or what the largest tensor takes alone."""
+    build.build()
+    L, fmt = B.lib(), B.pq_format(B.KIND_INT, 4, group)
+    size = lambda r, n_rows: L.pq_calibrate_workspace_bytes(len(r), (C.c_int64 * len(r))(*r), n_rows, K, fmt, J)
+    alone = max(size([max(rows)], 1), size([1], N))
+    assert size(rows, N) <= max((64 << 20) + 4 * K + 256, alone)
+
+
 gpu = pytest.mark.gpu
 
 

@@ -105,3 +105,15 @@ def test_one_call_equals_the_separate_calls(rows, N, K, fmt, J):
     assert c.rows_a == sum(rows)
     for name, t in want.items():
         assert torch.equal(getattr(c, name), t), name
+
+
+@pytest.mark.parametrize("n", [40, 26])      # 1440 slabs in two rounds; 936 in one, and the weight in one of its own
+def test_rounds_of_many_slabs_equal_the_separate_calls(n):
+    """More partial sums than one round's 64 MiB hold (1213 slabs of these widths)."""
+    g = torch.Generator(device=DEV).manual_seed(n)
+    x = torch.randn(4608, 3072, generator=g, device=DEV).mul_(3).to(torch.bfloat16)
+    W = torch.randn(36864, 3072, generator=g, device=DEV).to(torch.bfloat16)
+    batches = [x] * n
+    c = pipeline.calibrate(batches, W, J=7)
+    for name, t in separate_calls(batches, W, pipeline.NVFP4, 7, 0.0).items():
+        assert torch.equal(getattr(c, name), t), name

@@ -14,7 +14,7 @@
 //   candidate orders: persistent blocks of thread groups; a group stages a chunk's rows in shared memory four at a time,
 //     interleaved per channel, for all orders of its share of the (chunk, order) pairs, and a lane gathers the 16 channels
 //     of its run for four rows with 64-bit loads, two rows side by side in packed registers; the tensor is fetched from HBM
-//     about once.
+//     about once.  Few (chunk, order) pairs go to one block each instead (group_error_chunk).
 #include <type_traits>
 
 #include "pq_common.cuh"
@@ -22,6 +22,7 @@
 namespace {
 
 // ---------------------------------------------------------------- original order
+constexpr int64_t kErrMaxK = 16384;
 constexpr int kDirectThreads = 128;
 constexpr int kDirectRows = 4;  // rows in flight per thread (2 x 16 bytes each)
 
@@ -477,6 +478,95 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     }
 }
 
+// ---------------------------------------------------------------- candidate orders, few pairs
+// One block per (chunk, order), several per SM.  The chunk goes through shared memory four rows at a time, interleaved per
+// channel as above; a thread owns whole 16-channel runs (GPT of them, blockDim apart), keeps their slots packed in registers,
+// and for every row rebuilds the two 16-byte words the original-order kernel loads, so the error of a run is computed by
+// the same routine, in row order.  It prepares no tables, and the blocks of an SM fill each other's waits; what it costs is
+// staging the chunk once per order.  While its blocks are all resident at once it is the faster one (chunk_kernel_serves).
+constexpr int kChunkThreads = 256, kChunkMaxGpt = 4;  // 256 threads x 4 runs x 16 channels = 16384 channels
+
+// one run per thread (up to 4096 channels): held to 64 registers, five 192-thread blocks per SM instead of four
+template <int KIND, int TEAM16, int GPT>
+__global__ void __launch_bounds__(kChunkThreads, GPT == 1 ? 4 : 1)
+group_error_chunk(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int64_t ld,
+                  const float *__restrict__ ts_ptr, float Qf, const int32_t *__restrict__ perms, int P,
+                  float *__restrict__ part /*[chunks, P, K/g]*/) {
+    extern __shared__ __align__(16) uint16_t quad_s[];  // [K][4 rows]
+    __shared__ float2 scale_table[KIND == 0 ? 256 : 1];
+    pq::dependents_may_launch();
+    const int64_t chunk = blockIdx.x;
+    const int p = blockIdx.y;
+    const int32_t *perm = perms + static_cast<int64_t>(p) * K;
+    const int octs = static_cast<int>(K >> 3), runs = static_cast<int>(K >> 4);
+    const int64_t r0 = chunk * PQ_CHUNK_ROWS;
+    const float ts = (KIND == 0) ? __ldg(ts_ptr) : 1.0f;
+    const float c6 = __fmul_rn(6.0f, ts);
+    if (KIND == 0) build_scale_table(scale_table, ts);  // the first barrier below publishes it
+
+    // positions of this thread's channels in the interleaved image, two per register
+    uint32_t ch[GPT][8];
+    float acc[GPT];
+#pragma unroll
+    for (int t = 0; t < GPT; ++t) {
+        acc[t] = 0.0f;
+        const int q = threadIdx.x + t * blockDim.x;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            uint32_t lo = 0, hi = 0;
+            if (q < runs) {
+                lo = pq::quad_channel(static_cast<uint32_t>(perm[q * 16 + 2 * w]));
+                hi = pq::quad_channel(static_cast<uint32_t>(perm[q * 16 + 2 * w + 1]));
+            }
+            ch[t][w] = lo | (hi << 16);
+        }
+    }
+
+    uint4 *quad4 = reinterpret_cast<uint4 *>(quad_s);
+    const uint2 *quad2 = reinterpret_cast<const uint2 *>(quad_s);
+#pragma unroll 1
+    for (int quad = 0; quad < PQ_CHUNK_ROWS / 4; ++quad) {
+        const int64_t row = r0 + 4 * quad;
+        if (row >= rows) break;  // no rows left: their error is +0.0
+        __syncthreads();         // the previous four rows have been used
+        for (int o = threadIdx.x; o < octs; o += blockDim.x) {
+            uint4 v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)  // rows past the end are zeros: their error is +0.0 and adding it changes nothing
+                v[r] = row + r < rows ? __ldg(reinterpret_cast<const uint4 *>(T + (row + r) * ld) + o) : make_uint4(0, 0, 0, 0);
+            pq::store_quad_octet(quad4, o, v);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int t = 0; t < GPT; ++t) {
+            if (t * static_cast<int>(blockDim.x) >= runs) break;  // uniform over the block
+            uint2 g[16];
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                g[2 * w] = quad2[ch[t][w] & 0xFFFFu];
+                g[2 * w + 1] = quad2[ch[t][w] >> 16];
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                uint32_t pr[8];
+#pragma unroll
+                for (int w = 0; w < 8; ++w) {
+                    const uint32_t a = r < 2 ? g[2 * w].x : g[2 * w].y, b = r < 2 ? g[2 * w + 1].x : g[2 * w + 1].y;
+                    pr[w] = __byte_perm(a, b, (r & 1) ? 0x7632 : 0x5410);
+                }
+                acc[t] = __fadd_rn(acc[t], row_sse16<KIND, TEAM16>(make_uint4(pr[0], pr[1], pr[2], pr[3]),
+                                                                   make_uint4(pr[4], pr[5], pr[6], pr[7]), c6, scale_table, Qf));
+            }
+        }
+    }
+    const int64_t Kg = runs / TEAM16;
+#pragma unroll
+    for (int t = 0; t < GPT; ++t) {
+        const int q = threadIdx.x + t * blockDim.x;
+        if (q < runs && (q % TEAM16) == 0) part[(chunk * P + p) * Kg + q / TEAM16] = acc[t];
+    }
+}
+
 // Orders per block, groups per block and threads per group for `chunks` chunks of K channels under P orders:
 // the configuration with the shortest estimated schedule.  A group works through its share of the (chunk, order)
 // pairs; a pair costs one unit per run of each lane, a chunk a quarter of a unit of staging per run (and a share
@@ -515,6 +605,19 @@ int sm_count() {
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return sms;
+}
+
+int chunk_threads(int64_t K) {
+    const int64_t runs = K / 16;
+    return static_cast<int>(runs >= kChunkThreads ? kChunkThreads : pq_ceil_div(runs, 32) * 32);
+}
+// Few (chunk, order) pairs: all blocks of the kernel for them resident at once.  One block per chunk and order / thread groups
+// with tables, us with the fold, NVFP4: 37 x 3072 3 orders 12.6 / 21.5, 512 x 6400 3 orders 20.9 / 28.9, 4608 x 768 3 orders (864
+// pairs) 20.4 / 27.5, 4608 x 6400 1 order (288) 36.3 / 63.9, 512 x 16384 3 orders (96) 37.7 / 48.4; past the line
+// 4608 x 768 6 orders (1728) 29.2 / 25.9, 1357 x 6400 6 orders (510) 53.1 / 51.7, 512 x 16384 6 orders (192) 66.4 / 61.1,
+// 4608 x 12288 8 orders 540 / 237.  704 threads of it per SM; above 8192 channels one block, by registers and shared memory.
+bool chunk_kernel_serves(int64_t pairs, int64_t K) {
+    return pairs <= static_cast<int64_t>(sm_count()) * (K > 2 * 16 * kChunkThreads ? 1 : 704 / chunk_threads(K));
 }
 
 template <typename PT, int PER_SLAB>
@@ -561,6 +664,18 @@ pq_status launch(const uint16_t *T, int64_t rows, int64_t K, int64_t ld, const f
         if (pq_launch_status() != PQ_OK) return PQ_ERR_CUDA;
         return fold<double, 1>(ws, slabs, Kg, err, st);
     }
+    if (chunk_kernel_serves(chunks * P, K)) {
+        const int runs = static_cast<int>(K >> 4), threads = chunk_threads(K);
+        const size_t smem = static_cast<size_t>(K) * 8;  // four rows, interleaved per channel
+        const dim3 grid(static_cast<unsigned>(chunks), static_cast<unsigned>(P));
+        auto kern = runs <= threads       ? group_error_chunk<KIND, TEAM / 2, 1>
+                    : runs <= 2 * threads ? group_error_chunk<KIND, TEAM / 2, 2>
+                                          : group_error_chunk<KIND, TEAM / 2, kChunkMaxGpt>;
+        PQ_CUDA_OK(pq::allow_smem(kern, smem, kErrMaxK * 8, 4096));
+        kern<<<grid, threads, smem, st>>>(T, rows, K, ld, ts, Qf, perms, P, static_cast<float *>(ws));
+        if (pq_launch_status() != PQ_OK) return PQ_ERR_CUDA;
+        return fold<float, kSlabChunks>(ws, chunks, static_cast<int64_t>(P) * Kg, err, st);
+    }
     GatherParams p;
     p.list.add(T, rows, ld);
     p.list.n_x = 1;
@@ -599,7 +714,7 @@ extern "C" pq_status pq_group_error(const void *T, int64_t rows, int64_t K, int6
     } else {
         PQ_REQUIRE(ts, PQ_ERR_NULL);
     }
-    PQ_REQUIRE(rows > 0 && K > 0 && K % group == 0 && K <= 16384 && ld >= K, PQ_ERR_SHAPE);
+    PQ_REQUIRE(rows > 0 && K > 0 && K % group == 0 && K <= kErrMaxK && ld >= K, PQ_ERR_SHAPE);
     PQ_REQUIRE(P >= 1 && P <= 8 && (perms || P == 1), PQ_ERR_SHAPE);
     PQ_REQUIRE(pq_aligned16(T) && ld % 8 == 0, PQ_ERR_ALIGN);
     const int64_t chunks = pq_ceil_div(rows, PQ_CHUNK_ROWS);

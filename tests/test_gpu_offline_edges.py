@@ -50,6 +50,18 @@ def test_candidate_errors_match_the_original_order_on_gathered_columns(rows, K, 
         assert np.array_equal(got[p], errors(x[:, perms[p].long()].contiguous(), fmt, tsd, None)[0], equal_nan=True)
 
 
+@pytest.mark.parametrize("fmt", [(B.KIND_NVFP4, 4, 16), (B.KIND_INT, 3, 32), (B.KIND_INT, 4, 64), (B.KIND_INT, 8, 256)])
+@pytest.mark.parametrize("rows,K,P", [(6501, 512, 8), (6550, 512, 8), (912, 3072, 8), (900, 3072, 7), (901, 6400, 8), (288, 16384, 8), (294, 16384, 8)])
+def test_candidate_errors_around_the_number_of_pairs_where_kernels_change(rows, K, P, fmt):
+    """Both kernels of the candidate orders (pairs of 16-row chunks and orders on either side of the line on 148 SMs) against
+    the original-order kernel on gathered columns."""
+    x, ts = tensor_with_edges(rows, K, rows + K), torch.tensor([0.01], device=DEV)
+    perms = torch.stack([torch.randperm(K, generator=torch.Generator().manual_seed(p)) for p in range(P)]).to(DEV, torch.int32)
+    got = errors(x, fmt, ts, perms)
+    for p in range(P):
+        assert np.array_equal(got[p], errors(x[:, perms[p].long()].contiguous(), fmt, ts, None)[0], equal_nan=True)
+
+
 @pytest.mark.parametrize("K", [8, 1024, 1032, 3080, 8192, 8200, 16384])
 def test_orders_with_ties_across_chunks(K):
     rng = np.random.default_rng(K)

@@ -816,8 +816,13 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
 // One round of narrow tiles covers the product.  Measured on both sides of the line (narrow against wide, us):
 // 128 x 3072 x 3072 6.9 / 8.1, 512 x 3072 x 3072 7.4 / 8.3, 512 x 3072 x 12288 18.0 / 20.5; beyond one round the wide tile wins:
 // 512 x 9216 x 3072 12.2 / 10.9, 1024 x 3072 x 3072 11.2 / 9.4, 4608 x 9216 x 3072 72.8 / 56.9.
-bool narrow_tiles(int64_t M, int64_t N, int pairs) {
-    return pq_ceil_div(M, BM) * pq_ceil_div(N, 128) <= pairs;
+// Few rows: the CTAs of all pairs fetch the same few lines of X at every K step, and with more than half of the pairs at that the
+// narrow tile loses for one or two rows (1 x 5120 x 3072 8.6 / 7.6, 1 x 9216 x 12288 25.6 / 21.9, 2 x 7168 x 12288 21.0 / 18.3) and
+// for up to 16 on long rows (4 x 8192 x 12288 21.7 / 19.7); 8 x 5120 x 3072 7.2 / 8.0, 24 x 9216 x 12288 17.9 / 20.1.
+bool narrow_tiles(int64_t M, int64_t N, int64_t K, int pairs) {
+    const int64_t tiles = pq_ceil_div(M, BM) * pq_ceil_div(N, 128);
+    const bool few = M <= 2 || (M <= 16 && K > 3072);
+    return tiles <= (few ? pairs / 2 : pairs);
 }
 
 pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, const uint8_t *wq, const uint8_t *sfw,
@@ -836,7 +841,7 @@ pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, 
     const int pairs_max = resident_pairs<256>(), pairs_narrow = resident_pairs<128>();
     if (pairs_max <= 0 || pairs_narrow <= 0) return PQ_ERR_CUDA;
     const GemmArgs g{xq, sfx, wq, sfw, ts_x, ts_w, M, N, K, ldy, Y, ws, st};
-    return narrow_tiles(M, N, pairs_narrow) ? launch_tiles<128>(g, pairs_narrow) : launch_tiles<256>(g, pairs_max);
+    return narrow_tiles(M, N, K, pairs_narrow) ? launch_tiles<128>(g, pairs_narrow) : launch_tiles<256>(g, pairs_max);
 }
 }  // namespace
 

@@ -20,3 +20,8 @@ def test_exact_at_the_line(M, N, K):
     sfx, sfw = pow2[rng.integers(0, 4, (M, K // 16))], pow2[rng.integers(0, 4, (N, K // 16))]
     Y = gemm(pack(xn), sfx, 0.5, pack(wn), sfw, 4.0, ldy=N + 8)
     assert np.array_equal(Y, bf16_round(O.gemm_ref(pack(xn), sfx, 0.5, pack(wn), sfw, 4.0)))
+
+
+@pytest.mark.parametrize("M,N,K", [(2, 4736, 128), (2, 4744, 320), (3, 4744, 128), (1, 9472, 192), (16, 4744, 3136), (17, 4744, 3136)])   # 37 and 38 narrow tiles, few rows
+def test_few_rows_at_the_line(M, N, K):
+    test_exact_at_the_line(M, N, K)

@@ -182,11 +182,14 @@ group_error_direct(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int6
 // Blocks are persistent, one per SM; the groups of a block only share the slot and scale tables.
 //
 // NVFP4 is scalar arithmetic: packed f32x2 instructions save issue slots but run on one of the two FMA pipes only, and
-// with the f16 converts there too it was 59 % busy (9216 x 3072, six orders: 79 us scalar, 84 packed).  The integer
-// formats, without converts, are packed (4608 x 3072, INT4 g64: 53.4 us, 54.1 scalar).
-// What bounds it: shared-memory wavefronts (a 64-bit gather through a random order takes about 6 of them
-// where 2 would do: 0.05 per element) and instruction issue, in about equal parts.
-constexpr int kGatherThreads = 768;  // 80 registers per thread; 960 threads at 64 spill
+// with the f16 converts there too it was 59 % busy (9216 x 3072, six orders, with the fold of that time: 79 us scalar, 84
+// packed; 74 with the present fold).  The integer formats, without converts, are packed (4608 x 3072, INT4 g64: 53.4 us,
+// 54.1 scalar; 50.1 with the present fold).
+// What bounds it: instruction issue (67 % of the slots busy at 23 warps per SM) and shared-memory wavefronts (a 64-bit gather
+// through a random order takes about 6 of them where 2 would do: 0.069 per element and order).
+// Registers: 72 per thread, of which 56 to 92 bytes are spilled: the launch bounds count the one more warp that adds up the error
+// weights, 800 threads.  At 768 the compiler takes 80 and spills 48 to 52 bytes; not timed.  960 threads at 64 spill more.
+constexpr int kGatherThreads = 768;
 constexpr int kMaxOrders = 9;      // eight candidates and the original order
 constexpr int kMaxGroups = 15;                                           // named barriers 1..15
 constexpr int kSfTabMax = 2624;  // bf16 magnitudes from "scale byte 0" to "saturated": 19 binades and the edges
@@ -407,7 +410,7 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     // An equal part of the (chunk, order) pairs of the first p.split chunks, then p.full whole chunks.  Without the first
     // part a group that has work for a few chunks only would wait for the one that has a whole chunk more; without the
     // second a group would stage one more chunk of which it uses some orders (eight batches of 4608 x 3072 and a
-    // 9216 x 3072 weight: 535 us a calibration all in pairs, 518 like this).
+    // 9216 x 3072 weight: 535 us a calibration all in pairs, 518 like this; 473 with the present fold).
     const uint32_t shares = gridDim.x * p.groups, share = blockIdx.x * p.groups + grp;
     const uint32_t base = p.base[o0 + no == p.P], rem = p.rem[o0 + no == p.P];
     const uint32_t first = share * base + min(share, rem);

@@ -475,10 +475,12 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
 // order of every floating-point operation is that of the one-row kernel.
 // What bounds it: instruction issue at 20-24 warps per SM (ncu: issue slots 58 % busy, stalls on shared memory,
 // fixed latencies and barriers).  Several small blocks share an SM and drift apart, so that some wait for memory while
-// others compute.  RMSNorm / adaptive LayerNorm, us, against the kernel above: 512 x 3072 4.5 / 6.0 against 10.6 / 13.4,
-// 4608 x 6144 35.0 / 46.2 against 42.9 / 53.7; 2304 x 12288 35.9 / 45.8 against 69.5 / 81.5 one row per warp; but
-// 4608 x 3072 17.8 / 22.3 against 17.4 / 21.9 and 4608 x 1088 11.2 / 13.9 against 10.3 / 12.3.  Without a norm: 4608 x 3072
-// 12.7 against 14.4, 18432 x 3072 37.7 against 49.4.
+// others compute.  RMSNorm / adaptive LayerNorm, us from HBM, against the kernel above: 512 x 3072 5.1 / 6.0 against
+// 10.8 / 13.5, 2304 x 3072 10.4 / 12.5 against 12.1 / 14.8; 4608 x 3072 18.1 / 22.0 against 17.3 / 21.6, 4608 x 1088
+// 10.9 / 13.5 against 9.4 / 11.4, 4608 x 512 8.4 / 10.5 against 5.2 / 6.3; but 3072 x 3072 15.0 / 19.1 against 16.3 / 20.5 and
+// 9216 x 3072 31.8 / 39.1 against 32.5 / 41.4, where the rule below still takes the kernel above.  4608 x 6144 35.5 / 44.6,
+// 2304 x 12288 34.0 / 45.4 (69.5 / 81.5 one row per warp).  The adaptive-LayerNorm instances spill 104 to 148 bytes at 80 registers.
+// Without a norm: 4608 x 3072 13.1, 18432 x 3072 41.0 (14.4, 49.4 with the sixteen-row kernel of that time).
 template <int KIND, int SF_LAYOUT, int ITER>  // ITER = groups per lane
 __global__ void __maxnreg__(kQuadRegs)
 norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
@@ -807,7 +809,8 @@ pq_status launch(const uint16_t *H, int64_t M, int64_t rows_pad, int K, int64_t 
         return pq_launch_status();
     }
     // several rows per warp while two blocks of sixteen rows fit on an SM and there is one for every SM at least;
-    // otherwise four rows per block (measurements at that kernel)
+    // otherwise four rows per block (both sides measured at that kernel: right up to 2304 rows and at 4608, up to 8 % off at
+    // 2368 to 3072 rows and at 9216)
     const size_t group_smem = static_cast<size_t>(kGroupWarps) * kGroupRows * K * 2;
     const int64_t group_blocks = pq_ceil_div(rows_pad, kGroupWarps * kGroupRows);
     if (group_smem <= kGroupSmemMax && group_blocks >= sms) {

@@ -6,49 +6,53 @@
 // 256 x 256, persistent over the tile list: tcgen05.mma.cta_group::2 lets each CTA hold 128 rows
 // of the accumulator while the B operand is split between the two shared memories, so a CTA
 // fetches 128 rows of X codes and 128 rows of W codes per 256-channel K step (38 KB with the
-// scales, for 512 cycles of MMA).  What bounds the main loop is the rate at which the SMs can take
-// operands in from L2 (about 70 bytes per clock each when all of them pull), so the tile is as
-// large as tensor memory allows.  Roles of the 18 warps of a CTA:
-//   warp 0       producer: TMA loads of the packed E2M1 operand tiles (128-byte swizzle) and bulk
-//                copies of the scale-factor blocks into a 5-stage shared-memory ring.  Operand
-//                loads of both CTAs signal the pair leader's barrier (cp.async.bulk.tensor with
-//                .cta_group::2).
-//   warp 1       (leader CTA) issues tcgen05.mma.kind::mxf4nvf4.block_scale, K = 64 per instruction,
-//                4 per stage, into the 256-column fp32 accumulator in tensor memory.
+// scales, for 512 cycles of MMA).  Roles of the 10 warps of a CTA:
+//   warp 0       producer: TMA loads of the packed E2M1 operand tiles (128-byte swizzle) and of the
+//                scale-factor blocks into a 5-stage shared-memory ring.  The loads of both CTAs signal
+//                the pair leader's barrier (cp.async.bulk.tensor with .cta_group::2).
+//   warp 1       (leader CTA) copies the stage's scale blocks of both CTAs to tensor memory (tcgen05.cp) and
+//                issues tcgen05.mma.kind::mxf4nvf4.block_scale, K = 64 per instruction, 4 per stage, into the
+//                256-column fp32 accumulator in tensor memory.
 //   warps 2..9   epilogue (lane quadrant x column half): tcgen05.ld the finished accumulator (own
 //                CTA's 128 rows) 16 columns at a time, scale by ts_x*ts_w, round to bf16 and keep the
 //                32 x 128 piece as 64 packed registers; hand the accumulator back; then stage 32 x 64
 //                boxes in swizzled shared memory and write them with TMA stores (full 128-byte
-//                lines) while the next tile's main loop runs.
-//   warps 10..17 scale-factor stagers: read the stage's scale blocks from shared memory and write
-//                them into one of the scale slots in tensor memory with tcgen05.st (one warp per
-//                lane quadrant; two sets of four warps take alternate K iterations).
+//                lines), spread over the next tile's main loop.
 // 256 divides every FLUX output width (3072, 9216, 12288).  The 512 tensor-memory columns hold one
-// 256-column accumulator plus three scale slots (3 x 48); the epilogue warps pull the accumulator
-// into registers as packed bf16 within a few hundred cycles and store it from there.
+// 256-column accumulator plus a scale slot of 48 columns per stage.
 //
-// Measurements on B200 behind these choices:
-//   - a tcgen05.cp of one 512-byte scale block occupies the tensor pipe for about 80 cycles and
-//     twelve are needed per stage, more than the stage's four MMAs (384 cycles); the register path
-//     (ld.shared + tcgen05.st, 7 to 16 cycles per store) costs the pipe nothing;
-//   - TMA and tcgen05 instructions take their operands from uniform registers.  Issued from a
-//     divergent single-lane loop (`if (lane == 0) for (...)`) every operand is moved there one by
-//     one and an MMA costs about 190 cycles of issue time instead of 96; the producer and the MMA
-//     issuer therefore run their loops with the whole warp and single out one lane with
-//     elect.sync only around those instructions;
+// What bounds it.  The main loop runs at 523 cycles per stage of 512 MMA cycles: waiting for the stage, issuing
+// (about 340 cycles, a tcgen05.cp about 6 and an MMA about 50 of them) and the loop around it take that long, and a
+// stage's loads land 700 to 1000 cycles after they were asked for with 2500 to spare.  A tile boundary costs about
+// 1000 cycles (the last stage's MMAs, the read-out, the signals).  At that rate the chip is at its power limit:
+// 1.55 GHz of 1.965.
+//
+// Measurements on B200 behind these choices (4608 x 3072 x 9216 / 4608 x 12288 x 3072 / 18432 x 3072 x 12288, us):
+//   - scales by tcgen05.cp from the issuing warp 52.8 / 59.6 / 275; by eight more warps through registers (ld.shared +
+//     tcgen05.st, three slots, 96 registers a thread) 55.9 / 62.7 / 289;
+//   - stores spread over the next main loop (kPaceCycles, 30 to 32) 50.7 / 59.0 / 255.  All SMs finish their tiles together, and
+//     while 16 stores of each went out at once the loads behind them took 2000 to 3500 cycles to land: the ring ran dry
+//     for three or four stages of every tile.  24 cycles per box and stage 51.2 / 59.0 / 264, 14: 53.3 / 59.0 / 276,
+//     40: 52.6 / 61.1 / 268 (the last store is then later than the next tile);
+//   - two accumulators that overlap by 144 columns, so that a tile starts when those have been read: 51.4 / 59.0 / 265
+//     against 51.2 / 59.0 / 264, not worth the fewer scale slots; four stages 53.3 / 62.5 / 271;
+//   - tiles walked in groups of 6 to 16 rows of tiles: no better (50.9 to 51.1 / 59.1 to 59.4 / 257);
+//   - TMA and tcgen05 instructions take their operands from uniform registers.  The issuing warps run their loops with
+//     the whole warp, with the warp index from a shuffle so that the branch is known to be uniform, and single out one
+//     lane with elect.sync around those instructions.  Predicated instructions instead of that branch: 56.1 / 67.6 / 283;
+//   - all copies of a stage in front of its MMAs: 512 x 3072 x 3072 6.6, copies and MMAs in turn 6.9;
 //   - a remote mbarrier arrive with cluster-scope release semantics costs 500 to 2500 cycles;
 //     what the arrivals here publish has already completed (tcgen05.wait) when they are issued,
 //     so the default semantics are used.
 //
 // Scale factors live in global memory in 512-byte blocks of 128 rows x 4 groups (see pq.h); a
 // block occupies 4 tensor-memory columns (row r of the block -> lane r%32, column r/32, the same
-// in all four lane quadrants), which is the layout the MMA reads: lane l of every stager warp
-// loads the 16 bytes at offset 16 l of the block and stores them as columns of its quadrant.
+// in all four lane quadrants), which is the layout the MMA reads and what tcgen05.cp.32x128b.warpx4 makes of it.
 // The 256 B-scale rows of a tile are two whole blocks: 8 columns per K block.
 //
-// Cross-CTA signalling uses plain remote mbarrier arrives and, for the completion of a stage's
-// MMAs and of a tile's accumulator, one tcgen05.commit per CTA (issued by the pair leader's MMA
-// warp onto each CTA's own copy of the barrier).  Every wait on an mbarrier is bounded.  If one
+// Completion of a stage's MMAs and of a tile's accumulator is one tcgen05.commit by the pair leader's MMA warp, onto
+// both CTAs' copies of the barrier; the epilogue warps hand the accumulator back by plain remote arrives.
+// Every wait on an mbarrier is bounded.  If one
 // expires the CTA records PQ_ERR_TIMEOUT in the status word, raises a shared abort flag that every role polls,
 // and falls through to the common teardown (cluster barrier, tensor-memory release).
 #include <cuda.h>
@@ -70,38 +74,18 @@ constexpr int kEpiWarps = 8;               // lane quadrant x column half of the
 constexpr int kBoxCols = 64;               // output staging box: 32 rows x 64 bf16, one TMA store
 constexpr int kEpiBox = 32 * kBoxCols * 2;
 constexpr int kEpiBytes = kEpiWarps * kEpiBox;      // one staging box per epilogue warp: 32 KB
-constexpr int kStagerSets = 2;             // sets of four stager warps taking alternate K iterations
-constexpr int kFirstStager = 2 + kEpiWarps;
-constexpr int kThreads = 32 * (kFirstStager + 4 * kStagerSets);   // producer, MMA issuer, 8 epilogue and 8 stager warps
-// One 256-column accumulator, then the scale slots.  A slot holds the scales of one stage: per 64-channel
-// K block 4 columns of A scales (128 rows) and 8 columns of B scales (256 rows).  Slot it % kSfSlots
-// serves iteration it; it is rewritten only after the MMAs of iteration it - kSfSlots have completed
-// (their commit releases that iteration's stage).
+// SM clock cycles per K step between the stores of a tile's 2 * kEpiWarps boxes: the last one starts at 15 / 17 of the
+// next tile's main loop.
+constexpr int kPaceCycles = 30;
+constexpr int kThreads = 32 * (2 + kEpiWarps);      // producer, MMA issuer, 8 epilogue warps
+// One 256-column accumulator, then the scale slots, one per stage: per 64-channel K block 4 columns of A scales (128
+// rows) and 8 columns of B scales (256 rows).  A slot is written after the wait for its stage's data, which the producer
+// asked for only when the MMAs that read the stage (and the slot) before had completed.
 //
-// Why the slot count is tied to the stage count.  Every wait here is a PARITY wait: it tells "phase n
-// of this barrier has completed" from "it has not" only if the barrier cannot still be in phase n - 1,
-// i.e. only if the waiter already knows that phase n - 1 has completed.  A role that waits on every
-// phase of a barrier in turn (producer on stage_free, MMA issuer on stage_full and acc_empty, each
-// epilogue warp on acc_full) knows it from its own previous wait.  The stagers do not: the stage
-// count is odd and the two stager sets take alternate iterations, so the previous phase of
-// sf_ready(s), iteration it - kStages, was waited for by the OTHER set.  What a set knows when it
-// reaches iteration `it` is what its own iteration it - kStagerSets waited for: the MMAs of
-// it - kStagerSets - kSfSlots have completed.  Those of it - kStages (hence that iteration's scale
-// copies, which its stagers had to see before its MMAs could be issued) are then known complete only if
-//     it - kStagerSets - kSfSlots >= it - kStages,   i.e.  kSfSlots + kStagerSets <= kStages.
-// With 4 slots, 2 sets and 5 stages the condition fails: when the scale copies of it - kStages were
-// still in flight the wait for phase n returned true one phase early, the warp read the previous
-// occupant's scale bytes from shared memory and stored them to tensor memory -- one lane quadrant of
-// one CTA, all columns, wrong by the ratio of two scale factors -- about once in 450 launches of the
-// 4608 x 3072 x 9216 product.  2 and 3 slots, and 4 slots with the stagers held to three stages
-// ahead, satisfy the condition and never failed.  The stagers also wait for the release of iteration
-// it - kStages (stage_free, which the producer waited for before it refilled the stage) in front of
-// the sf_ready wait, so that wait is sound whatever the slot count; the assertions keep the original
-// condition as well.
-//
-// Three slots for the wide tile are what the condition allows with five stages: 57.5 -> 56.8 us (4608 x 3072 x 9216)
-// and 66.3 -> 64.1 us (4608 x 12288 x 3072) against two.  A third set of stagers (80 registers per thread) made both
-// slower, 59.5 and 67.3 us.
+// Every wait here is a PARITY wait: it tells "phase n of this barrier has completed" from "it has not" only if the
+// barrier cannot still be in phase n - 1, i.e. only if the waiter already knows that phase n - 1 has completed.  Every role
+// waits on every phase of its barriers in turn (producer on stage_free, MMA issuer on stage_full and acc_empty, each
+// epilogue warp on acc_full), so it knows it from its own previous wait.
 //
 // Two tile widths.  The wide tile (256 columns) needs the fewest operand bytes per flop and is what every
 // product of more than one round of tiles runs on.  The narrow tile (128 columns) is for products that have at
@@ -112,32 +96,27 @@ struct Tile {
     static constexpr int kNCta = BN / 2;
     static constexpr bool kOneTile = BN == 128;             // a pair computes one tile; the epilogue stages in the ring
     static constexpr int kStages = BN == 256 ? 5 : 8;
-    static constexpr int kSfSlots = BN == 256 ? 3 : 4;
     static constexpr int kNB = BN / 128;                  // 128-row scale blocks of B per tile
     static constexpr int kBBytes = kNCta * BK / 2;
     static constexpr int kSfbBytes = kNB * kSfaBytes;     // the 128-row blocks of the tile's B rows
     static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38 or 28 * 1024
     static constexpr uint32_t kSfSlotCol0 = BN, kSfbColsPerKb = 4 * kNB, kSfbOfs = 16;
     static constexpr uint32_t kSfSlotCols = 4 * (4 + kSfbColsPerKb);   // 48 or 32
-    static constexpr int kNumBars = 3 * kStages + 2;      // stage_full[S] sf_ready[S] stage_free[S] acc_full acc_empty
+    static constexpr int kNumBars = 2 * kStages + 2;      // stage_full[S] stage_free[S] acc_full acc_empty
     static constexpr int kRingBytes = kStages * kStageBytes, kEpi = kOneTile ? 0 : kRingBytes;  // where the boxes start
     static constexpr size_t kSmemBytes = kRingBytes + (kOneTile ? 0 : kEpiBytes) + 1024 /*alignment slack*/ + 8 * kNumBars + 64;
     // Instruction descriptor: E2M1 x E2M1, UE4M3 scales, both K-major, M = 256 (pair), N = BN, K = 64.
     static constexpr uint32_t kIdesc = (1u << 7) | (1u << 10) | (static_cast<uint32_t>(BN >> 3) << 17) | (0u << 23) |
                                        (static_cast<uint32_t>(BM >> 4) << 24);
     static_assert(kStageBytes % 1024 == 0, "swizzled operand tiles start on 1024-byte boundaries");
-    static_assert(kSfSlotCol0 + kSfSlots * kSfSlotCols <= 512, "tensor memory columns");
-    static_assert(kSfSlots + kStagerSets <= kStages, "a stager set must know that the previous phase of sf_ready has completed");
-    static_assert(kSfSlots <= 2 * kStages - 2, "the stagers' parity waits on stage_free must be unambiguous");
+    static_assert(kSfSlotCol0 + kStages * kSfSlotCols <= 512, "tensor memory columns");
     static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 };
 
 struct GemmParams {
-    const uint8_t *sfx, *sfw;
     const float *ts_x, *ts_w;
-    int M, N, K;
-    int m_tiles, n_tiles, k_tiles, kb_total, kb4;
-    int m_rowblocks, n_rowblocks;
+    int M, N;
+    int m_tiles, n_tiles, k_tiles, kb_total;
     long long wait_cycles;  // limit of every mbarrier wait, in SM clock cycles
     int *status;
 };
@@ -256,11 +235,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster)
         : "memory");
 }
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int x, int y, uint32_t src) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
                  ::"l"(map), "r"(x), "r"(y), "r"(src)
@@ -275,10 +249,15 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// Arrive on `bar` (cluster-window address: this CTA's or the peer's) once every tcgen05 operation
-// issued so far by this thread has completed in both CTAs of the pair.
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+// Arrive on both CTAs' copies of `bar` once every tcgen05 operation issued so far by this thread has completed in the pair.
+__device__ __forceinline__ void tc_commit_both(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(bar), "h"(static_cast<uint16_t>(3))
+                 : "memory");
+}
+// Copies a 512-byte scale block of either CTA to four columns of its tensor memory, replicated over the lane quadrants.
+__device__ __forceinline__ void tc_cp_scales(uint32_t tmem_col, uint64_t desc) {
+    asm volatile("tcgen05.cp.cta_group::2.32x128b.warpx4 [%0], %1;" ::"r"(tmem_col), "l"(desc) : "memory");
 }
 __device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t sfa,
                                             uint32_t sfb, uint32_t accumulate) {
@@ -311,17 +290,6 @@ __device__ __forceinline__ void tc_wait_ld(uint32_t (&v)[16]) {
                  :
                  : "memory");
 }
-__device__ __forceinline__ void tc_st4(uint32_t taddr, const uint4 &v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v.x), "r"(v.y),
-                 "r"(v.z), "r"(v.w)
-                 : "memory");
-}
-__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
-}
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
@@ -332,13 +300,13 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t smem_addr) {
     return static_cast<uint64_t>((smem_addr & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) |
            (2ull << 61);
 }
+// ... of scale blocks: no swizzle, 16-byte rows, 8-row groups 128 bytes apart.
+__device__ __forceinline__ uint64_t scale_desc(uint32_t smem_addr) {
+    return static_cast<uint64_t>((smem_addr & 0x3FFFFu) >> 4) | (1ull << 16) | (8ull << 32) | (1ull << 46);
+}
 // Two accumulator values times alpha, each rounded to bf16 (nearest even), packed low | high.
-#ifndef PQ_GEMM_EPI_PACKED
-#define PQ_GEMM_EPI_PACKED 1
-#endif
 __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo_bits, uint32_t hi_bits, float alpha) {
     uint32_t r;
-#if PQ_GEMM_EPI_PACKED
     // one packed multiply (two IEEE products per issue slot), then the two-way convert
     asm("{\n"
         ".reg .b64 v, a;\n"
@@ -351,26 +319,20 @@ __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo_bits, uint32_t hi_bits
         "}\n"
         : "=r"(r)
         : "r"(lo_bits), "r"(hi_bits), "f"(alpha));
-#else
-    const float lo = __fmul_rn(__uint_as_float(lo_bits), alpha);
-    const float hi = __fmul_rn(__uint_as_float(hi_bits), alpha);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-#endif
     return r;
 }
 
 // ---------------------------------------------------------------- kernel
-// Register budget: the register file is split over the four SM sub-partitions (16384 registers
-// each) and two of them receive five of this CTA's 18 warps: 5 x 32 x 96 = 15360 fits, 104 would not.
-// The 1024 registers left there take one warp of a 32-register kernel, so 128-thread blocks of
-// other kernels can still run on the SM beside the GEMM.
-constexpr int kMaxRegs = 96;
+// Register budget: the register file is split over the four SM sub-partitions (16384 registers each) and two of them
+// receive three of this CTA's ten warps: 3 x 32 x 128 = 12288.  The rest takes blocks of a 32-register kernel beside the GEMM.
+constexpr int kMaxRegs = 128;
 template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kMaxRegs)
 gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                 const __grid_constant__ CUtensorMap map_sfa, const __grid_constant__ CUtensorMap map_sfb,
                  const __grid_constant__ CUtensorMap map_y, const GemmParams p) {
     using T = Tile<BN>;
-    constexpr int kStages = T::kStages, kSfSlots = T::kSfSlots, kNB = T::kNB, BN_CTA = T::kNCta;
+    constexpr int kStages = T::kStages, kNB = T::kNB, BN_CTA = T::kNCta;
     constexpr int kBBytes = T::kBBytes, kStageBytes = T::kStageBytes, kNumBars = T::kNumBars;
     constexpr uint32_t kSfbOfs = T::kSfbOfs, kSfbColsPerKb = T::kSfbColsPerKb;
     extern __shared__ uint8_t smem_raw[];
@@ -381,26 +343,23 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     const uint32_t epi = base + T::kEpi;
     const uint32_t bars = base + kBarOfs;
     uint8_t *bars_ptr = base_ptr + kBarOfs;
-    // stage_full: operand bytes of both CTAs have landed (1 arrival + transaction bytes) and the
-    // stage's scales are in tensor memory in both CTAs (8 stager-warp arrivals); leader's copy only
+    // stage_full: operand and scale bytes of both CTAs have landed (1 arrival + transaction bytes); leader's copy only
     auto stage_full_bar = [&](int s) { return bars + 8u * s; };
-    auto sf_ready_bar = [&](int s) { return bars + 8u * (kStages + s); };     // scale blocks landed (own CTA)
-    auto stage_free_bar = [&](int s) { return bars + 8u * (2 * kStages + s); };  // the stage's MMAs have run
-    const uint32_t acc_full_bar = bars + 8u * (3 * kStages);       // one copy per CTA, both signalled by the issuer
-    const uint32_t acc_empty_bar = bars + 8u * (3 * kStages + 1);  // leader's copy only
+        auto stage_free_bar = [&](int s) { return bars + 8u * (kStages + s); };  // the stage's MMAs have run
+    const uint32_t acc_full_bar = bars + 8u * (2 * kStages);       // one copy per CTA, both signalled by the issuer
+    const uint32_t acc_empty_bar = bars + 8u * (2 * kStages + 1);  // leader's copy only
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars_ptr + 8 * kNumBars);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_ptr + 8 * kNumBars + 8);
     const WaitCtx wctx{abort_flag, p.status, p.wait_cycles};
     auto sf_slot_col = [](uint32_t t) { return T::kSfSlotCol0 + t * T::kSfSlotCols; };
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_ctarank();  // 0 = pair leader
+    const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const uint32_t rank = __shfl_sync(0xFFFFFFFFu, cluster_ctarank(), 0);  // 0 = pair leader
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(stage_full_bar(s), 9);  // producer + 4 stager warps in each CTA
-            mbar_init(sf_ready_bar(s), 1);
+            mbar_init(stage_full_bar(s), 1);
             mbar_init(stage_free_bar(s), 1);
         }
         mbar_init(acc_full_bar, 1);
@@ -409,6 +368,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_b);
+        prefetch_tensormap(&map_sfa);
+        prefetch_tensormap(&map_sfb);
         prefetch_tensormap(&map_y);
     }
     if (warp == 1) {
@@ -421,7 +382,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     __syncthreads();
     cluster_sync();  // both CTAs' barriers are initialised before anyone signals across
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot, 0);
     // When launched as a programmatic dependent of the activation quantizer, everything above ran
     // while that kernel was finishing; its output (and any earlier work in the stream) is complete
     // and visible from here on.  A no-op for an ordinary launch.
@@ -440,51 +401,37 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             const int m_blk = tile % p.m_tiles, n_blk = tile / p.m_tiles;
             const int m0 = m_blk * BM + static_cast<int>(rank) * BM_CTA;
             const int n0 = n_blk * BN;
-            const int ra = min(m0 >> 7, p.m_rowblocks - 1);
-            const int nb0 = n0 >> 7;
-            const uint8_t *sfa_src = p.sfx + static_cast<int64_t>(ra) * p.kb4 * kSfBlock;
-            const uint8_t *sfb_src[kNB];
-#pragma unroll
-            for (int j = 0; j < kNB; ++j)
-                sfb_src[j] = p.sfw + static_cast<int64_t>(min(nb0 + j, p.n_rowblocks - 1)) * p.kb4 * kSfBlock;
             for (int kt = 0; kt < p.k_tiles; ++kt, ++it) {
                 const int s = it % kStages;
                 const uint32_t par = (it / kStages) & 1u;
                 ok = mbar_wait_warp(stage_free_bar(s), par ^ 1u, wctx);
                 if (!ok) break;
-                const int kb_valid = min(4, p.kb_total - kt * 4);
-                const uint32_t sf_bytes = static_cast<uint32_t>(kb_valid) * kSfBlock;
                 const uint32_t stage = base + s * kStageBytes;
                 const uint32_t sf_stage = stage + kABytes + kBBytes;
                 const uint32_t full_leader = mapa(stage_full_bar(s), 0);
-                const int64_t kofs = static_cast<int64_t>(kt) * 4 * kSfBlock;
                 if (elect_one()) {
-                    if (rank == 0) mbar_expect_tx(stage_full_bar(s), 2u * (kABytes + kBBytes));
-                    mbar_expect_tx(sf_ready_bar(s), (1u + kNB) * sf_bytes);
-                    bulk_load(sf_stage, sfa_src + kofs, sf_bytes, sf_ready_bar(s));
-#pragma unroll
-                    for (int j = 0; j < kNB; ++j)
-                        bulk_load(sf_stage + (1 + j) * kSfaBytes, sfb_src[j] + kofs, sf_bytes, sf_ready_bar(s));
+                    if (rank == 0) mbar_expect_tx(stage_full_bar(s), 2u * kStageBytes);
                     tma_load_2d_pair(stage, &map_a, kt * (BK / 2), m0, full_leader);
                     tma_load_2d_pair(stage + kABytes, &map_b, kt * (BK / 2), n0 + static_cast<int>(rank) * BN_CTA,
                                      full_leader);
+                    tma_load_2d_pair(sf_stage, &map_sfa, kt * (4 * kSfBlock / 8), m0 >> 7, full_leader);
+                    tma_load_2d_pair(sf_stage + kSfaBytes, &map_sfb, kt * (4 * kSfBlock / 8), n0 >> 7, full_leader);
                 }
                 __syncwarp();
             }
         }
-        if (!ok && lane == 0) {
-            // give the scale copies already issued a bounded chance to land before leaving
+        if (!ok && lane == 0 && rank == 0) {
+            // give the copies already issued (both CTAs': they count on this barrier) a bounded chance to land before leaving
             const uint32_t first = it > kStages ? it - kStages : 0;
             for (uint32_t j = first; j < it; ++j)
-                for (uint32_t i = 0; i < 4096 && !mbar_try(sf_ready_bar(j % kStages), (j / kStages) & 1u); ++i) {}
+                for (uint32_t i = 0; i < 4096 && !mbar_try(stage_full_bar(j % kStages), (j / kStages) & 1u); ++i) {}
         }
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (pair leader)
         if (rank == 0) {
-            // Ring positions are kept incrementally: operand stage s with phase ph, scale slot t.
-            const uint32_t peer = mapa(bars, 1) - bars;  // cluster-window offset of the peer's shared memory
-            uint32_t s = 0, ph = 0, t = 0, tcount = 0;
+            // Ring positions are kept incrementally: stage (and scale slot) s with phase ph.
+            uint32_t s = 0, ph = 0, tcount = 0;
             bool ok = true;
             for (int tile = pair; tile < total_tiles && ok; tile += num_pairs, ++tcount) {
                 // the accumulator is free once the epilogue has read the previous tile out of it
@@ -499,9 +446,18 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     tc_fence_after();
                     const uint32_t stage = base + s * kStageBytes;
                     const uint64_t da = operand_desc(stage), db = operand_desc(stage + kABytes);
-                    const uint32_t sfa_t = tmem_base + sf_slot_col(t), sfb_t = sfa_t + kSfbOfs;
+                    const uint64_t ds = scale_desc(stage + kABytes + kBBytes);
+                    const uint32_t sfa_t = tmem_base + sf_slot_col(s), sfb_t = sfa_t + kSfbOfs;
                     const int kb_valid = min(4, p.kb_total - kt * 4);
                     if (elect_one()) {
+                        // (blocks past the last channel are zeros and belong to no MMA)
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            tc_cp_scales(sfa_t + 4 * kk, ds + kk * (kSfBlock / 16));
+#pragma unroll
+                            for (int j = 0; j < kNB; ++j)
+                                tc_cp_scales(sfb_t + kSfbColsPerKb * kk + 4 * j, ds + ((1 + j) * kSfaBytes + kk * kSfBlock) / 16);
+                        }
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
                             if (kk < kb_valid) {
@@ -511,72 +467,14 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                             }
                         }
                         // the stage (and its scale slot) is free in both CTAs once these MMAs have run
-                        tc_commit_pair(stage_free_bar(s));
-                        tc_commit_pair(stage_free_bar(s) + peer);
-                        if (kt == p.k_tiles - 1) {  // ... and with them the tile's accumulator is complete
-                            tc_commit_pair(acc_full_bar);
-                            tc_commit_pair(acc_full_bar + peer);
-                        }
+                        tc_commit_both(stage_free_bar(s));
+                        if (kt == p.k_tiles - 1) tc_commit_both(acc_full_bar);  // ... and the tile's accumulator is complete
                     }
                     __syncwarp();
                     acc = 1u;
                     s = (s + 1 == kStages) ? 0u : s + 1;
                     ph ^= (s == 0) ? 1u : 0u;
-                    t = (t + 1 == kSfSlots) ? 0u : t + 1;
                 }
-            }
-        }
-    } else if (warp >= kFirstStager) {
-        // ------------------------------------------------------------ scale-factor stagers
-        // Two sets of four warps (one warp per tensor-memory lane quadrant) take alternate K
-        // iterations, so a set has two stages' worth of MMA time for one stage of scales.
-        const uint32_t q = warp & 3;  // tensor-memory lane quadrant this warp may write
-        const uint32_t set = static_cast<uint32_t>(warp - kFirstStager) >> 2;
-        const uint32_t lane_ofs = (q * 32u) << 16;
-        uint32_t it = 0;
-        bool ok = true;
-        for (int tile = pair; tile < total_tiles && ok; tile += num_pairs) {
-            for (int kt = 0; kt < p.k_tiles; ++kt, ++it) {
-                if ((it % kStagerSets) != set) continue;
-                const int s = it % kStages;
-                const uint32_t t = it % kSfSlots;
-                // The stage's previous occupant has been released (which makes the parity wait that
-                // follows unambiguous: see kSfSlots), then: this iteration's scale blocks have landed.
-                if (it >= kStages) ok = mbar_wait_warp(stage_free_bar(s), ((it - kStages) / kStages) & 1u, wctx);
-                ok = ok && mbar_wait_warp(sf_ready_bar(s), (it / kStages) & 1u, wctx);
-                if (!ok) break;
-                const int kb_valid = min(4, p.kb_total - kt * 4);
-                const uint32_t sf_s = base + s * kStageBytes + kABytes + kBBytes + lane * 16u;
-                const uint32_t sf_t = tmem_base + lane_ofs + sf_slot_col(t);
-                // the shared-memory reads do not depend on the slot: start them before waiting for it
-                uint4 sa[4], sb[kNB][4];
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    if (kk < kb_valid) {
-                        sa[kk] = lds128(sf_s + kk * kSfBlock);
-#pragma unroll
-                        for (int j = 0; j < kNB; ++j) sb[j][kk] = lds128(sf_s + (1 + j) * kSfaBytes + kk * kSfBlock);
-                    }
-                }
-                // the MMAs that read this slot kSfSlots iterations ago have completed (their commit
-                // released that iteration's stage)
-                if (it >= kSfSlots)
-                    ok = mbar_wait_warp(stage_free_bar((it - kSfSlots) % kStages), ((it - kSfSlots) / kStages) & 1u, wctx);
-                if (!ok) break;
-                tc_fence_after();
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    if (kk < kb_valid) {
-                        tc_st4(sf_t + 4 * kk, sa[kk]);
-#pragma unroll
-                        for (int j = 0; j < kNB; ++j)
-                            tc_st4(sf_t + kSfbOfs + kSfbColsPerKb * kk + 4 * j, sb[j][kk]);
-                    }
-                }
-                tc_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_leader(stage_full_bar(s), rank);
             }
         }
     } else {
@@ -584,8 +482,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         // Eight warps: lane quadrant q x column half h.  A warp reads its 32 rows x BN / 2 columns out of
         // tensor memory, scales and rounds them to bf16 and keeps them packed in BN / 4 registers; the
         // accumulator goes back to the MMA issuer after those loads (a few hundred cycles), and the
-        // 64-column boxes leave through one staging box and TMA stores behind the next tile's
-        // main loop.
+        // 64-column boxes leave through one staging box and TMA stores, the warps and boxes one after the other over
+        // the next tile's main loop (at once if there is none).
         constexpr int kCols = BN / 2, kBoxes = kCols / kBoxCols, kChunks = kBoxCols / 8;  // boxes per warp, 16-byte chunks per box row
         const int q = warp & 3;                // tensor-memory lane quadrant this warp may read
         const int h = (warp - 2) >> 2;         // column half
@@ -600,6 +498,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             const bool got = mbar_wait(acc_full_bar, tcount & 1u, wctx);
             if (!__all_sync(0xFFFFFFFFu, got)) break;
             tc_fence_after();
+            const bool more = tile + num_pairs < total_tiles;
+            const long long t0 = clock64();
             const uint32_t acc = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + h * kCols;
             uint32_t pk[kCols / 2];  // pk[8 c + i] = columns 16 c + 2 i, 16 c + 2 i + 1 of this lane's row
             // two loads in flight: chunk c + 1 is on its way while chunk c is scaled and packed
@@ -622,6 +522,10 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             if (lane == 0) mbar_arrive_leader(acc_empty_bar, rank);
 #pragma unroll
             for (int c = 0; c < kBoxes; ++c) {
+                if (more) {
+                    const long long until = t0 + static_cast<long long>(c * kEpiWarps + warp - 2) * p.k_tiles * kPaceCycles;
+                    while (clock64() < until) __nanosleep(64);
+                }
                 // the store that read the box before (previous box or previous tile) must be done with it
                 if (lane == 0) bulk_wait_read<0>();
                 __syncwarp();
@@ -688,7 +592,8 @@ EncodeTiledFn encode_tiled() {
 }
 
 // A row-major 2-D tensor [rows, row_bytes / elem] cut into 128-byte-swizzled boxes of 128 bytes x
-// box_rows rows.  Loads read out-of-range rows / columns as zero, stores skip them.
+// box_rows rows; with elem = 8 (scale blocks, a row of blocks per row of the map) plain boxes of 2 KB x box_rows.  Loads read
+// out-of-range rows / columns as zero, stores skip them.
 struct MapKey {
     const void *ptr;
     int64_t rows, row_bytes, pitch;
@@ -700,31 +605,44 @@ struct MapSlot {
     bool used;
 };
 // Encoding a tensor map costs several microseconds of host time; a layer calls the GEMM with
-// the same buffers over and over, so the last few encodings are kept.
+// the same buffers over and over, so a thread keeps the encodings of the last few layers: five maps a call, found by a hash of
+// the whole key in one of four neighbouring slots.
 bool make_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t row_bytes, int64_t pitch, int box_rows,
               int elem) {
-    constexpr int kSlots = 16;
+    constexpr uint32_t kSlots = 64, kProbes = 4;
     static thread_local MapSlot cache[kSlots];
-    static thread_local int next = 0;
-    for (MapSlot &c : cache)
+    static thread_local uint32_t next = 0;
+    const uint64_t mix = (reinterpret_cast<uintptr_t>(ptr) >> 4) ^ (static_cast<uint64_t>(rows) << 20) ^
+                         (static_cast<uint64_t>(pitch) << 40) ^ static_cast<uint64_t>(box_rows);
+    const uint32_t home = static_cast<uint32_t>((mix * 0x9E3779B97F4A7C15ull) >> 58);
+    for (uint32_t i = 0; i < kProbes; ++i) {
+        const MapSlot &c = cache[(home + i) % kSlots];
         if (c.used && c.key.ptr == ptr && c.key.rows == rows && c.key.row_bytes == row_bytes && c.key.pitch == pitch &&
             c.key.box_rows == box_rows && c.key.elem == elem) {
             *map = c.map;
             return true;
         }
+    }
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return false;
     const cuuint64_t dims[2] = {static_cast<cuuint64_t>(row_bytes / elem), static_cast<cuuint64_t>(rows)};
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(pitch)};
-    const cuuint32_t box[2] = {static_cast<cuuint32_t>(128 / elem), static_cast<cuuint32_t>(box_rows)};
+    const cuuint32_t box[2] = {static_cast<cuuint32_t>(elem == 8 ? 256 : 128 / elem), static_cast<cuuint32_t>(box_rows)};
     const cuuint32_t estr[2] = {1, 1};
-    const CUtensorMapDataType dt = elem == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    const CUtensorMapDataType dt = elem == 1   ? CU_TENSOR_MAP_DATA_TYPE_UINT8
+                                   : elem == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                               : CU_TENSOR_MAP_DATA_TYPE_UINT64;
     if (enc(map, dt, 2, const_cast<void *>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            elem == 8 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
-    MapSlot &slot = cache[next];
-    next = (next + 1) % kSlots;
+    uint32_t at = home + next++ % kProbes;  // an empty slot, or one of the four in turn
+    for (uint32_t i = 0; i < kProbes; ++i)
+        if (!cache[(home + i) % kSlots].used) {
+            at = home + i;
+            break;
+        }
+    MapSlot &slot = cache[at % kSlots];
     slot.key = MapKey{ptr, rows, row_bytes, pitch, box_rows, elem};
     slot.map = *map;
     slot.used = true;
@@ -776,20 +694,19 @@ struct GemmArgs {
 
 template <int BN>
 pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
-    CUtensorMap map_a, map_b, map_y;
+    CUtensorMap map_a, map_b, map_sfa, map_sfb, map_y;
+    const int64_t sf_pitch = g.K / 64 * kSfBlock;
     if (!make_map(&map_a, g.xq, g.M, g.K / 2, g.K / 2, BM_CTA, 1) || !make_map(&map_b, g.wq, g.N, g.K / 2, g.K / 2, Tile<BN>::kNCta, 1) ||
-        !make_map(&map_y, g.Y, g.M, g.N * 2, g.ldy * 2, 32, 2))
+        !make_map(&map_sfa, g.sfx, pq_ceil_div(g.M, 128), sf_pitch, sf_pitch, 1, 8) ||
+        !make_map(&map_sfb, g.sfw, pq_ceil_div(g.N, 128), sf_pitch, sf_pitch, Tile<BN>::kNB, 8) || !make_map(&map_y, g.Y, g.M, g.N * 2, g.ldy * 2, 32, 2))
         return PQ_ERR_CUDA;
     GemmParams p;
-    p.sfx = g.sfx, p.sfw = g.sfw, p.ts_x = g.ts_x, p.ts_w = g.ts_w;
-    p.M = static_cast<int>(g.M), p.N = static_cast<int>(g.N), p.K = static_cast<int>(g.K);
+    p.ts_x = g.ts_x, p.ts_w = g.ts_w;
+    p.M = static_cast<int>(g.M), p.N = static_cast<int>(g.N);
     p.m_tiles = static_cast<int>(pq_ceil_div(g.M, BM));
     p.n_tiles = static_cast<int>(pq_ceil_div(g.N, BN));
     p.k_tiles = static_cast<int>(pq_ceil_div(g.K, BK));
     p.kb_total = static_cast<int>(g.K / 64);
-    p.kb4 = p.kb_total;
-    p.m_rowblocks = static_cast<int>(pq_ceil_div(g.M, 128));
-    p.n_rowblocks = static_cast<int>(pq_ceil_div(g.N, 128));
     p.wait_cycles = kWaitCycles;
     p.status = static_cast<int *>(g.ws);
     const int64_t tiles = static_cast<int64_t>(p.m_tiles) * p.n_tiles;
@@ -809,7 +726,7 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    PQ_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel<BN>, map_a, map_b, map_y, p));
+    PQ_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel<BN>, map_a, map_b, map_sfa, map_sfb, map_y, p));
     return PQ_OK;
 }
 

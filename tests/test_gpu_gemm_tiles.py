@@ -25,3 +25,8 @@ def test_exact_at_the_line(M, N, K):
 @pytest.mark.parametrize("M,N,K", [(2, 4736, 128), (2, 4744, 320), (3, 4744, 128), (1, 9472, 192), (16, 4744, 3136), (17, 4744, 3136)])   # 37 and 38 narrow tiles, few rows
 def test_few_rows_at_the_line(M, N, K):
     test_exact_at_the_line(M, N, K)
+
+
+@pytest.mark.parametrize("M,N,K", [(2200, 2440, 64), (4700, 1288, 320), (1025, 8200, 576)])   # two and three rounds of wide tiles;
+def test_rounds_at_ragged_edges(M, N, K):           # 1 to 4 blocks of channels in the last K step, a last row block of either
+    test_exact_at_the_line(M, N, K)                 # operand that is the second of its tile or past the end

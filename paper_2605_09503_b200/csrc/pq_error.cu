@@ -181,9 +181,10 @@ group_error_direct(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int6
 // and divide once per group and row (the scale tables below take a clamp and two loads).
 // Blocks are persistent, one per SM; the groups of a block only share the slot and scale tables.
 //
-// NVFP4 is scalar arithmetic: packed f32x2 instructions save issue slots but run on one of the two FMA pipes only, and
+// NVFP4 is scalar arithmetic but for the sums: packed f32x2 instructions save issue slots but run on one of the two FMA pipes only, and
 // with the f16 converts there too it was 59 % busy (9216 x 3072, six orders, with the fold of that time: 79 us scalar, 84
-// packed; 74 with the present fold).  The integer formats, without converts, are packed (4608 x 3072, INT4 g64: 53.4 us,
+// packed; 74 with the present fold); only the sums of squares are packed, which leaves that pipe room (9216 x 3072 72.9 -> 71.6, 4608 x
+// 12288 197.6 -> 194.7; the multiplication packed 81.2, the residual 74.6).  The integer formats, without converts, are packed (4608 x 3072, INT4 g64: 53.4 us,
 // 54.1 scalar; 50.1 with the present fold).
 // What bounds it: instruction issue (67 % of the slots busy at 23 warps per SM) and shared-memory wavefronts (a 64-bit gather
 // through a random order takes about 6 of them where 2 would do: 0.069 per element and order).
@@ -300,7 +301,7 @@ __device__ __forceinline__ void row_pair_sse(const uint32_t (&u)[16], const Scal
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (KIND == 0) {
-            float acc0 = 0.0f, acc1 = 0.0f;
+            uint64_t acc2 = 0;  // {+0, +0}
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const uint32_t w = u[8 * h + i];
@@ -308,9 +309,10 @@ __device__ __forceinline__ void row_pair_sse(const uint32_t (&u)[16], const Scal
                 float q0 = __fmul_rn(x0, r0), q1 = __fmul_rn(x1, r1);
                 e2m1_pair(q0, q1);
                 const float d0 = __fmaf_rn(q0, nd0, x0), d1 = __fmaf_rn(q1, nd1, x1);
-                acc0 = __fmaf_rn(d0, d0, acc0), acc1 = __fmaf_rn(d1, d1, acc1);
+                const uint64_t d2 = pack2(d0, d1);
+                acc2 = fma2(d2, d2, acc2);
             }
-            run0[h] = acc0, run1[h] = acc1;
+            unpack2(acc2, run0[h], run1[h]);
         } else {
             const uint64_t r2 = pack2(r0, r1), nd2 = pack2(nd0, nd1), one2 = pack2(1.0f, 1.0f);
             const uint64_t magic = pack2(12582912.0f, 12582912.0f), unmagic = pack2(-12582912.0f, -12582912.0f);

@@ -240,6 +240,8 @@ fakequant_int_kernel(const uint16_t *__restrict__ T, int64_t rows, int64_t K, in
     const int64_t oct = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
     const int64_t row = row_block_index() * kTileRows + threadIdx.y;
     const bool live = row < rows && oct * 8 < K;
+    pq::dependents_may_launch();
+    pq::wait_for_prior_grid();
     float x[8];
     if (live) {
         pq::unpack8(__ldcs(reinterpret_cast<const uint4 *>(T + row * ld + oct * 8)), x);
@@ -256,7 +258,9 @@ fakequant_int_kernel(const uint16_t *__restrict__ T, int64_t rows, int64_t K, in
 // side in packed fp32 registers.  Everything works on magnitudes (sign-symmetric, round to nearest even), the
 // sign bits come back at the end; the scale comes from a table by the mantissa of the absmax.  A block is one
 // group of four rows and five of them share an SM at 3072 channels (192 threads, 64 registers), so some load while others
-// compute: 16.6 us for 4608 x 3072, INT4 g64, from HBM; 12.8 without an order.
+// compute: 16.6 us for 4608 x 3072, INT4 g64, from HBM; 12.8 without an order.  Calls one behind the other overlap (programmatic
+// dependent launch): 16.2 us a call in a loop, 18.3 without.  Persistent blocks with the next rows copied ahead, and slots from
+// a table, were slower at every size (600 x 3072 8.1 against 4.7, 18432 x 3072 49.4 against 46.6).
 // The kernel before it staged one row per block and gathered two bytes at a time, about four shared-memory
 // wavefronts per 32 elements and two divisions per eight: 30.7 us for 4608 x 3072, INT4 g64.
 constexpr int kFqThreads = 512;
@@ -322,9 +326,11 @@ fakequant_int_gather_kernel(const uint16_t *__restrict__ T, int64_t rows, int K,
         for (int r = 0; r < 4; ++r)
             v[r] = o < octs && r < live_rows ? __ldg(reinterpret_cast<const uint4 *>(T + r * ld) + o) : make_uint4(0, 0, 0, 0);
     };
+    pq::build_int_tab(tab, Qf, false);  // needs nothing of the kernel in front
+    pq::dependents_may_launch();
+    pq::wait_for_prior_grid();
     uint4 v[4];
     load_octet(threadIdx.x, v);
-    pq::build_int_tab(tab, Qf, false);  // while the first rows are on their way
     for (int o = threadIdx.x; o < octs; o += blockDim.x) {
         pq::store_quad_octet(quad_s, o, v);
         load_octet(o + blockDim.x, v);
@@ -535,10 +541,10 @@ extern "C" pq_status pq_fakequant_int(const void *T, int64_t rows, int64_t K, in
 #define PQ_FQ_CASE(TEAM)                                                                              \
     if (perm) {                                                                                       \
         PQ_CUDA_OK(pq::allow_smem(fakequant_int_gather_kernel<TEAM>, smem, kOrderMaxK * 8, 1024));    \
-        fakequant_int_gather_kernel<TEAM><<<static_cast<unsigned>(grid_g), threads_g, smem, st>>>(    \
-            t, rows, static_cast<int>(K), ld, perm, Qf, o, ldo);                                      \
+        PQ_CUDA_OK(pq::launch_dependent(fakequant_int_gather_kernel<TEAM>, dim3(static_cast<unsigned>(grid_g)), dim3(threads_g), smem, st, \
+                                        t, rows, static_cast<int>(K), ld, perm, Qf, o, ldo));         \
     } else {                                                                                          \
-        fakequant_int_kernel<TEAM><<<grid, dim3(32, kTileRows), 0, st>>>(t, rows, K, ld, Qf, o, ldo); \
+        PQ_CUDA_OK(pq::launch_dependent(fakequant_int_kernel<TEAM>, grid, dim3(32, kTileRows), 0, st, t, rows, K, ld, Qf, o, ldo)); \
     }
     switch (fmt.group) {
         case 16: PQ_FQ_CASE(2) break;

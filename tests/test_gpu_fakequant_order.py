@@ -22,3 +22,24 @@ def test_order_matches_gathered_columns(rows, K, shift, bits, group):
     B.pq_fakequant_int(x, (B.KIND_INT, bits, group), held[shift:shift + K], out)
     B.pq_fakequant_int(x[:, perm.to(DEV)].contiguous(), (B.KIND_INT, bits, group), None, want)
     assert torch.equal(out.contiguous().view(torch.int16), want.view(torch.int16))
+
+
+@pytest.mark.parametrize("rows,K", [(30, 768), (2501, 3072)])
+def test_chain_of_calls(rows, K):
+    """Blocks start before the call in front has finished: a chain, in place in parts, gives what it gives call by call."""
+    perm = torch.randperm(K, generator=torch.Generator().manual_seed(5)).to(DEV).to(torch.int32)
+    fmt = (B.KIND_INT, 4, 64)
+
+    def chain(wait):
+        x, y = tensor_with_edges(rows, K, 5), torch.empty(rows, K, dtype=torch.bfloat16, device=DEV)
+        for i in range(12):
+            B.pq_fakequant_int(x, fmt, perm if i % 3 else None, y)
+            if wait:
+                torch.cuda.synchronize()
+            B.pq_fakequant_int(y, fmt, perm if i % 2 else None, y)
+            if wait:
+                torch.cuda.synchronize()
+            x, y = y, x
+        return x
+
+    assert torch.equal(chain(False).view(torch.int16), chain(True).view(torch.int16))

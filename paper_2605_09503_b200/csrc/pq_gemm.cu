@@ -594,35 +594,7 @@ EncodeTiledFn encode_tiled() {
 // A row-major 2-D tensor [rows, row_bytes / elem] cut into 128-byte-swizzled boxes of 128 bytes x
 // box_rows rows; with elem = 8 (scale blocks, a row of blocks per row of the map) plain boxes of 2 KB x box_rows.  Loads read
 // out-of-range rows / columns as zero, stores skip them.
-struct MapKey {
-    const void *ptr;
-    int64_t rows, row_bytes, pitch;
-    int box_rows, elem;
-};
-struct MapSlot {
-    MapKey key;
-    CUtensorMap map;
-    bool used;
-};
-// Encoding a tensor map costs several microseconds of host time; a layer calls the GEMM with
-// the same buffers over and over, so a thread keeps the encodings of the last few layers: five maps a call, found by a hash of
-// the whole key in one of four neighbouring slots.
-bool make_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t row_bytes, int64_t pitch, int box_rows,
-              int elem) {
-    constexpr uint32_t kSlots = 64, kProbes = 4;
-    static thread_local MapSlot cache[kSlots];
-    static thread_local uint32_t next = 0;
-    const uint64_t mix = (reinterpret_cast<uintptr_t>(ptr) >> 4) ^ (static_cast<uint64_t>(rows) << 20) ^
-                         (static_cast<uint64_t>(pitch) << 40) ^ static_cast<uint64_t>(box_rows);
-    const uint32_t home = static_cast<uint32_t>((mix * 0x9E3779B97F4A7C15ull) >> 58);
-    for (uint32_t i = 0; i < kProbes; ++i) {
-        const MapSlot &c = cache[(home + i) % kSlots];
-        if (c.used && c.key.ptr == ptr && c.key.rows == rows && c.key.row_bytes == row_bytes && c.key.pitch == pitch &&
-            c.key.box_rows == box_rows && c.key.elem == elem) {
-            *map = c.map;
-            return true;
-        }
-    }
+bool encode_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t row_bytes, int64_t pitch, int box_rows, int elem) {
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return false;
     const cuuint64_t dims[2] = {static_cast<cuuint64_t>(row_bytes / elem), static_cast<cuuint64_t>(rows)};
@@ -632,33 +604,68 @@ bool make_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t row_bytes
     const CUtensorMapDataType dt = elem == 1   ? CU_TENSOR_MAP_DATA_TYPE_UINT8
                                    : elem == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                                : CU_TENSOR_MAP_DATA_TYPE_UINT64;
-    if (enc(map, dt, 2, const_cast<void *>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            elem == 8 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
-    uint32_t at = home + next++ % kProbes;  // an empty slot, or one of the four in turn
-    for (uint32_t i = 0; i < kProbes; ++i)
-        if (!cache[(home + i) % kSlots].used) {
+    return enc(map, dt, 2, const_cast<void *>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               elem == 8 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// What the maps of an operand (codes and scale blocks; rows x K) or of the output (sf = NULL; rows x K, ld) depend on.
+struct MapKey {
+    const void *ptr, *sf;
+    int64_t rows, K, ld;
+    int box_rows, sf_box_rows;
+    bool operator==(const MapKey &o) const {
+        return ptr == o.ptr && sf == o.sf && rows == o.rows && K == o.K && ld == o.ld && box_rows == o.box_rows && sf_box_rows == o.sf_box_rows;
+    }
+};
+struct MapSlot {
+    MapKey key;
+    CUtensorMap map, scales;
+    bool used;
+};
+// Encoding a tensor map costs several microseconds of host time; a layer calls the GEMM with the same buffers over and over, so
+// a thread keeps the encodings of the last layers: three entries a call, each in one of four neighbouring slots found by a
+// hash of its key.
+const MapSlot *find_maps(const MapKey &key) {
+    constexpr uint32_t kSlots = 64, kProbes = 4;
+    static thread_local MapSlot cache[kSlots];
+    static thread_local uint32_t next = 0;
+    const uint64_t mix = (reinterpret_cast<uintptr_t>(key.ptr) >> 4) ^ (static_cast<uint64_t>(key.rows) << 20) ^
+                         (static_cast<uint64_t>(key.ld) << 40) ^ static_cast<uint64_t>(key.box_rows);
+    const uint32_t home = static_cast<uint32_t>((mix * 0x9E3779B97F4A7C15ull) >> 58);
+    uint32_t at = home + next % kProbes;  // an empty slot, or one of the four in turn
+    for (uint32_t i = 0; i < kProbes; ++i) {
+        const MapSlot &c = cache[(home + i) % kSlots];
+        if (c.used && c.key == key) return &c;
+        if (!c.used) {
             at = home + i;
             break;
         }
+    }
+    ++next;
     MapSlot &slot = cache[at % kSlots];
-    slot.key = MapKey{ptr, rows, row_bytes, pitch, box_rows, elem};
-    slot.map = *map;
-    slot.used = true;
-    return true;
+    slot.used = false;
+    slot.key = key;
+    if (key.sf) {
+        const int64_t sf_pitch = key.K / 64 * kSfBlock;
+        slot.used = encode_map(&slot.map, key.ptr, key.rows, key.K / 2, key.K / 2, key.box_rows, 1) &&
+                    encode_map(&slot.scales, key.sf, pq_ceil_div(key.rows, 128), sf_pitch, sf_pitch, key.sf_box_rows, 8);
+    } else {
+        slot.used = encode_map(&slot.map, key.ptr, key.rows, key.K * 2, key.ld * 2, key.box_rows, 2);
+    }
+    return slot.used ? &slot : nullptr;
 }
 
 // Number of CTA pairs that can be resident at once on the current device (a cluster must fit inside
 // one GPC), after opting the kernel in to its dynamic shared memory there.  Both are per device.
 template <int BN>
-int resident_pairs() {
+int resident_pairs(int dev) {
     constexpr size_t kSmemBytes = Tile<BN>::kSmemBytes;
     static PqPerDevice cache;
-    const int dev = pq_device_slot();
     if (dev < 0) return 0;
+    if (const int known = cache.value[dev]) return known;
     std::lock_guard<std::mutex> guard(cache.lock);
-    if (cache.value[dev]) return cache.value[dev];
+    if (const int known = cache.value[dev]) return known;
     if (cudaFuncSetAttribute(gemm_w4a4_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kSmemBytes)) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -694,11 +701,18 @@ struct GemmArgs {
 
 template <int BN>
 pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
+    // copied one by one: a later entry may take an earlier one's slot
     CUtensorMap map_a, map_b, map_sfa, map_sfb, map_y;
-    const int64_t sf_pitch = g.K / 64 * kSfBlock;
-    if (!make_map(&map_a, g.xq, g.M, g.K / 2, g.K / 2, BM_CTA, 1) || !make_map(&map_b, g.wq, g.N, g.K / 2, g.K / 2, Tile<BN>::kNCta, 1) ||
-        !make_map(&map_sfa, g.sfx, pq_ceil_div(g.M, 128), sf_pitch, sf_pitch, 1, 8) ||
-        !make_map(&map_sfb, g.sfw, pq_ceil_div(g.N, 128), sf_pitch, sf_pitch, Tile<BN>::kNB, 8) || !make_map(&map_y, g.Y, g.M, g.N * 2, g.ldy * 2, 32, 2))
+    auto operand = [&](CUtensorMap &map, CUtensorMap *scales, const MapKey &key) {
+        const MapSlot *slot = find_maps(key);
+        if (!slot) return false;
+        map = slot->map;
+        if (scales) *scales = slot->scales;
+        return true;
+    };
+    if (!operand(map_a, &map_sfa, MapKey{g.xq, g.sfx, g.M, g.K, g.K, BM_CTA, 1}) ||
+        !operand(map_b, &map_sfb, MapKey{g.wq, g.sfw, g.N, g.K, g.K, Tile<BN>::kNCta, Tile<BN>::kNB}) ||
+        !operand(map_y, nullptr, MapKey{g.Y, nullptr, g.M, g.N, g.ldy, 32, 0}))
         return PQ_ERR_CUDA;
     GemmParams p;
     p.ts_x = g.ts_x, p.ts_w = g.ts_w;
@@ -755,7 +769,7 @@ pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, 
     PQ_REQUIRE(pq_aligned256(ws), PQ_ERR_ALIGN);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-    const int pairs_max = resident_pairs<256>(), pairs_narrow = resident_pairs<128>();
+    const int dev = pq_device_slot(), pairs_max = resident_pairs<256>(dev), pairs_narrow = resident_pairs<128>(dev);
     if (pairs_max <= 0 || pairs_narrow <= 0) return PQ_ERR_CUDA;
     const GemmArgs g{xq, sfx, wq, sfw, ts_x, ts_w, M, N, K, ldy, Y, ws, st};
     return narrow_tiles(M, N, K, pairs_narrow) ? launch_tiles<128>(g, pairs_narrow) : launch_tiles<256>(g, pairs_max);

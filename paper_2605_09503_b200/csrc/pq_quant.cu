@@ -404,7 +404,7 @@ pq_status quant_act_launch(const uint16_t *x, int64_t M, int64_t K, int64_t ld, 
     // has to drain before it can switch between the two configurations.
     static PqPerDevice carveout;
     const int dev = pq_device_slot();
-    if (dev >= 0) {
+    if (dev >= 0 && !carveout.value[dev]) {
         std::lock_guard<std::mutex> guard(carveout.lock);
         if (!carveout.value[dev]) {
             cudaFuncSetAttribute(quant_nvfp4_kernel<PQ_SF_TCGEN05, true, TILE_ROWS>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);

@@ -370,19 +370,42 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     pq::dependents_may_launch();
     pq::wait_for_prior_grid();
 
-    for (int j = threadIdx.x; j < K; j += blockDim.x) {
-        // the channel of every order at position j, all loads in flight (one after the other they cost 10 us a launch)
-        uint32_t ch[kMaxOrders];
+    // Slots of the orders.  The two 16-byte halves of a run's lie in separate planes: lanes read consecutive 16-byte words.
+    auto slots_at = [&](int j) { return slot_s + ((j >> 3) & 1) * (K >> 1) + (j >> 4) * 8 + (j & 7); };
+    if (K <= static_cast<int>(blockDim.x) || (reinterpret_cast<uintptr_t>(p.perms) & 15u)) {
+        for (int j = threadIdx.x; j < K; j += blockDim.x) {
+            // the channel of every order at position j, all loads in flight (one after the other they cost 10 us a launch)
+            uint32_t ch[kMaxOrders];
 #pragma unroll
-        for (int o = 0; o < kMaxOrders; ++o) {
-            const int order = o0 + o - p.identity;
-            ch[o] = o < no && order >= 0 ? static_cast<uint32_t>(__ldg(p.perms + static_cast<int64_t>(order) * K + j)) : static_cast<uint32_t>(j);
+            for (int o = 0; o < kMaxOrders; ++o) {
+                const int order = o0 + o - p.identity;
+                ch[o] = o < no && order >= 0 ? static_cast<uint32_t>(__ldg(p.perms + static_cast<int64_t>(order) * K + j)) : static_cast<uint32_t>(j);
+            }
+#pragma unroll
+            for (int o = 0; o < kMaxOrders; ++o)
+                if (o < no) slots_at(j)[o * K] = static_cast<uint16_t>(pq::quad_channel(ch[o]));
         }
-        // the two 16-byte halves of a run's slots lie in separate planes: lanes read consecutive 16-byte words
-        uint16_t *slot = slot_s + ((j >> 3) & 1) * (K >> 1) + (j >> 4) * 8 + (j & 7);
+    } else {
+        // four positions a thread, half of the orders at a time (3072 channels: 1.2 us, one position a thread 3.6)
+        for (int j = 4 * threadIdx.x; j < K; j += 4 * blockDim.x) {
+            constexpr int kHalf = (kMaxOrders + 1) / 2;
 #pragma unroll
-        for (int o = 0; o < kMaxOrders; ++o)
-            if (o < no) slot[o * K] = static_cast<uint16_t>(pq::quad_channel(ch[o]));
+            for (int h = 0; h < kMaxOrders; h += kHalf) {
+                int4 ch[kHalf];
+#pragma unroll
+                for (int u = 0; u < kHalf; ++u) {
+                    const int order = o0 + h + u - p.identity;
+                    ch[u] = h + u < no && order >= 0 ? __ldg(reinterpret_cast<const int4 *>(p.perms + static_cast<int64_t>(order) * K + j))
+                                                     : make_int4(j, j + 1, j + 2, j + 3);
+                }
+#pragma unroll
+                for (int u = 0; u < kHalf; ++u)
+                    if (h + u < no)
+                        *reinterpret_cast<uint2 *>(slots_at(j) + (h + u) * K) =
+                            make_uint2(pq::quad_channel(static_cast<uint32_t>(ch[u].x)) | pq::quad_channel(static_cast<uint32_t>(ch[u].y)) << 16,
+                                       pq::quad_channel(static_cast<uint32_t>(ch[u].z)) | pq::quad_channel(static_cast<uint32_t>(ch[u].w)) << 16);
+            }
+        }
     }
     const int sides = p.ts[1] ? 2 : 1;
     if (KIND == 0) {

@@ -188,8 +188,9 @@ group_error_direct(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int6
 // 54.1 scalar; 50.1 with the present fold).
 // What bounds it: instruction issue (67 % of the slots busy at 23 warps per SM) and shared-memory wavefronts (a 64-bit gather
 // through a random order takes about 6 of them where 2 would do: 0.069 per element and order).
-// Registers: 72 per thread, of which 56 to 92 bytes are spilled: the launch bounds count the one more warp that adds up the error
-// weights, 800 threads.  At 768 the compiler takes 80 and spills 48 to 52 bytes; not timed.  960 threads at 64 spill more.
+// Registers: 80 per thread, of which 36 to 56 bytes are spilled.  The weights of the acceptance rule, two chains of K additions, have a
+// block of their own and the gather one SM less: with a 25th warp on every SM for them the compiler had 72 (60 to 96 bytes), and
+// the chain, among the gather's warps, outlasted short passes (3 x 500 x 2560 in INT3).
 constexpr int kGatherThreads = 768;
 constexpr int kMaxOrders = 9;      // eight candidates and the original order
 constexpr int kMaxGroups = 15;                                           // named barriers 1..15
@@ -340,13 +341,14 @@ struct GatherParams {
     const int32_t *perms;      // [P - identity, K]
     int opb;                   // orders per block (blockIdx.y picks the subset)
     int groups, group_threads;
+    int blocks;                // per subset of the orders; behind them one for the error weights, if they are asked for
     uint32_t base[2], rem[2];  // pairs of the first `split` chunks / shares and its remainder: subsets of opb orders, the last
     uint32_t split;
     int full;                  // whole chunks per share behind them
     int chunks;                // eight per slab; the chunks of a last slab that hold no rows may be left out
     float Qf;
     float *part;               // [chunks, P, K/g]
-    PqErrorWeights weights;    // added up by one more warp of the block(s) in front, behind the gather's back
+    PqErrorWeights weights;    // added up by a block of their own, beside the gather
 };
 
 constexpr size_t kGatherSmemMax = 226 * 1024;
@@ -358,7 +360,7 @@ inline size_t gather_smem_bytes(int64_t K, int opb, int groups, int sides) {
 }
 
 template <int KIND, int TEAM16>
-__global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(const __grid_constant__ GatherParams p) {
+__global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __grid_constant__ GatherParams p) {
     // [groups][K][4 rows] bf16 magnitudes | [opb][K] 16-bit slots | scale tables | [groups][opb][runs] fp32 chunk sums
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.K, octs = K >> 3, runs = K >> 4;
@@ -369,6 +371,14 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     if (KIND == 1) pq::build_int_tab(int_tab, p.Qf, true);  // needs nothing of the kernel in front
     pq::dependents_may_launch();
     pq::wait_for_prior_grid();
+
+    if (blockIdx.x == static_cast<unsigned>(p.blocks)) {  // the block of the error weights: a warp per side
+        for (int s = threadIdx.x >> 5; blockIdx.y == 0 && s < 2; s += blockDim.x >> 5) {
+            const double sum = pq::ordered_sum(s ? p.weights.sumsq_w : p.weights.sumsq_a, K);
+            if ((threadIdx.x & 31) == 0) p.weights.lambda[s] = __ddiv_rn(1.0, sum);
+        }
+        return;
+    }
 
     // Slots of the orders.  The two 16-byte halves of a run's lie in separate planes: lanes read consecutive 16-byte words.
     auto slots_at = [&](int j) { return slot_s + ((j >> 3) & 1) * (K >> 1) + (j >> 4) * 8 + (j & 7); };
@@ -414,14 +424,6 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     __syncthreads();
 
     const int grp = threadIdx.x / p.group_threads, tid = threadIdx.x - grp * p.group_threads;
-    if (grp >= p.groups) {  // the extra warp
-        for (int s = 0; s < 2; ++s)
-            if (blockIdx.y == 0 && blockIdx.x == min(static_cast<unsigned>(s), gridDim.x - 1)) {
-                const double sum = pq::ordered_sum(s ? p.weights.sumsq_w : p.weights.sumsq_a, K);
-                if ((threadIdx.x & 31) == 0) p.weights.lambda[s] = __ddiv_rn(1.0, sum);
-            }
-        return;
-    }
     auto group_sync = [&]() {
         if (p.group_threads == 32) __syncwarp();
         else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(p.group_threads) : "memory");
@@ -436,7 +438,7 @@ __global__ void __launch_bounds__(kGatherThreads + 32, 1) group_error_gather(con
     // part a group that has work for a few chunks only would wait for the one that has a whole chunk more; without the
     // second a group would stage one more chunk of which it uses some orders (eight batches of 4608 x 3072 and a
     // 9216 x 3072 weight: 535 us a calibration all in pairs, 518 like this; 473 with the present fold).
-    const uint32_t shares = gridDim.x * p.groups, share = blockIdx.x * p.groups + grp;
+    const uint32_t shares = p.blocks * p.groups, share = blockIdx.x * p.groups + grp;
     const uint32_t base = p.base[o0 + no == p.P], rem = p.rem[o0 + no == p.P];
     const uint32_t first = share * base + min(share, rem);
     int pairs = static_cast<int>(base + (share < rem)), full = p.full * no;
@@ -657,7 +659,7 @@ pq_status fold(const void *part, int64_t count, int64_t n, double *err, cudaStre
 // list, ts, identity, perms, chunks and weights of p are set by the caller.
 template <int KIND, int TEAM>
 pq_status launch_gather(GatherParams &p, int64_t K, int P, float Qf, float *part, cudaStream_t st) {
-    const int sms = sm_count(), sides = KIND == 0 && p.ts[1] ? 2 : 1;
+    const int weights = p.weights.lambda ? 1 : 0, sms = sm_count() - weights, sides = KIND == 0 && p.ts[1] ? 2 : 1;
     const GatherConfig cfg = gather_config(p.chunks, K, P, sides, sms);
     if (!cfg.groups) return PQ_ERR_SHAPE;
     p.K = static_cast<int>(K), p.P = P, p.Qf = Qf, p.part = part;
@@ -675,9 +677,9 @@ pq_status launch_gather(GatherParams &p, int64_t K, int P, float Qf, float *part
     const size_t smem = gather_smem_bytes(K, cfg.opb, cfg.groups, sides);
     auto kern = group_error_gather<KIND, TEAM / 2>;
     PQ_CUDA_OK(pq::allow_smem(kern, smem, kGatherSmemMax));
-    const unsigned threads = static_cast<unsigned>(cfg.groups * cfg.group_threads + (p.weights.lambda ? 32 : 0));
-    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(subsets)),
-                                    dim3(threads), smem, st, p));
+    p.blocks = static_cast<int>(blocks);
+    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks + weights), static_cast<unsigned>(subsets)),
+                                    dim3(static_cast<unsigned>(cfg.groups * cfg.group_threads)), smem, st, p));
     return pq_launch_status();
 }
 

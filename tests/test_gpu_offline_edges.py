@@ -119,6 +119,12 @@ def test_one_call_equals_the_separate_calls(rows, N, K, fmt, J):
         assert torch.equal(getattr(c, name), t), name
 
 
+@pytest.mark.parametrize("rows,N,K,fmt,J", [([2500], 264, 3072, (B.KIND_NVFP4, 4, 16), 5),         # all SMs but one gather
+                                            ([700], 136, 16384, (B.KIND_INT, 4, 128), 7)])          # ... in subsets of the orders
+def test_weights_beside_a_full_chip(rows, N, K, fmt, J):
+    test_one_call_equals_the_separate_calls(rows, N, K, fmt, J)
+
+
 @pytest.mark.parametrize("n", [40, 26])      # 1440 slabs in two rounds; 936 in one, and the weight in one of its own
 def test_rounds_of_many_slabs_equal_the_separate_calls(n):
     """More partial sums than one round's 64 MiB hold (1213 slabs of these widths)."""

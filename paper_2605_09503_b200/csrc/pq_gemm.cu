@@ -102,7 +102,7 @@ struct Tile {
     static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38 or 28 * 1024
     static constexpr uint32_t kSfSlotCol0 = BN, kSfbColsPerKb = 4 * kNB, kSfbOfs = 16;
     static constexpr uint32_t kSfSlotCols = 4 * (4 + kSfbColsPerKb);   // 48 or 32
-    static constexpr int kNumBars = 2 * kStages + 2;      // stage_full[S] stage_free[S] acc_full acc_empty
+    static constexpr int kNumBars = (kOneTile ? 3 : 2) * kStages + 2;  // stage_full[S] stage_free[S] acc_full acc_empty, narrow: sf_ready[S]
     static constexpr int kRingBytes = kStages * kStageBytes, kEpi = kOneTile ? 0 : kRingBytes;  // where the boxes start
     static constexpr size_t kSmemBytes = kRingBytes + (kOneTile ? 0 : kEpiBytes) + 1024 /*alignment slack*/ + 8 * kNumBars + 64;
     // Instruction descriptor: E2M1 x E2M1, UE4M3 scales, both K-major, M = 256 (pair), N = BN, K = 64.
@@ -111,6 +111,18 @@ struct Tile {
     static_assert(kStageBytes % 1024 == 0, "swizzled operand tiles start on 1024-byte boundaries");
     static_assert(kSfSlotCol0 + kStages * kSfSlotCols <= 512, "tensor memory columns");
     static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
+};
+
+// What the kernel reads its operands by.  The wide tile's scale blocks come by tensor maps, too; the narrow tile's as plain bulk
+// copies, which spares a small product 256 bytes of launch parameters (0.35 us of host time a launch).
+template <int BN>
+struct Maps {
+    CUtensorMap a, b, y, sfa, sfb;
+};
+template <>
+struct Maps<128> {
+    CUtensorMap a, b, y;
+    const uint8_t *sfx, *sfw;
 };
 
 struct GemmParams {
@@ -235,6 +247,11 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster)
         : "memory");
 }
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int x, int y, uint32_t src) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
                  ::"l"(map), "r"(x), "r"(y), "r"(src)
@@ -328,9 +345,7 @@ __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo_bits, uint32_t hi_bits
 constexpr int kMaxRegs = 128;
 template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kMaxRegs)
-gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                 const __grid_constant__ CUtensorMap map_sfa, const __grid_constant__ CUtensorMap map_sfb,
-                 const __grid_constant__ CUtensorMap map_y, const GemmParams p) {
+gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
     using T = Tile<BN>;
     constexpr int kStages = T::kStages, kNB = T::kNB, BN_CTA = T::kNCta;
     constexpr int kBBytes = T::kBBytes, kStageBytes = T::kStageBytes, kNumBars = T::kNumBars;
@@ -343,11 +358,13 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     const uint32_t epi = base + T::kEpi;
     const uint32_t bars = base + kBarOfs;
     uint8_t *bars_ptr = base_ptr + kBarOfs;
-    // stage_full: operand and scale bytes of both CTAs have landed (1 arrival + transaction bytes); leader's copy only
+    // stage_full: operand and scale bytes of both CTAs have landed; leader's copy only.  Wide: 1 arrival + transaction bytes.  Narrow:
+    // a bulk copy reports to its own CTA, so the other CTA's scales report to its sf_ready, and its warp 1 passes that on (2 arrivals).
     auto stage_full_bar = [&](int s) { return bars + 8u * s; };
         auto stage_free_bar = [&](int s) { return bars + 8u * (kStages + s); };  // the stage's MMAs have run
     const uint32_t acc_full_bar = bars + 8u * (2 * kStages);       // one copy per CTA, both signalled by the issuer
     const uint32_t acc_empty_bar = bars + 8u * (2 * kStages + 1);  // leader's copy only
+    auto sf_ready_bar = [&](int s) { return bars + 8u * (2 * kStages + 2 + s); };  // narrow tile
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars_ptr + 8 * kNumBars);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_ptr + 8 * kNumBars + 8);
     const WaitCtx wctx{abort_flag, p.status, p.wait_cycles};
@@ -359,18 +376,18 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(stage_full_bar(s), 1);
+            mbar_init(stage_full_bar(s), T::kOneTile ? 2 : 1);
+            if (T::kOneTile) mbar_init(sf_ready_bar(s), 1);
             mbar_init(stage_free_bar(s), 1);
         }
         mbar_init(acc_full_bar, 1);
         mbar_init(acc_empty_bar, 2 * kEpiWarps);  // the epilogue warps of both CTAs
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        prefetch_tensormap(&map_a);
-        prefetch_tensormap(&map_b);
-        prefetch_tensormap(&map_sfa);
-        prefetch_tensormap(&map_sfb);
-        prefetch_tensormap(&map_y);
+        prefetch_tensormap(&maps.a);
+        prefetch_tensormap(&maps.b);
+        if constexpr (!T::kOneTile) prefetch_tensormap(&maps.sfa), prefetch_tensormap(&maps.sfb);
+        prefetch_tensormap(&maps.y);
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -410,21 +427,30 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 const uint32_t sf_stage = stage + kABytes + kBBytes;
                 const uint32_t full_leader = mapa(stage_full_bar(s), 0);
                 if (elect_one()) {
-                    if (rank == 0) mbar_expect_tx(stage_full_bar(s), 2u * kStageBytes);
-                    tma_load_2d_pair(stage, &map_a, kt * (BK / 2), m0, full_leader);
-                    tma_load_2d_pair(stage + kABytes, &map_b, kt * (BK / 2), n0 + static_cast<int>(rank) * BN_CTA,
-                                     full_leader);
-                    tma_load_2d_pair(sf_stage, &map_sfa, kt * (4 * kSfBlock / 8), m0 >> 7, full_leader);
-                    tma_load_2d_pair(sf_stage + kSfaBytes, &map_sfb, kt * (4 * kSfBlock / 8), n0 >> 7, full_leader);
+                    if constexpr (T::kOneTile) {
+                        // the other CTA's rows may lie past the last block of rows: any block will do for them
+                        const uint32_t sf_bytes = static_cast<uint32_t>(min(4, p.kb_total - kt * 4)) * kSfBlock;
+                        const int64_t kofs = static_cast<int64_t>(kt) * 4 * kSfBlock, pitch = static_cast<int64_t>(p.kb_total) * kSfBlock;
+                        const uint32_t sf_bar = rank == 0 ? stage_full_bar(s) : sf_ready_bar(s);
+                        mbar_expect_tx(sf_bar, 2u * sf_bytes + (rank == 0 ? 2u * (kABytes + kBBytes) : 0u));
+                        bulk_load(sf_stage, maps.sfx + min(m0 >> 7, (p.M - 1) >> 7) * pitch + kofs, sf_bytes, sf_bar);
+                        bulk_load(sf_stage + kSfaBytes, maps.sfw + (n0 >> 7) * pitch + kofs, sf_bytes, sf_bar);
+                    } else {
+                        if (rank == 0) mbar_expect_tx(stage_full_bar(s), 2u * kStageBytes);
+                        tma_load_2d_pair(sf_stage, &maps.sfa, kt * (4 * kSfBlock / 8), m0 >> 7, full_leader);
+                        tma_load_2d_pair(sf_stage + kSfaBytes, &maps.sfb, kt * (4 * kSfBlock / 8), n0 >> 7, full_leader);
+                    }
+                    tma_load_2d_pair(stage, &maps.a, kt * (BK / 2), m0, full_leader);
+                    tma_load_2d_pair(stage + kABytes, &maps.b, kt * (BK / 2), n0 + static_cast<int>(rank) * BN_CTA, full_leader);
                 }
                 __syncwarp();
             }
         }
-        if (!ok && lane == 0 && rank == 0) {
-            // give the copies already issued (both CTAs': they count on this barrier) a bounded chance to land before leaving
+        if (!ok && lane == 0 && (rank == 0 || T::kOneTile)) {
+            // give the copies already issued (they count on these barriers) a bounded chance to land before leaving
             const uint32_t first = it > kStages ? it - kStages : 0;
             for (uint32_t j = first; j < it; ++j)
-                for (uint32_t i = 0; i < 4096 && !mbar_try(stage_full_bar(j % kStages), (j / kStages) & 1u); ++i) {}
+                for (uint32_t i = 0; i < 4096 && !mbar_try(rank == 0 ? stage_full_bar(j % kStages) : sf_ready_bar(j % kStages), (j / kStages) & 1u); ++i) {}
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -450,7 +476,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     const uint32_t sfa_t = tmem_base + sf_slot_col(s), sfb_t = sfa_t + kSfbOfs;
                     const int kb_valid = min(4, p.kb_total - kt * 4);
                     if (elect_one()) {
-                        // (blocks past the last channel are zeros and belong to no MMA)
+                        // (what lies behind the last channel, zeros or an older stage, belongs to no MMA)
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
                             tc_cp_scales(sfa_t + 4 * kk, ds + kk * (kSfBlock / 16));
@@ -475,6 +501,13 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     s = (s + 1 == kStages) ? 0u : s + 1;
                     ph ^= (s == 0) ? 1u : 0u;
                 }
+            }
+        } else if (T::kOneTile) {
+            // the other CTA: its scales have landed
+            bool ok = true;
+            for (int kt = 0; kt < p.k_tiles && ok; ++kt) {
+                ok = mbar_wait_warp(sf_ready_bar(kt % kStages), static_cast<uint32_t>(kt / kStages) & 1u, wctx);
+                if (ok && lane == 0) mbar_arrive_remote(stage_full_bar(kt % kStages), 0);
             }
         }
     } else {
@@ -536,7 +569,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    if (m0 < p.M && n0 + c * kBoxCols < p.N) tma_store_2d(&map_y, n0 + c * kBoxCols, m0, buf);
+                    if (m0 < p.M && n0 + c * kBoxCols < p.N) tma_store_2d(&maps.y, n0 + c * kBoxCols, m0, buf);
                     bulk_commit();
                 }
             }
@@ -609,7 +642,7 @@ bool encode_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t row_byt
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// What the maps of an operand (codes and scale blocks; rows x K) or of the output (sf = NULL; rows x K, ld) depend on.
+// What the maps of an operand (ld = 0: codes and, unless sf is NULL, scale blocks; rows x K) or of the output (rows x K, ld) depend on.
 struct MapKey {
     const void *ptr, *sf;
     int64_t rows, K, ld;
@@ -631,7 +664,7 @@ const MapSlot *find_maps(const MapKey &key) {
     static thread_local MapSlot cache[kSlots];
     static thread_local uint32_t next = 0;
     const uint64_t mix = (reinterpret_cast<uintptr_t>(key.ptr) >> 4) ^ (static_cast<uint64_t>(key.rows) << 20) ^
-                         (static_cast<uint64_t>(key.ld) << 40) ^ static_cast<uint64_t>(key.box_rows);
+                         (static_cast<uint64_t>(key.K) << 40) ^ static_cast<uint64_t>(key.box_rows);
     const uint32_t home = static_cast<uint32_t>((mix * 0x9E3779B97F4A7C15ull) >> 58);
     uint32_t at = home + next % kProbes;  // an empty slot, or one of the four in turn
     for (uint32_t i = 0; i < kProbes; ++i) {
@@ -646,12 +679,12 @@ const MapSlot *find_maps(const MapKey &key) {
     MapSlot &slot = cache[at % kSlots];
     slot.used = false;
     slot.key = key;
-    if (key.sf) {
+    if (key.ld) {
+        slot.used = encode_map(&slot.map, key.ptr, key.rows, key.K * 2, key.ld * 2, key.box_rows, 2);
+    } else {
         const int64_t sf_pitch = key.K / 64 * kSfBlock;
         slot.used = encode_map(&slot.map, key.ptr, key.rows, key.K / 2, key.K / 2, key.box_rows, 1) &&
-                    encode_map(&slot.scales, key.sf, pq_ceil_div(key.rows, 128), sf_pitch, sf_pitch, key.sf_box_rows, 8);
-    } else {
-        slot.used = encode_map(&slot.map, key.ptr, key.rows, key.K * 2, key.ld * 2, key.box_rows, 2);
+                    (!key.sf || encode_map(&slot.scales, key.sf, pq_ceil_div(key.rows, 128), sf_pitch, sf_pitch, key.sf_box_rows, 8));
     }
     return slot.used ? &slot : nullptr;
 }
@@ -701,19 +734,25 @@ struct GemmArgs {
 
 template <int BN>
 pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
+    Maps<BN> maps;
     // copied one by one: a later entry may take an earlier one's slot
-    CUtensorMap map_a, map_b, map_sfa, map_sfb, map_y;
-    auto operand = [&](CUtensorMap &map, CUtensorMap *scales, const MapKey &key) {
+    auto find = [&](CUtensorMap &map, CUtensorMap *scales, const MapKey &key) {
         const MapSlot *slot = find_maps(key);
         if (!slot) return false;
         map = slot->map;
         if (scales) *scales = slot->scales;
         return true;
     };
-    if (!operand(map_a, &map_sfa, MapKey{g.xq, g.sfx, g.M, g.K, g.K, BM_CTA, 1}) ||
-        !operand(map_b, &map_sfb, MapKey{g.wq, g.sfw, g.N, g.K, g.K, Tile<BN>::kNCta, Tile<BN>::kNB}) ||
-        !operand(map_y, nullptr, MapKey{g.Y, nullptr, g.M, g.N, g.ldy, 32, 0}))
-        return PQ_ERR_CUDA;
+    bool found = find(maps.y, nullptr, MapKey{g.Y, nullptr, g.M, g.N, g.ldy, 32, 0});
+    if constexpr (Tile<BN>::kOneTile) {
+        maps.sfx = g.sfx, maps.sfw = g.sfw;
+        found = found && find(maps.a, nullptr, MapKey{g.xq, nullptr, g.M, g.K, 0, BM_CTA, 0}) &&
+                find(maps.b, nullptr, MapKey{g.wq, nullptr, g.N, g.K, 0, Tile<BN>::kNCta, 0});
+    } else {
+        found = found && find(maps.a, &maps.sfa, MapKey{g.xq, g.sfx, g.M, g.K, 0, BM_CTA, 1}) &&
+                find(maps.b, &maps.sfb, MapKey{g.wq, g.sfw, g.N, g.K, 0, Tile<BN>::kNCta, Tile<BN>::kNB});
+    }
+    if (!found) return PQ_ERR_CUDA;
     GemmParams p;
     p.ts_x = g.ts_x, p.ts_w = g.ts_w;
     p.M = static_cast<int>(g.M), p.N = static_cast<int>(g.N);
@@ -740,7 +779,7 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    PQ_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel<BN>, map_a, map_b, map_sfa, map_sfb, map_y, p));
+    PQ_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel<BN>, maps, p));
     return PQ_OK;
 }
 

@@ -114,7 +114,8 @@ struct Tile {
 };
 
 // What the kernel reads its operands by.  The wide tile's scale blocks come by tensor maps, too; the narrow tile's as plain bulk
-// copies, which spares a small product 256 bytes of launch parameters (0.35 us of host time a launch).
+// copies of just the blocks a K step has: no two more descriptors to fetch at the start of a short kernel (quantize + GEMM of
+// 512 x 3072 x 3072 8.7 us against 9.2 with maps; on the wide tile not tried).
 template <int BN>
 struct Maps {
     CUtensorMap a, b, y, sfa, sfb;
@@ -783,16 +784,15 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
     return PQ_OK;
 }
 
-// One round of narrow tiles covers the product.  Measured on both sides of the line (narrow against wide, us):
-// 128 x 3072 x 3072 6.9 / 8.1, 512 x 3072 x 3072 7.4 / 8.3, 512 x 3072 x 12288 18.0 / 20.5; beyond one round the wide tile wins:
-// 512 x 9216 x 3072 12.2 / 10.9, 1024 x 3072 x 3072 11.2 / 9.4, 4608 x 9216 x 3072 72.8 / 56.9.
+// One round of narrow tiles covers the product.  Measured on both sides of the line (M x N x K, narrow against wide, us):
+// 128 x 3072 x 3072 6.2 / 7.6, 512 x 3072 x 3072 6.6 / 7.7, 512 x 3072 x 12288 16.1 / 19.3, 512 x 4736 x 3072 7.3 / 8.1; beyond one
+// round the wide tile wins (512 x 9216 x 3072 12.2 / 10.9, 1024 x 3072 x 3072 11.2 / 9.4 before the scales came by tcgen05.cp).
 // Few rows: the CTAs of all pairs fetch the same few lines of X at every K step, and with more than half of the pairs at that the
-// narrow tile loses for one or two rows (1 x 5120 x 3072 8.6 / 7.6, 1 x 9216 x 12288 25.6 / 21.9, 2 x 7168 x 12288 21.0 / 18.3) and
-// for up to 16 on long rows (4 x 8192 x 12288 21.7 / 19.7); 8 x 5120 x 3072 7.2 / 8.0, 24 x 9216 x 12288 17.9 / 20.1.
-bool narrow_tiles(int64_t M, int64_t N, int64_t K, int pairs) {
+// narrow tile loses up to 16 rows (1 x 5120 x 3072 8.4 / 6.8, 4 x 9216 x 3072 7.7 / 7.1, 8 x 5120 x 3072 7.0 / 6.7, 2 x 7168 x 12288
+// 22.8 / 21.2, 16 x 9216 x 12288 22.2 / 21.4; 24 x 9216 x 12288 16.0 / 19.6).
+bool narrow_tiles(int64_t M, int64_t N, int pairs) {
     const int64_t tiles = pq_ceil_div(M, BM) * pq_ceil_div(N, 128);
-    const bool few = M <= 2 || (M <= 16 && K > 3072);
-    return tiles <= (few ? pairs / 2 : pairs);
+    return tiles <= (M <= 16 ? pairs / 2 : pairs);
 }
 
 pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, const uint8_t *wq, const uint8_t *sfw,
@@ -811,7 +811,7 @@ pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, 
     const int dev = pq_device_slot(), pairs_max = resident_pairs<256>(dev), pairs_narrow = resident_pairs<128>(dev);
     if (pairs_max <= 0 || pairs_narrow <= 0) return PQ_ERR_CUDA;
     const GemmArgs g{xq, sfx, wq, sfw, ts_x, ts_w, M, N, K, ldy, Y, ws, st};
-    return narrow_tiles(M, N, K, pairs_narrow) ? launch_tiles<128>(g, pairs_narrow) : launch_tiles<256>(g, pairs_max);
+    return narrow_tiles(M, N, pairs_narrow) ? launch_tiles<128>(g, pairs_narrow) : launch_tiles<256>(g, pairs_max);
 }
 }  // namespace
 

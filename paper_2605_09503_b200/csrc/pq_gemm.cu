@@ -123,10 +123,10 @@ struct Maps {
 template <>
 struct Maps<128> {
     CUtensorMap a, b, y;
-    const uint8_t *sfx, *sfw;
 };
 
 struct GemmParams {
+    const uint8_t *sfx, *sfw;  // narrow tile
     const float *ts_x, *ts_w;
     int M, N;
     int m_tiles, n_tiles, k_tiles, kb_total;
@@ -434,8 +434,8 @@ gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
                         const int64_t kofs = static_cast<int64_t>(kt) * 4 * kSfBlock, pitch = static_cast<int64_t>(p.kb_total) * kSfBlock;
                         const uint32_t sf_bar = rank == 0 ? stage_full_bar(s) : sf_ready_bar(s);
                         mbar_expect_tx(sf_bar, 2u * sf_bytes + (rank == 0 ? 2u * (kABytes + kBBytes) : 0u));
-                        bulk_load(sf_stage, maps.sfx + min(m0 >> 7, (p.M - 1) >> 7) * pitch + kofs, sf_bytes, sf_bar);
-                        bulk_load(sf_stage + kSfaBytes, maps.sfw + (n0 >> 7) * pitch + kofs, sf_bytes, sf_bar);
+                        bulk_load(sf_stage, p.sfx + min(m0 >> 7, (p.M - 1) >> 7) * pitch + kofs, sf_bytes, sf_bar);
+                        bulk_load(sf_stage + kSfaBytes, p.sfw + (n0 >> 7) * pitch + kofs, sf_bytes, sf_bar);
                     } else {
                         if (rank == 0) mbar_expect_tx(stage_full_bar(s), 2u * kStageBytes);
                         tma_load_2d_pair(sf_stage, &maps.sfa, kt * (4 * kSfBlock / 8), m0 >> 7, full_leader);
@@ -746,7 +746,6 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
     };
     bool found = find(maps.y, nullptr, MapKey{g.Y, nullptr, g.M, g.N, g.ldy, 32, 0});
     if constexpr (Tile<BN>::kOneTile) {
-        maps.sfx = g.sfx, maps.sfw = g.sfw;
         found = found && find(maps.a, nullptr, MapKey{g.xq, nullptr, g.M, g.K, 0, BM_CTA, 0}) &&
                 find(maps.b, nullptr, MapKey{g.wq, nullptr, g.N, g.K, 0, Tile<BN>::kNCta, 0});
     } else {
@@ -755,7 +754,7 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
     }
     if (!found) return PQ_ERR_CUDA;
     GemmParams p;
-    p.ts_x = g.ts_x, p.ts_w = g.ts_w;
+    p.sfx = g.sfx, p.sfw = g.sfw, p.ts_x = g.ts_x, p.ts_w = g.ts_w;
     p.M = static_cast<int>(g.M), p.N = static_cast<int>(g.N);
     p.m_tiles = static_cast<int>(pq_ceil_div(g.M, BM));
     p.n_tiles = static_cast<int>(pq_ceil_div(g.N, BN));

@@ -415,7 +415,8 @@ pq_status pq_hadamard_quant_nvfp4(const void *X, int64_t M, int64_t K, int64_t l
                                   void *y_out, void *stream);
 
 /* Integer fake-quant of Eq. 1-2 (quantize, dequantize, round to bf16), optional gather.
- *   T : bf16 [rows, K], ld.  out : bf16 [rows, K], ldo.  perm : int32 [K] or NULL.
+ *   T : bf16 [rows, K], ld.  out : bf16 [rows, K], ldo; may be T itself (ldo == ld), otherwise apart from it.
+ *   perm : int32 [K] or NULL.
  *   fmt.kind must be 1; fmt.group in {16, 32, 64, 128, 256}; K % fmt.group == 0; K <= 16384 when perm != NULL. */
 pq_status pq_fakequant_int(const void *T, int64_t rows, int64_t K, int64_t ld, pq_format fmt,
                            const int32_t *perm, void *out, int64_t ldo, void *stream);

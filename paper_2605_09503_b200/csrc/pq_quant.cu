@@ -235,8 +235,7 @@ __device__ __forceinline__ uint4 fakequant8(const float (&x)[8], float Qf) {
 // warp (K % (8 TEAM) == 0 and 32 % TEAM == 0), dead lanes carry zeros through the shuffles.
 template <int TEAM>
 __global__ void __launch_bounds__(kQuantThreads)
-fakequant_int_kernel(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int64_t ld, float Qf,
-                     uint16_t *__restrict__ out, int64_t ldo) {
+fakequant_int_kernel(const uint16_t *T, int64_t rows, int64_t K, int64_t ld, float Qf, uint16_t *out, int64_t ldo) {
     const int64_t oct = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;
     const int64_t row = row_block_index() * kTileRows + threadIdx.y;
     const bool live = row < rows && oct * 8 < K;
@@ -311,9 +310,7 @@ __device__ __forceinline__ void fakequant_row_pair(const uint32_t (&u)[8], const
 
 template <int TEAM>
 __global__ void __launch_bounds__(kFqThreads, 2)
-fakequant_int_gather_kernel(const uint16_t *__restrict__ T, int64_t rows, int K, int64_t ld,
-                            const int32_t *__restrict__ perm, float Qf, uint16_t *__restrict__ out,
-                            int64_t ldo) {
+fakequant_int_gather_kernel(const uint16_t *T, int64_t rows, int K, int64_t ld, const int32_t *perm, float Qf, uint16_t *out, int64_t ldo) {
     extern __shared__ __align__(16) uint4 quad_s[];  // [K][4 rows]
     __shared__ uint2 tab[128];
     const int octs = K >> 3;
@@ -324,7 +321,7 @@ fakequant_int_gather_kernel(const uint16_t *__restrict__ T, int64_t rows, int K,
     auto load_octet = [&](int o, uint4 (&v)[4]) {
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-            v[r] = o < octs && r < live_rows ? __ldg(reinterpret_cast<const uint4 *>(T + r * ld) + o) : make_uint4(0, 0, 0, 0);
+            v[r] = o < octs && r < live_rows ? __ldca(reinterpret_cast<const uint4 *>(T + r * ld) + o) : make_uint4(0, 0, 0, 0);
     };
     pq::build_int_tab(tab, Qf, false);  // needs nothing of the kernel in front
     pq::dependents_may_launch();
@@ -344,11 +341,11 @@ fakequant_int_gather_kernel(const uint16_t *__restrict__ T, int64_t rows, int K,
         const int32_t *src = perm + (live ? 8 * o : 0);
         int idx[8];
         if (aligned) {
-            const int4 i0 = __ldg(reinterpret_cast<const int4 *>(src)), i1 = __ldg(reinterpret_cast<const int4 *>(src) + 1);
+            const int4 i0 = __ldca(reinterpret_cast<const int4 *>(src)), i1 = __ldca(reinterpret_cast<const int4 *>(src) + 1);
             idx[0] = i0.x, idx[1] = i0.y, idx[2] = i0.z, idx[3] = i0.w, idx[4] = i1.x, idx[5] = i1.y, idx[6] = i1.z, idx[7] = i1.w;
         } else {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) idx[i] = __ldg(src + i);
+            for (int i = 0; i < 8; ++i) idx[i] = __ldca(src + i);
         }
         uint32_t lo[8], hi[8];
 #pragma unroll

@@ -257,12 +257,18 @@ fakequant_int_kernel(const uint16_t *T, int64_t rows, int64_t K, int64_t ld, flo
 // side in packed fp32 registers.  Everything works on magnitudes (sign-symmetric, round to nearest even), the
 // sign bits come back at the end; the scale comes from a table by the mantissa of the absmax.  A block is one
 // group of four rows and five of them share an SM at 3072 channels (192 threads, 64 registers), so some load while others
-// compute: 16.6 us for 4608 x 3072, INT4 g64, from HBM; 12.8 without an order.  Calls one behind the other overlap (programmatic
-// dependent launch): 16.2 us a call in a loop, 18.3 without.  Persistent blocks with the next rows copied ahead, and slots from
-// a table, were slower at every size (600 x 3072 8.1 against 4.7, 18432 x 3072 49.4 against 46.6).
+// compute.  Persistent blocks with the next rows copied ahead, and slots from
+// a table, were slower at every size (600 x 3072 8.1 us against 4.7, 18432 x 3072 49.4 against 46.6).
+// Launched as a programmatic dependent.  More than a block per SM: nothing is allowed to start before this grid's last blocks
+// end, and the scale table is built while the first rows are on their way.  The next call's blocks, let in early, take the places that
+// are free and not the ones that balance the SMs: 2000 x 1024 6.1 us a call in a graph against 4.3, 1200 x 3072 8.4 / 6.7, and the
+// table in front of the loads adds to every block: 18432 x 3072 50.0 / 46.7, 57.5 / 54.1 for a call alone.  A block
+// per SM at most: the next call's are let in and build their tables early, 256 x 512 1.9 / 2.2.  (4608 x 3072, INT4 g64: 15.7 us a
+// call in a stream, 18.2 by an ordinary launch; 15.6 against 15.7 in a graph.)
 // The kernel before it staged one row per block and gathered two bytes at a time, about four shared-memory
 // wavefronts per 32 elements and two divisions per eight: 30.7 us for 4608 x 3072, INT4 g64.
 constexpr int kFqThreads = 512;
+constexpr unsigned kFqFewBlocks = 148;  // one per SM
 
 // Eight positions of two rows: u[i] = position i of row 0 (low half) and row 1 (high half), w0 / w1 = the rows' results.
 template <int TEAM>
@@ -323,11 +329,13 @@ fakequant_int_gather_kernel(const uint16_t *T, int64_t rows, int K, int64_t ld, 
         for (int r = 0; r < 4; ++r)
             v[r] = o < octs && r < live_rows ? __ldca(reinterpret_cast<const uint4 *>(T + r * ld) + o) : make_uint4(0, 0, 0, 0);
     };
-    pq::build_int_tab(tab, Qf, false);  // needs nothing of the kernel in front
-    pq::dependents_may_launch();
+    const bool few = gridDim.x <= kFqFewBlocks;
+    if (few) pq::build_int_tab(tab, Qf, false);
     pq::wait_for_prior_grid();
+    if (few) pq::dependents_may_launch();
     uint4 v[4];
     load_octet(threadIdx.x, v);
+    if (!few) pq::build_int_tab(tab, Qf, false);
     for (int o = threadIdx.x; o < octs; o += blockDim.x) {
         pq::store_quad_octet(quad_s, o, v);
         load_octet(o + blockDim.x, v);

@@ -24,7 +24,7 @@ def test_order_matches_gathered_columns(rows, K, shift, bits, group):
     assert torch.equal(out.contiguous().view(torch.int16), want.view(torch.int16))
 
 
-@pytest.mark.parametrize("rows,K", [(30, 768), (2501, 3072)])
+@pytest.mark.parametrize("rows,K", [(30, 768), (592, 512), (593, 512), (2501, 3072)])      # 148 and 149 blocks with an order
 def test_chain_of_calls(rows, K):
     """Blocks start before the call in front has finished: a chain, in place in parts, gives what it gives call by call."""
     perm = torch.randperm(K, generator=torch.Generator().manual_seed(5)).to(DEV).to(torch.int32)

@@ -521,7 +521,7 @@ gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
         constexpr int kCols = BN / 2, kBoxes = kCols / kBoxCols, kChunks = kBoxCols / 8;  // boxes per warp, 16-byte chunks per box row
         const int q = warp & 3;                // tensor-memory lane quadrant this warp may read
         const int h = (warp - 2) >> 2;         // column half
-        const float alpha = __fmul_rn(__ldg(p.ts_x), __ldg(p.ts_w));
+        const float alpha = __fmul_rn(__ldca(p.ts_x), __ldca(p.ts_w));
         const uint32_t buf = epi + static_cast<uint32_t>(warp - 2) * kEpiBox;
         // 128-byte swizzle of the staging box (what the store's tensor map expects): chunk ^ (row & 7)
         const uint32_t row_ofs = static_cast<uint32_t>(lane) * (kBoxCols * 2), sw = static_cast<uint32_t>(lane & 7);

@@ -231,8 +231,8 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) hadamard_quant_kernel(
     // where each output position reads its channel in a row's (swizzled) shared-memory image, as a byte
     // offset: the same for every row, so it is worked out once per block (K <= 16384: 16 bits)
     for (int j = threadIdx.x; j < p.K; j += THREADS)
-        offset_s[j] = static_cast<uint16_t>(swz(p.perm ? __ldg(p.perm + j) : j, p.sw) << 2);
-    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldg(p.ts) : 1.0f);
+        offset_s[j] = static_cast<uint16_t>(swz(p.perm ? p.perm[j] : j, p.sw) << 2);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldca(p.ts) : 1.0f);
 
     for (int64_t batch = blockIdx.x; batch < batches; batch += gridDim.x) {
         const int64_t row0 = batch * kRows;
@@ -560,8 +560,8 @@ __global__ void __launch_bounds__(32 * kRowWarps, 2) hadamard_quant_rows_kernel(
     // so that the lanes' 16-byte reads are adjacent
     for (int j = threadIdx.x; j < K; j += 32 * kRowWarps)
         offset_s[((j >> 3) & 1) * (K / 2) + (j >> 4) * 8 + (j & 7)] =
-            static_cast<uint16_t>(row_image_index<N>(p.perm ? __ldg(p.perm + j) : j) << 2);
-    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldg(p.ts) : 1.0f);
+            static_cast<uint16_t>(row_image_index<N>(p.perm ? p.perm[j] : j) << 2);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldca(p.ts) : 1.0f);
     __syncthreads();
 
     // warps of different blocks first, so that few rows spread over all SMs
@@ -630,8 +630,8 @@ __global__ void __launch_bounds__(512, 1) hadamard_quant_team_kernel(const HadPa
     pq::dependents_may_launch();
     for (int j = threadIdx.x; j < K; j += 512)
         offset_s[((j >> 3) & 1) * (K / 2) + (j >> 4) * 8 + (j & 7)] =
-            static_cast<uint16_t>(row_image_index<N>(p.perm ? __ldg(p.perm + j) : j) << 2);
-    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldg(p.ts) : 1.0f);
+            static_cast<uint16_t>(row_image_index<N>(p.perm ? p.perm[j] : j) << 2);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldca(p.ts) : 1.0f);
     __syncthreads();
     auto team_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(NT) : "memory"); };
 
@@ -704,8 +704,8 @@ __global__ void __launch_bounds__(32 * WARPS, 2) hadamard_quant_pow2_kernel(cons
     pq::dependents_may_launch();
     for (int j = threadIdx.x; j < K; j += 32 * WARPS)
         offset_s[((j >> 3) & 1) * (K / 2) + (j >> 4) * 8 + (j & 7)] =
-            static_cast<uint16_t>(pow2_image_index<P1>(p.perm ? __ldg(p.perm + j) : j) << 2);
-    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldg(p.ts) : 1.0f);
+            static_cast<uint16_t>(pow2_image_index<P1>(p.perm ? p.perm[j] : j) << 2);
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(p.codes ? __ldca(p.ts) : 1.0f);
     __syncthreads();
 
     const int64_t batches = (p.rows_pad + RPW - 1) / RPW, step = static_cast<int64_t>(gridDim.x) * WARPS;
@@ -720,7 +720,7 @@ __global__ void __launch_bounds__(32 * WARPS, 2) hadamard_quant_pow2_kernel(cons
                 const bool have = row0 + r < p.rows;  // rows past the end are zeros
                 uint4 raw[BL / 8];
 #pragma unroll
-                for (int q = 0; q < BL / 8; ++q) raw[q] = have ? __ldg(src + q) : make_uint4(0, 0, 0, 0);
+                for (int q = 0; q < BL / 8; ++q) raw[q] = have ? __ldca(src + q) : make_uint4(0, 0, 0, 0);
                 uint64_t v[BL / 2];
 #pragma unroll
                 for (int q = 0; q < BL / 8; ++q) {

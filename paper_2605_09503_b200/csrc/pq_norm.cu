@@ -262,10 +262,10 @@ __device__ __forceinline__ float row_minus(const uint2 &g, int r, float c) {
 
 template <int KIND, int SF_LAYOUT>
 __global__ void __launch_bounds__(32 * kGroupWarps * kSplit, 2)
-norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
-                        const float *__restrict__ a, const float *__restrict__ b, float eps,
-                        const int32_t *__restrict__ perm,
-                        const float *__restrict__ ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
+norm_quant_grouped_kernel(const uint16_t *H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
+                        const float *a, const float *b, float eps,
+                        const int32_t *perm,
+                        const float *ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
                         uint16_t *__restrict__ y_out) {
     extern __shared__ __align__(16) uint16_t row_s[];  // [row groups][K][R rows] bf16 bit patterns
     __shared__ float stat_s[kGroupWarps][2 * kGroupRows];
@@ -281,7 +281,7 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
     const int octs = K >> 3, gpr = K >> 4;
     pq::wait_for_prior_grid();
     pq::dependents_may_launch();
-    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldca(ts_ptr));
     float inv[R], mu[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) inv[r] = 0.0f, mu[r] = 0.0f;
@@ -390,13 +390,13 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
                 for (int h = 0; h < POS / 4; ++h) {
                     const int j0 = POS * q + 4 * h;
                     int4 idx = make_int4(j0, j0 + 1, j0 + 2, j0 + 3);
-                    if (perm) idx = __ldg(reinterpret_cast<const int4 *>(perm) + (POS / 4) * q + h);
+                    if (perm) idx = __ldca(reinterpret_cast<const int4 *>(perm) + (POS / 4) * q + h);
                     g[4 * h + 0] = channel_rows<R>(xs, idx.x), g[4 * h + 1] = channel_rows<R>(xs, idx.y);
                     g[4 * h + 2] = channel_rows<R>(xs, idx.z), g[4 * h + 3] = channel_rows<R>(xs, idx.w);
-                    const float4 a4 = __ldg(reinterpret_cast<const float4 *>(a) + (POS / 4) * q + h);
+                    const float4 a4 = __ldca(reinterpret_cast<const float4 *>(a) + (POS / 4) * q + h);
                     w[4 * h + 0] = a4.x, w[4 * h + 1] = a4.y, w[4 * h + 2] = a4.z, w[4 * h + 3] = a4.w;
                     if (KIND == 1) {
-                        const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b) + (POS / 4) * q + h);
+                        const float4 b4 = __ldca(reinterpret_cast<const float4 *>(b) + (POS / 4) * q + h);
                         sh[4 * h + 0] = b4.x, sh[4 * h + 1] = b4.y, sh[4 * h + 2] = b4.z, sh[4 * h + 3] = b4.w;
                     }
                 }
@@ -483,10 +483,10 @@ norm_quant_grouped_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
 // Without a norm: 4608 x 3072 13.1, 18432 x 3072 41.0 (14.4, 49.4 with the sixteen-row kernel of that time).
 template <int KIND, int SF_LAYOUT, int ITER>  // ITER = groups per lane
 __global__ void __maxnreg__(kQuadRegs)
-norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
-                       const float *__restrict__ a, const float *__restrict__ b, float eps,
-                       const int32_t *__restrict__ perm, const int32_t *__restrict__ perm_select,
-                       const float *__restrict__ ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
+norm_quant_quad_kernel(const uint16_t *H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
+                       const float *a, const float *b, float eps,
+                       const int32_t *perm, const int32_t *perm_select,
+                       const float *ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
                        uint16_t *__restrict__ y_out) {
     extern __shared__ __align__(16) uint4 quad_s[];  // [4 rows][K] bf16, then [K][4 rows]
     __shared__ float stat_s[8];                      // inv, mu of the four rows
@@ -499,7 +499,7 @@ norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t row
     // perm_select given: perm is a table of candidate orders [., K] and {best, accept} on the device name the
     // row best - 1, or the original order (the offline weight quantizer, whose decision never visits the host)
     if (perm_select) perm = perm_select[1] ? perm + static_cast<int64_t>(perm_select[0] - 1) * K : nullptr;
-    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldca(ts_ptr));
     const uint16_t *src = H + row0 * ld;
 
     if (KIND == 2) {  // no statistics: straight into the interleaved image
@@ -571,16 +571,16 @@ norm_quant_quad_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t row
             for (int h = 0; h < 4; ++h) {
                 const int j0 = have ? 16 * q + 4 * h : 0;
                 int4 idx = make_int4(j0, j0 + 1, j0 + 2, j0 + 3);
-                if (perm) idx = __ldg(reinterpret_cast<const int4 *>(perm + j0));
+                if (perm) idx = __ldca(reinterpret_cast<const int4 *>(perm + j0));
                 g[4 * h + 0] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.x))];
                 g[4 * h + 1] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.y))];
                 g[4 * h + 2] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.z))];
                 g[4 * h + 3] = quad2[pq::quad_channel(static_cast<uint32_t>(idx.w))];
                 if (KIND != 2) {
-                    float4 a4 = __ldg(reinterpret_cast<const float4 *>(a + j0));
+                    float4 a4 = __ldca(reinterpret_cast<const float4 *>(a + j0));
                     if (KIND == 1) {
                         a4 = make_float4(__fadd_rn(1.0f, a4.x), __fadd_rn(1.0f, a4.y), __fadd_rn(1.0f, a4.z), __fadd_rn(1.0f, a4.w));
-                        const float4 b4 = __ldg(reinterpret_cast<const float4 *>(b + j0));
+                        const float4 b4 = __ldca(reinterpret_cast<const float4 *>(b + j0));
                         sh2[2 * h] = pq::pack2(b4.x, b4.y), sh2[2 * h + 1] = pq::pack2(b4.z, b4.w);
                     }
                     w2[2 * h] = pq::pack2(a4.x, a4.y), w2[2 * h + 1] = pq::pack2(a4.z, a4.w);
@@ -677,11 +677,12 @@ pq_status launch_quad(const uint16_t *H, int64_t rows, int64_t rows_pad, int K, 
 constexpr int kDirectMaxOcts = 16;  // octets per lane: rows of up to 4096 channels
 constexpr int kDirectThreads = 128;
 
+// (RMS norm at eight octets a lane: 72 registers, seven blocks per SM; left alone it takes 80 and 9216 x 1536 13.3 us instead of 12.9)
 template <int KIND, int SF_LAYOUT, int NOCT>  // NOCT = octets per lane the registers are sized for
-__global__ void __launch_bounds__(kDirectThreads)
-norm_quant_ordered_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
-                          const float *__restrict__ a, const float *__restrict__ b, float eps,
-                          const float *__restrict__ ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
+__global__ void __launch_bounds__(kDirectThreads, KIND == 0 && NOCT == 8 ? 7 : 0)
+norm_quant_ordered_kernel(const uint16_t *H, int64_t rows, int64_t rows_pad, int K, int64_t ld,
+                          const float *a, const float *b, float eps,
+                          const float *ts_ptr, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf,
                           uint16_t *__restrict__ y_out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     pq::wait_for_prior_grid();
@@ -690,7 +691,7 @@ norm_quant_ordered_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
     if (row >= rows_pad) return;  // whole warps only
     const bool live = row < rows;
     const int octs = K >> 3, gpr = K >> 4;
-    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldca(ts_ptr));
     uint4 raw[NOCT];
 #pragma unroll
     for (int u = 0; u < NOCT; ++u) {
@@ -744,13 +745,13 @@ norm_quant_ordered_kernel(const uint16_t *__restrict__ H, int64_t rows, int64_t 
             if (live && have) {
                 float x[8];
                 pq::unpack8(raw[u], x);
-                const float4 a0 = __ldg(reinterpret_cast<const float4 *>(a) + 2 * o), a1 = __ldg(reinterpret_cast<const float4 *>(a) + 2 * o + 1);
+                const float4 a0 = *(reinterpret_cast<const float4 *>(a) + 2 * o), a1 = *(reinterpret_cast<const float4 *>(a) + 2 * o + 1);
                 const float w[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
                 if (KIND == 0) {
 #pragma unroll
                     for (int e = 0; e < 8; ++e) out[e] = __fmul_rn(__fmul_rn(x[e], inv), w[e]);
                 } else {
-                    const float4 b0 = __ldg(reinterpret_cast<const float4 *>(b) + 2 * o), b1 = __ldg(reinterpret_cast<const float4 *>(b) + 2 * o + 1);
+                    const float4 b0 = *(reinterpret_cast<const float4 *>(b) + 2 * o), b1 = *(reinterpret_cast<const float4 *>(b) + 2 * o + 1);
                     const float sh[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
                     for (int e = 0; e < 8; ++e)

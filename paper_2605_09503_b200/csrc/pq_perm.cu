@@ -215,7 +215,7 @@ pq_status launch_sort(const SortParams &p, cudaStream_t st) {
 // inside the chain took 22 us for 7 orders of 192 groups.
 constexpr int kAcceptWarps = 16;
 __global__ void __launch_bounds__(32 * kAcceptWarps)
-accept_kernel(const double *__restrict__ ex, const double *__restrict__ ew, const double *__restrict__ lambda, int P, int64_t Kg,
+accept_kernel(const double *ex, const double *ew, const double *lambda, int P, int64_t Kg,
               double tau, int32_t *best, int32_t *accept, double *E_out) {
     __shared__ double sums[2][32], E[32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

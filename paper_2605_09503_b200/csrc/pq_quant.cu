@@ -44,7 +44,7 @@ inline dim3 tile_grid(int64_t col_chunks, int64_t row_blocks) {
 template <bool WIDE>
 __device__ __forceinline__ void load_group(const uint16_t *p, uint4 &lo, uint4 &hi) {
     if (WIDE) {
-        asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                      : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
                      : "l"(p));
     } else {
@@ -61,8 +61,8 @@ constexpr int kActRows = PQ_ACT_ROWS;  // rows per thread: their loads are issue
 // 32 registers per thread (eight 256-thread blocks per SM): all 2048 thread slots of an SM carry a load
 template <int SF_LAYOUT, bool WIDE, int kActTileRows>
 __global__ void __launch_bounds__(kActThreads, 2048 / kActThreads)
-quant_nvfp4_kernel(const uint16_t *__restrict__ X, int64_t rows, int64_t rows_pad, int64_t K,
-                   int64_t ld, const float *__restrict__ ts_ptr, uint8_t *__restrict__ codes,
+quant_nvfp4_kernel(const uint16_t *X, int64_t rows, int64_t rows_pad, int64_t K,
+                   int64_t ld, const float *ts_ptr, uint8_t *__restrict__ codes,
                    uint8_t *__restrict__ sf) {
     const uint32_t gpr = static_cast<uint32_t>(K >> 4);  // groups per row
     const uint32_t g = blockIdx.x * 32u + threadIdx.x;
@@ -81,7 +81,7 @@ quant_nvfp4_kernel(const uint16_t *__restrict__ X, int64_t rows, int64_t rows_pa
         lo[i] = make_uint4(0, 0, 0, 0), hi[i] = lo[i];
         if (row < rows && g < gpr) load_group<WIDE>(X + row * ld + static_cast<int64_t>(g) * 16, lo[i], hi[i]);
     }
-    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldg(ts_ptr));
+    const pq::Nvfp4Scaler scaler = pq::nvfp4_scaler(__ldca(ts_ptr));
     auto quantize = [&](auto fast) {
 #pragma unroll
         for (int i = 0; i < kActRows; ++i) {

@@ -199,7 +199,7 @@ __global__ void tensor_scale_kernel(const float *__restrict__ amax, int64_t K, f
 }
 
 // lambda[s] = 1 / (sequential fp64 sum of side s in ascending channel order), one warp per side.
-__global__ void __launch_bounds__(64) error_weights_kernel(const double *__restrict__ sa, const double *__restrict__ sw,
+__global__ void __launch_bounds__(64) error_weights_kernel(const double *sa, const double *sw,
                                                            int64_t K, double *lambda) {
     pq::dependents_may_launch();
     pq::wait_for_prior_grid();

@@ -339,9 +339,9 @@ struct GatherParams {
     const float *ts[2];        // tensor scale per side (NVFP4)
     int K, P, identity;        // P orders; identity != 0: order 0 is the original one and perms holds the others
     const int32_t *perms;      // [P - identity, K]
-    int opb;                   // orders per block (blockIdx.y picks the subset)
+    int opb;                   // orders per block, a subset of them
     int groups, group_threads;
-    int blocks;                // per subset of the orders; behind them one for the error weights, if they are asked for
+    int blocks;                // per subset of the orders; behind all of them one for the error weights, if they are asked for
     uint32_t base[2], rem[2];  // pairs of the first `split` chunks / shares and its remainder: subsets of opb orders, the last
     uint32_t split;
     int full;                  // whole chunks per share behind them
@@ -372,7 +372,8 @@ __global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __
     // [groups][K][4 rows] bf16 magnitudes | [opb][K] 16-bit slots | scale tables | [groups][opb][runs] fp32 chunk sums
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = p.K, octs = K >> 3, runs = K >> 4;
-    const int o0 = blockIdx.y * p.opb, no = min(p.opb, p.P - o0);
+    const uint32_t subset = blockIdx.x / static_cast<uint32_t>(p.blocks), block = blockIdx.x - subset * p.blocks;
+    const int o0 = static_cast<int>(subset) * p.opb, no = min(p.opb, p.P - o0);
     uint16_t *slot_s = reinterpret_cast<uint16_t *>(smem + static_cast<size_t>(p.groups) * K * 8);
     unsigned char *tab_s = reinterpret_cast<unsigned char *>(slot_s + static_cast<size_t>(p.opb) * K);
     uint2 *int_tab = reinterpret_cast<uint2 *>(tab_s);
@@ -380,8 +381,8 @@ __global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __
     pq::dependents_may_launch();
     pq::wait_for_prior_grid();
 
-    if (blockIdx.x == static_cast<unsigned>(p.blocks)) {  // the block of the error weights: a warp per side
-        for (int s = threadIdx.x >> 5; blockIdx.y == 0 && s < 2; s += blockDim.x >> 5) {
+    if (o0 >= p.P) {  // the block of the error weights: a warp per side
+        for (int s = threadIdx.x >> 5; s < 2; s += blockDim.x >> 5) {
             const double sum = pq::ordered_sum(s ? p.weights.sumsq_w : p.weights.sumsq_a, K);
             if ((threadIdx.x & 31) == 0) p.weights.lambda[s] = __ddiv_rn(1.0, sum);
         }
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __
     // part a group that has work for a few chunks only would wait for the one that has a whole chunk more; without the
     // second a group would stage one more chunk of which it uses some orders (eight batches of 4608 x 3072 and a
     // 9216 x 3072 weight: 535 us a calibration all in pairs, 518 like this; 473 with the present fold).
-    const uint32_t shares = p.blocks * p.groups, share = blockIdx.x * p.groups + grp;
+    const uint32_t shares = p.blocks * p.groups, share = block * p.groups + grp;
     const uint32_t base = p.base[o0 + no == p.P], rem = p.rem[o0 + no == p.P];
     const uint32_t first = share * base + min(share, rem);
     int pairs = static_cast<int>(base + (share < rem)), full = p.full * no;
@@ -686,7 +687,7 @@ pq_status launch_gather(GatherParams &p, int64_t K, int P, float Qf, float *part
     auto kern = group_error_gather<KIND, TEAM / 2>;
     PQ_CUDA_OK(pq::allow_smem(kern, smem, kGatherSmemMax));
     p.blocks = static_cast<int>(blocks);
-    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks + weights), static_cast<unsigned>(subsets)),
+    PQ_CUDA_OK(pq::launch_dependent(kern, dim3(static_cast<unsigned>(blocks * subsets + weights)),
                                     dim3(static_cast<unsigned>(cfg.groups * cfg.group_threads)), smem, st, p));
     return pq_launch_status();
 }

@@ -41,9 +41,11 @@
 //     the whole warp, with the warp index from a shuffle so that the branch is known to be uniform, and single out one
 //     lane with elect.sync around those instructions.  Predicated instructions instead of that branch: 56.1 / 67.6 / 283;
 //   - all copies of a stage in front of its MMAs: 512 x 3072 x 3072 6.6, copies and MMAs in turn 6.9;
-//   - a remote mbarrier arrive with cluster-scope release semantics costs 500 to 2500 cycles;
-//     what the arrivals here publish has already completed (tcgen05.wait) when they are issued,
-//     so the default semantics are used.
+//   - a remote mbarrier arrive with cluster-scope release semantics costs 500 to 2500 cycles.  The only remote arrives here hand
+//     the accumulator back, whose reads have completed (tcgen05.wait::ld) when they are issued, so they have the default semantics;
+//   - the narrow tile's scales by plain bulk copies, which report to their own CTA, so that the other CTA has to pass them on to the
+//     leader: by an arrive with default semantics 1 % slower (512 x 3072 x 3072 6.61 us, 6.57 by the pair's tensor loads) and of CTA
+//     scope only; by release and acquire of the cluster, which is what it takes, 9.96.
 //
 // Scale factors live in global memory in 512-byte blocks of 128 rows x 4 groups (see pq.h); a
 // block occupies 4 tensor-memory columns (row r of the block -> lane r%32, column r/32, the same
@@ -102,7 +104,7 @@ struct Tile {
     static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;  // 38 or 28 * 1024
     static constexpr uint32_t kSfSlotCol0 = BN, kSfbColsPerKb = 4 * kNB, kSfbOfs = 16;
     static constexpr uint32_t kSfSlotCols = 4 * (4 + kSfbColsPerKb);   // 48 or 32
-    static constexpr int kNumBars = (kOneTile ? 3 : 2) * kStages + 2;  // stage_full[S] stage_free[S] acc_full acc_empty, narrow: sf_ready[S]
+    static constexpr int kNumBars = 2 * kStages + 2;      // stage_full[S] stage_free[S] acc_full acc_empty
     static constexpr int kRingBytes = kStages * kStageBytes, kEpi = kOneTile ? 0 : kRingBytes;  // where the boxes start
     static constexpr size_t kSmemBytes = kRingBytes + (kOneTile ? 0 : kEpiBytes) + 1024 /*alignment slack*/ + 8 * kNumBars + 64;
     // Instruction descriptor: E2M1 x E2M1, UE4M3 scales, both K-major, M = 256 (pair), N = BN, K = 64.
@@ -113,20 +115,11 @@ struct Tile {
     static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 };
 
-// What the kernel reads its operands by.  The wide tile's scale blocks come by tensor maps, too; the narrow tile's as plain bulk
-// copies of just the blocks a K step has: no two more descriptors to fetch at the start of a short kernel (quantize + GEMM of
-// 512 x 3072 x 3072 8.7 us against 9.2 with maps; on the wide tile not tried).
-template <int BN>
 struct Maps {
     CUtensorMap a, b, y, sfa, sfb;
 };
-template <>
-struct Maps<128> {
-    CUtensorMap a, b, y;
-};
 
 struct GemmParams {
-    const uint8_t *sfx, *sfw;  // narrow tile
     const float *ts_x, *ts_w;
     int M, N;
     int m_tiles, n_tiles, k_tiles, kb_total;
@@ -229,7 +222,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
     return mbar_wait_slow(bar, parity, w);
 }
 // Wait of a converged warp: every lane returns the same answer and the warp is converged again
-// afterwards, so .sync.aligned instructions (elect, tcgen05.st / ld) may follow on either outcome.
+// afterwards, so .sync.aligned instructions (elect, tcgen05.ld) may follow on either outcome.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx w) {
     bool ok = mbar_try(bar, parity);
     if (__all_sync(0xFFFFFFFFu, ok)) return true;
@@ -247,11 +240,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar_cluster)
         : "memory");
-}
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
 }
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int x, int y, uint32_t src) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
@@ -346,7 +334,7 @@ __device__ __forceinline__ uint32_t pack_bf16(uint32_t lo_bits, uint32_t hi_bits
 constexpr int kMaxRegs = 128;
 template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(kMaxRegs)
-gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
+gemm_w4a4_kernel(const __grid_constant__ Maps maps, const GemmParams p) {
     using T = Tile<BN>;
     constexpr int kStages = T::kStages, kNB = T::kNB, BN_CTA = T::kNCta;
     constexpr int kBBytes = T::kBBytes, kStageBytes = T::kStageBytes, kNumBars = T::kNumBars;
@@ -359,13 +347,11 @@ gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
     const uint32_t epi = base + T::kEpi;
     const uint32_t bars = base + kBarOfs;
     uint8_t *bars_ptr = base_ptr + kBarOfs;
-    // stage_full: operand and scale bytes of both CTAs have landed; leader's copy only.  Wide: 1 arrival + transaction bytes.  Narrow:
-    // a bulk copy reports to its own CTA, so the other CTA's scales report to its sf_ready, and its warp 1 passes that on (2 arrivals).
+    // stage_full: operand and scale bytes of both CTAs have landed (1 arrival + transaction bytes); leader's copy only
     auto stage_full_bar = [&](int s) { return bars + 8u * s; };
-        auto stage_free_bar = [&](int s) { return bars + 8u * (kStages + s); };  // the stage's MMAs have run
+    auto stage_free_bar = [&](int s) { return bars + 8u * (kStages + s); };  // the stage's MMAs have run
     const uint32_t acc_full_bar = bars + 8u * (2 * kStages);       // one copy per CTA, both signalled by the issuer
     const uint32_t acc_empty_bar = bars + 8u * (2 * kStages + 1);  // leader's copy only
-    auto sf_ready_bar = [&](int s) { return bars + 8u * (2 * kStages + 2 + s); };  // narrow tile
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars_ptr + 8 * kNumBars);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_ptr + 8 * kNumBars + 8);
     const WaitCtx wctx{abort_flag, p.status, p.wait_cycles};
@@ -377,8 +363,7 @@ gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(stage_full_bar(s), T::kOneTile ? 2 : 1);
-            if (T::kOneTile) mbar_init(sf_ready_bar(s), 1);
+            mbar_init(stage_full_bar(s), 1);
             mbar_init(stage_free_bar(s), 1);
         }
         mbar_init(acc_full_bar, 1);
@@ -387,7 +372,8 @@ gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         prefetch_tensormap(&maps.a);
         prefetch_tensormap(&maps.b);
-        if constexpr (!T::kOneTile) prefetch_tensormap(&maps.sfa), prefetch_tensormap(&maps.sfb);
+        prefetch_tensormap(&maps.sfa);
+        prefetch_tensormap(&maps.sfb);
         prefetch_tensormap(&maps.y);
     }
     if (warp == 1) {
@@ -428,30 +414,20 @@ gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
                 const uint32_t sf_stage = stage + kABytes + kBBytes;
                 const uint32_t full_leader = mapa(stage_full_bar(s), 0);
                 if (elect_one()) {
-                    if constexpr (T::kOneTile) {
-                        // the other CTA's rows may lie past the last block of rows: any block will do for them
-                        const uint32_t sf_bytes = static_cast<uint32_t>(min(4, p.kb_total - kt * 4)) * kSfBlock;
-                        const int64_t kofs = static_cast<int64_t>(kt) * 4 * kSfBlock, pitch = static_cast<int64_t>(p.kb_total) * kSfBlock;
-                        const uint32_t sf_bar = rank == 0 ? stage_full_bar(s) : sf_ready_bar(s);
-                        mbar_expect_tx(sf_bar, 2u * sf_bytes + (rank == 0 ? 2u * (kABytes + kBBytes) : 0u));
-                        bulk_load(sf_stage, p.sfx + min(m0 >> 7, (p.M - 1) >> 7) * pitch + kofs, sf_bytes, sf_bar);
-                        bulk_load(sf_stage + kSfaBytes, p.sfw + (n0 >> 7) * pitch + kofs, sf_bytes, sf_bar);
-                    } else {
-                        if (rank == 0) mbar_expect_tx(stage_full_bar(s), 2u * kStageBytes);
-                        tma_load_2d_pair(sf_stage, &maps.sfa, kt * (4 * kSfBlock / 8), m0 >> 7, full_leader);
-                        tma_load_2d_pair(sf_stage + kSfaBytes, &maps.sfb, kt * (4 * kSfBlock / 8), n0 >> 7, full_leader);
-                    }
+                    if (rank == 0) mbar_expect_tx(stage_full_bar(s), 2u * kStageBytes);
+                    tma_load_2d_pair(sf_stage, &maps.sfa, kt * (4 * kSfBlock / 8), m0 >> 7, full_leader);
+                    tma_load_2d_pair(sf_stage + kSfaBytes, &maps.sfb, kt * (4 * kSfBlock / 8), n0 >> 7, full_leader);
                     tma_load_2d_pair(stage, &maps.a, kt * (BK / 2), m0, full_leader);
                     tma_load_2d_pair(stage + kABytes, &maps.b, kt * (BK / 2), n0 + static_cast<int>(rank) * BN_CTA, full_leader);
                 }
                 __syncwarp();
             }
         }
-        if (!ok && lane == 0 && (rank == 0 || T::kOneTile)) {
+        if (!ok && lane == 0 && rank == 0) {
             // give the copies already issued (they count on these barriers) a bounded chance to land before leaving
             const uint32_t first = it > kStages ? it - kStages : 0;
             for (uint32_t j = first; j < it; ++j)
-                for (uint32_t i = 0; i < 4096 && !mbar_try(rank == 0 ? stage_full_bar(j % kStages) : sf_ready_bar(j % kStages), (j / kStages) & 1u); ++i) {}
+                for (uint32_t i = 0; i < 4096 && !mbar_try(stage_full_bar(j % kStages), (j / kStages) & 1u); ++i) {}
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -502,13 +478,6 @@ gemm_w4a4_kernel(const __grid_constant__ Maps<BN> maps, const GemmParams p) {
                     s = (s + 1 == kStages) ? 0u : s + 1;
                     ph ^= (s == 0) ? 1u : 0u;
                 }
-            }
-        } else if (T::kOneTile) {
-            // the other CTA: its scales have landed
-            bool ok = true;
-            for (int kt = 0; kt < p.k_tiles && ok; ++kt) {
-                ok = mbar_wait_warp(sf_ready_bar(kt % kStages), static_cast<uint32_t>(kt / kStages) & 1u, wctx);
-                if (ok && lane == 0) mbar_arrive_remote(stage_full_bar(kt % kStages), 0);
             }
         }
     } else {
@@ -643,7 +612,7 @@ bool encode_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t row_byt
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// What the maps of an operand (ld = 0: codes and, unless sf is NULL, scale blocks; rows x K) or of the output (rows x K, ld) depend on.
+// What the maps of an operand (ld = 0: codes and scale blocks; rows x K) or of the output (rows x K, ld) depend on.
 struct MapKey {
     const void *ptr, *sf;
     int64_t rows, K, ld;
@@ -685,7 +654,7 @@ const MapSlot *find_maps(const MapKey &key) {
     } else {
         const int64_t sf_pitch = key.K / 64 * kSfBlock;
         slot.used = encode_map(&slot.map, key.ptr, key.rows, key.K / 2, key.K / 2, key.box_rows, 1) &&
-                    (!key.sf || encode_map(&slot.scales, key.sf, pq_ceil_div(key.rows, 128), sf_pitch, sf_pitch, key.sf_box_rows, 8));
+                    encode_map(&slot.scales, key.sf, pq_ceil_div(key.rows, 128), sf_pitch, sf_pitch, key.sf_box_rows, 8);
     }
     return slot.used ? &slot : nullptr;
 }
@@ -735,7 +704,7 @@ struct GemmArgs {
 
 template <int BN>
 pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
-    Maps<BN> maps;
+    Maps maps;
     // copied one by one: a later entry may take an earlier one's slot
     auto find = [&](CUtensorMap &map, CUtensorMap *scales, const MapKey &key) {
         const MapSlot *slot = find_maps(key);
@@ -744,17 +713,12 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
         if (scales) *scales = slot->scales;
         return true;
     };
-    bool found = find(maps.y, nullptr, MapKey{g.Y, nullptr, g.M, g.N, g.ldy, 32, 0});
-    if constexpr (Tile<BN>::kOneTile) {
-        found = found && find(maps.a, nullptr, MapKey{g.xq, nullptr, g.M, g.K, 0, BM_CTA, 0}) &&
-                find(maps.b, nullptr, MapKey{g.wq, nullptr, g.N, g.K, 0, Tile<BN>::kNCta, 0});
-    } else {
-        found = found && find(maps.a, &maps.sfa, MapKey{g.xq, g.sfx, g.M, g.K, 0, BM_CTA, 1}) &&
-                find(maps.b, &maps.sfb, MapKey{g.wq, g.sfw, g.N, g.K, 0, Tile<BN>::kNCta, Tile<BN>::kNB});
-    }
+    const bool found = find(maps.y, nullptr, MapKey{g.Y, nullptr, g.M, g.N, g.ldy, 32, 0}) &&
+                       find(maps.a, &maps.sfa, MapKey{g.xq, g.sfx, g.M, g.K, 0, BM_CTA, 1}) &&
+                       find(maps.b, &maps.sfb, MapKey{g.wq, g.sfw, g.N, g.K, 0, Tile<BN>::kNCta, Tile<BN>::kNB});
     if (!found) return PQ_ERR_CUDA;
     GemmParams p;
-    p.sfx = g.sfx, p.sfw = g.sfw, p.ts_x = g.ts_x, p.ts_w = g.ts_w;
+    p.ts_x = g.ts_x, p.ts_w = g.ts_w;
     p.M = static_cast<int>(g.M), p.N = static_cast<int>(g.N);
     p.m_tiles = static_cast<int>(pq_ceil_div(g.M, BM));
     p.n_tiles = static_cast<int>(pq_ceil_div(g.N, BN));

@@ -77,7 +77,8 @@ def test_streaming_entry_points_repeat_bit_for_bit():
     assert _repeat(lambda: B.pq_output_error(yref, yq, eo, wso), [eo]) == 0
 
 
-@pytest.mark.parametrize("m,k,n", [(4608, 12288, 3072), (1000, 3072, 3080)])
+@pytest.mark.parametrize("m,k,n", [(4608, 12288, 3072), (1000, 3072, 3080),                 # wide tiles
+                                   (512, 3072, 3072), (300, 1088, 4736), (100, 12288, 1288)])  # narrow ones
 def test_linear_repeats_bit_for_bit_on_long_and_ragged_shapes(m, k, n):
     g = torch.Generator(device=DEV)
     g.manual_seed(m + n)

@@ -182,10 +182,10 @@ group_error_direct(const uint16_t *__restrict__ T, int64_t rows, int64_t K, int6
 // Blocks are persistent, one per SM; the groups of a block only share the slot and scale tables.
 //
 // NVFP4 is scalar arithmetic but for the sums: packed f32x2 instructions save issue slots but run on one of the two FMA pipes only, and
-// with the f16 converts there too it was 59 % busy (9216 x 3072, six orders, with the fold of that time: 79 us scalar, 84
-// packed; 74 with the present fold); only the sums of squares are packed, which leaves that pipe room (9216 x 3072 72.9 -> 71.6, 4608 x
-// 12288 197.6 -> 194.7; the multiplication packed 81.2, the residual 74.6).  The integer formats, without converts, are packed (4608 x 3072, INT4 g64: 53.4 us,
-// 54.1 scalar; 50.1 with the present fold).
+// with the f16 converts there too it was 59 % busy (9216 x 3072, six orders, with an earlier fold: 79 us scalar, 84
+// packed); only the sums of squares are packed, which leaves that pipe room (9216 x 3072 72.9 -> 71.6, 4608 x
+// 12288 197.6 -> 194.7; the multiplication packed 81.2, the residual 74.6).  The integer formats, without converts, are packed (4608 x 3072,
+// INT4 g64, with that fold: 53.4 us, 54.1 scalar).
 // What bounds it: instruction issue (67 % of the slots busy at 23 warps per SM) and shared-memory wavefronts (a 64-bit gather
 // through a random order takes about 6 of them where 2 would do: 0.069 per element and order).
 // Registers: 80 per thread, of which 36 to 56 bytes are spilled.  The weights of the acceptance rule, two chains of K additions, have a
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) group_error_gather(const __
     // An equal part of the (chunk, order) pairs of the first p.split chunks, then p.full whole chunks.  Without the first
     // part a group that has work for a few chunks only would wait for the one that has a whole chunk more; without the
     // second a group would stage one more chunk of which it uses some orders (eight batches of 4608 x 3072 and a
-    // 9216 x 3072 weight: 535 us a calibration all in pairs, 518 like this; 473 with the present fold).
+    // 9216 x 3072 weight, with an earlier fold: 535 us a calibration all in pairs, 518 like this).
     const uint32_t shares = p.blocks * p.groups, share = block * p.groups + grp;
     const uint32_t base = p.base[o0 + no == p.P], rem = p.rem[o0 + no == p.P];
     const uint32_t first = share * base + min(share, rem);

@@ -27,6 +27,8 @@ def test_few_rows_at_the_line(M, N, K):
     test_exact_at_the_line(M, N, K)
 
 
-@pytest.mark.parametrize("M,N,K", [(2200, 2440, 64), (4700, 1288, 320), (1025, 8200, 576)])   # two and three rounds of wide tiles;
-def test_rounds_at_ragged_edges(M, N, K):           # 1 to 4 blocks of channels in the last K step, a last row block of either
-    test_exact_at_the_line(M, N, K)                 # operand that is the second of its tile or past the end
+# Two and three rounds of wide tiles; 1, 2, 3 and 4 blocks of 64 channels in the last K step; six K steps, so that the ring of five stages
+# (and the scale slots) wraps inside a tile; a last row block of either operand that is the second of its tile or past the end.
+@pytest.mark.parametrize("M,N,K", [(2200, 2440, 64), (4700, 1288, 384), (1025, 8200, 704), (2200, 2440, 512), (1100, 4744, 1472)])
+def test_rounds_at_ragged_edges(M, N, K):
+    test_exact_at_the_line(M, N, K)

@@ -88,6 +88,15 @@ def hadamard(K):
     return producer(K, 9, lambda x, perm, a, ts, codes, sf: B.pq_hadamard_quant_nvfp4(x, perm, ts, codes, sf, B.PQ_SF_TCGEN05))
 
 
+def linear(M, K, N):
+    x, w = matrix(M, K, 8), matrix(N, K, 9)
+    wq, sfw = torch.empty(N, K // 2, dtype=torch.uint8, device=DEV), torch.empty(B.sf_bytes(N, K, B.PQ_SF_TCGEN05), dtype=torch.uint8, device=DEV)
+    ts = torch.empty(1, device=DEV)
+    B.pq_quant_weight(w, None, None, wq, sfw, B.PQ_SF_TCGEN05, ts, B.workspace(B.OP_QUANT_WEIGHT, N, K))
+    layer = pipeline.QuantLinear(wq, sfw, ts, torch.full((1,), 0.01, device=DEV), M)
+    return lambda: (layer(x),)
+
+
 PAIRS = {
     "calibrate": lambda: (calibrate(3072, pipeline.NVFP4), calibrate(12288, pipeline.NVFP4)),
     "calibrate_int": lambda: (calibrate(1024, INT4_G64), calibrate(8192, INT4_G64)),
@@ -99,6 +108,7 @@ PAIRS = {
     "norm_group": lambda: (norm(2048, 2400), norm(3072, 2400)),
     "norm_wide": lambda: (norm(20480, 9), norm(32768, 9)),
     "hadamard": lambda: (hadamard(8192), hadamard(16384)),
+    "linear": lambda: (linear(200, 512, 520), linear(520, 1088, 9480)),   # narrow and wide tiles: maps found per thread
 }
 
 

@@ -749,13 +749,19 @@ pq_status launch_tiles(const GemmArgs &g, int pairs_max) {
 
 // One round of narrow tiles covers the product.  Measured on both sides of the line (M x N x K, narrow against wide, us):
 // 128 x 3072 x 3072 6.2 / 7.6, 512 x 3072 x 3072 6.6 / 7.7, 512 x 3072 x 12288 16.1 / 19.3, 512 x 4736 x 3072 7.3 / 8.1; beyond one
-// round the wide tile wins (512 x 9216 x 3072 12.2 / 10.9, 1024 x 3072 x 3072 11.2 / 9.4 before the scales came by tcgen05.cp).
+// round, in a second wave of CTAs, the narrow tile loses by a third and more (512 x 4744 x 3072 12.0 / 8.2, 512 x 9216 x 3072 14.2 / 9.2,
+// 1357 x 4744 x 1088 18.3 / 7.9, 2048 x 3072 x 12288 47.4 / 34.5).
 // Few rows: the CTAs of all pairs fetch the same few lines of X at every K step, and with more than half of the pairs at that the
-// narrow tile loses up to 16 rows (1 x 5120 x 3072 8.4 / 6.8, 4 x 9216 x 3072 7.7 / 7.1, 8 x 5120 x 3072 7.0 / 6.7, 2 x 7168 x 12288
-// 22.8 / 21.2, 16 x 9216 x 12288 22.2 / 21.4; 24 x 9216 x 12288 16.0 / 19.6).
-bool narrow_tiles(int64_t M, int64_t N, int pairs) {
-    const int64_t tiles = pq_ceil_div(M, BM) * pq_ceil_div(N, 128);
-    return tiles <= (M <= 16 ? pairs / 2 : pairs);
+// narrow tile loses up to 16 rows (1 x 5120 x 3072 8.4 / 6.8, 4 x 9216 x 3072 7.7 / 7.1, 2 x 7168 x 12288 22.8 / 21.2, 16 x 9216 x 12288
+// 22.2 / 21.4; 24 x 9216 x 12288 16.0 / 19.6).  It does so the later the fewer K steps there are and the more rows, as long as the rows of codes
+// start on 128-byte lines: 3 to 16 rows of 256, 512 or 768 channels keep it up to two thirds of the pairs (wide 1.00 to 1.16 x the narrow
+// time at 38 to 49 tiles), 8 to 16 rows of 1024 to 2048 for one tile more than half (wide 1.03 to 1.15 x; at 40 tiles 0.95 to 1.1 x).  Other
+// row lengths do not (3 x 5120 x 960 5.2 narrow, 4.4 wide).
+bool narrow_tiles(int64_t M, int64_t N, int64_t K, int pairs) {
+    int most = pairs;
+    if (M <= 2 || (M <= 16 && K > 3072)) most = pairs / 2;
+    else if (M <= 16) most = K % 256 ? pairs / 2 : K < 1024 ? pairs * 2 / 3 : pairs / 2 + (M >= 8 && K <= 2048 ? 1 : 0);
+    return pq_ceil_div(M, BM) * pq_ceil_div(N, 128) <= most;
 }
 
 pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, const uint8_t *wq, const uint8_t *sfw,
@@ -774,7 +780,7 @@ pq_status gemm_launch(const uint8_t *xq, const uint8_t *sfx, const float *ts_x, 
     const int dev = pq_device_slot(), pairs_max = resident_pairs<256>(dev), pairs_narrow = resident_pairs<128>(dev);
     if (pairs_max <= 0 || pairs_narrow <= 0) return PQ_ERR_CUDA;
     const GemmArgs g{xq, sfx, wq, sfw, ts_x, ts_w, M, N, K, ldy, Y, ws, st};
-    return narrow_tiles(M, N, pairs_narrow) ? launch_tiles<128>(g, pairs_narrow) : launch_tiles<256>(g, pairs_max);
+    return narrow_tiles(M, N, K, pairs_narrow) ? launch_tiles<128>(g, pairs_narrow) : launch_tiles<256>(g, pairs_max);
 }
 }  // namespace
 

@@ -22,7 +22,8 @@ def test_exact_at_the_line(M, N, K):
     assert np.array_equal(Y, bf16_round(O.gemm_ref(pack(xn), sfx, 0.5, pack(wn), sfw, 4.0)))
 
 
-@pytest.mark.parametrize("M,N,K", [(2, 4736, 128), (2, 4744, 320), (3, 4744, 128), (1, 9472, 192), (16, 4744, 3136), (17, 4744, 3136)])   # 37 and 38 narrow tiles, few rows
+@pytest.mark.parametrize("M,N,K", [(2, 4736, 128), (2, 4744, 320), (3, 4744, 128), (1, 9472, 192), (16, 4744, 3136), (17, 4744, 3136),    # 37 and 38 narrow tiles, few rows
+                                   (8, 4864, 1280), (8, 4872, 1280), (7, 4744, 1088), (16, 6272, 768), (3, 6280, 768)])    # 38 and 39; 49 and 50
 def test_few_rows_at_the_line(M, N, K):
     test_exact_at_the_line(M, N, K)
 
